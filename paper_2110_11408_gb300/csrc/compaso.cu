@@ -1,8 +1,11 @@
-// CompaSO levels (Sec. 2.2.2): one thread block per group runs the nucleus
-// loop of steps 1-4 over the group's members in key order (Sigma desc, id asc).
+// CompaSO levels (Sec. 2.2.2): the nucleus loop of steps 1-4 inside every
+// group.  The nuclei come from the group's density peaks (peaks.cu), found
+// beforehand by the whole GPU: the loop takes the peak first in key order
+// (Sigma desc, id asc) among those still eligible until none is left.  The
+// members of a group lie in cell order.
 //
 // Per nucleus:
-//   pass A  squared distances d_j of all members to the nucleus;
+//   pass A  squared distances d_j of the members to the nucleus;
 //   select  R^2 = the smallest member distance d with n(<d)^2 u^6 < K d^3
 //           (exact), found without a full sort: a 1024-bin histogram over a
 //           window of d (first window binned by the threshold count
@@ -11,11 +14,20 @@
 //           sorted in shared memory and scanned, or narrowed further when it
 //           holds more than 2048 members; small groups are sorted whole;
 //   pass B  tentative membership / competitive reassignment (Eq. 3) and
-//           eligibility marking.
+//           eligibility of the peaks left.
+//
+// Groups above small_n (2,048) members are walked in tiles of 128 members,
+// which are neighbours in space.  Where a group has several peaks, every tile
+// has a bounding box, and a nucleus' passes visit only the tiles its radius
+// can reach: the members of all tiles whose box is nearer than r are at least
+// n(<r), so the first r (two steps an octave of r^2) at which that count is
+// below the threshold density bounds the search, and R^2 bounds pass B.
 #include <cooperative_groups.h>
 #include <atomic>
 #include <float.h>
 #include <limits.h>
+
+#include <algorithm>
 
 #include "cells.cuh"
 #include "compaso.cuh"
@@ -212,7 +224,6 @@ __device__ __forceinline__ int first_bin(unsigned long long d, const PredConst& 
   return g < (float)(nb - 1) ? (int)g : nb - 1;
 }
 
-// R^2 of nucleus pc over the n members at epos[0..n); distances left in ed.
 // The bin's smallest and largest distance.  A bound read without the atomic
 // can only be stale in the safe direction (the minimum only falls, the
 // maximum only rises), so a member that does not beat it is skipped: per bin
@@ -232,9 +243,133 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
   return v;
 }
 
+// ---------------------------------------------------------------------------
+// tiles of a group: TILE consecutive members, their bounding boxes and the
+// passes over the tiles within reach of a nucleus
+// ---------------------------------------------------------------------------
+constexpr int TILE = 128;
+constexpr int LEVELS = 88;  // squared radii tried for the search bound: two per octave up to 2^43
+
+__device__ __forceinline__ int fold21(int v) { return (int)((unsigned)v << 11) >> 11; }  // nearest image
+
+// squared radius at the lower edge of level k, and the level of d
+__device__ __forceinline__ unsigned long long level_edge(int k) {
+  return k < 2 ? (unsigned long long)k : (k & 1 ? 3ull << (k / 2 - 1) : 1ull << (k / 2));
+}
+__device__ __forceinline__ int level_of(unsigned long long d) {
+  if (d < 2) return (int)d;
+  const int m = 63 - __clzll((long long)d);
+  return 2 * m + (int)((d >> (m - 1)) & 1);
+}
+
+// The tiles a CTA owns: rank, rank + cs, ... of the group's nt (cs = 1 for a block).
+struct Tiles {
+  int nt, rank, cs;
+  const int4* lo;  // boxes of the group's tiles, offsets from the group's first member; null: none
+  const int4* hi;
+  int4 q;          // the nucleus in those offsets
+  __device__ __forceinline__ int own() const { return nt > rank ? (nt - rank + cs - 1) / cs : 0; }
+};
+
+__device__ __forceinline__ unsigned long long axis_gap2(int q, int lo, int hi) {
+  // over the three images of the box's interval, which is shorter than a box side
+  int g = max(max(lo - q, q - hi), 0);
+  g = min(g, max(max(lo + CSO_BOX - q, q - hi - CSO_BOX), 0));
+  g = min(g, max(max(lo - CSO_BOX - q, q - hi + CSO_BOX), 0));
+  return (unsigned long long)g * (unsigned long long)g;
+}
+
+// squared distance from the nucleus to tile t's box: no member of it is nearer
+__device__ __forceinline__ unsigned long long tile_gap2(const Tiles& T, int t) {
+  const int4 a = T.lo[t], b = T.hi[t];
+  return axis_gap2(T.q.x, a.x, b.x) + axis_gap2(T.q.y, a.y, b.y) + axis_gap2(T.q.z, a.z, b.z);
+}
+
+// f(j) for every member j < n of the CTA's tiles nearer than lim (0: of all
+// its tiles).  Warps take chunks of up to 32 tiles that lie a whole chunk
+// count apart, so that the tiles in reach, neighbours of one another, spread
+// over the warps.
+template <class F>
+__device__ __forceinline__ void for_members(const Tiles& T, int n, unsigned long long lim, F f) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int own = T.own();
+  const int per = min(32, (own + nw - 1) / nw);
+  const int nchunk = per > 0 ? (own + per - 1) / per : 0;
+  for (int c = threadIdx.x >> 5; c < nchunk; c += nw) {
+    const int i = lane * nchunk + c;
+    const bool act = lane < per && i < own && (!lim || tile_gap2(T, T.rank + i * T.cs) < lim);
+    for (unsigned m = __ballot_sync(0xffffffffu, act); m; m &= m - 1) {
+      const int t = T.rank + ((__ffs(m) - 1) * nchunk + c) * T.cs;
+#pragma unroll
+      for (int k = 0; k < TILE / 32; ++k) {
+        const int j = t * TILE + k * 32 + lane;
+        if (j < n) f(j);
+      }
+    }
+  }
+}
+
+// boxes of the CTA's own tiles, a warp per tile
+__device__ void tile_boxes(const Tiles& T, const int4* __restrict__ epos, int n, int4* lo, int4* hi) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int4 ref = epos[0];
+  for (int i = threadIdx.x >> 5; i < T.own(); i += nw) {
+    const int t = T.rank + i * T.cs;
+    int a[3] = {INT_MAX, INT_MAX, INT_MAX}, b[3] = {INT_MIN, INT_MIN, INT_MIN};
+#pragma unroll
+    for (int k = 0; k < TILE / 32; ++k) {
+      const int j = t * TILE + k * 32 + lane;
+      if (j >= n) continue;
+      const int4 p = epos[j];
+      const int o[3] = {fold21(p.x - ref.x), fold21(p.y - ref.y), fold21(p.z - ref.z)};
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        a[x] = min(a[x], o[x]);
+        b[x] = max(b[x], o[x]);
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      a[x] = __reduce_min_sync(0xffffffffu, a[x]);
+      b[x] = __reduce_max_sync(0xffffffffu, b[x]);
+    }
+    if (lane == 0) {
+      lo[t] = make_int4(a[0], a[1], a[2], 0);
+      hi[t] = make_int4(b[0], b[1], b[2], 0);
+    }
+  }
+}
+
+// The squared radius that bounds the nucleus' search: the first level edge e
+// at which the members of all tiles nearer than e are below the threshold
+// density (then so are the members nearer than e, and R^2 is the smallest
+// member distance below e that qualifies, or the first one past it); 0 if
+// there is none.  Every thread of the block calls it; h: LEVELS counters.
+__device__ unsigned long long search_bound(const Tiles& T, int n, const PredConst& c, unsigned* h, int* best) {
+  for (int k = threadIdx.x; k < LEVELS; k += blockDim.x) h[k] = 0;
+  if (threadIdx.x == 0) *best = LEVELS;
+  __syncthreads();
+  for (int t = threadIdx.x; t < T.nt; t += blockDim.x)
+    atomicAdd(&h[min(level_of(tile_gap2(T, t)), LEVELS - 1)], (unsigned)min(TILE, n - t * TILE));
+  __syncthreads();
+  for (int k = 1 + threadIdx.x; k < LEVELS; k += blockDim.x) {
+    unsigned long long cnt = 0;
+    for (int q = 0; q < k; ++q) cnt += h[q];
+    if (pred(cnt, level_edge(k), c)) atomicMin(best, k);
+  }
+  __syncthreads();
+  const int k = *best;
+  __syncthreads();
+  return k < LEVELS ? level_edge(k) : 0;
+}
+
+// R^2 of nucleus pc over the n members at epos[0..n); the distances of the
+// members the search visited are left in ed.  lim > 0 bounds the search (the
+// boxes of T are there).
 template <int NT>
 __device__ long long r_search(const int4* __restrict__ epos, long long* __restrict__ ed, int n, int4 pc,
-                              const PredConst& c, SelShared& S, const int small_n, const int cap, const int nb) {
+                              const PredConst& c, SelShared& S, const int small_n, const int cap, const int nb,
+                              const Tiles& T, unsigned long long lim) {
   const int tid = threadIdx.x;
   if (n <= small_n && n <= COUNT_N) {
     // every member's strictly enclosed count, counted directly: n(<d_i) =
@@ -297,7 +432,7 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
 
   // ---- windowed histogram select ----
   // window [wlo, whi] of d; base = members with d < wlo; mode 0 = threshold-count bins
-  unsigned long long wlo = 0, whi = ~0ull, base = 0;
+  unsigned long long wlo = 0, whi = lim ? lim - 1 : ~0ull, base = 0;
   int mode = 0;
   const float scale0 = c.bin_scale0 / (float)((n + nb - 2) / (nb - 1));  // n/(nb-1) members of threshold per bin
   bool first_pass = true;
@@ -311,7 +446,7 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
     __syncthreads();
     unsigned long long span = whi - wlo + 1;  // mode 1 only
     unsigned long long dmax = 0;              // this thread's farthest member (first pass)
-    for (int j = tid; j < n; j += blockDim.x) {
+    for_members(T, n, lim, [&](int j) {
       unsigned long long d;
       if (first_pass) {
         d = (unsigned long long)dist2(pc, epos[j]);
@@ -320,7 +455,7 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
       } else {
         d = (unsigned long long)ed[j];
       }
-      if (d < wlo || d > whi) continue;
+      if (d < wlo || d > whi) return;
       int b;
       if (mode == 0) {
         b = first_bin(d, c, scale0, nb);
@@ -329,7 +464,7 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
       }
       atomicAdd(&S.cnt[b], 1u);
       bin_minmax(S, b, d);
-    }
+    });
     if (first_pass) {
       // one shared atomic per warp (per member it serialised on one address)
       const unsigned long long m = warp_max_u64(dmax);
@@ -388,10 +523,10 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
       if (cntb <= (unsigned)cap) {
         if (tid == 0) S.nlist = 0;
         __syncthreads();
-        for (int j = tid; j < n; j += blockDim.x) {
+        for_members(T, n, lim, [&](int j) {
           unsigned long long d = (unsigned long long)ed[j];
           if (d >= lo && d <= hi) S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
-        }
+        });
         __syncthreads();
         int m = S.nlist;
         int p2 = pow2_at_least(m);
@@ -417,11 +552,22 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
     }
     if (narrowed) continue;
     // nothing in [wlo, whi]: move past it
-    base += in_window;
-    if (whi >= S.dmax_all) break;
-    wlo = whi + 1;
-    whi = S.dmax_all;
-    mode = 1;
+    const unsigned long long top = lim ? lim - 1 : S.dmax_all;
+    if (whi < top) {
+      base += in_window;
+      wlo = whi + 1;
+      whi = top;
+      mode = 1;
+    } else if (lim) {  // nothing below the bound: all members, from the start
+      __syncthreads();  // every thread has read dmax_all
+      lim = 0;
+      wlo = base = 0;
+      whi = ~0ull;
+      mode = 0;
+      first_pass = true;
+    } else {
+      break;
+    }
   }
   long long r = 0;
   if (tid == 0) S.list[0] = exhaust_radius((unsigned long long)n, (long long)S.dmax_all, c);
@@ -431,265 +577,273 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
   return r;
 }
 
-// Step 2's density criterion for cell-sorted particle se of group glabel: no
-// particle of the same group within d < b2 comes before it in key order
-// (Sigma desc, id asc).  The neighbours are the runs of the 27-cell stencil,
-// nine rows (own row first, where a denser neighbour usually sits), each one
-// run plus one where the row wraps; rows and end cells that cannot reach
-// within b are dropped.
-struct PeakRows {
-  uint32_t lo0, hi0, lo1, hi1;  // lanes 0-8: row lane's runs (rows in walk order)
-  int qx1, qy, qz;              // the query in that row's image
-  uint32_t pre;                 // lanes 0-9: neighbours in the rows before this one
+// ---------------------------------------------------------------------------
+// the choice of the next nucleus among a group's peaks
+// ---------------------------------------------------------------------------
+struct Best {
+  long long sig;
+  uint64_t id;
+  int i;  // -1: none
 };
 
-__device__ __forceinline__ int peak_row_of(int o) { return o == 0 ? 4 : (o <= 4 ? o - 1 : o); }
+__device__ __forceinline__ void best_of(Best& a, const Best& b) {  // key order: Sigma desc, id asc
+  if (b.i >= 0 && (a.i < 0 || b.sig > a.sig || (b.sig == a.sig && b.id < a.id))) a = b;
+}
 
-__device__ PeakRows peak_rows(const LevelArgs& a, int4 p) {
-  const int lane = threadIdx.x & 31;
-  const CellGrid& g = a.grid;
-  const int nc = g.nc;
-  const int cy = cell_coord(p.y, nc), cz = cell_coord(p.z, nc);
-  const int tc = grid_col(g, p.x);
-  const XCells X = x_cells(g, tc);
-  PeakRows R{0, 0, 0, 0, p.x, p.y, p.z, 0};
-  if (lane < 9) {
-    const int r = peak_row_of(lane);
-    const int dz = r / 3 - 1, dy = r % 3 - 1;
-    const int gx = (p.x + g.x0) & (CSO_BOX - 1), gcx = cell_coord(gx, nc);
-    const long long zl = p.z - cell_lo(cz, nc) + 1, zr = cell_lo(cz + 1, nc) - p.z;
-    const long long yl = p.y - cell_lo(cy, nc) + 1, yr = cell_lo(cy + 1, nc) - p.y;
-    const long long xl = gx - cell_lo(gcx, nc) + 1, xr = cell_lo(gcx + 1, nc) - gx;
-    const long long m = (dz < 0 ? zl * zl : (dz > 0 ? zr * zr : 0)) + (dy < 0 ? yl * yl : (dy > 0 ? yr * yr : 0));
-    if (m < (long long)a.b2) {
-      int sz, sy;
-      const int zz = wrap_yz(cz + dz, nc, sz), yy = wrap_yz(cy + dy, nc, sy);
-      R.qz += sz;
-      R.qy += sy;
-      const uint32_t* row = grid_row(g, zz, yy);
-      const bool left = m + xl * xl < (long long)a.b2, right = m + xr * xr < (long long)a.b2;
-      const int ca = left ? X.a : tc, cb = right ? X.b : tc;
-      if (left && X.wl >= 0) { R.lo1 = row[X.wl]; R.hi1 = row[X.wl + 1]; R.qx1 = p.x + CSO_BOX; }
-      if (right && X.wr >= 0) { R.lo1 = row[X.wr]; R.hi1 = row[X.wr + 1]; R.qx1 = p.x - CSO_BOX; }
-      R.lo0 = row[ca];
-      R.hi0 = row[cb + 1];
+__device__ __forceinline__ void warp_best(Best& a) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    Best b;
+    b.sig = __shfl_xor_sync(0xffffffffu, a.sig, o);
+    b.id = __shfl_xor_sync(0xffffffffu, a.id, o);
+    b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
+    best_of(a, b);
+  }
+}
+
+struct PickShared {
+  Best w[32];
+  Best all;
+};
+
+// Marks the peaks that nucleus pc of squared radius R2 makes ineligible (step
+// 1: nearer than alpha R; `cur` is the nucleus itself) and returns the first
+// of the others in key order, or -1.  cur < 0: the first choice.  Each CTA of
+// a cluster calls it with the same arguments and gets the same answer; the
+// flags they write are the same too, and none of them is a nucleus ahead.
+__device__ int next_nucleus(const LevelArgs& a, unsigned p0, int m, int cur, int4 pc, long long R2, PickShared& K) {
+  const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
+  Best mine{0, 0, -1};
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    if (cur >= 0) {
+      if (a.peaks.out[p0 + i]) continue;
+      if (i == cur || (__int128)aden2 * dist2(pc, a.peaks.pos[p0 + i]) < (__int128)anum2 * R2) {
+        a.peaks.out[p0 + i] = 1;
+        continue;
+      }
     }
+    best_of(mine, Best{a.peaks.sig[p0 + i], a.peaks.id[p0 + i], i});
   }
-  // exclusive prefix of the rows' neighbour counts (lane 9 holds the total)
-  const uint32_t cnt = lane < 9 ? (R.hi0 - R.lo0) + (R.hi1 - R.lo1) : 0u;
-  uint32_t inc = cnt;
-#pragma unroll
-  for (int o = 1; o < 16; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  R.pre = inc - cnt;
-  return R;
-}
-
-// One load step of the peak test: neighbours f0 + k * 32 + lane (k < U) of
-// the flattened rows; true if any lane found a beater.  Every load of the
-// step is issued before any comparison, so a step costs one memory round trip.
-constexpr int PEAK_U = 4;
-__device__ __forceinline__ bool peak_step(const LevelArgs& a, const PeakRows& R, uint32_t f0, uint32_t total, uint32_t se,
-                                          int glabel, int4 p, long long sp, uint64_t idp) {
-  const int lane = threadIdx.x & 31;
-  int4 q[PEAK_U];
-  int lab[PEAK_U];
-  long long st[PEAK_U];
-  uint32_t tt[PEAK_U];
-  int ow[PEAK_U];  // row (walk order) | 16 for the wrapped run
-#pragma unroll
-  for (int k = 0; k < PEAK_U; ++k) {
-    const uint32_t f = f0 + k * 32 + lane;
-    // the row holding f: the last o with pre[o] <= f
-    int o = 0;
-#pragma unroll
-    for (int oo = 1; oo < 9; ++oo)
-      if (__shfl_sync(0xffffffffu, R.pre, oo) <= f) o = oo;
-    const uint32_t r = f - __shfl_sync(0xffffffffu, R.pre, o);
-    const uint32_t l0 = __shfl_sync(0xffffffffu, R.lo0, o), n0 = __shfl_sync(0xffffffffu, R.hi0, o) - l0;
-    const uint32_t l1 = __shfl_sync(0xffffffffu, R.lo1, o);
-    tt[k] = f < total ? (r < n0 ? l0 + r : l1 + (r - n0)) : se;
-    ow[k] = o | (r < n0 ? 0 : 16);
-    q[k] = a.spos[tt[k]];
-    lab[k] = a.slab[tt[k]];
-    st[k] = a.ssig[tt[k]];
-  }
-  bool beat = false;
-#pragma unroll
-  for (int k = 0; k < PEAK_U; ++k) {
-    const int o = ow[k] & 15;
-    const int x1 = __shfl_sync(0xffffffffu, R.qx1, o), yq = __shfl_sync(0xffffffffu, R.qy, o),
-              zq = __shfl_sync(0xffffffffu, R.qz, o);
-    if (tt[k] == se || lab[k] != glabel) continue;  // past the end (tt = se), self, or another group
-    const int dx = (ow[k] & 16 ? x1 : p.x) - q[k].x, dy = yq - q[k].y, dz = zq - q[k].z;
-    const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
-    if (d < a.b2) beat = beat || st[k] > sp || (st[k] == sp && a.sid[tt[k]] < idp);
-  }
-  return __any_sync(0xffffffffu, beat);
-}
-
-enum : int { PEAK_NO = 0, PEAK_YES = 1, PEAK_OPEN = 2 };
-
-// The test by one warp, at most `steps` load steps: PEAK_NO (a beater was
-// found), PEAK_YES (no beater among all neighbours) or PEAK_OPEN (not
-// finished; peak_part finishes it with many warps).
-__device__ __forceinline__ int warp_peak(const LevelArgs& a, uint32_t se, int glabel, int steps) {
-  const int4 p = a.spos[se];
-  const long long sp = a.ssig[se];
-  const uint64_t idp = a.sid[se];
-  const PeakRows R = peak_rows(a, p);
-  const uint32_t total = __shfl_sync(0xffffffffu, R.pre, 9);
-  for (uint32_t f0 = 0; f0 < total; f0 += 32 * PEAK_U) {
-    if (steps-- <= 0) return PEAK_OPEN;
-    if (peak_step(a, R, f0, total, se, glabel, p, sp, idp)) return PEAK_NO;
-  }
-  return PEAK_YES;
-}
-
-// Part `part` of `parts` of the test (warps of a block or of a cluster
-// share the neighbours step by step): true if this part holds a beater.
-__device__ __forceinline__ bool peak_part_beaten(const LevelArgs& a, uint32_t se, int glabel, int part, int parts) {
-  const int4 p = a.spos[se];
-  const long long sp = a.ssig[se];
-  const uint64_t idp = a.sid[se];
-  const PeakRows R = peak_rows(a, p);
-  const uint32_t total = __shfl_sync(0xffffffffu, R.pre, 9);
-  for (uint32_t f0 = (uint32_t)part * 32 * PEAK_U; f0 < total; f0 += (uint32_t)parts * 32 * PEAK_U)
-    if (peak_step(a, R, f0, total, se, glabel, p, sp, idp)) return true;
-  return false;
-}
-
-// load steps a warp spends on a candidate before the test goes to all warps
-constexpr int PEAK_STEPS = 4;
-
-__device__ bool warp_is_peak(const LevelArgs& a, uint32_t se, int glabel) {
-  return warp_peak(a, se, glabel, INT_MAX) == PEAK_YES;
-}
-
-template <int NT>
-__device__ void level_block(const LevelArgs& a, const int seg) {
-  constexpr int NW = NT / 32;
-  __shared__ SelShared S;
-  __shared__ int sP;
-  __shared__ int list[NT];
-  __shared__ int peak_of[NW];
-  __shared__ int coop_beat;
-  const unsigned base = a.seg_off[seg];
-  const int n = (int)(a.seg_off[seg + 1] - base);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int4* epos = a.epos + base;
-  const long long* esig = a.esig + base;
-  const uint32_t* egs = a.egs + base;
-  int* eslot = a.eslot + base;
-  long long* edold = a.edold + base;
-  uint8_t* einel = a.einel + base;
-  long long* ed = a.ed + base;
-
-  for (int j = tid; j < n; j += blockDim.x) {
-    eslot[j] = -1;
-    einel[j] = 0;
-  }
-  // step 4: candidates are the members above the stop level: a prefix in key order
-  if (tid == 0) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-      int mid = (lo + hi) >> 1;
-      if (esig[mid] > a.T_min) lo = mid + 1;
-      else hi = mid;
-    }
-    sP = lo;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  warp_best(mine);
+  if (lane == 0) K.w[w] = mine;
+  __syncthreads();
+  if (w == 0) {
+    Best b = lane < (int)(blockDim.x >> 5) ? K.w[lane] : Best{0, 0, -1};
+    warp_best(b);
+    if (lane == 0) K.all = b;
   }
   __syncthreads();
-  const int P = sP;
-  const int glabel = a.slab[egs[0]];  // every member carries the group's label
-  const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
+  return K.all.i;
+}
+
+// steps 1 and 3 for member j at squared distance d < R2: tentative membership
+// or reassignment (Eq. 3)
+__device__ __forceinline__ void assign_member(const LevelArgs& a, unsigned base, int* eslot, long long* edold, int j,
+                                              long long d, long long R2, int nn) {
+  const int s = eslot[j];
+  bool take = s < 0;
+  if (!take) {
+    const long long R2old = __ldcg(&a.nuc_R2[base + s]);
+    take = (__int128)R2 * edold[j] * a.roche_den >= (__int128)a.roche_num * R2old * d;
+  }
+  if (take) {
+    eslot[j] = nn;
+    edold[j] = d;
+  }
+}
+
+__device__ __forceinline__ Tiles group_tiles(const LevelArgs& a, int seg, unsigned base, int n, int rank, int cs) {
+  // tiles of different groups never share a slot: a group of n members takes
+  // at most n / TILE + 1 of them
+  const size_t at = base / TILE + (size_t)seg;
+  return Tiles{(n + TILE - 1) / TILE, rank, cs, a.tlo + at, a.thi + at, make_int4(0, 0, 0, 0)};
+}
+
+__device__ __forceinline__ int4 tile_origin(const int4* epos, int4 pc) {
+  const int4 ref = epos[0];
+  return make_int4(fold21(pc.x - ref.x), fold21(pc.y - ref.y), fold21(pc.z - ref.z), 0);
+}
+
+struct BlockShared {
+  SelShared S;
+  PickShared K;
+  unsigned h[LEVELS];
+  int hbest;
+};
+
+template <int NT>
+__device__ void level_block(const LevelArgs& a, const int seg, BlockShared& B) {
+  const unsigned p0 = a.peaks.off[seg];
+  const int m = (int)(a.peaks.off[seg + 1] - p0);
+  const int tid = threadIdx.x;
+  if (m == 0) {
+    if (tid == 0) a.nnuc[seg] = 0;
+    return;
+  }
+  const unsigned base = a.seg_off[seg];
+  const int n = (int)(a.seg_off[seg + 1] - base);
+  const int4* epos = a.epos + base;
+  int* eslot = a.eslot + base;
+  long long* edold = a.edold + base;
+  long long* ed = a.ed + base;
+  Tiles T = group_tiles(a, seg, base, n, 0, 1);
+  const bool boxes = m > 1 && n > a.small_n;
+  if (boxes) tile_boxes(T, epos, n, a.tlo + (T.lo - a.tlo), a.thi + (T.hi - a.thi));
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
   int nn = 0;
-  for (int c0 = 0; c0 < P; c0 += NT) {
-    // the eligible candidates of this chunk, in key order
-    const int j = c0 + tid;
-    const unsigned f = (j < P && !einel[j]) ? 1u : 0u;
-    unsigned excl;
-    const unsigned m = block_scan<NT>(f, excl, S.sw);
-    if (f) list[excl] = j;
-    __syncthreads();
-    for (int g0 = 0; g0 < (int)m; g0 += NW) {
-      // step 2 for up to NW of them at once, one warp each for at most
-      // PEAK_STEPS load steps (peak-ness never changes)
-      const int k = g0 + warp;
-      if (k < (int)m) {
-        const int e = list[k];
-        const int st = einel[e] ? PEAK_NO : warp_peak(a, egs[e], glabel, PEAK_STEPS);
-        if (lane == 0) peak_of[warp] = st;
-      }
-      __syncthreads();
-      const int kmax = min(NW, (int)m - g0);
-      for (int kk = 0; kk < kmax; ++kk) {
-        const int e = list[g0 + kk];
-        // eligibility may have been lost to a nucleus found earlier in this walk
-        if (peak_of[kk] == PEAK_NO || einel[e]) continue;
-        if (peak_of[kk] == PEAK_OPEN) {
-          // a test one warp did not finish: every warp of the block takes a share
-          if (tid == 0) coop_beat = 0;
-          __syncthreads();
-          if (peak_part_beaten(a, egs[e], glabel, warp, NW) && lane == 0) coop_beat = 1;
-          __syncthreads();
-          const bool beaten = coop_beat != 0;
-          __syncthreads();
-          if (beaten) continue;
-        }
-        const int4 pc = epos[e];
-        const long long R2 = r_search<NT>(epos, ed, n, pc, a.pc, S, a.small_n, a.cap, a.nb);
-        // steps 1 and 3
-        for (int jj = tid; jj < n; jj += blockDim.x) {
-          long long d = ed[jj];
-          if (d >= R2) continue;
-          int s = eslot[jj];
-          bool take;
-          if (s < 0) {
-            take = true;
-          } else {
-            long long R2old = a.nuc_R2[base + s];
-            __int128 lhs = (__int128)R2 * edold[jj] * a.roche_den;
-            __int128 rhs = (__int128)a.roche_num * R2old * d;
-            take = lhs >= rhs;
-          }
-          if (take) {
-            eslot[jj] = nn;
-            edold[jj] = d;
-          }
-          if ((__int128)aden2 * d < (__int128)anum2 * R2) einel[jj] = 1;
-        }
-        if (tid == 0) {
-          a.nuc_member[base + nn] = (uint32_t)e;
-          a.nuc_R2[base + nn] = R2;
-        }
-        ++nn;
-        __syncthreads();
-      }
-      __syncthreads();
+  while (cur >= 0) {
+    const int4 pc = a.peaks.pos[p0 + cur];
+    unsigned long long lim = 0;
+    if (boxes) {
+      T.q = tile_origin(epos, pc);
+      lim = search_bound(T, n, a.pc, B.h, &B.hbest);
     }
+    const long long R2 = r_search<NT>(epos, ed, n, pc, a.pc, B.S, a.small_n, a.cap, a.nb, T, lim);
+    if (n <= a.small_n) {
+      for (int j = tid; j < n; j += NT)
+        if (ed[j] < R2) assign_member(a, base, eslot, edold, j, ed[j], R2, nn);
+    } else {
+      for_members(T, n, boxes ? (unsigned long long)R2 : 0, [&](int j) {
+        const long long d = ed[j];
+        if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
+      });
+    }
+    if (tid == 0) {
+      a.nuc_member[base + nn] = (uint32_t)pc.w;
+      a.nuc_R2[base + nn] = R2;
+    }
+    ++nn;
+    if (m == 1) break;
+    __syncthreads();
+    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
   }
   if (tid == 0) {
     a.nnuc[seg] = (uint32_t)nn;
-    if (a.work && nn) atomicAdd(a.work, (unsigned long long)nn * (unsigned long long)n);
+    if (a.work) atomicAdd(a.work, (unsigned long long)nn * (unsigned long long)n);
   }
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT) k_level(LevelArgs a, const uint32_t* __restrict__ segs) {
-  level_block<NT>(a, segs ? (int)segs[blockIdx.x] : (int)blockIdx.x);
+__global__ void __launch_bounds__(NT) k_level(LevelArgs a) {
+  __shared__ BlockShared B;
+  level_block<NT>(a, (int)blockIdx.x, B);
+}
+
+// ---------------------------------------------------------------------------
+// Groups of up to 512 members: 128 threads, members, distances and slots in
+// registers (four per thread), every member's strictly enclosed count counted
+// directly: n(<d_i) = #{j : d_j < d_i}, R^2 the smallest d_i whose count
+// satisfies the predicate.  4 KB of shared memory instead of the histogram's
+// 40, so sixteen such groups are in flight on an SM instead of four.
+// ---------------------------------------------------------------------------
+constexpr int SM_NT = 128;
+constexpr int SM_PER = COUNT_N / SM_NT;
+
+struct SmallShared {
+  long long d[COUNT_N];
+  PickShared K;
+  unsigned long long r;     // smallest qualifying distance
+  unsigned long long dmax;  // farthest member
+};
+
+__device__ void level_small(const LevelArgs& a, const int seg, SmallShared& B) {
+  const int tid = threadIdx.x;
+  const unsigned base = a.seg_off[seg];
+  const int n = (int)(a.seg_off[seg + 1] - base);
+  const unsigned p0 = a.peaks.off[seg];
+  const int m = (int)(a.peaks.off[seg + 1] - p0);
+  int4 p[SM_PER];
+  long long d[SM_PER], dold[SM_PER];
+  int slot[SM_PER];
+#pragma unroll
+  for (int k = 0; k < SM_PER; ++k) {
+    const int j = tid + k * SM_NT;
+    p[k] = j < n ? a.epos[base + j] : make_int4(0, 0, 0, 0);
+    slot[k] = -1;
+    dold[k] = 0;
+  }
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
+  int nn = 0;
+  while (cur >= 0) {
+    const int4 pc = a.peaks.pos[p0 + cur];
+    unsigned long long dmax = 0;
+#pragma unroll
+    for (int k = 0; k < SM_PER; ++k) {
+      const int j = tid + k * SM_NT;
+      d[k] = j < n ? dist2(pc, p[k]) : LLONG_MAX;
+      if (j < n) {
+        B.d[j] = d[k];
+        dmax = max(dmax, (unsigned long long)d[k]);
+      }
+    }
+    if (tid == 0) {
+      B.r = ~0ull;
+      B.dmax = 0;
+    }
+    __syncthreads();
+    unsigned cnt[SM_PER] = {};
+    for (int j = 0; j < n; ++j) {
+      const long long v = B.d[j];
+#pragma unroll
+      for (int k = 0; k < SM_PER; ++k) cnt[k] += v < d[k];
+    }
+    unsigned long long best = ~0ull;
+#pragma unroll
+    for (int k = 0; k < SM_PER; ++k)
+      if (tid + k * SM_NT < n && (unsigned long long)d[k] < best && pred(cnt[k], (unsigned long long)d[k], a.pc))
+        best = (unsigned long long)d[k];
+    if (best != ~0ull) atomicMin(&B.r, best);
+    dmax = warp_max_u64(dmax);
+    if ((tid & 31) == 0) atomicMax(&B.dmax, dmax);
+    __syncthreads();
+    if (B.r == ~0ull) {
+      __syncthreads();
+      if (tid == 0) B.r = (unsigned long long)exhaust_radius((unsigned long long)n, (long long)B.dmax, a.pc);
+      __syncthreads();
+    }
+    const long long R2 = (long long)B.r;
+#pragma unroll
+    for (int k = 0; k < SM_PER; ++k) {
+      if (d[k] >= R2) continue;  // past the end: LLONG_MAX
+      bool take = slot[k] < 0;
+      if (!take) {
+        const long long R2old = __ldcg(&a.nuc_R2[base + slot[k]]);
+        take = (__int128)R2 * dold[k] * a.roche_den >= (__int128)a.roche_num * R2old * d[k];
+      }
+      if (take) {
+        slot[k] = nn;
+        dold[k] = d[k];
+      }
+    }
+    if (tid == 0) {
+      a.nuc_member[base + nn] = (uint32_t)pc.w;
+      a.nuc_R2[base + nn] = R2;
+    }
+    ++nn;
+    if (m == 1) break;
+    __syncthreads();
+    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
+  }
+#pragma unroll
+  for (int k = 0; k < SM_PER; ++k)
+    if (tid + k * SM_NT < n) a.eslot[base + tid + k * SM_NT] = slot[k];
+  if (tid == 0) {
+    a.nnuc[seg] = (uint32_t)nn;
+    if (a.work) atomicAdd(a.work, (unsigned long long)nn * (unsigned long long)n);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Giant groups: one thread-block cluster of CS CTAs per group.  CTA r owns
-// the members [r n / CS, (r + 1) n / CS) for the distance, histogram, gather
-// and assignment passes; CTA 0 (the leader) runs the nucleus loop and the
-// select decisions and broadcasts them through its shared memory, which the
-// other CTAs read (and add their histograms into) over DSMEM.  Every CTA
-// passes every cluster barrier, in the same order: all control decisions are
-// read from the leader after a barrier.
+// the tiles r, r + CS, ... for the distance, histogram, gather and assignment
+// passes (interleaved, so that the tiles in reach of a nucleus spread over the
+// CTAs); CTA 0 (the leader) takes the select's decisions and broadcasts them
+// through its shared memory, which the other CTAs read over DSMEM.  A phase
+// of the select is: own work, barrier, the leader's decision from everyone's
+// shares, barrier.  Every CTA passes every cluster barrier, in the same order:
+// all control decisions are read from the leader after a barrier, or computed
+// by every CTA from the same data.
 // ---------------------------------------------------------------------------
 namespace cg = cooperative_groups;
 
@@ -697,61 +851,22 @@ constexpr int CL_CS = 8;      // CTAs per cluster (giant groups)
 constexpr int CL_HUGE_CS = 16;  // CTAs per cluster for huge groups (non-portable size, where it fits)
 constexpr int CL_NT = 1024;   // threads per CTA
 
-enum : int { OP_DONE = 0, OP_HIST = 1, OP_GATHER = 2 };
+enum : int { OP_DONE = 0, OP_HIST = 1, OP_GATHER = 2, OP_RESTART = 3 };
 
 struct ClusterCtl {
   int op;
-  int e;                    // next nucleus (member index) or -1
   int mode;                 // histogram binning of the window
-  int P;                    // members above the stop level
   long long R2;
   unsigned long long wlo, whi, base;  // window and members below it
   unsigned long long lo, hi, cb;      // bin to gather and its enclosed count
-  int from;                 // next bin to examine after a gather
   int bin;                  // bin being gathered
   unsigned in_window;
-  int blo, bn, bend;        // candidate batch of the nucleus walk
-  int coop;                 // batch entry whose peak test every warp shares, or -1
-  int cbeat;                // that test found a beater
 };
-
-struct ClusterGen {  // the leader's resumable walk over eligible candidates
-  int list[CL_NT];
-  int8_t peak_of[CL_NT];
-  int m, pos, c0;
-};
-
-// Leader only: refill the candidate list when it is used up (the eligible
-// members among the next CL_NT above the stop level, in key order) and
-// publish the next batch of up to cs * 32 untested candidates in C.blo /
-// C.bn, or C.bend = 1 when none remain.  Every CTA of the cluster then tests
-// one candidate of the batch per warp.
-__device__ void leader_next_batch(const uint8_t* einel, int P, ClusterGen& G, ClusterCtl& C, SelShared& S, int cs) {
-  const int tid = threadIdx.x;
-  while (G.pos >= G.m && G.c0 < P) {
-    const int j = G.c0 + tid;
-    const unsigned f = (j < P && !einel[j]) ? 1u : 0u;
-    unsigned excl;
-    const unsigned m = block_scan<CL_NT>(f, excl, S.sw);
-    if (f) G.list[excl] = j;
-    __syncthreads();
-    if (tid == 0) {
-      G.m = (int)m;
-      G.pos = 0;
-      G.c0 += CL_NT;
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    C.bend = G.pos >= G.m;
-    C.blo = G.pos;
-    C.bn = min(G.m - G.pos, cs * 32);
-  }
-}
 
 // leader only: decide the next step of the select from bin `from` of the
 // merged histogram (S.cnt / S.dmn / S.dmx / S.clo, window in Ctl)
-__device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int cap, int n, const PredConst& c) {
+__device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int cap, int n, const PredConst& c,
+                              unsigned long long lim) {
   const int tid = threadIdx.x;
   if (tid == 0) S.best = NB;
   __syncthreads();
@@ -779,15 +894,22 @@ __device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int
         C.mode = 1;
       }
     } else {  // nothing in the window: move past it
-      C.base += C.in_window;
-      if (C.whi >= S.dmax_all) {
+      const unsigned long long top = lim ? lim - 1 : S.dmax_all;
+      if (C.whi < top) {
+        C.op = OP_HIST;
+        C.base += C.in_window;
+        C.wlo = C.whi + 1;
+        C.whi = top;
+        C.mode = 1;
+      } else if (lim) {  // nothing below the bound: all members, from the start
+        C.op = OP_RESTART;
+        C.base = 0;
+        C.wlo = 0;
+        C.whi = ~0ull;
+        C.mode = 0;
+      } else {
         C.op = OP_DONE;
         C.R2 = exhaust_radius((unsigned long long)n, (long long)S.dmax_all, c);
-      } else {
-        C.op = OP_HIST;
-        C.wlo = C.whi + 1;
-        C.whi = S.dmax_all;
-        C.mode = 1;
       }
     }
   }
@@ -799,26 +921,24 @@ __device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int
 // memory; after the barrier the leader reads the others' with plain DSMEM
 // loads and combines them.
 __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __restrict__ epos,
-                                      long long* __restrict__ ed, int n, int lo_r, int hi_r, int4 pc,
-                                      const PredConst& c, SelShared& S, ClusterCtl& C, int cap, int nb) {
+                                      long long* __restrict__ ed, int n, const Tiles& T, int4 pc, const PredConst& c,
+                                      SelShared& S, ClusterCtl& C, int cap, int nb, unsigned long long lim) {
   const int tid = threadIdx.x;
   const bool leader = cluster.block_rank() == 0;
   const int cs = (int)cluster.num_blocks();
   ClusterCtl* LC = cluster.map_shared_rank(&C, 0);
   const float scale0 = c.bin_scale0 / (float)((n + nb - 2) / (nb - 1));
-  // the first pass: threshold-count bins over every distance
-  unsigned long long wlo = 0, whi = ~0ull;
+  // the first pass: threshold-count bins over every distance below the bound
+  unsigned long long wlo = 0, whi = lim ? lim - 1 : ~0ull;
   int mode = 0;
   bool first = true;
-  if (leader && tid == 0) {
-    C.base = 0;
-    C.wlo = 0;
-    C.whi = ~0ull;
-    C.mode = 0;
-  }
   int op = OP_HIST;
   while (true) {
-    if (op == OP_HIST) {
+    if (op != OP_GATHER) {
+      if (op == OP_RESTART) {
+        first = true;
+        lim = 0;
+      }
       for (int b = tid; b < NB; b += blockDim.x) {
         S.cnt[b] = 0;
         S.dmn[b] = ~0ull;
@@ -828,7 +948,7 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
       __syncthreads();
       const unsigned long long span = whi - wlo + 1;
       unsigned long long dmax = 0;  // this thread's farthest member (first pass)
-      for (int j = lo_r + tid; j < hi_r; j += blockDim.x) {
+      for_members(T, n, lim, [&](int j) {
         unsigned long long d;
         if (first) {
           d = (unsigned long long)dist2(pc, epos[j]);
@@ -837,7 +957,7 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
         } else {
           d = (unsigned long long)ed[j];
         }
-        if (d < wlo || d > whi) continue;
+        if (d < wlo || d > whi) return;
         int b;
         if (mode == 0) {
           b = first_bin(d, c, scale0, nb);
@@ -846,14 +966,19 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
         }
         atomicAdd(&S.cnt[b], 1u);
         bin_minmax(S, b, d);
-      }
+      });
       if (first) {
         const unsigned long long m = warp_max_u64(dmax);
         if ((tid & 31) == 0) atomicMax(&S.dmax_all, m);
       }
-      __syncthreads();
       cluster.sync();  // every CTA's histogram of its members is complete
       if (leader) {
+        if (op == OP_HIST && first && tid == 0) {  // (a restart's window is set already)
+          C.base = 0;
+          C.wlo = wlo;
+          C.whi = whi;
+          C.mode = 0;
+        }
         // combine the CTAs' histograms (the leader's own is the first share)
         for (int b = tid; b < NB; b += blockDim.x) {
           unsigned cn = S.cnt[b];
@@ -878,36 +1003,23 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
           S.dmax_all = m;
         }
         __syncthreads();
-        constexpr int per = NB / CL_NT;
-        unsigned loc[per > 0 ? per : 1];
-        unsigned sum = 0;
-#pragma unroll
-        for (int q = 0; q < per; ++q) {
-          loc[q] = S.cnt[tid * per + q];
-          sum += loc[q];
-        }
+        static_assert(NB == CL_NT, "one bin per thread");
         unsigned excl;
-        const unsigned tot = block_scan<CL_NT>(sum, excl, S.sw);
-        unsigned run = excl;
-#pragma unroll
-        for (int q = 0; q < per; ++q) {
-          S.clo[tid * per + q] = run;
-          run += loc[q];
-        }
+        const unsigned tot = block_scan<CL_NT>(S.cnt[tid], excl, S.sw);
+        S.clo[tid] = excl;
         if (tid == 0) C.in_window = tot;
         __syncthreads();
-        leader_decide(C, S, 0, nb, cap, n, c);
+        leader_decide(C, S, 0, nb, cap, n, c, lim);
       }
       first = false;
     } else {  // OP_GATHER: every CTA lists its members of the bin, the leader collects them
       const unsigned long long glo = LC->lo, ghi = LC->hi;
       if (tid == 0) S.nlist = 0;
       __syncthreads();
-      for (int j = lo_r + tid; j < hi_r; j += blockDim.x) {
+      for_members(T, n, lim, [&](int j) {
         const unsigned long long d = (unsigned long long)ed[j];
         if (d >= glo && d <= ghi) S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
-      }
-      __syncthreads();
+      });
       cluster.sync();  // every CTA's list is complete
       if (leader) {
         int off = S.nlist;
@@ -931,233 +1043,207 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
           }
           __syncthreads();
         } else {
-          leader_decide(C, S, C.bin + 1, nb, cap, n, c);
+          leader_decide(C, S, C.bin + 1, nb, cap, n, c, lim);
         }
       }
     }
-    cluster.sync();  // the leader's decision is published (and it has read everyone's shares)
+    // the leader's decision is published, and it has read everyone's shares;
+    // it writes the next one only after the next phase's first barrier, which
+    // no CTA reaches before it has read this one
+    cluster.sync();
     op = LC->op;
     if (op == OP_DONE) break;
     wlo = LC->wlo;
     whi = LC->whi;
     mode = LC->mode;
-    cluster.sync();  // everyone has read it before the leader writes the next one
   }
-  const long long R2 = LC->R2;
-  cluster.sync();
-  return R2;
+  return LC->R2;
 }
 
-// Step 2 walk of the cluster tier: the next candidate in key order that is
-// eligible and a local peak (member index), or -1.  The leader hands out
-// batches; every warp of every CTA peak-tests one candidate for at most
-// PEAK_STEPS load steps and stores the state in the leader's shared memory;
-// the leader's thread 0 takes the first candidate of the batch still in
-// play, and a test no warp finished is finished by every warp of the cluster
-// before it is decided (no nucleus is accepted during the walk, so a batch
-// is settled in order).  Every CTA passes the same barriers: the exits are
-// read from the leader after a barrier.
-__device__ __forceinline__ int cluster_walk(const LevelArgs& a, const uint32_t* __restrict__ egs,
-                                         const uint8_t* __restrict__ einel, int glabel, SelShared& S,
-                                         ClusterCtl& C, ClusterGen& G) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const bool leader = rank == 0;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cs = (int)cluster.num_blocks();
-  ClusterCtl* LC = cluster.map_shared_rank(&C, 0);
-  ClusterGen* LG = cluster.map_shared_rank(&G, 0);
-  int e = -1;
-  while (true) {
-    if (leader) leader_next_batch(einel, C.P, G, C, S, cs);
-    cluster.sync();  // batch published
-    if (LC->bend) break;
-    const int blo = LC->blo, bn = LC->bn;
-    const int k = blo + rank * 32 + warp;
-    if (k < blo + bn) {
-      const int ek = LG->list[k];
-      const int st = einel[ek] ? PEAK_NO : warp_peak(a, egs[ek], glabel, PEAK_STEPS);
-      if (lane == 0) LG->peak_of[k] = (int8_t)st;
-    }
-    cluster.sync();  // peak states in the leader's shared memory
-    int from = blo;
-    while (true) {
-      // the leader takes the first candidate of the batch still in play: a
-      // settled peak is the nucleus; an open test goes to every warp of
-      // the cluster first
-      if (leader && tid == 0) {
-        int kk = from, found = -1, coop = -1;
-        for (const int kend = C.blo + C.bn; kk < kend; ++kk) {
-          const int ec = G.list[kk];
-          if (G.peak_of[kk] == PEAK_NO || einel[ec]) continue;
-          if (G.peak_of[kk] == PEAK_OPEN) {
-            coop = kk;
-            break;
-          }
-          found = ec;
-          ++kk;
-          break;
-        }
-        G.pos = kk;
-        C.e = found;
-        C.coop = coop;
-        C.cbeat = 0;
-      }
-      cluster.sync();  // walk decision (or the shared test) published
-      const int kc = LC->coop;
-      if (kc < 0) break;
-      if (peak_part_beaten(a, egs[LG->list[kc]], glabel, rank * 32 + warp, cs * 32) && lane == 0)
-        atomicExch(&LC->cbeat, 1);
-      cluster.sync();  // every share of the shared test done
-      if (leader && tid == 0) G.peak_of[kc] = (int8_t)(C.cbeat ? PEAK_NO : PEAK_YES);
-      from = kc;
-    }
-    e = LC->e;
-    if (e >= 0) break;
-  }
-  return e;
-}
+struct ClusterShared {
+  SelShared S;
+  ClusterCtl C;
+  PickShared K;
+  unsigned h[LEVELS];
+  int hbest;
+};
 
-__device__ void cluster_level(const LevelArgs& a, const int seg, SelShared& S, ClusterCtl& C, ClusterGen& G) {
+__device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& B) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const bool leader = rank == 0;
   const unsigned base = a.seg_off[seg];
   const int n = (int)(a.seg_off[seg + 1] - base);
+  const unsigned p0 = a.peaks.off[seg];
+  const int m = (int)(a.peaks.off[seg + 1] - p0);
   const int tid = threadIdx.x;
   const int cs = (int)cluster.num_blocks();
-  const int lo_r = (int)((long long)n * rank / cs), hi_r = (int)((long long)n * (rank + 1) / cs);
   const int4* epos = a.epos + base;
-  const long long* esig = a.esig + base;
-  const uint32_t* egs = a.egs + base;
   int* eslot = a.eslot + base;
   long long* edold = a.edold + base;
-  uint8_t* einel = a.einel + base;
   long long* ed = a.ed + base;
-  ClusterCtl* LC = cluster.map_shared_rank(&C, 0);
-
-  for (int j = lo_r + tid; j < hi_r; j += blockDim.x) {
-    eslot[j] = -1;
-    einel[j] = 0;
+  Tiles T = group_tiles(a, seg, base, n, rank, cs);
+  const bool boxes = m > 1;
+  if (boxes) {
+    tile_boxes(T, epos, n, a.tlo + (T.lo - a.tlo), a.thi + (T.hi - a.thi));
+    cluster.sync();  // every CTA reads all boxes
   }
-  if (leader && tid == 0) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (esig[mid] > a.T_min) lo = mid + 1;
-      else hi = mid;
-    }
-    C.P = lo;
-    G.m = 0;
-    G.pos = 0;
-    G.c0 = 0;
-  }
-  ClusterGen* LG = cluster.map_shared_rank(&G, 0);
-  const int warp = tid >> 5, lane = tid & 31;
-  const int glabel = a.slab[egs[0]];
-  const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
-  cluster.sync();  // slots and flags initialised everywhere
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
   int nn = 0;
-  while (true) {
-    const int e = cluster_walk(a, egs, einel, glabel, S, C, G);
-    if (e < 0) break;
-    const int4 pc = epos[e];
-    const long long R2 = cluster_r_search(cluster, epos, ed, n, lo_r, hi_r, pc, a.pc, S, C, a.cap, a.nb);
-    // steps 1 and 3 on this CTA's share of the members
-    for (int j = lo_r + tid; j < hi_r; j += blockDim.x) {
-      const long long d = ed[j];
-      if (d >= R2) continue;
-      const int sl = eslot[j];
-      bool take;
-      if (sl < 0) {
-        take = true;
-      } else {
-        const long long R2old = a.nuc_R2[base + sl];
-        take = (__int128)R2 * edold[j] * a.roche_den >= (__int128)a.roche_num * R2old * d;
-      }
-      if (take) {
-        eslot[j] = nn;
-        edold[j] = d;
-      }
-      if ((__int128)aden2 * d < (__int128)anum2 * R2) einel[j] = 1;
+  while (cur >= 0) {
+    const int4 pc = a.peaks.pos[p0 + cur];
+    unsigned long long lim = 0;
+    if (boxes) {
+      T.q = tile_origin(epos, pc);
+      lim = search_bound(T, n, a.pc, B.h, &B.hbest);
     }
+    const long long R2 = cluster_r_search(cluster, epos, ed, n, T, pc, a.pc, B.S, B.C, a.cap, a.nb, lim);
+    // steps 1 and 3 on this CTA's share of the members
+    for_members(T, n, boxes ? (unsigned long long)R2 : 0, [&](int j) {
+      const long long d = ed[j];
+      if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
+    });
     if (leader && tid == 0) {
-      a.nuc_member[base + nn] = (uint32_t)e;
+      a.nuc_member[base + nn] = (uint32_t)pc.w;
       a.nuc_R2[base + nn] = R2;
     }
     ++nn;
-    cluster.sync();  // assignments and eligibility visible to the leader's next walk
+    if (m == 1) break;
+    __syncthreads();
+    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
   }
   if (leader && tid == 0) {
     a.nnuc[seg] = (uint32_t)nn;
-    if (a.work && nn) atomicAdd(a.work, (unsigned long long)nn * (unsigned long long)n);
+    if (a.work) atomicAdd(a.work, (unsigned long long)nn * (unsigned long long)n);
   }
-  // no CTA may exit while another can still read its shared memory (the last
-  // read of the leader's C.e happens after the final barrier of the loop)
-  cluster.sync();
 }
 
 // ---------------------------------------------------------------------------
-// The batched schedule's work queue: the groups sorted by size (largest
-// first) and cut into four size bins on the device -- giants, large, medium
-// and small -- with one fetch counter per bin.  Four persistent kernels pull
-// from it concurrently: 8-CTA clusters take giants, 1024-thread blocks large
-// groups, 256-thread blocks medium ones and warps the small ones, each taking
-// the next group of its bin when it finishes one, so no launch size depends
-// on a count read back by the host.
+// The batched schedule's work queue: the groups that have peaks, filed by
+// tier and size (four bins an octave) on the device, largest first, with one
+// fetch counter per tier.  Six persistent kernels pull from it concurrently:
+// 16-CTA clusters take huge groups, 8-CTA clusters giants, 1024-thread blocks
+// large groups, 256-thread blocks medium ones, 128-thread blocks those of up
+// to 512 members and warps the smallest, each taking the next group of its
+// tier when it finishes one, so no launch size depends on a count read back
+// by the host.
 // ---------------------------------------------------------------------------
+enum : int { TIER_HUGE = 0, TIER_GIANT, TIER_LARGE, TIER_MEDIUM, TIER_SMALL, TIER_WARP, TIERS };
+constexpr int SIZE_BINS = 128;
+constexpr int QBINS = TIERS * SIZE_BINS;
+
 struct TierQueue {
-  unsigned count[4];  // giant (huge included), large, small, huge (from k_seg_sizes)
-  unsigned next[5];   // fetch counters: giant, large, medium, small, huge
-  unsigned nseg;
+  unsigned count[QBINS];  // groups per bin
+  unsigned next[TIERS];   // fetch counters
+  unsigned first[TIERS], cnt[TIERS];
 };
 
-// first index in the size-sorted order and count of bin t
-__device__ __forceinline__ void tier_range(const TierQueue& q, int t, unsigned& first, unsigned& cnt) {
-  const unsigned ng = q.count[0], nl = q.count[1], ns = q.count[2], nh = q.count[3];
-  const unsigned nm = q.nseg - ng - nl - ns;
-  if (t == 4) { first = 0; cnt = nh; }
-  else if (t == 0) { first = nh; cnt = ng - nh; }
-  else if (t == 1) { first = ng; cnt = nl; }
-  else if (t == 2) { first = ng + nl; cnt = nm; }
-  else { first = q.nseg - ns; cnt = ns; }
+struct TierBounds {
+  int huge, giant, large, medium, small;  // groups above `huge` members are TIER_HUGE, ...
+};
+
+// bin of every group with peaks and its rank there; groups without any have no nuclei
+__global__ void __launch_bounds__(1024) k_seg_bins(const uint32_t* __restrict__ seg_off,
+                                                   const uint32_t* __restrict__ peak_off, int nseg, TierBounds b,
+                                                   int* __restrict__ bin, uint32_t* __restrict__ rank,
+                                                   uint32_t* __restrict__ nnuc, TierQueue* q) {
+  __shared__ unsigned sc[QBINS];
+  for (int i = threadIdx.x; i < QBINS; i += blockDim.x) sc[i] = 0;
+  __syncthreads();
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  int k = -1;
+  unsigned local = 0;
+  if (g < nseg) {
+    if (peak_off[g + 1] == peak_off[g]) {
+      nnuc[g] = 0;
+    } else {
+      const int n = (int)(seg_off[g + 1] - seg_off[g]);
+      const int tier = n > b.huge ? TIER_HUGE : n > b.giant ? TIER_GIANT : n > b.large ? TIER_LARGE
+                       : n > b.medium ? TIER_MEDIUM : n > b.small ? TIER_SMALL : TIER_WARP;
+      const int msb = 31 - __clz(n);
+      const int size = 4 * msb + (int)(((unsigned)n << (31 - msb)) >> 29 & 3u);
+      k = tier * SIZE_BINS + SIZE_BINS - 1 - size;
+      local = atomicAdd(&sc[k], 1u);
+    }
+    bin[g] = k;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < QBINS; i += blockDim.x)
+    if (sc[i]) sc[i] = atomicAdd(&q->count[i], sc[i]);
+  __syncthreads();
+  if (k >= 0) rank[g] = sc[k] + local;
 }
 
-// tier 0 (giants) on 8-CTA clusters, tier 4 (huge groups) on 16-CTA clusters
+// order[position] = group, bins in order; the tiers' ranges
+__global__ void __launch_bounds__(1024) k_seg_order(const int* __restrict__ bin, const uint32_t* __restrict__ rank,
+                                                    int nseg, uint32_t* __restrict__ order, TierQueue* q) {
+  __shared__ unsigned first[QBINS + 1];
+  __shared__ unsigned sw[33];
+  static_assert(QBINS < 1024, "one thread per bin");
+  const unsigned v = threadIdx.x < QBINS ? q->count[threadIdx.x] : 0u;
+  unsigned excl;
+  block_scan<1024>(v, excl, sw);
+  if (threadIdx.x <= QBINS) first[threadIdx.x] = excl;
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x < TIERS) {
+    const unsigned f = first[threadIdx.x * SIZE_BINS];
+    q->first[threadIdx.x] = f;
+    q->cnt[threadIdx.x] = first[(threadIdx.x + 1) * SIZE_BINS] - f;
+  }
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g < nseg && bin[g] >= 0) order[first[bin[g]] + rank[g]] = (uint32_t)g;
+}
+
+// giants on 8-CTA clusters, huge groups on 16-CTA clusters
 template <int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(CL_NT)
     k_level_cluster_q(LevelArgs a, const uint32_t* __restrict__ order, TierQueue* q, int tier) {
-  __shared__ SelShared S;
-  __shared__ ClusterCtl C;
-  __shared__ ClusterGen G;
+  __shared__ ClusterShared B;
   __shared__ unsigned item;
   cg::cluster_group cluster = cg::this_cluster();
   const bool leader = cluster.block_rank() == 0;
-  unsigned first, cnt;
-  tier_range(*q, tier, first, cnt);
+  const unsigned first = q->first[tier], cnt = q->cnt[tier];
   for (;;) {
+    // (the first barrier also ends the previous group: its last reads of the
+    // leader's shared memory are done)
     if (leader && threadIdx.x == 0) item = atomicAdd(&q->next[tier], 1u);
     cluster.sync();
     const unsigned it = *cluster.map_shared_rank(&item, 0);
     cluster.sync();  // every CTA has read the leader's item before it changes
     if (it >= cnt) return;
-    cluster_level(a, (int)order[first + it], S, C, G);
+    cluster_level(a, (int)order[first + it], B);
   }
 }
 
 template <int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_level_q(LevelArgs a, const uint32_t* __restrict__ order, TierQueue* q,
                                                 int tier) {
+  __shared__ BlockShared B;
   __shared__ unsigned item;
-  unsigned first, cnt;
-  tier_range(*q, tier, first, cnt);
+  const unsigned first = q->first[tier], cnt = q->cnt[tier];
   for (;;) {
     if (threadIdx.x == 0) item = atomicAdd(&q->next[tier], 1u);
     __syncthreads();
     const unsigned it = item;
     __syncthreads();
     if (it >= cnt) return;
-    level_block<NT>(a, (int)order[first + it]);
+    level_block<NT>(a, (int)order[first + it], B);
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(SM_NT, 8) k_level_small_q(LevelArgs a, const uint32_t* __restrict__ order,
+                                                          TierQueue* q) {
+  __shared__ SmallShared B;
+  __shared__ unsigned item;
+  const unsigned first = q->first[TIER_SMALL], cnt = q->cnt[TIER_SMALL];
+  for (;;) {
+    if (threadIdx.x == 0) item = atomicAdd(&q->next[TIER_SMALL], 1u);
+    __syncthreads();
+    const unsigned it = item;
+    __syncthreads();
+    if (it >= cnt) return;
+    level_small(a, (int)order[first + it], B);
     __syncthreads();
   }
 }
@@ -1192,41 +1278,48 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
   const int lane = threadIdx.x & 31;
   const unsigned base = a.seg_off[seg];
   const int n = (int)(a.seg_off[seg + 1] - base);
+  const unsigned p0 = a.peaks.off[seg];
+  const int m = (int)(a.peaks.off[seg + 1] - p0);  // at most n <= 64
   const bool v0 = lane < n, v1 = lane + 32 < n;
-  const int4 p0 = v0 ? a.epos[base + lane] : make_int4(0, 0, 0, 0);
-  const int4 p1 = v1 ? a.epos[base + lane + 32] : make_int4(0, 0, 0, 0);
-  const long long s0 = v0 ? a.esig[base + lane] : LLONG_MIN;
-  const long long s1 = v1 ? a.esig[base + lane + 32] : LLONG_MIN;
-  const uint32_t g0 = v0 ? a.egs[base + lane] : 0, g1 = v1 ? a.egs[base + lane + 32] : 0;
+  const int4 p0v = v0 ? a.epos[base + lane] : make_int4(0, 0, 0, 0);
+  const int4 p1v = v1 ? a.epos[base + lane + 32] : make_int4(0, 0, 0, 0);
   int slot0 = -1, slot1 = -1;
-  bool in0 = false, in1 = false;
   long long do0 = 0, do1 = 0;
-  // step 4: the members above the stop level form a prefix in key order
-  const int P = __popc(__ballot_sync(0xffffffffu, s0 > a.T_min)) + __popc(__ballot_sync(0xffffffffu, s1 > a.T_min));
-  const int glabel = a.slab[__shfl_sync(0xffffffffu, g0, 0)];
   const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
+  // the group's peaks, two per lane, and whether each may still become a nucleus
+  Best k0{0, 0, -1}, k1{0, 0, -1};
+  int4 c0 = make_int4(0, 0, 0, 0), c1 = make_int4(0, 0, 0, 0);
+  if (lane < m) {
+    k0 = Best{a.peaks.sig[p0 + lane], a.peaks.id[p0 + lane], lane};
+    c0 = a.peaks.pos[p0 + lane];
+  }
+  if (lane + 32 < m) {
+    k1 = Best{a.peaks.sig[p0 + lane + 32], a.peaks.id[p0 + lane + 32], lane + 32};
+    c1 = a.peaks.pos[p0 + lane + 32];
+  }
   int nn = 0;
-  for (int c = 0; c < P; ++c) {
-    const int src = c & 31;
-    const bool hi = c >= 32;
-    const bool inel = __shfl_sync(0xffffffffu, hi ? in1 : in0, src);
-    if (inel) continue;
-    const uint32_t se = __shfl_sync(0xffffffffu, hi ? g1 : g0, src);
-    if (!warp_is_peak(a, se, glabel)) continue;
+  while (true) {
+    Best b = k0;
+    best_of(b, k1);
+    warp_best(b);
+    if (b.i < 0) break;
+    const int src = b.i & 31;
+    const bool hi = b.i >= 32;
     int4 pc;
-    pc.x = __shfl_sync(0xffffffffu, hi ? p1.x : p0.x, src);
-    pc.y = __shfl_sync(0xffffffffu, hi ? p1.y : p0.y, src);
-    pc.z = __shfl_sync(0xffffffffu, hi ? p1.z : p0.z, src);
-    const long long d0 = v0 ? dist2(pc, p0) : D_INF, d1 = v1 ? dist2(pc, p1) : D_INF;
+    pc.x = __shfl_sync(0xffffffffu, hi ? c1.x : c0.x, src);
+    pc.y = __shfl_sync(0xffffffffu, hi ? c1.y : c0.y, src);
+    pc.z = __shfl_sync(0xffffffffu, hi ? c1.z : c0.z, src);
+    pc.w = __shfl_sync(0xffffffffu, hi ? c1.w : c0.w, src);
+    const long long d0 = v0 ? dist2(pc, p0v) : D_INF, d1 = v1 ? dist2(pc, p1v) : D_INF;
     // strictly enclosed counts
-    unsigned k0 = 0, k1 = 0;
+    unsigned n0 = 0, n1 = 0;
     for (int j = 0; j < n; ++j) {
       const long long dj = __shfl_sync(0xffffffffu, j >= 32 ? d1 : d0, j & 31);
-      k0 += dj < d0;
-      k1 += dj < d1;
+      n0 += dj < d0;
+      n1 += dj < d1;
     }
-    const bool ok0 = v0 && pred(k0, (unsigned long long)d0, a.pc);
-    const bool ok1 = v1 && pred(k1, (unsigned long long)d1, a.pc);
+    const bool ok0 = v0 && pred(n0, (unsigned long long)d0, a.pc);
+    const bool ok1 = v1 && pred(n1, (unsigned long long)d1, a.pc);
     long long R2 = warp_min_ll(min(ok0 ? d0 : D_INF, ok1 ? d1 : D_INF));
     if (R2 == D_INF) {
       const long long dmax = warp_max_ll(max(v0 ? d0 : 0ll, v1 ? d1 : 0ll));
@@ -1234,7 +1327,7 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
       if (lane == 0) r = exhaust_radius((unsigned long long)n, dmax, a.pc);
       R2 = __shfl_sync(0xffffffffu, r, 0);
     }
-    // steps 1 and 3 on the two members of this lane
+    // step 3 on the two members of this lane
     if (v0 && d0 < R2) {
       bool take = slot0 < 0;
       if (!take) {
@@ -1245,7 +1338,6 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
         slot0 = nn;
         do0 = d0;
       }
-      if ((__int128)aden2 * d0 < (__int128)anum2 * R2) in0 = true;
     }
     if (v1 && d1 < R2) {
       bool take = slot1 < 0;
@@ -1257,14 +1349,17 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
         slot1 = nn;
         do1 = d1;
       }
-      if ((__int128)aden2 * d1 < (__int128)anum2 * R2) in1 = true;
     }
+    // step 1: peaks nearer than alpha R (and the nucleus itself) are out
+    if (k0.i >= 0 && (k0.i == b.i || (__int128)aden2 * dist2(pc, c0) < (__int128)anum2 * R2)) k0.i = -1;
+    if (k1.i >= 0 && (k1.i == b.i || (__int128)aden2 * dist2(pc, c1) < (__int128)anum2 * R2)) k1.i = -1;
     if (lane == 0) {
-      a.nuc_member[base + nn] = (uint32_t)c;
+      a.nuc_member[base + nn] = (uint32_t)pc.w;
       a.nuc_R2[base + nn] = R2;
     }
     __syncwarp();
     ++nn;
+    if (m == 1) break;
   }
   if (v0) a.eslot[base + lane] = slot0;
   if (v1) a.eslot[base + lane + 32] = slot1;
@@ -1275,32 +1370,15 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
 }
 
 __global__ void __launch_bounds__(256) k_level_warp_q(LevelArgs a, const uint32_t* __restrict__ order, TierQueue* q) {
-  unsigned first, cnt;
-  tier_range(*q, 3, first, cnt);
+  const unsigned first = q->first[TIER_WARP], cnt = q->cnt[TIER_WARP];
   const int lane = threadIdx.x & 31;
   for (;;) {
     unsigned it = 0;
-    if (lane == 0) it = atomicAdd(&q->next[3], 1u);
+    if (lane == 0) it = atomicAdd(&q->next[TIER_WARP], 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= cnt) return;  // whole warps leave together
     level_warp(a, (int)order[first + it]);
   }
-}
-
-// segment sizes as descending sort keys, and the size-bin counts
-__global__ void k_seg_sizes(const uint32_t* __restrict__ seg_off, int nseg, int huge, int giant, int large, int small,
-                            uint32_t* __restrict__ key, uint32_t* __restrict__ val, unsigned* __restrict__ counts,
-                            unsigned* __restrict__ nseg_out) {
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g == 0) *nseg_out = (unsigned)nseg;
-  if (g >= nseg) return;
-  const uint32_t sz = seg_off[g + 1] - seg_off[g];
-  key[g] = 0xffffffffu - sz;
-  val[g] = (uint32_t)g;
-  if (sz > (uint32_t)huge) atomicAdd(&counts[3], 1u);
-  if (sz > (uint32_t)giant) atomicAdd(&counts[0], 1u);
-  else if (sz > (uint32_t)large) atomicAdd(&counts[1], 1u);
-  else if (sz <= (uint32_t)small) atomicAdd(&counts[2], 1u);
 }
 
 // largest g with off[g] <= k (off ascending, off[0] = 0)
@@ -1314,42 +1392,31 @@ __device__ __forceinline__ int seg_of(const uint32_t* __restrict__ off, int nseg
   return lo;
 }
 
-// global halo index of every member (or -1): one thread per member
-__global__ void k_level_halo_members(const uint32_t* __restrict__ seg_off, int nseg, const uint32_t* __restrict__ hbase,
-                                     const int* __restrict__ eslot, int* __restrict__ ehalo) {
-  const unsigned j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= seg_off[nseg]) return;
-  const int s = eslot[j];
-  ehalo[j] = s < 0 ? -1 : (int)(hbase[seg_of(seg_off, nseg, j)] + s);
-}
-
 // per-halo nucleus records: one thread per halo (halos of segment g start at
 // hbase[g])
 __global__ void k_level_halo_nuclei(const uint32_t* __restrict__ seg_off, int nseg, const uint32_t* __restrict__ hbase,
                                     const uint32_t* __restrict__ nuc_member, const long long* __restrict__ nuc_R2,
-                                    uint32_t* __restrict__ hnuc, long long* __restrict__ hR2,
-                                    uint32_t* __restrict__ hseg) {
+                                    uint32_t* __restrict__ hnuc, long long* __restrict__ hR2) {
   const unsigned h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= hbase[nseg]) return;
   const int g = seg_of(hbase, nseg, h);  // hbase ascending; segments without nuclei repeat a value
   const unsigned base = seg_off[g], q = h - hbase[g];
-  hnuc[h] = base + nuc_member[base + q];
+  hnuc[h] = nuc_member[base + q];
   hR2[h] = nuc_R2[base + q];
-  hseg[h] = (uint32_t)g;
 }
 
 }  // namespace
 
 // resident blocks per SM of the persistent level kernels (same for every
 // device of one build; queried once)
-static std::atomic<int> g_occ_l{0}, g_occ_m{0}, g_occ_w{0};
+static std::atomic<int> g_occ_l{0}, g_occ_m{0}, g_occ_s{0}, g_occ_w{0};
 // 16-CTA clusters that can be resident at once (0: that size does not fit
 // this device, and huge groups stay on 8-CTA clusters)
 static std::atomic<int> g_cl16{0};
 
 void level_prepare() {
   if (g_occ_l.load()) return;
-  int l = 0, m = 0, w = 0;
+  int l = 0, m = 0, s = 0, w = 0;
   int c16 = 0;
   if (cudaFuncSetAttribute(k_level_cluster_q<CL_HUGE_CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
       cudaSuccess) {
@@ -1362,8 +1429,10 @@ void level_prepare() {
   g_cl16.store(c16 > 0 ? c16 : 0);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&l, k_level_q<1024>, 1024, 0) != cudaSuccess || l < 1) l = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_level_q<256>, 256, 0) != cudaSuccess || m < 1) m = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s, k_level_small_q, SM_NT, 0) != cudaSuccess || s < 1) s = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&w, k_level_warp_q, 256, 0) != cudaSuccess || w < 1) w = 1;
   g_occ_m.store(m);
+  g_occ_s.store(s);
   g_occ_w.store(w);
   g_occ_l.store(l);
   cso_sm_count();
@@ -1371,23 +1440,23 @@ void level_prepare() {
 
 int level_run(const LevelArgs& a, cudaStream_t st) {
   if (a.nseg <= 0) return CSO_OK;
-  k_level<256><<<CL(a.nseg), 256, 0, st>>>(a, nullptr);
+  k_level<256><<<CL(a.nseg), 256, 0, st>>>(a);
   CSO_CUDA(cudaGetLastError());
   return CSO_OK;
 }
 
+size_t level_tiles(long long members, long long nseg) { return (size_t)(members / TILE + nseg + 2); }
+
 int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws, cudaStream_t st,
                       cudaStream_t side, cudaStream_t side2, cudaStream_t side3, cudaEvent_t fork,
-                      cudaEvent_t join, cudaEvent_t join2, cudaEvent_t join3, unsigned* host_counts) {
-  (void)host_counts;
+                      cudaEvent_t join, cudaEvent_t join2, cudaEvent_t join3) {
   if (a.nseg <= 0) return CSO_OK;
   size_t mark = ws.off;
-  uint32_t* key = ws.get<uint32_t>(a.nseg);
-  uint32_t* val = ws.get<uint32_t>(a.nseg);
-  uint32_t* key2 = ws.get<uint32_t>(a.nseg);
-  uint32_t* val2 = ws.get<uint32_t>(a.nseg);
+  int* bin = ws.get<int>(a.nseg);
+  uint32_t* rank = ws.get<uint32_t>(a.nseg);
+  uint32_t* order = ws.get<uint32_t>(a.nseg);
   TierQueue* q = ws.get<TierQueue>(1);
-  if (!key || !val || !key2 || !val2 || !q) {
+  if (!bin || !rank || !order || !q) {
     cso_set_error("workspace exhausted in the batched schedule");
     return CSO_ERR_BUDGET;
   }
@@ -1395,36 +1464,41 @@ int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws
   level_prepare();
   const int c16 = g_cl16;
   // groups above the huge bound (and the giant bound) run on 16-CTA clusters
-  // where the device holds them
-  const int huge = c16 > 0 ? std::max(sc.giant, sc.huge) : INT_MAX;
-  k_seg_sizes<<<CL(cdiv(a.nseg, 256)), 256, 0, st>>>(a.seg_off, a.nseg, huge, sc.giant, sc.large(), sc.small, key,
-                                                     val, q->count, &q->nseg);
-  // largest groups first: giants start at once, the rest fill in behind them
-  uint32_t *pk = key, *pv = val;
-  CSO_TRY(radix_sort_32(&pk, &pv, key2, val2, a.nseg, 32, ws, st));
+  // where the device holds them; the direct count of the small tier needs
+  // groups that the select would count directly too
+  TierBounds b;
+  b.huge = c16 > 0 ? std::max(sc.giant, sc.huge) : INT_MAX;
+  b.giant = sc.giant;
+  b.large = sc.large();
+  b.small = sc.small;
+  b.medium = a.small_n >= COUNT_N ? std::max(b.small, COUNT_N) : b.small;
+  k_seg_bins<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(a.seg_off, a.peaks.off, a.nseg, b, bin, rank, a.nnuc, q);
+  k_seg_order<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(bin, rank, a.nseg, order, q);
   CSO_CUDA(cudaGetLastError());
-  // persistent grids sized to the device; blocks of a bin leave when its
+  // persistent grids sized to the device; blocks of a tier leave when its
   // queue is empty
-  const int occ_l = g_occ_l, occ_m = g_occ_m, occ_w = g_occ_w;
+  const int occ_l = g_occ_l, occ_m = g_occ_m, occ_s = g_occ_s, occ_w = g_occ_w;
   const int sms = cso_sm_count();
   const int n_clusters = sms / CL_CS > 0 ? sms / CL_CS : 1;
   const int nseg = a.nseg;
-  // no bin can hold more groups than there are: grids never exceed nseg
+  // no tier can hold more groups than there are: grids never exceed nseg
   auto cap = [nseg](long long g) { return (unsigned)(g < nseg ? g : nseg); };
   CSO_CUDA(cudaEventRecord(fork, st));
   CSO_CUDA(cudaStreamWaitEvent(side, fork, 0));
-  k_level_cluster_q<CL_CS><<<CL(cap(n_clusters) * CL_CS), CL_NT, 0, side>>>(a, pv, q, 0);
+  k_level_cluster_q<CL_CS><<<CL(cap(n_clusters) * CL_CS), CL_NT, 0, side>>>(a, order, q, TIER_GIANT);
   CSO_CUDA(cudaGetLastError());
   if (c16 > 0) {
     // at most two: huge groups are few, and every 16-CTA cluster holds 16 SMs
     CSO_CUDA(cudaStreamWaitEvent(side3, fork, 0));
-    k_level_cluster_q<CL_HUGE_CS><<<CL(cap(c16 < 2 ? c16 : 2) * CL_HUGE_CS), CL_NT, 0, side3>>>(a, pv, q, 4);
+    k_level_cluster_q<CL_HUGE_CS><<<CL(cap(c16 < 2 ? c16 : 2) * CL_HUGE_CS), CL_NT, 0, side3>>>(a, order, q, TIER_HUGE);
     CSO_CUDA(cudaGetLastError());
   }
   CSO_CUDA(cudaStreamWaitEvent(side2, fork, 0));
-  k_level_q<1024><<<CL(cap((long long)sms * occ_l)), 1024, 0, side2>>>(a, pv, q, 1);
-  k_level_q<256><<<CL(cap((long long)sms * occ_m)), 256, 0, st>>>(a, pv, q, 2);
-  k_level_warp_q<<<CL(cdiv(cap((long long)sms * occ_w * 8), 8)), 256, 0, st>>>(a, pv, q);
+  k_level_q<1024><<<CL(cap((long long)sms * occ_l)), 1024, 0, side2>>>(a, order, q, TIER_LARGE);
+  k_level_q<256><<<CL(cap((long long)sms * occ_m)), 256, 0, st>>>(a, order, q, TIER_MEDIUM);
+  if (b.medium > b.small)
+    k_level_small_q<<<CL(cap((long long)sms * occ_s)), SM_NT, 0, st>>>(a, order, q);
+  k_level_warp_q<<<CL(cdiv(cap((long long)sms * occ_w * 8), 8)), 256, 0, st>>>(a, order, q);
   CSO_CUDA(cudaGetLastError());
   CSO_CUDA(cudaEventRecord(join, side));
   CSO_CUDA(cudaStreamWaitEvent(st, join, 0));
@@ -1438,16 +1512,10 @@ int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws
   return CSO_OK;
 }
 
-int level_halo(int nseg, const uint32_t* seg_off, const uint32_t* nnuc, const uint32_t* hbase, const int* eslot,
-               const uint32_t* nuc_member, const long long* nuc_R2, int* ehalo, uint32_t* hnuc, long long* hR2,
-               uint32_t* hseg, long long n_members, long long n_halos, cudaStream_t st) {
-  (void)nnuc;
-  if (nseg <= 0) return CSO_OK;
-  if (n_members > 0)
-    k_level_halo_members<<<CL(cdiv(n_members, 256)), 256, 0, st>>>(seg_off, nseg, hbase, eslot, ehalo);
-  if (n_halos > 0)
-    k_level_halo_nuclei<<<CL(cdiv(n_halos, 256)), 256, 0, st>>>(seg_off, nseg, hbase, nuc_member, nuc_R2, hnuc, hR2,
-                                                                hseg);
+int level_halo(int nseg, const uint32_t* seg_off, const uint32_t* hbase, const uint32_t* nuc_member,
+               const long long* nuc_R2, uint32_t* hnuc, long long* hR2, long long n_halos, cudaStream_t st) {
+  if (nseg <= 0 || n_halos <= 0) return CSO_OK;
+  k_level_halo_nuclei<<<CL(cdiv(n_halos, 256)), 256, 0, st>>>(seg_off, nseg, hbase, nuc_member, nuc_R2, hnuc, hR2);
   CSO_CUDA(cudaGetLastError());
   return CSO_OK;
 }

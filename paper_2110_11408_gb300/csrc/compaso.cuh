@@ -1,6 +1,7 @@
 // CompaSO level kernels (compaso.cu).
 #pragma once
 #include "cells.cuh"
+#include "peaks.cuh"
 
 // constants of the exact predicate n^2 u^6 < K d^3
 struct PredConst {
@@ -18,24 +19,16 @@ PredConst make_pred_const(double K, long long u);
 struct LevelArgs {
   int nseg;
   const uint32_t* seg_off;  // nseg + 1 offsets into the element arrays
-  const int4* epos;         // member positions, key order within a segment
-  const long long* esig;    // kernel sums (descending within a segment)
-  const uint32_t* egs;      // cell-sorted index of each member
-  long long T_min;
+  const int4* epos;         // member positions, cell order within a segment
   PredConst pc;
   int alpha_num, alpha_den, roche_num, roche_den;
-  int* eslot;               // out: nucleus ordinal within the segment, or -1
+  PeakList peaks;           // nucleus candidates of every segment
+  int* eslot;               // out: nucleus ordinal within the segment, or -1 (preset)
   long long* edold;         // scratch: squared distance to the current nucleus
-  uint8_t* einel;           // scratch: ineligible flags
   long long* ed;            // scratch: distances to the nucleus being processed
-  // cell-sorted particle data for the local-peak test of step 2
-  CellGrid grid;
-  const int4* spos;
-  const long long* ssig;
-  const uint64_t* sid;
-  const int* slab;          // group label per cell-sorted particle (-1: none)
-  uint32_t b2;
-  uint32_t* nuc_member;     // out: [seg_off + q] member offset of nucleus q
+  int4* tlo;                // scratch: tile boxes, level_tiles() entries each
+  int4* thi;
+  uint32_t* nuc_member;     // out: [seg_off + q] cell-sorted index of nucleus q
   long long* nuc_R2;        // out: [seg_off + q] its squared radius
   uint32_t* nnuc;           // out: nuclei per segment
   unsigned long long* work; // optional: sum over nuclei of the segment size
@@ -60,15 +53,16 @@ struct LevelSchedule {
 };
 
 int level_run(const LevelArgs& a, cudaStream_t st);
+// entries of the tile-box arrays for so many members and segments
+size_t level_tiles(long long members, long long nseg);
 // one-time set-up of the batched schedule's launch sizes (occupancy queries),
 // kept out of stream capture
 void level_prepare();
 int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws, cudaStream_t st,
                       cudaStream_t side, cudaStream_t side2, cudaStream_t side3, cudaEvent_t fork,
-                      cudaEvent_t join, cudaEvent_t join2, cudaEvent_t join3, unsigned* host_counts);
-// ehalo[j] = global halo of member j (hbase[g] + its nucleus ordinal, or -1)
-// and the nucleus records of every halo; n_members = seg_off[nseg] and
-// n_halos = hbase[nseg] as the host knows them (launch sizes)
-int level_halo(int nseg, const uint32_t* seg_off, const uint32_t* nnuc, const uint32_t* hbase, const int* eslot,
-               const uint32_t* nuc_member, const long long* nuc_R2, int* ehalo, uint32_t* hnuc, long long* hR2,
-               uint32_t* hseg, long long n_members, long long n_halos, cudaStream_t st);
+                      cudaEvent_t join, cudaEvent_t join2, cudaEvent_t join3);
+// the nucleus records of every halo (halos of segment g start at hbase[g]):
+// its cell-sorted index and squared radius; n_halos = hbase[nseg] as the host
+// knows it (launch size)
+int level_halo(int nseg, const uint32_t* seg_off, const uint32_t* hbase, const uint32_t* nuc_member,
+               const long long* nuc_R2, uint32_t* hnuc, long long* hR2, long long n_halos, cudaStream_t st);

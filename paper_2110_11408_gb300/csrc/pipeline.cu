@@ -4,11 +4,11 @@
 //   bin      counting sort of particles into the dense cell table
 //   density  Sigma per particle (Eq. 1)
 //   fof      L0 groups over dense particles (Sec. 2.2.1)
-//   gather   dense particles sorted by (L0 group, Sigma desc, id asc)
-//   level1   CompaSO L1 per L0 group (steps 1-4; the local-peak test of
-//            step 2 runs inside, only for eligible candidates): a block per
-//            group, or by size a warp, block or thread-block cluster
-//   prep2    members of each L1 halo in key order and their L1 labels
+//   gather   dense particles grouped by L0 group, cell order within one
+//   level1   CompaSO L1 per L0 group: the density peaks of every group (step
+//            2), then the nucleus loop (steps 1, 3 and 4) over them: a block
+//            per group, or by size a warp, block or thread-block cluster
+//   prep2    members of each L1 halo and their L1 labels
 //   level2   CompaSO L2 per L1 halo, scheduled as level1
 //   halos    per-halo statistics and the catalogue (optionally the radial
 //            statistics and the shrinking-sphere centre)
@@ -48,17 +48,22 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
   return v;
 }
 
-// compact the dense particles; block maxima of Sigma and id, one atomic per block
+// compact the dense particles taking part, each with its group's index; block
+// maxima of Sigma and id, one atomic per block
 __global__ void __launch_bounds__(256) k_compact_dense(const int* __restrict__ root, const uint8_t* __restrict__ select,
                                                        int n, const uint32_t* __restrict__ dscan,
+                                                       const uint32_t* __restrict__ rscan,
                                                        const long long* __restrict__ sigma,
                                                        const uint64_t* __restrict__ sid, uint32_t* __restrict__ dl,
-                                                       Meta* meta) {
+                                                       uint32_t* __restrict__ grp, Meta* meta) {
   __shared__ unsigned long long sh[8];
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long ms = 0, mid = 0;
-  if (s < n && root[s] >= 0 && (!select || select[s])) {
-    dl[dscan[s]] = (uint32_t)s;
+  const int r = s < n ? root[s] : -1;
+  if (r >= 0 && (!select || select[s])) {
+    const uint32_t k = dscan[s];
+    dl[k] = (uint32_t)s;
+    grp[k] = rscan[r];
     ms = (unsigned long long)sigma[s];
     mid = (unsigned long long)sid[s];
   }
@@ -70,77 +75,6 @@ __global__ void __launch_bounds__(256) k_compact_dense(const int* __restrict__ r
   }
 }
 
-// key = group | (Sigma_max - Sigma) | id, packed low to high: id, Sigma', group
-__global__ void k_make_keys(const uint32_t* __restrict__ dl, int nd, const int* __restrict__ root,
-                            const uint32_t* __restrict__ rscan, const long long* __restrict__ sigma,
-                            const uint64_t* __restrict__ sid, unsigned long long sigma_max, int bits_id,
-                            int bits_sig, uint64_t* __restrict__ khi, uint64_t* __restrict__ klo,
-                            uint32_t* __restrict__ val) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  uint32_t s = dl[k];
-  unsigned __int128 g = rscan[root[s]];
-  unsigned __int128 sp = sigma_max - (unsigned long long)sigma[s];
-  unsigned __int128 key = (g << (bits_sig + bits_id)) | (sp << bits_id) | (unsigned __int128)sid[s];
-  khi[k] = (uint64_t)(key >> 64);
-  klo[k] = (uint64_t)key;
-  val[k] = s;
-}
-
-// (group, Sigma desc) in one 64-bit key; the id tie-break is settled after
-// the sort by k_tie_fix
-__global__ void k_make_keys64(const uint32_t* __restrict__ dl, int nd, const int* __restrict__ root,
-                              const uint32_t* __restrict__ rscan, const long long* __restrict__ sigma,
-                              unsigned long long sigma_max, int bits_sig, uint64_t* __restrict__ key,
-                              uint32_t* __restrict__ val) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  uint32_t s = dl[k];
-  key[k] = ((uint64_t)rscan[root[s]] << bits_sig) | (sigma_max - (unsigned long long)sigma[s]);
-  val[k] = s;
-}
-
-// Runs of equal (group, Sigma) keys, ordered by id: the first thread of a run
-// sorts it by insertion (runs are almost always single elements).  A run
-// longer than TIE_RUN_MAX is left alone and raises *overflow, and the caller
-// sorts again with the id inside the key.
-constexpr int TIE_RUN_MAX = 64;
-
-__global__ void k_tie_fix(const uint64_t* __restrict__ key, uint32_t* __restrict__ val, int nd,
-                          const uint64_t* __restrict__ sid, int* __restrict__ overflow) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k + 1 >= nd || key[k + 1] != key[k] || (k > 0 && key[k - 1] == key[k])) return;
-  int e = k + 1;
-  while (e < nd && key[e] == key[k] && e - k <= TIE_RUN_MAX) ++e;
-  if (e - k > TIE_RUN_MAX) {
-    atomicExch(overflow, 1);
-    return;
-  }
-  for (int i = k + 1; i < e; ++i) {
-    const uint32_t v = val[i];
-    const uint64_t id = sid[v];
-    int j = i - 1;
-    while (j >= k && sid[val[j]] > id) {
-      val[j + 1] = val[j];
-      --j;
-    }
-    val[j + 1] = v;
-  }
-}
-
-__global__ void k_seg_bounds128(const uint64_t* __restrict__ khi, const uint64_t* __restrict__ klo, int nd,
-                                int gshift, int nseg, uint32_t* __restrict__ seg_off) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  auto grp = [&](int i) -> unsigned long long {
-    unsigned __int128 key = ((unsigned __int128)(khi ? khi[i] : 0) << 64) | klo[i];
-    return (unsigned long long)(key >> gshift);
-  };
-  unsigned long long g = grp(k);
-  if (k == 0 || grp(k - 1) != g) seg_off[g] = k;
-  if (k == nd - 1) seg_off[nseg] = nd;
-}
-
 __global__ void k_seg_bounds32(const uint32_t* __restrict__ key, int m, int nseg, uint32_t* __restrict__ seg_off) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= m) return;
@@ -149,43 +83,34 @@ __global__ void k_seg_bounds32(const uint32_t* __restrict__ key, int m, int nseg
   if (k == m - 1) seg_off[nseg] = m;
 }
 
-__global__ void k_gather1(const uint32_t* __restrict__ val, int nd, const int4* __restrict__ spos,
-                          const long long* __restrict__ sigma, const uint64_t* __restrict__ sid,
-                          int4* __restrict__ epos, long long* __restrict__ esig, uint64_t* __restrict__ eid) {
+__global__ void k_gather_pos(const uint32_t* __restrict__ gs, int nd, const int4* __restrict__ spos,
+                             int4* __restrict__ epos) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  uint32_t s = val[k];
-  epos[k] = spos[s];
-  esig[k] = sigma[s];
-  eid[k] = sid[s];
+  if (k < nd) epos[k] = spos[gs[k]];
 }
 
-__global__ void k_flag_assigned(const int* __restrict__ ehalo, int nd, uint32_t* __restrict__ f) {
+__global__ void k_flag_assigned(const int* __restrict__ eslot, int nd, uint32_t* __restrict__ f) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nd) f[k] = ehalo[k] >= 0;
+  if (k < nd) f[k] = eslot[k] >= 0;
 }
 
-__global__ void k_compact_assigned(const int* __restrict__ ehalo, int nd, const uint32_t* __restrict__ scan,
+// the members of L1 haloes, each with its halo's index; their L1 labels, on
+// the device by cell-sorted index and (optional) in input order
+__global__ void k_compact_assigned(const int* __restrict__ eslot, const uint32_t* __restrict__ grp,
+                                   const uint32_t* __restrict__ hbase, int nd, const uint32_t* __restrict__ scan,
                                    const uint32_t* __restrict__ gs, uint32_t* __restrict__ key,
-                                   uint32_t* __restrict__ val, int* __restrict__ lab1) {
+                                   uint32_t* __restrict__ val, int* __restrict__ lab1, const int4* __restrict__ spos,
+                                   const uint32_t* __restrict__ hnuc, const uint64_t* __restrict__ sid,
+                                   uint64_t* __restrict__ ol1) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nd) return;
-  int h = ehalo[k];
-  if (h < 0) return;
-  key[scan[k]] = (uint32_t)h;
-  val[scan[k]] = (uint32_t)k;
-  lab1[gs[k]] = h;
-}
-
-__global__ void k_gather2(const uint32_t* __restrict__ ek, int m, const int4* __restrict__ epos,
-                          const long long* __restrict__ esig, const uint32_t* __restrict__ gs,
-                          int4* __restrict__ epos2, long long* __restrict__ esig2, uint32_t* __restrict__ egs2) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  uint32_t k = ek[i];
-  epos2[i] = epos[k];
-  esig2[i] = esig[k];
-  egs2[i] = gs[k];
+  const int q = eslot[k];
+  if (q < 0) return;
+  const uint32_t h = hbase[grp[k]] + (uint32_t)q, s = gs[k], d = scan[k];
+  key[d] = h;
+  val[d] = s;
+  lab1[s] = (int)h;
+  if (ol1) ol1[spos[s].w] = sid[hnuc[h]];
 }
 
 __global__ void k_fill_u64(uint64_t* p, long long n, uint64_t v) {
@@ -208,27 +133,19 @@ __global__ void k_out_cells(const uint32_t* __restrict__ inv, int n, const long 
   }
 }
 
-__global__ void k_out_l1(const int* __restrict__ ehalo, int nd, const uint32_t* __restrict__ gs,
-                         const int4* __restrict__ spos, const uint32_t* __restrict__ hnuc,
-                         const uint64_t* __restrict__ eid, uint64_t* __restrict__ ol1) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  int h = ehalo[k];
-  if (h >= 0) ol1[spos[gs[k]].w] = eid[hnuc[h]];
-}
-
-__global__ void k_out_l2(const int* __restrict__ ehalo2, int m, const uint32_t* __restrict__ ek2,
-                         const uint32_t* __restrict__ gs, const int4* __restrict__ spos,
-                         const uint32_t* __restrict__ hnuc2, const uint64_t* __restrict__ eid,
-                         uint64_t* __restrict__ ol2, unsigned* __restrict__ h2size) {
+__global__ void k_out_l2(const int* __restrict__ eslot2, const uint32_t* __restrict__ ehal2,
+                         const uint32_t* __restrict__ hbase2, int m, const int4* __restrict__ epos2,
+                         const uint32_t* __restrict__ hnuc2,
+                         const uint64_t* __restrict__ sid, uint64_t* __restrict__ ol2, unsigned* __restrict__ h2size) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
-  int h = ehalo2[i];
+  const int q = eslot2[i];
+  const int h = q < 0 ? -1 : (int)hbase2[ehal2[i]] + q;
   // one atomic per distinct halo in the warp (members of a halo are mostly adjacent)
   const unsigned peers = __match_any_sync(__activemask(), h);
   if (h >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h2size[h], (unsigned)__popc(peers));
   if (h < 0) return;
-  if (ol2) ol2[spos[gs[ek2[i]]].w] = eid[ek2[hnuc2[h]]];
+  if (ol2) ol2[epos2[i].w] = sid[hnuc2[h]];
 }
 
 __device__ __forceinline__ int mi(int v) {
@@ -258,9 +175,8 @@ __device__ __forceinline__ double wrap_box(double c) {
 // sum exactly in 32 bits.
 constexpr int SUM_ITEMS = 16;
 __global__ void __launch_bounds__(256) k_summary_sums(const uint32_t* __restrict__ ehal2, int na,
-                                                      const int4* __restrict__ epos2, const int* __restrict__ ehalo2,
-                                                      const uint32_t* __restrict__ hnuc, const int4* __restrict__ epos,
-                                                      const uint32_t* __restrict__ nnuc2,
+                                                      const int4* __restrict__ epos2, const int* __restrict__ eslot2,
+                                                      const uint32_t* __restrict__ hnuc, const int4* __restrict__ spos,
                                                       const uint32_t* __restrict__ hbase2,
                                                       const uint32_t* __restrict__ hnuc2,
                                                       unsigned long long* __restrict__ acc) {
@@ -275,12 +191,12 @@ __global__ void __launch_bounds__(256) k_summary_sums(const uint32_t* __restrict
     int s[6] = {0, 0, 0, 0, 0, 0};
     if (v) {
       const int4 q = epos2[i];
-      const int4 pn = epos[hnuc[h]];
+      const int4 pn = spos[hnuc[h]];
       s[0] = mi(q.x - pn.x);
       s[1] = mi(q.y - pn.y);
       s[2] = mi(q.z - pn.z);
-      if (nnuc2[h] > 0 && ehalo2[i] == (int)hbase2[h]) {
-        const int4 p2 = epos2[hnuc2[hbase2[h]]];
+      if (eslot2[i] == 0) {  // the halo's first L2 nucleus
+        const int4 p2 = spos[hnuc2[hbase2[h]]];
         s[3] = mi(q.x - p2.x);
         s[4] = mi(q.y - p2.y);
         s[5] = mi(q.z - p2.z);
@@ -313,40 +229,39 @@ __global__ void __launch_bounds__(256) k_summary_sums(const uint32_t* __restrict
       if (run[k]) atomicAdd(&acc[6 * (size_t)open_h + k], (unsigned long long)run[k]);
 }
 
-__global__ void k_summary(const uint32_t* __restrict__ seg2, int H1, const int4* __restrict__ epos2,
-                          const uint32_t* __restrict__ hnuc, const long long* __restrict__ hR2,
-                          const int4* __restrict__ epos, const uint64_t* __restrict__ eid,
-                          const uint32_t* __restrict__ gs, const int* __restrict__ root,
+__global__ void k_summary(const uint32_t* __restrict__ seg2, int H1, const uint32_t* __restrict__ hnuc,
+                          const long long* __restrict__ hR2, const int4* __restrict__ spos,
+                          const uint64_t* __restrict__ sid, const int* __restrict__ root,
                           const unsigned long long* __restrict__ minid, const uint32_t* __restrict__ nnuc2,
                           const uint32_t* __restrict__ hbase2, const uint32_t* __restrict__ hnuc2,
                           const unsigned* __restrict__ h2size, const unsigned long long* __restrict__ acc,
-                          const uint32_t* __restrict__ ek2, double inv_u, int np_min, int x0,
+                          double inv_u, int np_min, int x0,
                           cso_halo* __restrict__ rows, uint32_t* __restrict__ keep) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= H1) return;
   const int n = (int)(seg2[h + 1] - seg2[h]);
   const uint32_t kn = hnuc[h];
-  const int4 pn = epos[kn];
+  const int4 pn = spos[kn];
   const int nl2 = (int)nnuc2[h];
   const int first2 = (int)hbase2[h];
   const long long sx = (long long)acc[6 * (size_t)h], sy = (long long)acc[6 * (size_t)h + 1],
                   sz = (long long)acc[6 * (size_t)h + 2], tx = (long long)acc[6 * (size_t)h + 3],
                   ty = (long long)acc[6 * (size_t)h + 4], tz = (long long)acc[6 * (size_t)h + 5];
   cso_halo r;
-  r.nucleus_id = eid[kn];
+  r.nucleus_id = sid[kn];
   r.N = n;
   r.R2 = hR2[h];
   r.R_delta = sqrt((double)r.R2) * inv_u;
   r.com[0] = wrap_box((double)((pn.x + x0) & (CSO_BOX - 1)) + (double)sx / (double)n);
   r.com[1] = wrap_box((double)pn.y + (double)sy / (double)n);
   r.com[2] = wrap_box((double)pn.z + (double)sz / (double)n);
-  r.l0_id = minid[root[gs[kn]]];
+  r.l0_id = minid[root[kn]];
   r.n_l2 = nl2;
   for (int k = 0; k < 5; ++k) r.l2_top5_N[k] = 0;
   if (nl2 > 0) {
-    const int4 p2 = epos2[hnuc2[first2]];
+    const int4 p2 = spos[hnuc2[first2]];
     long long n2 = h2size[first2];
-    r.l2max_id = eid[ek2[hnuc2[first2]]];
+    r.l2max_id = sid[hnuc2[first2]];
     r.l2max_N = n2;
     r.l2max_com[0] = wrap_box((double)((p2.x + x0) & (CSO_BOX - 1)) + (double)tx / (double)n2);
     r.l2max_com[1] = wrap_box((double)p2.y + (double)ty / (double)n2);
@@ -380,14 +295,14 @@ __global__ void k_catalogue_keys(const cso_halo* __restrict__ rows, const uint32
 
 // rows in nucleus-id order; optionally the input index of each row's nucleus
 __global__ void k_catalogue_write(const cso_halo* __restrict__ rows, const uint32_t* __restrict__ order, int m,
-                                  const uint32_t* __restrict__ hnuc, const int4* __restrict__ epos,
+                                  const uint32_t* __restrict__ hnuc, const int4* __restrict__ spos,
                                   cso_halo* __restrict__ out, uint32_t* __restrict__ out_w,
                                   const cso_radial* __restrict__ rad, cso_radial* __restrict__ rad_out) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   const uint32_t h = order[i];
   out[i] = rows[h];
-  if (out_w) out_w[i] = (uint32_t)epos[hnuc[h]].w;
+  if (out_w) out_w[i] = (uint32_t)spos[hnuc[h]].w;
   if (rad_out) rad_out[i] = rad[h];
 }
 
@@ -401,11 +316,10 @@ int readback(cso_ctx* c, const void* dev, size_t bytes) {
 
 }  // namespace
 
-int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched, unsigned* host_counts) {
+int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched) {
   cudaStream_t st = c->stream;
   if (!(c->flags & CSO_FLAG_GRAPH))
-    return level_run_batched(L, sched, c->ws, st, c->side, c->side2, c->side3, c->fork, c->join, c->join2, c->join3,
-                             host_counts);
+    return level_run_batched(L, sched, c->ws, st, c->side, c->side2, c->side3, c->fork, c->join, c->join2, c->join3);
   for (int i = 0; i < CSO_LEVEL_GRAPHS; ++i) {
     LevelGraph& G = c->graphs[i];
     if (G.exec && G.giant == sched.giant && G.small == sched.small && G.huge == sched.huge &&
@@ -420,7 +334,7 @@ int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched, unsi
   level_prepare();
   CSO_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   const int rc = level_run_batched(L, sched, c->ws, st, c->side, c->side2, c->side3, c->fork, c->join, c->join2,
-                                   c->join3, host_counts);
+                                   c->join3);
   cudaGraph_t graph = nullptr;
   const cudaError_t e = cudaStreamEndCapture(st, &graph);
   if (rc != CSO_OK) {
@@ -464,7 +378,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
     cso_set_error("workspace exhausted (%s)", #name);    \
     return CSO_ERR_BUDGET;                               \
   }
-  // ---- gather: dense particles by (group, Sigma desc, id asc) ----
+  // ---- gather: dense particles by group ----
   S.mark("gather");
   ALLOC(uint32_t, dscan, n + 1);
   ALLOC(uint32_t, rscan, n + 1);
@@ -472,7 +386,8 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   CSO_TRY(scan_u32(dscan, n, dscan + n, ws, st));
   CSO_TRY(scan_u32(rscan, n, rscan + n, ws, st));
   ALLOC(uint32_t, dl, n);
-  k_compact_dense<<<G1(n)>>>(root, gi.select, N, dscan, sigma, sid, dl, meta);
+  ALLOC(uint32_t, grp, n);
+  k_compact_dense<<<G1(n)>>>(root, gi.select, N, dscan, rscan, sigma, sid, dl, grp, meta);
   CSO_CUDA(cudaGetLastError());
   // counters: n_dense, G, sigma_max, id_max, bad
   {
@@ -503,54 +418,31 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
     cso_set_error("sort key of %d bits exceeds 128", bits_id + bits_sig + bits_g);
     return CSO_ERR_ARG;
   }
-  ALLOC(uint64_t, khi, nd);
-  ALLOC(uint64_t, klo, nd);
-  ALLOC(uint32_t, kval, nd);
-  ALLOC(uint64_t, khi2, nd);
-  ALLOC(uint64_t, klo2, nd);
-  ALLOC(uint32_t, kval2, nd);
+  ALLOC(uint32_t, dl2, nd);
+  ALLOC(uint32_t, grp2, nd);
   ALLOC(uint32_t, seg1, G + 1);
   ALLOC(int4, epos, nd);
-  ALLOC(long long, esig, nd);
-  ALLOC(uint64_t, eid, nd);
-  uint32_t* gs = kval;
+  uint32_t *gs = dl, *gseg = grp;  // cell-sorted index and group of every member
   if (nd > 0) {
-    // (group, Sigma desc) fits one 64-bit key in every box the cell table
-    // admits: sort by it, then order the rare runs of equal sums by id
-    bool full = bits_sig + bits_g > 64;
-    uint64_t *ph = nullptr, *pl = klo;
-    uint32_t* pv = kval;
-    if (!full) {
-      k_make_keys64<<<G1(nd)>>>(dl, nd, root, rscan, sigma, hm.sigma_max, bits_sig, klo, kval);
-      CSO_TRY(radix_sort_128(&ph, &pl, &pv, nullptr, klo2, kval2, nd, bits_sig + bits_g, ws, st));
-      int* overflow = &meta->tie_overflow;
-      k_tie_fix<<<G1(nd)>>>(pl, pv, nd, sid, overflow);
-      CSO_CUDA(cudaMemcpyAsync(c->pinned, overflow, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CSO_CUDA(cudaStreamSynchronize(st));
-      full = *(int*)c->pinned != 0;
-      if (full) CSO_CUDA(cudaMemsetAsync(overflow, 0, sizeof(int), st));
-      else k_seg_bounds128<<<G1(nd)>>>(nullptr, pl, nd, bits_sig, G, seg1);
-    }
-    if (full) {
-      k_make_keys<<<G1(nd)>>>(dl, nd, root, rscan, sigma, sid, hm.sigma_max, bits_id, bits_sig, khi, klo, kval);
-      ph = khi;
-      pl = klo;
-      pv = kval;
-      int bits = bits_id + bits_sig + bits_g;
-      CSO_TRY(radix_sort_128(&ph, &pl, &pv, khi2, klo2, kval2, nd, bits, ws, st));
-      k_seg_bounds128<<<G1(nd)>>>(bits > 64 ? ph : nullptr, pl, nd, bits_sig + bits_id, G, seg1);
-    }
-    gs = pv;
-    k_gather1<<<G1(nd)>>>(gs, nd, spos, sigma, sid, epos, esig, eid);
+    CSO_TRY(radix_sort_32(&gseg, &gs, grp2, dl2, nd, bits_g, ws, st));
+    k_seg_bounds32<<<G1(nd)>>>(gseg, nd, G, seg1);
+    k_gather_pos<<<G1(nd)>>>(gs, nd, spos, epos);
     CSO_CUDA(cudaGetLastError());
   }
 
   // ---- level1 ----
   S.mark("level1");
+  ALLOC(int, beater, n);
+  PeakArgs pk{g, spos, sigma, sid, root, (uint32_t)p->b2, N};
+  PeakList peaks;
+  CSO_TRY(peaks_find(pk, gs, gseg, nd, G, p->T_min_L1, p->T_min_L1 < p->T_min_L2 ? p->T_min_L1 : p->T_min_L2, true,
+                     beater, peaks, ws, st));
   ALLOC(int, eslot, nd);
   ALLOC(long long, edold, nd);
-  ALLOC(uint8_t, einel, nd);
   ALLOC(long long, ed, nd);
+  ALLOC(int4, tlo, level_tiles(nd, G));
+  ALLOC(int4, thi, level_tiles(nd, G));
+  CSO_CUDA(cudaMemsetAsync(eslot, 0xff, sizeof(int) * (size_t)nd, st));
   ALLOC(uint32_t, nucm, nd);
   ALLOC(long long, nucR2, nd);
   ALLOC(uint32_t, nnuc, G + 1);
@@ -558,9 +450,6 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   L1.nseg = G;
   L1.seg_off = seg1;
   L1.epos = epos;
-  L1.esig = esig;
-  L1.egs = gs;
-  L1.T_min = p->T_min_L1;
   L1.pc = make_pred_const(p->K_L1, (long long)p->l_mean_grid);
   const bool radial_bins = (c->flags & CSO_FLAG_RADIAL_BINS) != 0;
   // radial bins of sqrt(3)/3 cell sides (cells of 2^21 / nc grid units)
@@ -571,16 +460,12 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   L1.alpha_den = p->alpha_den;
   L1.roche_num = p->roche_num;
   L1.roche_den = p->roche_den;
+  L1.peaks = peaks;
   L1.eslot = eslot;
   L1.edold = edold;
-  L1.einel = einel;
   L1.ed = ed;
-  L1.grid = g;
-  L1.spos = spos;
-  L1.ssig = sigma;
-  L1.sid = sid;
-  L1.slab = root;
-  L1.b2 = (uint32_t)p->b2;
+  L1.tlo = tlo;
+  L1.thi = thi;
   L1.nuc_member = nucm;
   L1.nuc_R2 = nucR2;
   L1.nnuc = nnuc;
@@ -591,17 +476,15 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   L1.nb = stress ? 16 : 1024;
   const bool batched = (c->flags & CSO_FLAG_BATCHED) != 0;
   const LevelSchedule sched = c->sched;
-  unsigned* hcounts = (unsigned*)(c->pinned + 32);
-  if (batched) CSO_TRY(level_stage(c, L1, sched, hcounts));
+  if (batched) CSO_TRY(level_stage(c, L1, sched));
   else CSO_TRY(level_run(L1, st));
 
-  // ---- prep2: L1 haloes, their members in key order, peaks within L1 ----
+  // ---- prep2: L1 haloes, their members and labels ----
   S.mark("prep2");
   ALLOC(uint32_t, hbase, G + 1);
   if (G > 0) CSO_CUDA(cudaMemcpyAsync(hbase, nnuc, sizeof(uint32_t) * G, cudaMemcpyDeviceToDevice, st));
   CSO_TRY(scan_u32(hbase, G, hbase + G, ws, st));
   ALLOC(uint32_t, aflag, nd + 1);
-  ALLOC(int, ehalo, nd);
   if (nd > 0) k_flag_assigned<<<G1(nd)>>>(eslot, nd, aflag);  // slot >= 0 <=> assigned
   CSO_TRY(scan_u32(aflag, nd, aflag + nd, ws, st));
   CSO_CUDA(cudaMemcpyAsync(c->pinned, hbase + G, 4, cudaMemcpyDeviceToHost, st));
@@ -612,8 +495,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   c->stats[3] = H1;
   ALLOC(uint32_t, hnuc, H1);
   ALLOC(long long, hR2, H1);
-  ALLOC(uint32_t, hseg, H1);
-  CSO_TRY(level_halo(G, seg1, nnuc, hbase, eslot, nucm, nucR2, ehalo, hnuc, hR2, hseg, nd, H1, st));
+  CSO_TRY(level_halo(G, seg1, hbase, nucm, nucR2, hnuc, hR2, H1, st));
   ALLOC(int, lab1, n);
   CSO_CUDA(cudaMemsetAsync(lab1, 0xff, sizeof(int) * n, st));
   ALLOC(uint32_t, akey, na);
@@ -621,25 +503,28 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   ALLOC(uint32_t, akey2, na);
   ALLOC(uint32_t, aval2, na);
   ALLOC(uint32_t, seg2, H1 + 1);
-  uint32_t* ek2 = aval;
-  uint32_t* ehal2 = akey;  // L1 halo of each member element, ascending
-  if (nd > 0) k_compact_assigned<<<G1(nd)>>>(ehalo, nd, aflag, gs, akey, aval, lab1);
+  uint32_t* egs2 = aval;   // cell-sorted index of each member
+  uint32_t* ehal2 = akey;  // its L1 halo, ascending
+  if (nd > 0)
+    k_compact_assigned<<<G1(nd)>>>(eslot, gseg, hbase, nd, aflag, gs, akey, aval, lab1, spos, hnuc, sid, ol1);
   if (na > 0) {
     uint32_t *pk = akey, *pv = aval;
     CSO_TRY(radix_sort_32(&pk, &pv, akey2, aval2, na, bit_length_u64(H1 > 0 ? H1 - 1 : 0), ws, st));
     k_seg_bounds32<<<G1(na)>>>(pk, na, H1, seg2);
-    ek2 = pv;
+    egs2 = pv;
     ehal2 = pk;
   }
   ALLOC(int4, epos2, na);
-  ALLOC(long long, esig2, na);
-  ALLOC(uint32_t, egs2, na);
-  if (na > 0) k_gather2<<<G1(na)>>>(ek2, na, epos, esig, gs, epos2, esig2, egs2);
+  if (na > 0) k_gather_pos<<<G1(na)>>>(egs2, na, spos, epos2);
   CSO_CUDA(cudaGetLastError());
 
   // ---- level2 ----
   S.mark("level2");
+  pk.slab = lab1;
+  PeakList peaks2;
+  CSO_TRY(peaks_find(pk, egs2, ehal2, na, H1, p->T_min_L2, p->T_min_L2, false, beater, peaks2, ws, st));
   ALLOC(int, eslot2, na);
+  CSO_CUDA(cudaMemsetAsync(eslot2, 0xff, sizeof(int) * (size_t)na, st));
   ALLOC(uint32_t, nucm2, na);
   ALLOC(long long, nucR22, na);
   ALLOC(uint32_t, nnuc2, H1 + 1);
@@ -647,10 +532,11 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   L2.nseg = H1;
   L2.seg_off = seg2;
   L2.epos = epos2;
-  L2.esig = esig2;
-  L2.egs = egs2;
-  L2.slab = lab1;
-  L2.T_min = p->T_min_L2;
+  L2.peaks = peaks2;
+  ALLOC(int4, tlo2, level_tiles(na, H1));
+  ALLOC(int4, thi2, level_tiles(na, H1));
+  L2.tlo = tlo2;
+  L2.thi = thi2;
   L2.pc = make_pred_const(p->K_L2, (long long)p->l_mean_grid);
   L2.pc.radial = radial_bins;
   L2.pc.rbin_inv_w = rbin_inv_w;
@@ -659,8 +545,8 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   L2.nuc_R2 = nucR22;
   L2.nnuc = nnuc2;
   L2.work = &meta->work2;
-  // edold / einel / ed are reused (na <= nd)
-  if (batched) CSO_TRY(level_stage(c, L2, sched, hcounts));
+  // edold / ed are reused (na <= nd)
+  if (batched) CSO_TRY(level_stage(c, L2, sched));
   else CSO_TRY(level_run(L2, st));
 
   // ---- output ----
@@ -671,16 +557,13 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   CSO_TRY(readback(c, hbase2 + H1, 4));
   const int H2 = (int)((uint32_t*)c->pinned)[0];
   c->stats[4] = H2;
-  ALLOC(int, ehalo2, na);
   ALLOC(uint32_t, hnuc2, H2);
   ALLOC(long long, hR2b, H2);
-  ALLOC(uint32_t, hseg2, H2);
   ALLOC(unsigned, h2size, H2);
-  CSO_TRY(level_halo(H1, seg2, nnuc2, hbase2, eslot2, nucm2, nucR22, ehalo2, hnuc2, hR2b, hseg2, na, H2, st));
+  CSO_TRY(level_halo(H1, seg2, hbase2, nucm2, nucR22, hnuc2, hR2b, H2, st));
   if (H2 > 0) CSO_CUDA(cudaMemsetAsync(h2size, 0, sizeof(unsigned) * H2, st));
 
-  if (ol1 && nd > 0) k_out_l1<<<G1(nd)>>>(ehalo, nd, gs, spos, hnuc, eid, ol1);
-  if (na > 0) k_out_l2<<<G1(na)>>>(ehalo2, na, ek2, gs, spos, hnuc2, eid, ol2, h2size);
+  if (na > 0) k_out_l2<<<G1(na)>>>(eslot2, ehal2, hbase2, na, epos2, hnuc2, sid, ol2, h2size);
   CSO_CUDA(cudaGetLastError());
 
   // per-halo rows and the catalogue
@@ -703,10 +586,10 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
       ALLOC(unsigned long long, acc, 6 * (size_t)H1);
       CSO_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 6 * (size_t)H1, st));
       if (na > 0)
-        k_summary_sums<<<CL(cdiv(na, 256 * SUM_ITEMS)), 256, 0, st>>>(ehal2, na, epos2, ehalo2, hnuc, epos, nnuc2,
-                                                                      hbase2, hnuc2, acc);
-      k_summary<<<G1(H1)>>>(seg2, H1, epos2, hnuc, hR2, epos, eid, gs, root, minid, nnuc2, hbase2, hnuc2, h2size,
-                            acc, ek2, 1.0 / p->l_mean_grid, p->np_min_L1, gi.x0, rows, keep);
+        k_summary_sums<<<CL(cdiv(na, 256 * SUM_ITEMS)), 256, 0, st>>>(ehal2, na, epos2, eslot2, hnuc, spos, hbase2,
+                                                                      hnuc2, acc);
+      k_summary<<<G1(H1)>>>(seg2, H1, hnuc, hR2, spos, sid, root, minid, nnuc2, hbase2, hnuc2, h2size, acc,
+                            1.0 / p->l_mean_grid, p->np_min_L1, gi.x0, rows, keep);
     }
     CSO_CUDA(cudaGetLastError());
     cso_radial* rad = nullptr;
@@ -714,7 +597,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
       S.mark("radial");
       ALLOC(cso_radial, r1, H1);
       rad = r1;
-      CSO_TRY(radial_run(seg2, ehal2, epos2, na, rows, H1, gi.x0, p->l_mean_grid, hnuc, epos, rad, c->pinned, ws,
+      CSO_TRY(radial_run(seg2, ehal2, epos2, na, rows, H1, gi.x0, p->l_mean_grid, hnuc, spos, rad, c->pinned, ws,
                          st));
       S.mark("catalogue");
     }
@@ -745,7 +628,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
         srad = r2;
         *radial_out = r2;
       }
-      k_catalogue_write<<<G1(nrows)>>>(rows, pv, nrows, hnuc, epos, sorted_rows, row_w, rad, srad);
+      k_catalogue_write<<<G1(nrows)>>>(rows, pv, nrows, hnuc, spos, sorted_rows, row_w, rad, srad);
       CSO_CUDA(cudaGetLastError());
     }
   }

@@ -64,15 +64,13 @@ struct cso_ctx {
 
 // The batched level stage; with CSO_FLAG_GRAPH captured once per distinct
 // argument set and replayed as a CUDA graph.
-int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched, unsigned* host_counts);
+int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched);
 
 struct Meta {  // device counters read back by the host
   unsigned long long sigma_max, id_max;
   unsigned long long pairs, work1, work2;
   int bad;
-  int tie_overflow;  // a run of equal (group, Sigma) keys too long for k_tie_fix
-  int timeout;       // a bounded device wait gave up (Workspace::err points here)
-  int pad_;
+  int timeout;  // a bounded device wait gave up (Workspace::err points here)
 };
 
 // dense particles taking part (all, or those of selected groups) and group roots
