@@ -8,11 +8,11 @@
 // ascending in the halo's own segment.  A block per halo then reads the four
 // enclosed-fraction radii by index and finds the circular-velocity peak
 // max N(<= r) / r with an exact 128-bit comparison.
+#include <cooperative_groups.h>
+
 #include "radial.cuh"
 
 namespace {
-
-constexpr int RAD_NT = 256;
 
 __device__ __forceinline__ long long min_image(int dx) {
   long long d = dx;
@@ -79,22 +79,37 @@ __device__ __forceinline__ bool vbetter(unsigned long long na_, unsigned long lo
   return l > r || (l == r && da < db);
 }
 
-__global__ void __launch_bounds__(RAD_NT) k_radial_stats(const uint64_t* __restrict__ key,
-                                                         unsigned long long dmask, const uint32_t* __restrict__ seg,
-                                                         double u, cso_radial* __restrict__ out) {
-  __shared__ unsigned long long sn[RAD_NT / 32], sd[RAD_NT / 32];
-  const int h = blockIdx.x;
-  const uint32_t b = seg[h];
-  const uint32_t n = seg[h + 1] - b;
+// Haloes by the work they need: a halo below SS_N_MIN members stops at its
+// first shrinking sphere, one of SS_BIG or more takes the biggest blocks.
+constexpr long long SS_N_MIN = 700;
+constexpr long long SS_BIG = 16384;
+
+struct SsLists {  // listed haloes of each kind and their fetch counters
+  unsigned n_mid, n_big, next_mid, next_big;
+};
+
+// Quantiles and the circular-velocity peak from a halo's sorted distances, a
+// block per halo: 256 threads, or 1024 for the listed big ones.  The exact
+// 128-bit comparison is made only for members whose n^2 / d comes within 1e-5
+// of the thread's best in float (relative error below 1e-6), which leaves out
+// almost all of them.
+template <int NT>
+__device__ void radial_stats(const uint64_t* __restrict__ key, unsigned long long dmask, uint32_t b, uint32_t n, double u,
+                             cso_radial& r, unsigned long long* sn, unsigned long long* sd) {
   const uint64_t* D = key + b;
   unsigned long long bn = 0, bd = 0;
-  for (uint32_t i = threadIdx.x; i < n; i += RAD_NT) {
+  float fn2 = 0.f, fd = 1.f;  // the best so far in float
+  for (uint32_t i = threadIdx.x; i < n; i += NT) {
     const unsigned long long di = D[i] & dmask;
     if (di == 0) continue;
+    const float cn = (float)(i + 1), cd = (float)di;
+    if (cn * cn * fd < fn2 * cd * (1.f - 1e-5f)) continue;
     if (i + 1 < n && (D[i + 1] & dmask) == di) continue;  // N(<= r) takes the whole shell
     if (vbetter(i + 1, di, bn, bd)) {
       bn = i + 1;
       bd = di;
+      fn2 = cn * cn;
+      fd = cd;
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -112,12 +127,11 @@ __global__ void __launch_bounds__(RAD_NT) k_radial_stats(const uint64_t* __restr
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
-  for (int k = 1; k < RAD_NT / 32; ++k)
+  for (int k = 1; k < NT / 32; ++k)
     if (vbetter(sn[k], sd[k], bn, bd)) {
       bn = sn[k];
       bd = sd[k];
     }
-  cso_radial& r = out[h];
   const int pct[4] = {25, 50, 75, 98};
   for (int q = 0; q < 4; ++q) {
     long long m = ((long long)pct[q] * n + 99) / 100;
@@ -132,91 +146,259 @@ __global__ void __launch_bounds__(RAD_NT) k_radial_stats(const uint64_t* __restr
   r.vmax = bn > 0 ? sqrt((double)bn / r.r_vmax) : 0.0;
 }
 
-// Shrinking-sphere centre, a block per halo: every step is one pass over the
-// halo's members (count and summed minimum-image offsets of those inside the
-// sphere, reduced over the block in one step), then thread 0 moves the
-// centre to the rounded centre of mass and shrinks the radius, or stops.  The
-// sums are exact integers, so the reduction order is free.  Haloes of at
-// least SS_BIG members (the ones that take many steps over many members) run
-// on 1024-thread blocks, the rest on 256-thread blocks; each launch skips the
-// other's haloes.
-constexpr long long SS_N_MIN = 700;
-constexpr long long SS_BIG = 16384;
-
-template <int NT>
-__global__ void __launch_bounds__(NT) k_shrink_sphere(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
-                                                      const int4* __restrict__ nuc_pos,
-                                                      const uint32_t* __restrict__ hnuc,
-                                                      const cso_halo* __restrict__ rows, int x0,
+__global__ void __launch_bounds__(256) k_radial_stats(const uint64_t* __restrict__ key, unsigned long long dmask,
+                                                      const uint32_t* __restrict__ seg, double u,
                                                       cso_radial* __restrict__ out) {
-  __shared__ long long sh[NT / 32][4];
-  __shared__ int sc[3];
-  __shared__ long long sR2, sm, siter;
-  __shared__ int sgo;
-  const int h = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ unsigned long long sn[8], sd[8];
+  const int h = blockIdx.x;
+  const uint32_t b = seg[h], n = seg[h + 1] - b;
+  if (n < SS_BIG) radial_stats<256>(key, dmask, b, n, u, out[h], sn, sd);
+}
+
+__global__ void __launch_bounds__(1024) k_radial_stats_big(const uint64_t* __restrict__ key, unsigned long long dmask,
+                                                           const uint32_t* __restrict__ seg, double u,
+                                                           const uint32_t* __restrict__ list, const SsLists* L,
+                                                           cso_radial* __restrict__ out) {
+  __shared__ unsigned long long sn[32], sd[32];
+  for (unsigned it = blockIdx.x; it < L->n_big; it += gridDim.x) {
+    const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
+    radial_stats<1024>(key, dmask, b, n, u, out[h], sn, sd);
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Shrinking-sphere centre.  A halo below SS_N_MIN members stops at its first
+// sphere, so a warp counts it.  For the others every step is one pass over
+// the members that can lie in the sphere (count and summed minimum-image
+// offsets of those inside), then the centre moves to the rounded centre of
+// mass and the radius shrinks, or the loop stops.  The sums are exact
+// integers, so neither the order nor the split of the members matters.
+//
+// A pass also lists the members it finds inside.  Where the next sphere lies
+// within the one just counted (the centre moved by no more than the radius
+// shrank, the usual case), that list is all the next pass needs; otherwise the
+// list before it serves if the next sphere lies within its sphere, and the
+// whole halo if not.  The lists shrink with the sphere, so a halo costs about
+// twenty passes over its members instead of eighty.  Haloes below SS_BIG
+// members take a 256-thread block, the others a cluster of eight 1024-thread
+// blocks, each with its own share of the members, which add up their sums in
+// one another's shared memory (one block per halo: 4.1 ms for a halo of
+// 150,000 members; now 0.2).
+// ---------------------------------------------------------------------------
+namespace cg = cooperative_groups;
+
+constexpr int SS_CS = 8;
+
+__global__ void __launch_bounds__(256) k_ss_small(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
+                                                  int H, const int4* __restrict__ nuc_pos,
+                                                  const uint32_t* __restrict__ hnuc,
+                                                  const cso_halo* __restrict__ rows, int x0, uint32_t* __restrict__ mid,
+                                                  uint32_t* __restrict__ big, SsLists* L,
+                                                  cso_radial* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int h = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (h >= H) return;
   const uint32_t b = seg[h];
   const long long N = seg[h + 1] - b;
-  if ((N >= SS_BIG) != (NT == 1024)) return;
+  if (N >= SS_N_MIN) {
+    if (lane == 0) {
+      if (N >= SS_BIG) big[atomicAdd(&L->n_big, 1u)] = (uint32_t)h;
+      else mid[atomicAdd(&L->n_mid, 1u)] = (uint32_t)h;
+    }
+    return;
+  }
+  const int4 c = nuc_pos[hnuc[h]];
+  const long long R2 = rows[h].R2;
+  unsigned cnt = 0;
+  for (long long j = lane; j < N; j += 32) {
+    const int4 q = epos[b + j];
+    const long long dx = min_image(q.x - c.x), dy = min_image(q.y - c.y), dz = min_image(q.z - c.z);
+    cnt += dx * dx + dy * dy + dz * dz < R2;
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) {
+    cso_radial& r = out[h];
+    r.ss_centre[0] = (c.x + x0) & (CSO_BOX - 1);
+    r.ss_centre[1] = c.y;
+    r.ss_centre[2] = c.z;
+    r.ss_n = cnt;
+    r.ss_R2 = R2;
+    r.ss_iter = 0;
+  }
+}
+
+struct Sphere {
+  int c[3];
+  long long R2;
+};
+
+// sphere a within sphere b, with a margin far above the rounding of the square roots
+__device__ __forceinline__ bool within(const Sphere& a, const Sphere& b) {
+  double m = 0;
+  for (int k = 0; k < 3; ++k) {
+    const double d = (double)min_image(a.c[k] - b.c[k]);
+    m += d * d;
+  }
+  return sqrt(m) + sqrt((double)a.R2) + 1.0 <= sqrt((double)b.R2);
+}
+
+struct SsShared {
+  long long w[32][4];   // the warps' sums
+  long long tot[4];     // the block's sums (read by the cluster's other blocks)
+  Sphere s;             // the sphere to count next
+  int src;              // which list it is counted in: 0, 1, or 2 for the whole halo
+  int go;
+  unsigned n[2];        // members of the two lists (this block's share)
+};
+
+// One halo by one block (CS = 1) or a cluster: members b + lo .. b + hi of
+// epos are this block's share, listed at l0 and l1.
+template <int CS>
+__device__ void shrink_halo(const int4* __restrict__ share, unsigned ns, int4* __restrict__ l0, int4* __restrict__ l1,
+                            long long N, int4 start, long long R2start, int x0, cso_radial* __restrict__ out,
+                            SsShared& B) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const long long stop = (N + 99) / 100 > SS_N_MIN ? (N + 99) / 100 : SS_N_MIN;
   if (threadIdx.x == 0) {
-    const int4 p = nuc_pos[hnuc[h]];
-    sc[0] = p.x;
-    sc[1] = p.y;
-    sc[2] = p.z;
-    sR2 = rows[h].R2;
-    siter = 0;
+    B.s = Sphere{{start.x, start.y, start.z}, R2start};
+    B.src = 2;
   }
   __syncthreads();
+  Sphere cover[2];  // what the lists hold: every member inside this sphere
+  bool have[2] = {false, false};
+  long long iter = 0;
   for (;;) {
-    const int cx = sc[0], cy = sc[1], cz = sc[2];
-    const long long R2 = sR2;
+    const Sphere s = B.s;
+    const int src = B.src, dst = src == 0 ? 1 : 0;
+    const int4* from = src == 2 ? share : src ? l1 : l0;
+    int4* to = dst ? l1 : l0;
+    const unsigned m = src == 2 ? ns : B.n[src];
+    __syncthreads();  // everyone has read the sphere and the list's length
+    if (threadIdx.x == 0) B.n[dst] = 0;
+    __syncthreads();
     long long v[4] = {0, 0, 0, 0};  // count, summed dx, dy, dz
-    for (long long j = threadIdx.x; j < N; j += blockDim.x) {
-      const int4 q = epos[b + j];
-      const long long dx = min_image(q.x - cx), dy = min_image(q.y - cy), dz = min_image(q.z - cz);
-      if (dx * dx + dy * dy + dz * dz >= R2) continue;
-      v[0] += 1;
-      v[1] += dx;
-      v[2] += dy;
-      v[3] += dz;
+    for (unsigned j0 = threadIdx.x & ~31u; j0 < m; j0 += blockDim.x) {
+      const unsigned j = j0 + lane;
+      int4 q = make_int4(0, 0, 0, 0);
+      bool in = false;
+      if (j < m) {
+        q = from[j];
+        const long long dx = min_image(q.x - s.c[0]), dy = min_image(q.y - s.c[1]), dz = min_image(q.z - s.c[2]);
+        in = dx * dx + dy * dy + dz * dz < s.R2;
+        if (in) {
+          v[0] += 1;
+          v[1] += dx;
+          v[2] += dy;
+          v[3] += dz;
+        }
+      }
+      const unsigned mask = __ballot_sync(0xffffffffu, in);
+      if (!mask) continue;
+      unsigned at = 0;
+      if (lane == 0) at = atomicAdd(&B.n[dst], (unsigned)__popc(mask));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (in) to[at + __popc(mask & ((1u << lane) - 1u))] = q;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-      for (int k = 0; k < 4; ++k) sh[w][k] = v[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane < 4) B.w[w][lane] = lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3];
     __syncthreads();
-    if (threadIdx.x == 0) {
-      long long t[4] = {0, 0, 0, 0};
-      for (int x = 0; x < (int)(blockDim.x >> 5); ++x)
-        for (int k = 0; k < 4; ++k) t[k] += sh[x][k];
-      const long long m = t[0];
-      sm = m;
-      if (m < stop) {
-        sgo = 0;
-      } else {
-        for (int a = 0; a < 3; ++a) {
-          double f = (double)sc[a] + (double)t[a + 1] / (double)m;
-          if (f < 0) f += (double)CSO_BOX;
-          if (f >= (double)CSO_BOX) f -= (double)CSO_BOX;
-          sc[a] = (int)(llround(f) & (CSO_BOX - 1));
-        }
-        sR2 = R2 * 9025 / 10000;
-        ++siter;
-        sgo = 1;
+    if (w == 0) {
+      // the block's sums: eight lanes per value, then across them
+      long long t = 0;
+      for (int x = lane >> 2; x < nw; x += 8) t += B.w[x][lane & 3];
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane < 4) B.tot[lane] = t;
+    }
+    long long t[4];
+    if (CS > 1) {
+      cg::cluster_group cluster = cg::this_cluster();
+      cluster.sync();  // every block's sums
+      for (int k = 0; k < 4; ++k) t[k] = 0;
+      for (int r = 0; r < CS; ++r) {
+        const long long* o = cluster.map_shared_rank(&B, r)->tot;
+        for (int k = 0; k < 4; ++k) t[k] += o[k];
       }
+      cluster.sync();  // read by all before the next step's sums
+    } else {
+      __syncthreads();
+      for (int k = 0; k < 4; ++k) t[k] = B.tot[k];
+    }
+    // every thread (of every block) takes the same decision from the same sums
+    if (t[0] < stop) {
+      if (out && threadIdx.x == 0) {
+        out->ss_centre[0] = (s.c[0] + x0) & (CSO_BOX - 1);
+        out->ss_centre[1] = s.c[1];
+        out->ss_centre[2] = s.c[2];
+        out->ss_n = t[0];
+        out->ss_R2 = s.R2;
+        out->ss_iter = iter;
+      }
+      break;
+    }
+    ++iter;
+    if (threadIdx.x == 0) {
+      Sphere nx;
+      for (int a = 0; a < 3; ++a) {
+        double f = (double)s.c[a] + (double)t[a + 1] / (double)t[0];
+        if (f < 0) f += (double)CSO_BOX;
+        if (f >= (double)CSO_BOX) f -= (double)CSO_BOX;
+        nx.c[a] = (int)(llround(f) & (CSO_BOX - 1));
+      }
+      nx.R2 = s.R2 * 9025 / 10000;
+      cover[dst] = s;
+      have[dst] = true;
+      // (a list that was only read keeps its cover)
+      B.src = within(nx, s) ? dst : (src != 2 && have[src] && within(nx, cover[src])) ? src : 2;
+      B.s = nx;
     }
     __syncthreads();
-    if (!sgo) break;
   }
-  if (threadIdx.x == 0) {
-    cso_radial& r = out[h];
-    r.ss_centre[0] = (sc[0] + x0) & (CSO_BOX - 1);
-    r.ss_centre[1] = sc[1];
-    r.ss_centre[2] = sc[2];
-    r.ss_n = sm;
-    r.ss_R2 = sR2;
-    r.ss_iter = siter;
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(256) k_ss_mid(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
+                                                const int4* __restrict__ nuc_pos, const uint32_t* __restrict__ hnuc,
+                                                const cso_halo* __restrict__ rows, int x0,
+                                                const uint32_t* __restrict__ list, SsLists* L, int4* __restrict__ l0,
+                                                int4* __restrict__ l1, cso_radial* __restrict__ out) {
+  __shared__ SsShared B;
+  __shared__ unsigned item;
+  for (;;) {
+    if (threadIdx.x == 0) item = atomicAdd(&L->next_mid, 1u);
+    __syncthreads();
+    const unsigned it = item;
+    __syncthreads();
+    if (it >= L->n_mid) return;
+    const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
+    shrink_halo<1>(epos + b, n, l0 + b, l1 + b, n, nuc_pos[hnuc[h]], rows[h].R2, x0, out + h, B);
+  }
+}
+
+__global__ void __cluster_dims__(SS_CS, 1, 1) __launch_bounds__(1024)
+    k_ss_big(const int4* __restrict__ epos, const uint32_t* __restrict__ seg, const int4* __restrict__ nuc_pos,
+             const uint32_t* __restrict__ hnuc, const cso_halo* __restrict__ rows, int x0,
+             const uint32_t* __restrict__ list, SsLists* L, int4* __restrict__ l0, int4* __restrict__ l1,
+             cso_radial* __restrict__ out) {
+  __shared__ SsShared B;
+  __shared__ unsigned item;
+  cg::cluster_group cluster = cg::this_cluster();
+  const unsigned rank = cluster.block_rank();
+  for (;;) {
+    if (rank == 0 && threadIdx.x == 0) item = atomicAdd(&L->next_big, 1u);
+    cluster.sync();
+    const unsigned it = *cluster.map_shared_rank(&item, 0);
+    cluster.sync();  // read by all before it changes
+    if (it >= L->n_big) return;
+    const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
+    const uint32_t lo = (uint32_t)((unsigned long long)n * rank / SS_CS);
+    const uint32_t hi = (uint32_t)((unsigned long long)n * (rank + 1) / SS_CS);
+    shrink_halo<SS_CS>(epos + b + lo, hi - lo, l0 + b + lo, l1 + b + lo, n, nuc_pos[hnuc[h]], rows[h].R2, x0,
+                       rank == 0 ? out + h : nullptr, B);
   }
 }
 
@@ -227,16 +409,22 @@ int radial_run(const uint32_t* seg, const uint32_t* ehal, const int4* epos, long
                Workspace& ws, cudaStream_t st) {
   if (H <= 0) return CSO_OK;
   const size_t mark = ws.off;
+  SsLists* lists = ws.get<SsLists>(1);
+  uint32_t* mid = ws.get<uint32_t>(H);
+  uint32_t* big = ws.get<uint32_t>(H);
+  const size_t after_lists = ws.off;
   int4* cen = ws.get<int4>(H);
   uint64_t* key = ws.get<uint64_t>(na);
   uint64_t* key2 = ws.get<uint64_t>(na);
   uint32_t* val = ws.get<uint32_t>(na);
   uint32_t* val2 = ws.get<uint32_t>(na);
   unsigned long long* dmax = ws.get<unsigned long long>(1);
-  if (!cen || !key || !key2 || !val || !val2 || !dmax) {
+  if (!lists || !mid || !big || !cen || !key || !key2 || !val || !val2 || !dmax) {
     cso_set_error("workspace exhausted in the radial statistics");
     return CSO_ERR_BUDGET;
   }
+  CSO_CUDA(cudaMemsetAsync(lists, 0, sizeof(SsLists), st));
+  k_ss_small<<<CL(cdiv(H, 8)), 256, 0, st>>>(epos, seg, H, nuc_pos, hnuc, rows, x0, mid, big, lists, out);
   k_radial_centre<<<CL(cdiv(H, 256)), 256, 0, st>>>(rows, H, x0, cen, out);
   CSO_CUDA(cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), st));
   if (na > 0) {
@@ -274,9 +462,22 @@ int radial_run(const uint32_t* seg, const uint32_t* ehal, const int4* epos, long
       sorted = pl;
     }
   }
-  k_radial_stats<<<CL(H), RAD_NT, 0, st>>>(sorted, dmask, seg, u, out);
-  k_shrink_sphere<1024><<<CL(H), 1024, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, out);
-  k_shrink_sphere<256><<<CL(H), 256, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, out);
+  if (na >= SS_BIG)
+    k_radial_stats_big<<<CL(cso_sm_count()), 1024, 0, st>>>(sorted, dmask, seg, u, big, lists, out);
+  k_radial_stats<<<CL(H), 256, 0, st>>>(sorted, dmask, seg, u, out);
+  // the shrinking spheres' lists take the place of the sort's buffers
+  ws.off = after_lists;
+  int4* l0 = ws.get<int4>(na);
+  int4* l1 = ws.get<int4>(na);
+  if (!l0 || !l1) {
+    cso_set_error("workspace exhausted in the shrinking spheres");
+    return CSO_ERR_BUDGET;
+  }
+  const unsigned clusters = (unsigned)(cso_sm_count() / SS_CS > 0 ? cso_sm_count() / SS_CS : 1);
+  if (na >= SS_BIG)
+    k_ss_big<<<CL(clusters * SS_CS), 1024, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, big, lists, l0, l1, out);
+  if (na >= SS_N_MIN)
+    k_ss_mid<<<CL(cso_sm_count() * 8), 256, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, mid, lists, l0, l1, out);
   CSO_CUDA(cudaGetLastError());
   ws.off = mark;
   return CSO_OK;
