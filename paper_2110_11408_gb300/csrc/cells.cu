@@ -931,86 +931,119 @@ __global__ void __launch_bounds__(256) k_fof_cells(CellGrid g, const int4* __res
                    lane);
 }
 
-// Pass three, the stragglers one by one (a list of them): against every neighbour cell in
-// l_FoF reach (its own included), the first link into the cell's main tree
-// (skipped when that tree is already the straggler's) and every link to a
-// later straggler (each straggler pair once).  Cells out of reach of the
-// particle (by its distance to the home cell's faces) are skipped.
+// Pass three, the stragglers: against every neighbour cell in l_FoF reach (its
+// own included), the first link into the cell's main tree (skipped when that
+// tree is already the straggler's) and every link to a later straggler (each
+// straggler pair once).  A warp per straggler: lanes 0-26 look up one cell
+// each (skipping those out of reach by the particle's distance to the home
+// cell's faces, and trimming the rest to l_FoF in x), so the lookups' chain
+// of dependent loads is paid once and not once per cell, and the slots of all
+// cells are tested as one flat sequence, 32 at a time (a lane per straggler
+// walking its cells in turn: 202 us for the 3,000 stragglers of the side-64
+// box, where the longest walk set the time).
+__device__ __forceinline__ int fold21(int v) { return (int)((unsigned)v << 11) >> 11; }  // nearest image
+
+// lane whose run of the flat sequence holds f (incl: inclusive ends of the lanes' runs)
+__device__ __forceinline__ int flat_owner(uint32_t incl, uint32_t f) {
+  int r = 0;
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+    if (__shfl_sync(0xffffffffu, incl, r + o - 1) <= f) r += o;
+  return r;
+}
+
+__device__ __forceinline__ uint32_t warp_incl_u32(uint32_t v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+
 __global__ void __launch_bounds__(256) k_fof_stragglers(CellGrid g, const int4* __restrict__ spos,
-                                                        const int* __restrict__ didx,
-                                                        const uint32_t* __restrict__ nd_ptr, uint32_t lfof2,
+                                                        const int* __restrict__ slist,
+                                                        const uint32_t* __restrict__ ns_ptr, uint32_t lfof2,
                                                         int lreach, int* __restrict__ parent,
                                                         const int* __restrict__ cell_root,
                                                         const uint8_t* __restrict__ strag,
                                                         const uint2* __restrict__ srange) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int)*nd_ptr) return;
-  const int s = didx[i];
-  const int4 p = spos[s];
-  const int nc = g.nc;
-  const int cy = cell_coord(p.y, nc), cz = cell_coord(p.z, nc), tc = grid_col(g, p.x);
-  const XCells X = x_cells(g, tc);
-  const int xcol[3] = {X.a < tc ? X.a : X.wl, tc, X.b > tc ? X.b : X.wr};
-  const int xsh[3] = {X.a < tc ? 0 : CSO_BOX, 0, X.b > tc ? 0 : -CSO_BOX};
-  const int gx = (p.x + g.x0) & (CSO_BOX - 1), gcx = cell_coord(gx, nc);
-  const long long xl = gx - cell_lo(gcx, nc) + 1, xr = cell_lo(gcx + 1, nc) - gx;
-  const long long yl = p.y - cell_lo(cy, nc) + 1, yr = cell_lo(cy + 1, nc) - p.y;
-  const long long zl = p.z - cell_lo(cz, nc) + 1, zr = cell_lo(cz + 1, nc) - p.z;
-  const long long mx[3] = {xl * xl, 0, xr * xr};
-  const long long R2 = lfof2;
-  int rs = uf_root(parent, s);
-  for (int dz = -1; dz <= 1; ++dz) {
-    const long long mz = dz < 0 ? zl * zl : (dz > 0 ? zr * zr : 0);
-    if (mz >= R2) continue;
-    int sz;
-    const int zz = wrap_yz(cz + dz, nc, sz);
-    for (int dy = -1; dy <= 1; ++dy) {
-      const long long my = mz + (dy < 0 ? yl * yl : (dy > 0 ? yr * yr : 0));
-      if (my >= R2) continue;
-      int sy;
-      const int yy = wrap_yz(cy + dy, nc, sy);
-      for (int k = 0; k < 3; ++k) {
-        if (xcol[k] < 0 || my + mx[k] >= R2) continue;
-        const size_t c = grid_cell(g, zz, yy, xcol[k]);
-        const uint32_t c_lo = g.start[c], c_hi = g.start[c + 1];
-        if (c_lo == c_hi) continue;
-        const int cm = cell_root[c_lo];
-        if (cm == CELL_EMPTY) continue;
-        const int xq = p.x + xsh[k], yq = p.y + sy, zq = p.z + sz;
-        // the main tree: the first link joins all of it (only the cell's
-        // slots within l_FoF in x can link; cells are sorted by x)
-        if (uf_root(parent, cm) != rs) {
-          uint32_t t0 = c_lo, t1 = c_hi;
-          if (t1 - t0 > 16u) x_trim(spos, t0, t1, xq - lreach, xq + lreach);
-          for (uint32_t t = t0; t < t1; ++t) {
-            const int pt = parent[t];
-            if (pt < 0 || strag[t]) continue;
-            const int4 q = spos[t];
-            const int ddx = xq - q.x, ddy = yq - q.y, ddz = zq - q.z;
-            const uint32_t d = (uint32_t)(ddx * ddx) + (uint32_t)(ddy * ddy) + (uint32_t)(ddz * ddz);
-            if (d >= lfof2) continue;
-            uf_unite(parent, rs, pt);
-            rs = uf_root(parent, rs);
-            break;
+  const int lane = threadIdx.x & 31;
+  const int ns = (int)*ns_ptr;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < ns; i += (gridDim.x * blockDim.x) >> 5) {
+    const int s = slist[i];
+    const int4 p = spos[s];
+    const int nc = g.nc;
+    const int cy = cell_coord(p.y, nc), cz = cell_coord(p.z, nc), tc = grid_col(g, p.x);
+    const int rs = uf_root(parent, s);
+    int cm = CELL_EMPTY;
+    uint32_t t0 = 0, t1 = 0;
+    uint2 sr = make_uint2(0, 0);
+    if (lane < 27) {
+      const XCells X = x_cells(g, tc);
+      const int dz = lane / 9 - 1, dy = lane / 3 % 3 - 1, dx = lane % 3 - 1;
+      const int gx = (p.x + g.x0) & (CSO_BOX - 1), gcx = cell_coord(gx, nc);
+      const long long fx = dx < 0 ? gx - cell_lo(gcx, nc) + 1 : dx > 0 ? cell_lo(gcx + 1, nc) - gx : 0;
+      const long long fy = dy < 0 ? p.y - cell_lo(cy, nc) + 1 : dy > 0 ? cell_lo(cy + 1, nc) - p.y : 0;
+      const long long fz = dz < 0 ? p.z - cell_lo(cz, nc) + 1 : dz > 0 ? cell_lo(cz + 1, nc) - p.z : 0;
+      const int col = dx < 0 ? (X.a < tc ? X.a : X.wl) : dx > 0 ? (X.b > tc ? X.b : X.wr) : tc;
+      if (col >= 0 && fx * fx + fy * fy + fz * fz < (long long)lfof2) {
+        int sh;
+        const size_t c = grid_cell(g, wrap_yz(cz + dz, nc, sh), wrap_yz(cy + dy, nc, sh), col);
+        t0 = g.start[c];
+        t1 = g.start[c + 1];
+        if (t0 < t1) cm = cell_root[t0];
+        if (cm != CELL_EMPTY) {
+          sr = srange[t0];
+          if (uf_root(parent, cm) == rs) {
+            t1 = t0;  // the main tree is the straggler's already
+          } else if (t1 - t0 > 16u) {
+            const int xq = dx < 0 && X.a == tc ? p.x + CSO_BOX : dx > 0 && X.b == tc ? p.x - CSO_BOX : p.x;
+            x_trim(spos, t0, t1, xq - lreach, xq + lreach);
           }
-        }
-        // the cell's stragglers after this one, from its run of the list
-        const uint2 sr = srange[c_lo];
-        for (uint32_t j = sr.x; j < sr.y; ++j) {
-          const int t = didx[j];
-          if (t <= s) continue;
-          const int4 q = spos[t];
-          const int ddx = xq - q.x, ddy = yq - q.y, ddz = zq - q.z;
-          const uint32_t d = (uint32_t)(ddx * ddx) + (uint32_t)(ddy * ddy) + (uint32_t)(ddz * ddz);
-          if (d >= lfof2) continue;
-          const int rt = uf_root(parent, t);
-          if (rt != rs) {
-            uf_unite(parent, rs, rt);
-            rs = uf_root(parent, rs);
-          }
+        } else {
+          t1 = t0;
         }
       }
     }
+    // main trees: any link joins all of one
+    uint32_t incl = warp_incl_u32(t1 - t0, lane);
+    uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned want = __ballot_sync(0xffffffffu, t1 > t0);
+    unsigned hits = 0;
+    for (uint32_t f0 = 0; f0 < total && hits != want; f0 += 32) {
+      const uint32_t f = f0 + lane;
+      const int r = flat_owner(incl, f) & 31;
+      const uint32_t end = __shfl_sync(0xffffffffu, incl, r), hi = __shfl_sync(0xffffffffu, t1, r);
+      bool hit = false;
+      if (f < total && !(hits >> r & 1u)) {
+        const uint32_t t = hi - (end - f);
+        if (parent[t] >= 0 && !strag[t]) {
+          const int4 q = spos[t];
+          const int ex = fold21(p.x - q.x), ey = fold21(p.y - q.y), ez = fold21(p.z - q.z);
+          hit = (uint32_t)(ex * ex) + (uint32_t)(ey * ey) + (uint32_t)(ez * ez) < lfof2;
+        }
+      }
+      hits |= __reduce_or_sync(0xffffffffu, hit ? 1u << r : 0u);
+    }
+    if (hits >> lane & 1u) uf_unite(parent, rs, cm);
+    // the cells' stragglers after this one, from their runs of the list
+    incl = warp_incl_u32(sr.y - sr.x, lane);
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    for (uint32_t f0 = 0; f0 < total; f0 += 32) {
+      const uint32_t f = f0 + lane;
+      const int r = flat_owner(incl, f) & 31;
+      const uint32_t end = __shfl_sync(0xffffffffu, incl, r), hi = __shfl_sync(0xffffffffu, sr.y, r);
+      if (f < total) {
+        const int t = slist[hi - (end - f)];
+        if (t > s) {
+          const int4 q = spos[t];
+          const int ex = fold21(p.x - q.x), ey = fold21(p.y - q.y), ez = fold21(p.z - q.z);
+          if ((uint32_t)(ex * ex) + (uint32_t)(ey * ey) + (uint32_t)(ez * ez) < lfof2) uf_unite(parent, s, t);
+        }
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -1024,12 +1057,11 @@ __global__ void k_fof_finish(int* __restrict__ parent, int n, const long long* _
   root[s] = r;
   // smallest id per root: reduce over the lanes that share a root first
   const unsigned peers = __match_any_sync(__activemask(), r);
-  unsigned long long v = r >= 0 ? (unsigned long long)sid[s] : ~0ull;
-  for (unsigned m = peers; m; m &= m - 1) {
-    const unsigned long long o = __shfl_sync(peers, v, __ffs(m) - 1);
-    v = o < v ? o : v;
-  }
-  if (r >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicMin(&minid[r], v);
+  const unsigned long long v = r >= 0 ? (unsigned long long)sid[s] : ~0ull;
+  // (the high words first, the low words among the lanes that hold the smallest)
+  const unsigned hi = __reduce_min_sync(peers, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_min_sync(peers, (unsigned)(v >> 32) == hi ? (unsigned)v : ~0u);
+  if (r >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicMin(&minid[r], (unsigned long long)hi << 32 | lo);
 }
 
 }  // namespace
@@ -1193,8 +1225,8 @@ int cells_fof(const CellGrid& g, const int4* spos, int n, const long long* sigma
   // pass two: main trees of adjacent cells; pass three: stragglers
   const int lreach = reach_below(lfof2);
   k_fof_cells<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, clist, ncl, lfof2, lreach, parent, cell_root, strag);
-  k_fof_stragglers<<<CL(cdiv(n, 256)), 256, 0, st>>>(g, spos, slist, sflag + n, lfof2, lreach, parent, cell_root, strag,
-                                                     srange);
+  k_fof_stragglers<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, slist, sflag + n, lfof2, lreach, parent, cell_root,
+                                                           strag, srange);
   CSO_CUDA(cudaMemsetAsync(minid, 0xff, sizeof(unsigned long long) * n, st));
   k_fof_finish<<<CL(cdiv(n, 256)), 256, 0, st>>>(parent, n, sigma, T_L0, sid, root, minid);
   CSO_CUDA(cudaGetLastError());
