@@ -255,7 +255,9 @@ int cso_autotune(cso_ctx* ctx, const cso_input* in, const cso_params* p, cso_out
                  int32_t* small);
 
 /* Set the batched schedule's size bins directly (giant >= 64, 1 <= small
- * <= 64); the defaults are 16384 and 64. */
+ * <= 64); the defaults are 16384 and 64, and until this or the autotuner is
+ * called only as many of the groups above 16384 go to clusters as clusters
+ * run at a time (and those of 131072 or more). */
 int cso_set_schedule(cso_ctx* ctx, int32_t giant, int32_t small);
 
 /* Groups above max(huge, giant) members run on 16-CTA thread-block clusters

@@ -185,13 +185,12 @@ __device__ void bitonic_sort(long long* a, int m) {  // m power of two
 struct SelShared {
   unsigned cnt[NB];
   unsigned clo[NB];
-  unsigned long long dmn[NB];
-  unsigned long long dmx[NB];
   long long list[CAP];
   unsigned sw[33];
   int best;
   int nlist;
-  unsigned long long dmax_all;
+  unsigned long long lo, hi;    // smallest and largest distance of a bin too big to list
+  unsigned long long dmax_all;  // farthest member visited
 };
 
 // In the sorted list s[0..m) with n(<s[0]) = base, the first element whose
@@ -217,8 +216,8 @@ __device__ __forceinline__ int pow2_at_least(int m) {
 }
 
 // Bin of distance d in the first window of the select.  Both binnings are
-// monotone in d, and the select only prunes with the exact predicate at each
-// bin's largest member distance, so both give the same R^2:
+// monotone in d, and the select only prunes with the exact predicate at an
+// upper bound of each bin's distances, so both give the same R^2:
 //   * threshold-count bins (default): bin = sqrt(K) d^1.5 / u^3 / w with
 //     w = n / (nb - 1) members of threshold count per bin;
 //   * radial bins (the paper's cell-bounded search, Sec. 2.3.4): bins of
@@ -230,14 +229,47 @@ __device__ __forceinline__ int first_bin(unsigned long long d, const PredConst& 
   return g < (float)(nb - 1) ? (int)g : nb - 1;
 }
 
-// The bin's smallest and largest distance.  A bound read without the atomic
-// can only be stale in the safe direction (the minimum only falls, the
-// maximum only rises), so a member that does not beat it is skipped: per bin
-// only the few members that move a bound pay a 64-bit shared atomic, not
-// every member.
-__device__ __forceinline__ void bin_minmax(SelShared& S, int b, unsigned long long d) {
-  if (d < *(volatile unsigned long long*)&S.dmn[b]) atomicMin(&S.dmn[b], d);
-  if (d > *(volatile unsigned long long*)&S.dmx[b]) atomicMax(&S.dmx[b], d);
+// bins per unit of first_bin's threshold count: w members of threshold per
+// bin, for the whole group or for a search bounded by lim
+__device__ __forceinline__ float bin_scale(int n, unsigned long long lim, const PredConst& c, int nb) {
+  float cnt = (float)n;
+  if (lim) {
+    const float f = (float)lim;
+    cnt = fminf(cnt, f * sqrtf(f) * c.bin_scale0 + 2.f);
+  }
+  return c.bin_scale0 / ceilf(cnt / (float)(nb - 1));
+}
+
+// A window of the select: members with wlo <= d <= whi in nb bins, by
+// first_bin (mode 0) or linearly (mode 1).
+struct Window {
+  unsigned long long wlo, whi, base;  // base = members below wlo
+  int mode;
+};
+
+__device__ __forceinline__ int window_bin(const Window& W, unsigned long long d, const PredConst& c, float scale0,
+                                          int nb) {
+  if (W.mode == 0) return first_bin(d, c, scale0, nb);
+  const unsigned long long span = W.whi - W.wlo + 1;
+  return (int)(((d - W.wlo) * (unsigned long long)nb) / span);
+}
+
+// An upper bound of the distances that fall into bin b of the window, at
+// most top (the inverse of first_bin in float, raised by far more than its
+// rounding; the last bin of mode 0 is open).
+__device__ __forceinline__ unsigned long long bin_top(const Window& W, int b, const PredConst& c, float scale0, int nb,
+                                                      unsigned long long top) {
+  if (b >= nb - 1) return top;
+  unsigned long long e;
+  if (W.mode == 0) {
+    const float g = (float)(b + 1);
+    const float f = c.radial ? (g / c.rbin_inv_w) * (g / c.rbin_inv_w) : powf(g / scale0, 2.f / 3.f);
+    e = f < 9e18f ? (unsigned long long)(f * (1.f + 1e-4f)) + 1 : top;
+  } else {
+    const unsigned long long span = W.whi - W.wlo + 1;
+    e = W.wlo + (unsigned long long)(b + 1) * (span / nb + 1);
+  }
+  return e < top ? e : top;
 }
 
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
@@ -254,6 +286,7 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 // passes over the tiles within reach of a nucleus
 // ---------------------------------------------------------------------------
 constexpr int TILE = 128;
+constexpr int TILE_LIST = 2048;  // tiles in reach that a block keeps as a list
 constexpr int LEVELS = 88;  // squared radii tried for the search bound: two per octave up to 2^43
 
 __device__ __forceinline__ int fold21(int v) { return (int)((unsigned)v << 11) >> 11; }  // nearest image
@@ -274,6 +307,8 @@ struct Tiles {
   const int4* lo;  // boxes of the group's tiles, offsets from the group's first member; null: none
   const int4* hi;
   int4 q;          // the nucleus in those offsets
+  const uint32_t* list;  // the group's tiles in reach of the nucleus, or
+  int nlist;             // -1: no list
   __device__ __forceinline__ int own() const { return nt > rank ? (nt - rank + cs - 1) / cs : 0; }
 };
 
@@ -292,27 +327,53 @@ __device__ __forceinline__ unsigned long long tile_gap2(const Tiles& T, int t) {
 }
 
 // f(j) for every member j < n of the CTA's tiles nearer than lim (0: of all
-// its tiles).  Warps take chunks of up to 32 tiles that lie a whole chunk
-// count apart, so that the tiles in reach, neighbours of one another, spread
-// over the warps.
+// its tiles): of those on the list if there is one, else warps take chunks
+// of up to 32 tiles that lie a whole chunk count apart, so that the tiles in
+// reach, neighbours of one another, spread over the warps.
+template <class F>
+__device__ __forceinline__ void tile_members(int t, int n, F f) {
+#pragma unroll
+  for (int k = 0; k < TILE / 32; ++k) {
+    const int j = t * TILE + k * 32 + (threadIdx.x & 31);
+    if (j < n) f(j);
+  }
+}
+
 template <class F>
 __device__ __forceinline__ void for_members(const Tiles& T, int n, unsigned long long lim, F f) {
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (T.nlist >= 0) {
+    for (int i = threadIdx.x >> 5; i < T.nlist; i += nw) tile_members((int)T.list[i], n, f);
+    return;
+  }
   const int own = T.own();
   const int per = min(32, (own + nw - 1) / nw);
   const int nchunk = per > 0 ? (own + per - 1) / per : 0;
   for (int c = threadIdx.x >> 5; c < nchunk; c += nw) {
     const int i = lane * nchunk + c;
     const bool act = lane < per && i < own && (!lim || tile_gap2(T, T.rank + i * T.cs) < lim);
-    for (unsigned m = __ballot_sync(0xffffffffu, act); m; m &= m - 1) {
-      const int t = T.rank + ((__ffs(m) - 1) * nchunk + c) * T.cs;
-#pragma unroll
-      for (int k = 0; k < TILE / 32; ++k) {
-        const int j = t * TILE + k * 32 + lane;
-        if (j < n) f(j);
-      }
-    }
+    for (unsigned m = __ballot_sync(0xffffffffu, act); m; m &= m - 1)
+      tile_members(T.rank + ((__ffs(m) - 1) * nchunk + c) * T.cs, n, f);
   }
+}
+
+// The CTA's tiles nearer than lim, listed (T.nlist = -1 if they are too many):
+// one look at every box, which the passes that follow then need not repeat.
+__device__ void list_tiles(Tiles& T, unsigned long long lim, uint32_t* list, int* count) {
+  if (threadIdx.x == 0) *count = 0;
+  __syncthreads();
+  const int own = T.own();
+  for (int i = threadIdx.x; i < own; i += blockDim.x) {
+    const int t = T.rank + i * T.cs;
+    if (tile_gap2(T, t) >= lim) continue;
+    const int k = atomicAdd(count, 1);
+    if (k < TILE_LIST) list[k] = (uint32_t)t;
+  }
+  __syncthreads();
+  const int k = *count;
+  T.list = list;
+  T.nlist = k <= TILE_LIST ? k : -1;
+  __syncthreads();
 }
 
 // boxes of the CTA's own tiles, a warp per tile
@@ -370,12 +431,14 @@ __device__ unsigned long long search_bound(const Tiles& T, int n, const PredCons
 }
 
 // R^2 of nucleus pc over the n members at epos[0..n); the distances of the
-// members the search visited are left in ed.  lim > 0 bounds the search (the
-// boxes of T are there).
+// members the search visited are left in ed (null: computed again where they
+// are needed).  lim > 0 bounds the search (the
+// boxes of T are there): if nothing qualifies below lim, the answer is -1, or
+// with `whole` the search goes on over all members.
 template <int NT>
 __device__ long long r_search(const int4* __restrict__ epos, long long* __restrict__ ed, int n, int4 pc,
                               const PredConst& c, SelShared& S, const int small_n, const int cap, const int nb,
-                              const Tiles& T, unsigned long long lim) {
+                              Tiles& T, unsigned long long lim, bool whole) {
   const int tid = threadIdx.x;
   if (n <= small_n && n <= COUNT_N) {
     // every member's strictly enclosed count, counted directly: n(<d_i) =
@@ -397,12 +460,12 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
       dmax = (unsigned long long)di > dmax ? (unsigned long long)di : dmax;
     }
     atomicMin(&S.dmax_all, best);
-    if (tid == 0) S.dmn[0] = 0;
+    if (tid == 0) S.hi = 0;
     __syncthreads();
-    atomicMax(&S.dmn[0], dmax);
+    atomicMax(&S.hi, dmax);
     __syncthreads();
     long long r = (long long)S.dmax_all;
-    const long long far = (long long)S.dmn[0];
+    const long long far = (long long)S.hi;
     __syncthreads();
     if (S.dmax_all == ~0ull || r < 0) {
       if (tid == 0) S.list[0] = exhaust_radius((unsigned long long)n, far, c);
@@ -437,39 +500,28 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
   }
 
   // ---- windowed histogram select ----
-  // window [wlo, whi] of d; base = members with d < wlo; mode 0 = threshold-count bins
-  unsigned long long wlo = 0, whi = lim ? lim - 1 : ~0ull, base = 0;
-  int mode = 0;
-  const float scale0 = c.bin_scale0 / (float)((n + nb - 2) / (nb - 1));  // n/(nb-1) members of threshold per bin
+  Window W{0, lim ? lim - 1 : ~0ull, 0, 0};
+  float scale0 = bin_scale(n, lim, c, nb);
   bool first_pass = true;
   while (true) {
-    for (int b = tid; b < NB; b += blockDim.x) {
-      S.cnt[b] = 0;
-      S.dmn[b] = ~0ull;
-      S.dmx[b] = 0;
+    for (int b = tid; b < NB; b += blockDim.x) S.cnt[b] = 0;
+    if (tid == 0) {
+      S.lo = ~0ull;
+      S.hi = 0;
+      if (first_pass) S.dmax_all = 0;
     }
-    if (tid == 0 && first_pass) S.dmax_all = 0;
     __syncthreads();
-    unsigned long long span = whi - wlo + 1;  // mode 1 only
-    unsigned long long dmax = 0;              // this thread's farthest member (first pass)
+    unsigned long long dmax = 0;  // this thread's farthest member (first pass)
     for_members(T, n, lim, [&](int j) {
       unsigned long long d;
       if (first_pass) {
         d = (unsigned long long)dist2(pc, epos[j]);
-        ed[j] = (long long)d;
+        if (ed) ed[j] = (long long)d;
         dmax = d > dmax ? d : dmax;
       } else {
-        d = (unsigned long long)ed[j];
+        d = (unsigned long long)(ed ? ed[j] : dist2(pc, epos[j]));
       }
-      if (d < wlo || d > whi) return;
-      int b;
-      if (mode == 0) {
-        b = first_bin(d, c, scale0, nb);
-      } else {
-        b = (int)(((d - wlo) * (unsigned long long)nb) / span);
-      }
-      atomicAdd(&S.cnt[b], 1u);
-      bin_minmax(S, b, d);
+      if (d >= W.wlo && d <= W.whi) atomicAdd(&S.cnt[window_bin(W, d, c, scale0, nb)], 1u);
     });
     if (first_pass) {
       // one shared atomic per warp (per member it serialised on one address)
@@ -478,6 +530,7 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
     }
     __syncthreads();
     first_pass = false;
+    const unsigned long long dtop = S.dmax_all < W.whi ? S.dmax_all : W.whi;
     // interior counts
     {
       constexpr int per = NB / NT;
@@ -507,32 +560,33 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
       if (tid == 0) S.best = NB;
       __syncthreads();
       for (int b = from + tid; b < NB; b += blockDim.x)
-        if (S.cnt[b] && pred(base + S.clo[b], S.dmx[b], c)) atomicMin(&S.best, b);
+        if (S.cnt[b] && pred(W.base + S.clo[b], bin_top(W, b, c, scale0, nb, dtop), c)) atomicMin(&S.best, b);
       __syncthreads();
       // read the chosen bin before the barrier: the next window pass rewrites it
       const int b = S.best;
-      unsigned long long lo = 0, hi = 0, cb = 0;
+      unsigned long long cb = 0;
       unsigned cntb = 0;
       if (b < NB) {
-        lo = S.dmn[b];
-        hi = S.dmx[b];
-        cb = base + S.clo[b];
+        cb = W.base + S.clo[b];
         cntb = S.cnt[b];
       }
       __syncthreads();
       if (b == NB) break;  // nothing in this window
-      if (lo == hi) {
-        // one distinct value: its enclosed count is cb, and the bin test above
-        // was the exact predicate at that value
-        return (long long)lo;
-      }
-      if (cntb <= (unsigned)cap) {
-        if (tid == 0) S.nlist = 0;
-        __syncthreads();
-        for_members(T, n, lim, [&](int j) {
-          unsigned long long d = (unsigned long long)ed[j];
-          if (d >= lo && d <= hi) S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
-        });
+      const bool listed = cntb <= (unsigned)cap;
+      if (listed && tid == 0) S.nlist = 0;
+      if (listed) __syncthreads();
+      unsigned long long lo = ~0ull, hi = 0;
+      for_members(T, n, lim, [&](int j) {
+        const unsigned long long d = (unsigned long long)(ed ? ed[j] : dist2(pc, epos[j]));
+        if (d < W.wlo || d > W.whi || window_bin(W, d, c, scale0, nb) != b) return;
+        if (listed) {
+          S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
+        } else {
+          lo = d < lo ? d : lo;
+          hi = d > hi ? d : hi;
+        }
+      });
+      if (listed) {
         __syncthreads();
         int m = S.nlist;
         int p2 = pow2_at_least(m);
@@ -549,27 +603,43 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
         continue;
       }
       // too many members in the bin: narrow the window to it
-      wlo = lo;
-      whi = hi;
-      base = cb;
-      mode = 1;
+      hi = warp_max_u64(hi);
+      lo = ~warp_max_u64(~lo);
+      if ((tid & 31) == 0) {
+        atomicMin(&S.lo, lo);
+        atomicMax(&S.hi, hi);
+      }
+      __syncthreads();
+      lo = S.lo;
+      hi = S.hi;
+      __syncthreads();
+      if (lo == hi) {
+        // one distinct value: its enclosed count is cb, and it qualifies or not
+        if (pred(cb, lo, c)) return (long long)lo;
+        if (tid == 0) {
+          S.lo = ~0ull;
+          S.hi = 0;
+        }
+        from = b + 1;
+        continue;
+      }
+      W = Window{lo, hi, cb, 1};
       narrowed = true;
       break;
     }
     if (narrowed) continue;
-    // nothing in [wlo, whi]: move past it
+    // nothing in the window: move past it
     const unsigned long long top = lim ? lim - 1 : S.dmax_all;
-    if (whi < top) {
-      base += in_window;
-      wlo = whi + 1;
-      whi = top;
-      mode = 1;
+    if (W.whi < top) {
+      W = Window{W.whi + 1, top, W.base + in_window, 1};
+    } else if (lim && !whole) {
+      return -1;
     } else if (lim) {  // nothing below the bound: all members, from the start
       __syncthreads();  // every thread has read dmax_all
       lim = 0;
-      wlo = base = 0;
-      whi = ~0ull;
-      mode = 0;
+      T.nlist = -1;
+      scale0 = bin_scale(n, 0, c, nb);
+      W = Window{0, ~0ull, 0, 0};
       first_pass = true;
     } else {
       break;
@@ -581,6 +651,15 @@ __device__ long long r_search(const int4* __restrict__ epos, long long* __restri
   r = S.list[0];
   __syncthreads();
   return r;
+}
+
+// Nuclei after a group's first mostly have small radii: squared radii to try
+// before the bounded search of the whole group, those whose threshold counts
+// are 256 and 4,096 (a try that finds nothing costs a fraction of the next).
+constexpr int TRIES = 2;
+__device__ __forceinline__ unsigned long long try_bound(int k, const PredConst& c) {
+  const float f = powf((k ? 4096.f : 256.f) / c.bin_scale0, 2.f / 3.f);
+  return f < 9e18f ? (unsigned long long)f + 1 : 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -615,16 +694,22 @@ struct PickShared {
 // Marks the peaks that nucleus pc of squared radius R2 makes ineligible (step
 // 1: nearer than alpha R; `cur` is the nucleus itself) and returns the first
 // of the others in key order, or -1.  cur < 0: the first choice.  Each CTA of
-// a cluster calls it with the same arguments and gets the same answer; the
-// flags they write are the same too, and none of them is a nucleus ahead.
-__device__ int next_nucleus(const LevelArgs& a, unsigned p0, int m, int cur, int4 pc, long long R2, PickShared& K) {
+// a cluster calls it with the same arguments and gets the same answer.  The
+// flags of up to 64 peaks per thread are bits of gone; those of longer lists
+// are in memory, and there a cluster's CTAs must not be a nucleus apart.
+__device__ __forceinline__ bool private_flags(int m) { return m <= 64 * (int)blockDim.x; }
+
+__device__ int next_nucleus(const LevelArgs& a, unsigned p0, int m, int cur, int4 pc, long long R2,
+                            unsigned long long& gone, PickShared& K) {
   const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
+  const bool priv = private_flags(m);
   Best mine{0, 0, -1};
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+  for (int i = threadIdx.x, k = 0; i < m; i += blockDim.x, ++k) {
     if (cur >= 0) {
-      if (a.peaks.out[p0 + i]) continue;
+      if (priv ? gone >> k & 1 : a.peaks.out[p0 + i] != 0) continue;
       if (i == cur || (__int128)aden2 * dist2(pc, a.peaks.pos[p0 + i]) < (__int128)anum2 * R2) {
-        a.peaks.out[p0 + i] = 1;
+        if (priv) gone |= 1ull << k;
+        else a.peaks.out[p0 + i] = 1;
         continue;
       }
     }
@@ -663,7 +748,7 @@ __device__ __forceinline__ Tiles group_tiles(const LevelArgs& a, int seg, unsign
   // tiles of different groups never share a slot: a group of n members takes
   // at most n / TILE + 1 of them
   const size_t at = base / TILE + (size_t)seg;
-  return Tiles{(n + TILE - 1) / TILE, rank, cs, a.tlo + at, a.thi + at, make_int4(0, 0, 0, 0)};
+  return Tiles{(n + TILE - 1) / TILE, rank, cs, a.tlo + at, a.thi + at, make_int4(0, 0, 0, 0), nullptr, -1};
 }
 
 __device__ __forceinline__ int4 tile_origin(const int4* epos, int4 pc) {
@@ -674,6 +759,8 @@ __device__ __forceinline__ int4 tile_origin(const int4* epos, int4 pc) {
 struct BlockShared {
   SelShared S;
   PickShared K;
+  uint32_t tiles[TILE_LIST];
+  int ntiles;
   unsigned h[LEVELS];
   int hbest;
 };
@@ -696,21 +783,28 @@ __device__ void level_block(const LevelArgs& a, const int seg, BlockShared& B) {
   Tiles T = group_tiles(a, seg, base, n, 0, 1);
   const bool boxes = m > 1 && n > a.small_n;
   if (boxes) tile_boxes(T, epos, n, a.tlo + (T.lo - a.tlo), a.thi + (T.hi - a.thi));
-  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
+  unsigned long long gone = 0;
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, gone, B.K);
   int nn = 0;
   while (cur >= 0) {
     const int4 pc = a.peaks.pos[p0 + cur];
-    unsigned long long lim = 0;
-    if (boxes) {
+    long long R2 = -1;
+    if (boxes && nn > 0) {
       T.q = tile_origin(epos, pc);
-      lim = search_bound(T, n, a.pc, B.h, &B.hbest);
+      for (int k = 0; k <= TRIES && R2 < 0; ++k) {
+        const unsigned long long lim = k < TRIES ? try_bound(k, a.pc) : search_bound(T, n, a.pc, B.h, &B.hbest);
+        T.nlist = -1;
+        if (lim) list_tiles(T, lim, B.tiles, &B.ntiles);
+        R2 = r_search<NT>(epos, ed, n, pc, a.pc, B.S, a.small_n, a.cap, a.nb, T, lim, k == TRIES);
+      }
+    } else {
+      R2 = r_search<NT>(epos, ed, n, pc, a.pc, B.S, a.small_n, a.cap, a.nb, T, 0, true);
     }
-    const long long R2 = r_search<NT>(epos, ed, n, pc, a.pc, B.S, a.small_n, a.cap, a.nb, T, lim);
     if (n <= a.small_n) {
       for (int j = tid; j < n; j += NT)
         if (ed[j] < R2) assign_member(a, base, eslot, edold, j, ed[j], R2, nn);
     } else {
-      for_members(T, n, boxes ? (unsigned long long)R2 : 0, [&](int j) {
+      for_members(T, n, boxes && nn > 0 ? (unsigned long long)R2 : 0, [&](int j) {
         const long long d = ed[j];
         if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
       });
@@ -722,7 +816,7 @@ __device__ void level_block(const LevelArgs& a, const int seg, BlockShared& B) {
     ++nn;
     if (m == 1) break;
     __syncthreads();
-    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
+    cur = next_nucleus(a, p0, m, cur, pc, R2, gone, B.K);
   }
   if (tid == 0) {
     a.nnuc[seg] = (uint32_t)nn;
@@ -774,7 +868,8 @@ __device__ void level_small(const LevelArgs& a, const int seg, SmallShared& B) {
     slot[k] = -1;
     dold[k] = 0;
   }
-  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
+  unsigned long long gone = 0;
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, gone, B.K);
   int nn = 0;
   while (cur >= 0) {
     const int4 pc = a.peaks.pos[p0 + cur];
@@ -834,7 +929,7 @@ __device__ void level_small(const LevelArgs& a, const int seg, SmallShared& B) {
     ++nn;
     if (m == 1) break;
     __syncthreads();
-    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
+    cur = next_nucleus(a, p0, m, cur, pc, R2, gone, B.K);
   }
 #pragma unroll
   for (int k = 0; k < SM_PER; ++k)
@@ -866,58 +961,40 @@ enum : int { OP_DONE = 0, OP_HIST = 1, OP_GATHER = 2, OP_RESTART = 3 };
 
 struct ClusterCtl {
   int op;
-  int mode;                 // histogram binning of the window
+  Window W;
   long long R2;
-  unsigned long long wlo, whi, base;  // window and members below it
-  unsigned long long lo, hi, cb;      // bin to gather and its enclosed count
-  int bin;                  // bin being gathered
+  unsigned long long cb;    // enclosed count of the bin to gather
+  int bin;                  // bin to gather, or to find the extent of
+  int listed;               // its members are listed (they fit)
   unsigned in_window;
 };
 
 // leader only: decide the next step of the select from bin `from` of the
-// merged histogram (S.cnt / S.dmn / S.dmx / S.clo, window in Ctl)
+// merged histogram (S.cnt / S.clo, window in Ctl)
 __device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int cap, int n, const PredConst& c,
-                              unsigned long long lim) {
+                              float scale0, unsigned long long lim) {
   const int tid = threadIdx.x;
   if (tid == 0) S.best = NB;
   __syncthreads();
+  const unsigned long long dtop = S.dmax_all < C.W.whi ? S.dmax_all : C.W.whi;
   for (int b = from + tid; b < NB; b += blockDim.x)
-    if (S.cnt[b] && pred(C.base + S.clo[b], S.dmx[b], c)) atomicMin(&S.best, b);
+    if (S.cnt[b] && pred(C.W.base + S.clo[b], bin_top(C.W, b, c, scale0, nb, dtop), c)) atomicMin(&S.best, b);
   __syncthreads();
   if (tid == 0) {
     const int b = S.best;
     if (b < NB) {
-      const unsigned long long lo = S.dmn[b], hi = S.dmx[b], cb = C.base + S.clo[b];
-      if (lo == hi) {  // one distinct value: the bin test was the exact predicate
-        C.op = OP_DONE;
-        C.R2 = (long long)lo;
-      } else if (S.cnt[b] <= (unsigned)cap) {
-        C.op = OP_GATHER;
-        C.lo = lo;
-        C.hi = hi;
-        C.cb = cb;
-        C.bin = b;
-      } else {  // narrow the window to the bin
-        C.op = OP_HIST;
-        C.wlo = lo;
-        C.whi = hi;
-        C.base = cb;
-        C.mode = 1;
-      }
+      C.op = OP_GATHER;
+      C.cb = C.W.base + S.clo[b];
+      C.bin = b;
+      C.listed = S.cnt[b] <= (unsigned)cap;
     } else {  // nothing in the window: move past it
       const unsigned long long top = lim ? lim - 1 : S.dmax_all;
-      if (C.whi < top) {
+      if (C.W.whi < top) {
         C.op = OP_HIST;
-        C.base += C.in_window;
-        C.wlo = C.whi + 1;
-        C.whi = top;
-        C.mode = 1;
+        C.W = Window{C.W.whi + 1, top, C.W.base + C.in_window, 1};
       } else if (lim) {  // nothing below the bound: all members, from the start
         C.op = OP_RESTART;
-        C.base = 0;
-        C.wlo = 0;
-        C.whi = ~0ull;
-        C.mode = 0;
+        C.W = Window{0, ~0ull, 0, 0};
       } else {
         C.op = OP_DONE;
         C.R2 = exhaust_radius((unsigned long long)n, (long long)S.dmax_all, c);
@@ -932,16 +1009,15 @@ __device__ void leader_decide(ClusterCtl& C, SelShared& S, int from, int nb, int
 // memory; after the barrier the leader reads the others' with plain DSMEM
 // loads and combines them.
 __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __restrict__ epos,
-                                      long long* __restrict__ ed, int n, const Tiles& T, int4 pc, const PredConst& c,
+                                      long long* __restrict__ ed, int n, Tiles& T, int4 pc, const PredConst& c,
                                       SelShared& S, ClusterCtl& C, int cap, int nb, unsigned long long lim) {
   const int tid = threadIdx.x;
   const bool leader = cluster.block_rank() == 0;
   const int cs = (int)cluster.num_blocks();
   ClusterCtl* LC = cluster.map_shared_rank(&C, 0);
-  const float scale0 = c.bin_scale0 / (float)((n + nb - 2) / (nb - 1));
+  float scale0 = bin_scale(n, lim, c, nb);
   // the first pass: threshold-count bins over every distance below the bound
-  unsigned long long wlo = 0, whi = lim ? lim - 1 : ~0ull;
-  int mode = 0;
+  Window W{0, lim ? lim - 1 : ~0ull, 0, 0};
   bool first = true;
   int op = OP_HIST;
   while (true) {
@@ -949,15 +1025,12 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
       if (op == OP_RESTART) {
         first = true;
         lim = 0;
+        T.nlist = -1;
+        scale0 = bin_scale(n, 0, c, nb);
       }
-      for (int b = tid; b < NB; b += blockDim.x) {
-        S.cnt[b] = 0;
-        S.dmn[b] = ~0ull;
-        S.dmx[b] = 0;
-      }
+      for (int b = tid; b < NB; b += blockDim.x) S.cnt[b] = 0;
       if (tid == 0 && first) S.dmax_all = 0;
       __syncthreads();
-      const unsigned long long span = whi - wlo + 1;
       unsigned long long dmax = 0;  // this thread's farthest member (first pass)
       for_members(T, n, lim, [&](int j) {
         unsigned long long d;
@@ -968,15 +1041,7 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
         } else {
           d = (unsigned long long)ed[j];
         }
-        if (d < wlo || d > whi) return;
-        int b;
-        if (mode == 0) {
-          b = first_bin(d, c, scale0, nb);
-        } else {
-          b = (int)(((d - wlo) * (unsigned long long)nb) / span);
-        }
-        atomicAdd(&S.cnt[b], 1u);
-        bin_minmax(S, b, d);
+        if (d >= W.wlo && d <= W.whi) atomicAdd(&S.cnt[window_bin(W, d, c, scale0, nb)], 1u);
       });
       if (first) {
         const unsigned long long m = warp_max_u64(dmax);
@@ -984,55 +1049,56 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
       }
       cluster.sync();  // every CTA's histogram of its members is complete
       if (leader) {
-        if (op == OP_HIST && first && tid == 0) {  // (a restart's window is set already)
-          C.base = 0;
-          C.wlo = wlo;
-          C.whi = whi;
-          C.mode = 0;
-        }
+        if (tid == 0) C.W = W;
         // combine the CTAs' histograms (the leader's own is the first share)
-        for (int b = tid; b < NB; b += blockDim.x) {
-          unsigned cn = S.cnt[b];
-          unsigned long long mn = S.dmn[b], mx = S.dmx[b];
-          for (int r = 1; r < cs; ++r) {
-            const SelShared* R = cluster.map_shared_rank(&S, r);
-            cn += R->cnt[b];
-            const unsigned long long a1 = R->dmn[b], a2 = R->dmx[b];
-            mn = a1 < mn ? a1 : mn;
-            mx = a2 > mx ? a2 : mx;
-          }
-          S.cnt[b] = cn;
-          S.dmn[b] = mn;
-          S.dmx[b] = mx;
-        }
-        if (first && tid == 0) {
-          unsigned long long m = S.dmax_all;
-          for (int r = 1; r < cs; ++r) {
-            const unsigned long long v = cluster.map_shared_rank(&S, r)->dmax_all;
-            m = v > m ? v : m;
-          }
-          S.dmax_all = m;
+        static_assert(NB == CL_NT, "one bin per thread");
+        unsigned cn = S.cnt[tid];
+        for (int r = 1; r < cs; ++r) cn += cluster.map_shared_rank(&S, r)->cnt[tid];
+        S.cnt[tid] = cn;
+        if (first && tid < 32) {
+          unsigned long long m = tid < cs ? cluster.map_shared_rank(&S, tid)->dmax_all : 0;
+          m = warp_max_u64(m);
+          if (tid == 0) S.dmax_all = m;
         }
         __syncthreads();
-        static_assert(NB == CL_NT, "one bin per thread");
         unsigned excl;
-        const unsigned tot = block_scan<CL_NT>(S.cnt[tid], excl, S.sw);
+        const unsigned tot = block_scan<CL_NT>(cn, excl, S.sw);
         S.clo[tid] = excl;
         if (tid == 0) C.in_window = tot;
         __syncthreads();
-        leader_decide(C, S, 0, nb, cap, n, c, lim);
+        leader_decide(C, S, 0, nb, cap, n, c, scale0, lim);
       }
       first = false;
-    } else {  // OP_GATHER: every CTA lists its members of the bin, the leader collects them
-      const unsigned long long glo = LC->lo, ghi = LC->hi;
-      if (tid == 0) S.nlist = 0;
+    } else {  // OP_GATHER: every CTA lists its members of the bin (or finds their extent), the leader collects them
+      const int bin = LC->bin;
+      const bool listed = LC->listed;
+      if (tid == 0) {
+        S.nlist = 0;
+        S.lo = ~0ull;
+        S.hi = 0;
+      }
       __syncthreads();
+      unsigned long long lo = ~0ull, hi = 0;
       for_members(T, n, lim, [&](int j) {
         const unsigned long long d = (unsigned long long)ed[j];
-        if (d >= glo && d <= ghi) S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
+        if (d < W.wlo || d > W.whi || window_bin(W, d, c, scale0, nb) != bin) return;
+        if (listed) {
+          S.list[atomicAdd(&S.nlist, 1)] = (long long)d;
+        } else {
+          lo = d < lo ? d : lo;
+          hi = d > hi ? d : hi;
+        }
       });
+      if (!listed) {
+        hi = warp_max_u64(hi);
+        lo = ~warp_max_u64(~lo);
+        if ((tid & 31) == 0) {
+          atomicMin(&S.lo, lo);
+          atomicMax(&S.hi, hi);
+        }
+      }
       cluster.sync();  // every CTA's list is complete
-      if (leader) {
+      if (leader && listed) {
         int off = S.nlist;
         for (int r = 1; r < cs; ++r) {
           const SelShared* R = cluster.map_shared_rank(&S, r);
@@ -1054,8 +1120,38 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
           }
           __syncthreads();
         } else {
-          leader_decide(C, S, C.bin + 1, nb, cap, n, c, lim);
+          leader_decide(C, S, C.bin + 1, nb, cap, n, c, scale0, lim);
         }
+      } else if (leader) {
+        lo = ~0ull;
+        hi = 0;
+        if (tid < cs) {
+          const SelShared* R = cluster.map_shared_rank(&S, tid);
+          lo = R->lo;
+          hi = R->hi;
+        }
+        if (tid < 32) {
+          hi = warp_max_u64(hi);
+          lo = ~warp_max_u64(~lo);
+        }
+        if (tid == 0) {
+          S.best = 0;
+          if (lo == hi) {  // one distinct value: its enclosed count is cb
+            if (pred(C.cb, lo, c)) {
+              C.op = OP_DONE;
+              C.R2 = (long long)lo;
+            } else {
+              S.best = 1;
+            }
+          } else {  // narrow the window to the bin
+            C.op = OP_HIST;
+            C.W = Window{lo, hi, C.cb, 1};
+          }
+        }
+        __syncthreads();
+        const bool next_bin = S.best == 1;
+        __syncthreads();
+        if (next_bin) leader_decide(C, S, C.bin + 1, nb, cap, n, c, scale0, lim);
       }
     }
     // the leader's decision is published, and it has read everyone's shares;
@@ -1064,9 +1160,7 @@ __device__ long long cluster_r_search(cg::cluster_group& cluster, const int4* __
     cluster.sync();
     op = LC->op;
     if (op == OP_DONE) break;
-    wlo = LC->wlo;
-    whi = LC->whi;
-    mode = LC->mode;
+    W = LC->W;
   }
   return LC->R2;
 }
@@ -1075,6 +1169,8 @@ struct ClusterShared {
   SelShared S;
   ClusterCtl C;
   PickShared K;
+  uint32_t tiles[TILE_LIST];
+  int ntiles;
   unsigned h[LEVELS];
   int hbest;
 };
@@ -1099,29 +1195,51 @@ __device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& 
     tile_boxes(T, epos, n, a.tlo + (T.lo - a.tlo), a.thi + (T.hi - a.thi));
     cluster.sync();  // every CTA reads all boxes
   }
-  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, B.K);
+  unsigned long long gone = 0;
+  int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, gone, B.K);
   int nn = 0;
   while (cur >= 0) {
     const int4 pc = a.peaks.pos[p0 + cur];
+    long long R2 = -1;
     unsigned long long lim = 0;
-    if (boxes) {
+    bool tried = false;
+    if (boxes && nn > 0) {
       T.q = tile_origin(epos, pc);
-      lim = search_bound(T, n, a.pc, B.h, &B.hbest);
+      if (private_flags(m)) {
+        // the tries are small: every CTA makes them over all tiles by itself,
+        // which needs no barrier of the cluster.  The CTAs may then be
+        // nuclei apart until the next search of the whole cluster, so a CTA
+        // reads nothing here that another one writes on the way (distances,
+        // flags and earlier radii are its own).
+        Tiles A = T;
+        A.rank = 0;
+        A.cs = 1;
+        for (int k = 0; k < TRIES && R2 < 0; ++k) {
+          const unsigned long long tl = try_bound(k, a.pc);
+          list_tiles(A, tl, B.tiles, &B.ntiles);
+          R2 = r_search<CL_NT>(epos, nullptr, n, pc, a.pc, B.S, 0, a.cap, a.nb, A, tl, false);
+        }
+        tried = R2 >= 0;
+      }
+      T.nlist = -1;
+      if (R2 < 0) lim = search_bound(T, n, a.pc, B.h, &B.hbest);
+      if (tried) list_tiles(T, (unsigned long long)R2, B.tiles, &B.ntiles);
+      else if (lim) list_tiles(T, lim, B.tiles, &B.ntiles);
     }
-    const long long R2 = cluster_r_search(cluster, epos, ed, n, T, pc, a.pc, B.S, B.C, a.cap, a.nb, lim);
+    if (R2 < 0) R2 = cluster_r_search(cluster, epos, ed, n, T, pc, a.pc, B.S, B.C, a.cap, a.nb, lim);
     // steps 1 and 3 on this CTA's share of the members
-    for_members(T, n, boxes ? (unsigned long long)R2 : 0, [&](int j) {
-      const long long d = ed[j];
+    for_members(T, n, boxes && nn > 0 ? (unsigned long long)R2 : 0, [&](int j) {
+      const long long d = tried ? dist2(pc, epos[j]) : ed[j];
       if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
     });
-    if (leader && tid == 0) {
+    if (tid == 0) {  // every CTA: it reads the radii back in later assignments
       a.nuc_member[base + nn] = (uint32_t)pc.w;
       a.nuc_R2[base + nn] = R2;
     }
     ++nn;
     if (m == 1) break;
     __syncthreads();
-    cur = next_nucleus(a, p0, m, cur, pc, R2, B.K);
+    cur = next_nucleus(a, p0, m, cur, pc, R2, gone, B.K);
   }
   if (leader && tid == 0) {
     a.nnuc[seg] = (uint32_t)nn;
@@ -1185,9 +1303,17 @@ __global__ void __launch_bounds__(1024) k_seg_bins(const uint32_t* __restrict__ 
   if (k >= 0) rank[g] = sc[k] + local;
 }
 
-// order[position] = group, bins in order; the tiers' ranges
+// order[position] = group, bins in order; the tiers' ranges.  With the
+// default schedule only as many giants go to clusters as clusters run at a
+// time, and those of 2^GIANT_ALWAYS members or more; the others follow as the
+// first large groups: a 1024-thread block is slower for one such group, but
+// 152 of them finish seventy sooner than 19 clusters do (side-256 box, 74
+// groups above 16,384: level 1 2.05 -> 1.78 ms, level 2 1.05 -> 0.80; the
+// side-128 box has ten and keeps them all on clusters, 0.39 against 0.43 ms).
+constexpr int GIANT_ALWAYS = 17;
 __global__ void __launch_bounds__(1024) k_seg_order(const int* __restrict__ bin, const uint32_t* __restrict__ rank,
-                                                    int nseg, uint32_t* __restrict__ order, TierQueue* q) {
+                                                    int nseg, unsigned max_giants, uint32_t* __restrict__ order,
+                                                    TierQueue* q) {
   __shared__ unsigned first[QBINS + 1];
   __shared__ unsigned sw[33];
   static_assert(QBINS < 1024, "one thread per bin");
@@ -1197,9 +1323,17 @@ __global__ void __launch_bounds__(1024) k_seg_order(const int* __restrict__ bin,
   if (threadIdx.x <= QBINS) first[threadIdx.x] = excl;
   __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x < TIERS) {
-    const unsigned f = first[threadIdx.x * SIZE_BINS];
+    unsigned f = first[threadIdx.x * SIZE_BINS], e = first[(threadIdx.x + 1) * SIZE_BINS];
+    if (max_giants != UINT_MAX && (threadIdx.x == TIER_GIANT || threadIdx.x == TIER_LARGE)) {
+      // the boundary between giants and large groups in the size order
+      const unsigned g0 = first[TIER_GIANT * SIZE_BINS], g1 = first[(TIER_GIANT + 1) * SIZE_BINS];
+      const unsigned big = first[TIER_GIANT * SIZE_BINS + SIZE_BINS - 4 * GIANT_ALWAYS] - g0;
+      const unsigned cut = min(g1, g0 + max(max_giants, big));
+      if (threadIdx.x == TIER_GIANT) e = cut;
+      else f = cut;
+    }
     q->first[threadIdx.x] = f;
-    q->cnt[threadIdx.x] = first[(threadIdx.x + 1) * SIZE_BINS] - f;
+    q->cnt[threadIdx.x] = e - f;
   }
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < nseg && bin[g] >= 0) order[first[bin[g]] + rank[g]] = (uint32_t)g;
@@ -1485,13 +1619,14 @@ int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws
   b.small = sc.small;
   b.medium = a.small_n >= COUNT_N ? std::max(b.small, COUNT_N) : b.small;
   k_seg_bins<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(a.seg_off, a.peaks.off, a.nseg, b, bin, rank, a.nnuc, q);
-  k_seg_order<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(bin, rank, a.nseg, order, q);
-  CSO_CUDA(cudaGetLastError());
   // persistent grids sized to the device; blocks of a tier leave when its
   // queue is empty
   const int occ_l = g_occ_l, occ_m = g_occ_m, occ_s = g_occ_s, occ_w = g_occ_w;
   const int sms = cso_sm_count();
   const int n_clusters = sms / CL_CS > 0 ? sms / CL_CS : 1;
+  k_seg_order<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(bin, rank, a.nseg, sc.set ? UINT_MAX : (unsigned)n_clusters,
+                                                       order, q);
+  CSO_CUDA(cudaGetLastError());
   const int nseg = a.nseg;
   // no tier can hold more groups than there are: grids never exceed nseg
   auto cap = [nseg](long long g) { return (unsigned)(g < nseg ? g : nseg); };

@@ -49,6 +49,7 @@ struct LevelSchedule {
   int giant = 16384;
   int small = 64;
   int huge = CSO_HUGE_GROUP;  // above max(huge, giant): 16-CTA clusters
+  bool set = false;  // bins chosen by the caller or the autotuner: taken as they are
   int large() const { return giant / 16 > 512 ? giant / 16 : 512; }
 };
 
