@@ -442,9 +442,10 @@ __global__ void __launch_bounds__(DENS_WARPS * 32, 4) k_density(CellGrid g, cons
       sum[i] = 0;
     }
     __syncwarp();
-    // past the last neighbour: a staged value no query counts (|b2 - |q|^2| is
-    // below 2^30 in the signed form, |q|^2 below 2^31 in the general one)
-    const int4 none = make_int4(0, 0, 0, SIGNED ? -(1 << 30) : INT_MIN);
+    // past the last neighbour: a staged value no query counts (b2 - d becomes
+    // -|q|^2 in the signed form, and d |q|^2 + 2^31 with |q|^2 below 2^31 in the
+    // general one)
+    const int4 none = make_int4(0, 0, 0, SIGNED ? -(int)b2 : INT_MIN);
     int r = 0;
     uint32_t rend = F.end[0], f = (uint32_t)lane;
     int4 next = make_int4(0, 0, 0, 0);

@@ -28,6 +28,10 @@ def points(u, n, shape, seed):
         r = b * 2.5 * rng.random(n) ** 2
         v = rng.normal(size=(n, 3))
         x = r[:, None] * v / np.linalg.norm(v, axis=1, keepdims=True)
+    elif shape.startswith("even"):  # the first 32 particles fill exactly so many cells of one row
+        side = BOX / int(BOX / np.sqrt(float(np.rint(b * b))))
+        x = np.column_stack([np.ceil(10 * side) + np.arange(n) * (int(shape[4:]) * side - 1) / 32,
+                             np.full((n, 2), 10.5 * side)])
     elif shape == "rod":  # one row of cells, many columns, across the x edge
         x = np.column_stack([rng.uniform(-6 * b, 6 * b, n), rng.uniform(0, 0.9 * b, n), rng.uniform(0, 0.9 * b, n)])
     elif shape == "spot":  # every particle on one grid point or beside it
@@ -38,10 +42,11 @@ def points(u, n, shape, seed):
 
 
 # cell sides around the bounds of the forms: 16,384 (largest), 13,190, 9,490
-# and 9,447 (either side of the signed form's bound), 6,575, 3,277, 1,626
-@pytest.mark.parametrize("u", [40960, 32768, 23640, 23600, 16384, 8192, 4064])
+# and 9,447 (either side of the signed form's bound), 6,575 (spans of up to 4
+# cells), 5,269 (6), 3,931 (8), 3,277, 1,626
+@pytest.mark.parametrize("u", [40960, 32768, 23640, 23600, 16384, 13147, 9822, 8192, 4064])
 @pytest.mark.parametrize("shape,n", [("ball", 3001), ("rod", 1500), ("patch", 2000), ("spot", 257), ("ball", 33),
-                                     ("ball", 1)])
+                                     ("ball", 1), ("even5", 45), ("even7", 45), ("even9", 45)])
 def test_sums_equal_brute_force(u, shape, n):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
