@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(1024) k_radial_stats_big(const uint64_t* __res
 namespace cg = cooperative_groups;
 
 constexpr int SS_CS = 8;
+constexpr int SS_U = 4;  // members a lane loads before it looks at the first
 
 __global__ void __launch_bounds__(256) k_ss_small(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
                                                   int H, const int4* __restrict__ nuc_pos,
@@ -233,130 +234,147 @@ struct Sphere {
   long long R2;
 };
 
-// sphere a within sphere b, with a margin far above the rounding of the square roots
+// sphere a within sphere b, in float with a margin far above its rounding
+// (radii are at most 2^21 grid units and shrink by 5% a step)
 __device__ __forceinline__ bool within(const Sphere& a, const Sphere& b) {
-  double m = 0;
+  float m = 0;
   for (int k = 0; k < 3; ++k) {
-    const double d = (double)min_image(a.c[k] - b.c[k]);
+    const float d = (float)min_image(a.c[k] - b.c[k]);
     m += d * d;
   }
-  return sqrt(m) + sqrt((double)a.R2) + 1.0 <= sqrt((double)b.R2);
+  return (sqrtf(m) + sqrtf((float)a.R2)) * (1.f + 1e-5f) + 2.f <= sqrtf((float)b.R2);
 }
 
 struct SsShared {
   long long w[32][4];   // the warps' sums
-  long long tot[4];     // the block's sums (read by the cluster's other blocks)
+  long long tot[2][4];  // the block's sums, by step parity (read by the cluster's other blocks)
   Sphere s;             // the sphere to count next
   int src;              // which list it is counted in: 0, 1, or 2 for the whole halo
   int go;
-  unsigned n[2];        // members of the two lists (this block's share)
 };
 
-// One halo by one block (CS = 1) or a cluster: members b + lo .. b + hi of
-// epos are this block's share, listed at l0 and l1.
+// One halo by one block (CS = 1) or a cluster: the ns members at `share` are
+// this block's, listed at l0 and l1.  Every warp keeps lists of its own part
+// of them, so a pass needs no counter the warps share, and a step two
+// barriers: after the sums, and after the first warp's decision.
 template <int CS>
 __device__ void shrink_halo(const int4* __restrict__ share, unsigned ns, int4* __restrict__ l0, int4* __restrict__ l1,
                             long long N, int4 start, long long R2start, int x0, cso_radial* __restrict__ out,
                             SsShared& B) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const long long stop = (N + 99) / 100 > SS_N_MIN ? (N + 99) / 100 : SS_N_MIN;
+  // this warp's part, and the members of its two lists
+  const unsigned w0 = (unsigned)((unsigned long long)ns * w / nw), w1 = (unsigned)((unsigned long long)ns * (w + 1) / nw);
+  share += w0;
+  l0 += w0;
+  l1 += w0;
+  unsigned m0 = 0, m1 = 0;
   if (threadIdx.x == 0) {
     B.s = Sphere{{start.x, start.y, start.z}, R2start};
     B.src = 2;
   }
   __syncthreads();
-  Sphere cover[2];  // what the lists hold: every member inside this sphere
-  bool have[2] = {false, false};
-  long long iter = 0;
-  for (;;) {
+  Sphere cover0, cover1;  // (first warp) what the lists hold: every member inside this sphere
+  bool have0 = false, have1 = false;
+  for (long long iter = 0;; ++iter) {
     const Sphere s = B.s;
-    const int src = B.src, dst = src == 0 ? 1 : 0;
+    const int src = B.src;
     const int4* from = src == 2 ? share : src ? l1 : l0;
-    int4* to = dst ? l1 : l0;
-    const unsigned m = src == 2 ? ns : B.n[src];
-    __syncthreads();  // everyone has read the sphere and the list's length
-    if (threadIdx.x == 0) B.n[dst] = 0;
-    __syncthreads();
+    int4* to = src == 0 ? l1 : l0;
+    const unsigned m = src == 2 ? w1 - w0 : src ? m1 : m0;
     long long v[4] = {0, 0, 0, 0};  // count, summed dx, dy, dz
-    for (unsigned j0 = threadIdx.x & ~31u; j0 < m; j0 += blockDim.x) {
-      const unsigned j = j0 + lane;
-      int4 q = make_int4(0, 0, 0, 0);
-      bool in = false;
-      if (j < m) {
-        q = from[j];
-        const long long dx = min_image(q.x - s.c[0]), dy = min_image(q.y - s.c[1]), dz = min_image(q.z - s.c[2]);
-        in = dx * dx + dy * dy + dz * dz < s.R2;
+    unsigned kept = 0;
+    for (unsigned j0 = 0; j0 < m; j0 += 32 * SS_U) {
+      int4 q[SS_U];
+#pragma unroll
+      for (int u = 0; u < SS_U; ++u) {
+        const unsigned j = j0 + u * 32 + lane;
+        q[u] = j < m ? from[j] : make_int4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < SS_U; ++u) {
+        const long long dx = min_image(q[u].x - s.c[0]), dy = min_image(q[u].y - s.c[1]),
+                        dz = min_image(q[u].z - s.c[2]);
+        const bool in = j0 + u * 32 + lane < m && dx * dx + dy * dy + dz * dz < s.R2;
+        const unsigned mask = __ballot_sync(0xffffffffu, in);
         if (in) {
-          v[0] += 1;
           v[1] += dx;
           v[2] += dy;
           v[3] += dz;
+          to[kept + __popc(mask & ((1u << lane) - 1u))] = q[u];
         }
+        kept += __popc(mask);
       }
-      const unsigned mask = __ballot_sync(0xffffffffu, in);
-      if (!mask) continue;
-      unsigned at = 0;
-      if (lane == 0) at = atomicAdd(&B.n[dst], (unsigned)__popc(mask));
-      at = __shfl_sync(0xffffffffu, at, 0);
-      if (in) to[at + __popc(mask & ((1u << lane) - 1u))] = q;
     }
+    if (src == 0) m1 = kept;
+    else m0 = kept;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 1; k < 4; ++k)
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane < 4) B.w[w][lane] = lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3];
-    __syncthreads();
+    if (lane < 4) B.w[w][lane] = lane == 0 ? (long long)kept : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3];
+    __syncthreads();  // (also: the warp's own list is written)
+    long long t = 0;  // value lane & 3 of the sums
     if (w == 0) {
       // the block's sums: eight lanes per value, then across them
-      long long t = 0;
       for (int x = lane >> 2; x < nw; x += 8) t += B.w[x][lane & 3];
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane < 4) B.tot[lane] = t;
+      if (CS > 1 && lane < 4) B.tot[iter & 1][lane] = t;
     }
-    long long t[4];
     if (CS > 1) {
+      // every block's sums; a block writes the other slot in the next step,
+      // and this one again only after that step's barrier
       cg::cluster_group cluster = cg::this_cluster();
-      cluster.sync();  // every block's sums
-      for (int k = 0; k < 4; ++k) t[k] = 0;
-      for (int r = 0; r < CS; ++r) {
-        const long long* o = cluster.map_shared_rank(&B, r)->tot;
-        for (int k = 0; k < 4; ++k) t[k] += o[k];
+      cluster.sync();
+      if (w == 0) {
+        static_assert(CS == 1 || CS == 8, "eight lanes per value");
+        t = cluster.map_shared_rank(&B, lane >> 2)->tot[iter & 1][lane & 3];
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       }
-      cluster.sync();  // read by all before the next step's sums
-    } else {
-      __syncthreads();
-      for (int k = 0; k < 4; ++k) t[k] = B.tot[k];
     }
-    // every thread (of every block) takes the same decision from the same sums
-    if (t[0] < stop) {
-      if (out && threadIdx.x == 0) {
-        out->ss_centre[0] = (s.c[0] + x0) & (CSO_BOX - 1);
-        out->ss_centre[1] = s.c[1];
-        out->ss_centre[2] = s.c[2];
-        out->ss_n = t[0];
-        out->ss_R2 = s.R2;
-        out->ss_iter = iter;
-      }
-      break;
-    }
-    ++iter;
-    if (threadIdx.x == 0) {
+    if (w == 0) {
+      // the first warp of every block takes the same decision from the same sums
+      const long long cnt = __shfl_sync(0xffffffffu, t, 0);
+      // lanes 1-3: the centre's coordinates
+      const int a = (lane & 3) > 0 ? (lane & 3) - 1 : 0;
+      double f = (double)s.c[a] + (double)t / (double)cnt;
+      if (f < 0) f += (double)CSO_BOX;
+      if (f >= (double)CSO_BOX) f -= (double)CSO_BOX;
+      const int c = (int)(llround(f) & (CSO_BOX - 1));
       Sphere nx;
-      for (int a = 0; a < 3; ++a) {
-        double f = (double)s.c[a] + (double)t[a + 1] / (double)t[0];
-        if (f < 0) f += (double)CSO_BOX;
-        if (f >= (double)CSO_BOX) f -= (double)CSO_BOX;
-        nx.c[a] = (int)(llround(f) & (CSO_BOX - 1));
-      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) nx.c[k] = __shfl_sync(0xffffffffu, c, k + 1);
       nx.R2 = s.R2 * 9025 / 10000;
-      cover[dst] = s;
-      have[dst] = true;
-      // (a list that was only read keeps its cover)
-      B.src = within(nx, s) ? dst : (src != 2 && have[src] && within(nx, cover[src])) ? src : 2;
-      B.s = nx;
+      if (src == 0) {
+        cover1 = s;
+        have1 = true;
+      } else {
+        cover0 = s;
+        have0 = true;
+      }
+      if (lane == 0) {
+        B.go = cnt >= stop;
+        if (cnt < stop) {
+          if (out) {
+            out->ss_centre[0] = (s.c[0] + x0) & (CSO_BOX - 1);
+            out->ss_centre[1] = s.c[1];
+            out->ss_centre[2] = s.c[2];
+            out->ss_n = cnt;
+            out->ss_R2 = s.R2;
+            out->ss_iter = iter;
+          }
+        } else {
+          const int dst = src == 0 ? 1 : 0;
+          const bool again = src == 0 ? have0 && within(nx, cover0) : src == 1 && have1 && within(nx, cover1);
+          B.src = within(nx, s) ? dst : again ? src : 2;
+          B.s = nx;
+        }
+      }
     }
     __syncthreads();
+    if (!B.go) break;
   }
   __syncthreads();
 }
