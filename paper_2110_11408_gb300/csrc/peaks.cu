@@ -268,10 +268,12 @@ __global__ void k_peak_place(PeakArgs a, const uint2* __restrict__ found, const 
 int peaks_find(const PeakArgs& a, const uint32_t* gs, const uint32_t* seg, int m, int nseg, long long T_min,
                long long T_test, bool first, int* beater, PeakList& P, Workspace& ws, cudaStream_t st) {
   P.off = ws.get<uint32_t>((size_t)nseg + 1);
-  P.pos = ws.get<int4>(m);
-  P.sig = ws.get<long long>(m);
-  P.id = ws.get<uint64_t>(m);
-  P.out = ws.get<uint8_t>(m);
+  if (!P.pos) {
+    P.pos = ws.get<int4>(m);
+    P.sig = ws.get<long long>(m);
+    P.id = ws.get<uint64_t>(m);
+    P.out = ws.get<uint8_t>(m);
+  }
   const size_t mark = ws.off;
   PeakOut o;
   o.found = ws.get<uint2>(m);

@@ -25,8 +25,9 @@ struct PeakList {
 
 // Members gs[0 .. m) (cell-sorted indices, seg[k] the segment of member k)
 // whose kernel sum is above T_min and that no denser member of the same
-// segment within b comes before (Sec. 2.2.2 step 2): fills P (allocated here
-// from ws, which keeps them).
+// segment within b comes before (Sec. 2.2.2 step 2): fills P, whose arrays are
+// allocated here from ws (which keeps them) unless P brings arrays of at
+// least m peaks.
 //
 // beater (one entry per cell-sorted particle) links the levels: with
 // `first`, every member above T_test is tested and beater[s] receives one

@@ -435,7 +435,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   S.mark("level1");
   ALLOC(int, beater, n);
   PeakArgs pk{g, spos, sigma, sid, root, (uint32_t)p->b2, N};
-  PeakList peaks;
+  PeakList peaks{};
   CSO_TRY(peaks_find(pk, gs, gseg, nd, G, p->T_min_L1, p->T_min_L1 < p->T_min_L2 ? p->T_min_L1 : p->T_min_L2, true,
                      beater, peaks, ws, st));
   ALLOC(int, eslot, nd);
@@ -522,7 +522,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   // ---- level2 ----
   S.mark("level2");
   pk.slab = lab1;
-  PeakList peaks2;
+  PeakList peaks2 = peaks;  // level 1 is done with its list: the same memory
   CSO_TRY(peaks_find(pk, egs2, ehal2, na, H1, p->T_min_L2, p->T_min_L2, false, beater, peaks2, ws, st));
   ALLOC(int, eslot2, na);
   CSO_CUDA(cudaMemsetAsync(eslot2, 0xff, sizeof(int) * (size_t)na, st));
@@ -599,7 +599,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
       ALLOC(cso_radial, r1, H1);
       rad = r1;
       CSO_TRY(radial_run(seg2, ehal2, epos2, na, rows, H1, gi.x0, p->l_mean_grid, hnuc, spos, rad, c->pinned, ws,
-                         st));
+                         st, SideStreams{{c->side, c->side2, c->side3}, c->fork, {c->join, c->join2, c->join3}}));
       S.mark("catalogue");
     }
     ALLOC(uint32_t, kscan, H1 + 1);

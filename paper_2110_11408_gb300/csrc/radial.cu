@@ -80,12 +80,15 @@ __device__ __forceinline__ bool vbetter(unsigned long long na_, unsigned long lo
 }
 
 // Haloes by the work they need: a halo below SS_N_MIN members stops at its
-// first shrinking sphere, one of SS_BIG or more takes the biggest blocks.
+// first shrinking sphere; the others take a 256-thread block, a 1024-thread
+// block from SS_LARGE members and a cluster of such blocks from SS_BIG.
 constexpr long long SS_N_MIN = 700;
+constexpr long long SS_LARGE = 4096;
 constexpr long long SS_BIG = 16384;
+enum : int { SS_MID = 0, SS_LRG, SS_CLU, SS_KINDS };
 
 struct SsLists {  // listed haloes of each kind and their fetch counters
-  unsigned n_mid, n_big, next_mid, next_big;
+  unsigned n[SS_KINDS], next[SS_KINDS];
 };
 
 // Quantiles and the circular-velocity peak from a halo's sorted distances, a
@@ -99,17 +102,24 @@ __device__ void radial_stats(const uint64_t* __restrict__ key, unsigned long lon
   const uint64_t* D = key + b;
   unsigned long long bn = 0, bd = 0;
   float fn2 = 0.f, fd = 1.f;  // the best so far in float
-  for (uint32_t i = threadIdx.x; i < n; i += NT) {
-    const unsigned long long di = D[i] & dmask;
-    if (di == 0) continue;
-    const float cn = (float)(i + 1), cd = (float)di;
-    if (cn * cn * fd < fn2 * cd * (1.f - 1e-5f)) continue;
-    if (i + 1 < n && (D[i + 1] & dmask) == di) continue;  // N(<= r) takes the whole shell
-    if (vbetter(i + 1, di, bn, bd)) {
-      bn = i + 1;
-      bd = di;
-      fn2 = cn * cn;
-      fd = cd;
+  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 4 * NT) {
+    unsigned long long dq[4];  // four loads in flight
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dq[k] = i0 + k * NT < n ? D[i0 + k * NT] & dmask : 0ull;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t i = i0 + k * NT;
+      const unsigned long long di = dq[k];
+      if (di == 0) continue;
+      const float cn = (float)(i + 1), cd = (float)di;
+      if (cn * cn * fd < fn2 * cd * (1.f - 1e-5f)) continue;
+      if (i + 1 < n && (D[i + 1] & dmask) == di) continue;  // N(<= r) takes the whole shell
+      if (vbetter(i + 1, di, bn, bd)) {
+        bn = i + 1;
+        bd = di;
+        fn2 = cn * cn;
+        fd = cd;
+      }
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -160,7 +170,7 @@ __global__ void __launch_bounds__(1024) k_radial_stats_big(const uint64_t* __res
                                                            const uint32_t* __restrict__ list, const SsLists* L,
                                                            cso_radial* __restrict__ out) {
   __shared__ unsigned long long sn[32], sd[32];
-  for (unsigned it = blockIdx.x; it < L->n_big; it += gridDim.x) {
+  for (unsigned it = blockIdx.x; it < L->n[SS_CLU]; it += gridDim.x) {
     const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
     radial_stats<1024>(key, dmask, b, n, u, out[h], sn, sd);
     __syncthreads();
@@ -180,11 +190,12 @@ __global__ void __launch_bounds__(1024) k_radial_stats_big(const uint64_t* __res
 // shrank, the usual case), that list is all the next pass needs; otherwise the
 // list before it serves if the next sphere lies within its sphere, and the
 // whole halo if not.  The lists shrink with the sphere, so a halo costs about
-// twenty passes over its members instead of eighty.  Haloes below SS_BIG
-// members take a 256-thread block, the others a cluster of eight 1024-thread
-// blocks, each with its own share of the members, which add up their sums in
-// one another's shared memory (one block per halo: 4.1 ms for a halo of
-// 150,000 members; now 0.2).
+// twenty passes over its members instead of eighty.  The blocks of a cluster
+// each have their own share of the members and add up their sums in one
+// another's shared memory.  The three kinds run at the same time, beside the
+// distances' sort (the loops are eighty dependent steps of a microsecond or
+// two, which leave the GPU idle).  One block per halo and a pass over all its
+// members per step took 4.1 ms for a halo of 150,000 members.
 // ---------------------------------------------------------------------------
 namespace cg = cooperative_groups;
 
@@ -194,8 +205,8 @@ constexpr int SS_U = 4;  // members a lane loads before it looks at the first
 __global__ void __launch_bounds__(256) k_ss_small(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
                                                   int H, const int4* __restrict__ nuc_pos,
                                                   const uint32_t* __restrict__ hnuc,
-                                                  const cso_halo* __restrict__ rows, int x0, uint32_t* __restrict__ mid,
-                                                  uint32_t* __restrict__ big, SsLists* L,
+                                                  const cso_halo* __restrict__ rows, int x0, uint32_t* __restrict__ list,
+                                                  SsLists* L,
                                                   cso_radial* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int h = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -203,10 +214,8 @@ __global__ void __launch_bounds__(256) k_ss_small(const int4* __restrict__ epos,
   const uint32_t b = seg[h];
   const long long N = seg[h + 1] - b;
   if (N >= SS_N_MIN) {
-    if (lane == 0) {
-      if (N >= SS_BIG) big[atomicAdd(&L->n_big, 1u)] = (uint32_t)h;
-      else mid[atomicAdd(&L->n_mid, 1u)] = (uint32_t)h;
-    }
+    const int kind = N >= SS_BIG ? SS_CLU : N >= SS_LARGE ? SS_LRG : SS_MID;
+    if (lane == 0) list[(size_t)kind * H + atomicAdd(&L->n[kind], 1u)] = (uint32_t)h;
     return;
   }
   const int4 c = nuc_pos[hnuc[h]];
@@ -379,19 +388,20 @@ __device__ void shrink_halo(const int4* __restrict__ share, unsigned ns, int4* _
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(256) k_ss_mid(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
-                                                const int4* __restrict__ nuc_pos, const uint32_t* __restrict__ hnuc,
-                                                const cso_halo* __restrict__ rows, int x0,
-                                                const uint32_t* __restrict__ list, SsLists* L, int4* __restrict__ l0,
-                                                int4* __restrict__ l1, cso_radial* __restrict__ out) {
+template <int NT, int KIND>
+__global__ void __launch_bounds__(NT) k_ss_block(const int4* __restrict__ epos, const uint32_t* __restrict__ seg,
+                                                 const int4* __restrict__ nuc_pos, const uint32_t* __restrict__ hnuc,
+                                                 const cso_halo* __restrict__ rows, int x0,
+                                                 const uint32_t* __restrict__ list, SsLists* L, int4* __restrict__ l0,
+                                                 int4* __restrict__ l1, cso_radial* __restrict__ out) {
   __shared__ SsShared B;
   __shared__ unsigned item;
   for (;;) {
-    if (threadIdx.x == 0) item = atomicAdd(&L->next_mid, 1u);
+    if (threadIdx.x == 0) item = atomicAdd(&L->next[KIND], 1u);
     __syncthreads();
     const unsigned it = item;
     __syncthreads();
-    if (it >= L->n_mid) return;
+    if (it >= L->n[KIND]) return;
     const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
     shrink_halo<1>(epos + b, n, l0 + b, l1 + b, n, nuc_pos[hnuc[h]], rows[h].R2, x0, out + h, B);
   }
@@ -407,11 +417,11 @@ __global__ void __cluster_dims__(SS_CS, 1, 1) __launch_bounds__(1024)
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned rank = cluster.block_rank();
   for (;;) {
-    if (rank == 0 && threadIdx.x == 0) item = atomicAdd(&L->next_big, 1u);
+    if (rank == 0 && threadIdx.x == 0) item = atomicAdd(&L->next[SS_CLU], 1u);
     cluster.sync();
     const unsigned it = *cluster.map_shared_rank(&item, 0);
     cluster.sync();  // read by all before it changes
-    if (it >= L->n_big) return;
+    if (it >= L->n[SS_CLU]) return;
     const uint32_t h = list[it], b = seg[h], n = seg[h + 1] - b;
     const uint32_t lo = (uint32_t)((unsigned long long)n * rank / SS_CS);
     const uint32_t hi = (uint32_t)((unsigned long long)n * (rank + 1) / SS_CS);
@@ -424,25 +434,51 @@ __global__ void __cluster_dims__(SS_CS, 1, 1) __launch_bounds__(1024)
 
 int radial_run(const uint32_t* seg, const uint32_t* ehal, const int4* epos, long long na, const cso_halo* rows,
                int H, int x0, double u, const uint32_t* hnuc, const int4* nuc_pos, cso_radial* out, void* pinned,
-               Workspace& ws, cudaStream_t st) {
+               Workspace& ws, cudaStream_t st, const SideStreams& side) {
   if (H <= 0) return CSO_OK;
   const size_t mark = ws.off;
   SsLists* lists = ws.get<SsLists>(1);
-  uint32_t* mid = ws.get<uint32_t>(H);
-  uint32_t* big = ws.get<uint32_t>(H);
-  const size_t after_lists = ws.off;
+  uint32_t* list = ws.get<uint32_t>((size_t)SS_KINDS * H);
+  int4* l0 = ws.get<int4>(na);
+  int4* l1 = ws.get<int4>(na);
   int4* cen = ws.get<int4>(H);
   uint64_t* key = ws.get<uint64_t>(na);
   uint64_t* key2 = ws.get<uint64_t>(na);
   uint32_t* val = ws.get<uint32_t>(na);
   uint32_t* val2 = ws.get<uint32_t>(na);
   unsigned long long* dmax = ws.get<unsigned long long>(1);
-  if (!lists || !mid || !big || !cen || !key || !key2 || !val || !val2 || !dmax) {
+  if (!lists || !list || !l0 || !l1 || !cen || !key || !key2 || !val || !val2 || !dmax) {
     cso_set_error("workspace exhausted in the radial statistics");
     return CSO_ERR_BUDGET;
   }
+  // the shrinking spheres on the side streams; no return leaves one running
+  struct Join {
+    const SideStreams& s;
+    bool on = false;
+    ~Join() {
+      if (on)
+        for (int k = 0; k < 3; ++k) cudaStreamSynchronize(s.stream[k]);
+    }
+  } join{side};
   CSO_CUDA(cudaMemsetAsync(lists, 0, sizeof(SsLists), st));
-  k_ss_small<<<CL(cdiv(H, 8)), 256, 0, st>>>(epos, seg, H, nuc_pos, hnuc, rows, x0, mid, big, lists, out);
+  k_ss_small<<<CL(cdiv(H, 8)), 256, 0, st>>>(epos, seg, H, nuc_pos, hnuc, rows, x0, list, lists, out);
+  CSO_CUDA(cudaEventRecord(side.fork, st));
+  join.on = true;
+  for (int k = 0; k < 3; ++k) CSO_CUDA(cudaStreamWaitEvent(side.stream[k], side.fork, 0));
+  const int sms = cso_sm_count();
+  const unsigned clusters = (unsigned)(sms / SS_CS > 0 ? sms / SS_CS : 1);
+  if (na >= SS_BIG)
+    k_ss_big<<<CL(clusters * SS_CS), 1024, 0, side.stream[0]>>>(epos, seg, nuc_pos, hnuc, rows, x0,
+                                                               list + (size_t)SS_CLU * H, lists, l0, l1, out);
+  if (na >= SS_LARGE)
+    k_ss_block<1024, SS_LRG><<<CL(sms), 1024, 0, side.stream[1]>>>(epos, seg, nuc_pos, hnuc, rows, x0,
+                                                                 list + (size_t)SS_LRG * H, lists, l0, l1, out);
+  if (na >= SS_N_MIN)
+    k_ss_block<256, SS_MID><<<CL(sms * 8), 256, 0, side.stream[2]>>>(epos, seg, nuc_pos, hnuc, rows, x0,
+                                                                   list + (size_t)SS_MID * H, lists, l0, l1, out);
+  CSO_CUDA(cudaGetLastError());
+  for (int k = 0; k < 3; ++k) CSO_CUDA(cudaEventRecord(side.join[k], side.stream[k]));
+  // distances to the centre, sorted by (halo, distance)
   k_radial_centre<<<CL(cdiv(H, 256)), 256, 0, st>>>(rows, H, x0, cen, out);
   CSO_CUDA(cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), st));
   if (na > 0) {
@@ -481,22 +517,11 @@ int radial_run(const uint32_t* seg, const uint32_t* ehal, const int4* epos, long
     }
   }
   if (na >= SS_BIG)
-    k_radial_stats_big<<<CL(cso_sm_count()), 1024, 0, st>>>(sorted, dmask, seg, u, big, lists, out);
+    k_radial_stats_big<<<CL(sms), 1024, 0, st>>>(sorted, dmask, seg, u, list + (size_t)SS_CLU * H, lists, out);
   k_radial_stats<<<CL(H), 256, 0, st>>>(sorted, dmask, seg, u, out);
-  // the shrinking spheres' lists take the place of the sort's buffers
-  ws.off = after_lists;
-  int4* l0 = ws.get<int4>(na);
-  int4* l1 = ws.get<int4>(na);
-  if (!l0 || !l1) {
-    cso_set_error("workspace exhausted in the shrinking spheres");
-    return CSO_ERR_BUDGET;
-  }
-  const unsigned clusters = (unsigned)(cso_sm_count() / SS_CS > 0 ? cso_sm_count() / SS_CS : 1);
-  if (na >= SS_BIG)
-    k_ss_big<<<CL(clusters * SS_CS), 1024, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, big, lists, l0, l1, out);
-  if (na >= SS_N_MIN)
-    k_ss_mid<<<CL(cso_sm_count() * 8), 256, 0, st>>>(epos, seg, nuc_pos, hnuc, rows, x0, mid, lists, l0, l1, out);
   CSO_CUDA(cudaGetLastError());
+  for (int k = 0; k < 3; ++k) CSO_CUDA(cudaStreamWaitEvent(st, side.join[k], 0));
+  join.on = false;
   ws.off = mark;
   return CSO_OK;
 }
