@@ -12,6 +12,7 @@
 #include <math.h>
 
 #include "cells.cuh"
+#include "rank2.cuh"
 
 namespace {
 
@@ -553,24 +554,85 @@ __device__ __forceinline__ void uf_unite(int* parent, int a, int b) {
   }
 }
 
-// parent[s] = s for dense particles, -1 for the rest (one load answers both);
-// flag[s] = dense, scanned into the positions of the dense list
-__global__ void k_fof_init(int* __restrict__ parent, uint32_t* __restrict__ flag, int n,
-                           const long long* __restrict__ sigma, long long T_L0) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const bool dense = sigma[s] > T_L0;
-  parent[s] = dense ? s : -1;
-  flag[s] = dense;
+// Every cell that holds dense particles has a main tree: the tree of its
+// first dense particle after pass one, kept at slot start[c] of a
+// per-particle array (the first slot of every non-empty cell is its own) so
+// the summary costs n entries instead of one per cell of the sparse table;
+// CELL_EMPTY marks cells without dense particles.  A dense particle outside
+// its cell's main tree at that point is a straggler.
+constexpr int CELL_EMPTY = -2;
+
+__device__ __forceinline__ uint32_t cell_id(const CellGrid& g, int4 p) {
+  return (uint32_t)grid_cell(g, cell_coord(p.z, g.nc), cell_coord(p.y, g.nc), grid_col(g, p.x));
 }
 
-// the dense particles in cell order: FoF threads take one each, so a warp
-// holds 32 dense particles (consecutive in their cells) instead of 32 slots
-// of which only the dense ones work
-__global__ void k_dense_list(const uint32_t* __restrict__ pos_in_list, const int* __restrict__ parent, int n,
-                             int* __restrict__ didx) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < n && parent[s] >= 0) didx[pos_in_list[s]] = s;
+// The forest's start (parent[s] = s for dense particles, -1 for the rest: one
+// load answers both), the cells' summaries and the groups' smallest ids
+// cleared, and two lists in cell order: the dense particles (FoF threads take
+// one each, so a warp holds 32 dense particles instead of 32 slots of which
+// only the dense ones work), and the first dense particle of every cell that
+// holds any.  counts[0] and counts[1] receive their lengths.  (A pass each
+// for the flags, their scans and the lists: 0.39 ms on the side-256 box, this
+// one 0.16.)
+__global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4* __restrict__ spos, int n,
+                                                          const long long* __restrict__ sigma, long long T_L0,
+                                                          int* __restrict__ parent, int* __restrict__ cell_root,
+                                                          unsigned long long* __restrict__ minid,
+                                                          int* __restrict__ didx, int* __restrict__ clist,
+                                                          uint32_t* __restrict__ counts,
+                                                          unsigned long long* __restrict__ status, long long ntiles,
+                                                          int* __restrict__ err) {
+  __shared__ Rank2Shared S;
+  const long long tile = rank2_tile(S, status, ntiles);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
+  unsigned dense[R2_ITEMS], head[R2_ITEMS];
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long i = base + q * 32 + lane;
+    const bool in = i < n;
+    const bool d = in && sigma[i] > T_L0;
+    dense[q] = __ballot_sync(0xffffffffu, d);
+    if (in) {
+      parent[i] = d ? (int)i : -1;
+      cell_root[i] = CELL_EMPTY;
+      minid[i] = ~0ull;
+    }
+  }
+  uint32_t na = 0, nb = 0;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    bool h = false;
+    if (dense[q] >> lane & 1u) {
+      // first of its cell: no dense slot before it there (the one next to it, mostly)
+      const long long i = base + q * 32 + lane;
+      const uint32_t c = cell_id(g, spos[i]);
+      h = true;
+      for (long long t = i - 1; t >= 0 && cell_id(g, spos[t]) == c; --t)
+        if (sigma[t] > T_L0) {
+          h = false;
+          break;
+        }
+    }
+    head[q] = __ballot_sync(0xffffffffu, h);
+    na += __popc(dense[q]);
+    nb += __popc(head[q]);
+  }
+  uint32_t ta, tb;
+  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const int i = (int)(base + q * 32 + lane);
+    if (dense[q] >> lane & 1u) didx[na + __popc(dense[q] & lt)] = i;
+    if (head[q] >> lane & 1u) clist[nb + __popc(head[q] & lt)] = i;
+    na += __popc(dense[q]);
+    nb += __popc(head[q]);
+  }
+  if (tile == ntiles - 1 && threadIdx.x == 0) {
+    counts[0] = ta;
+    counts[1] = tb;
+  }
 }
 
 // Pass one (in the spirit of Afforest, Sutton et al. 2018): each dense
@@ -663,104 +725,79 @@ __global__ void __launch_bounds__(256) k_fof_sample(CellGrid g, const int4* __re
   }
 }
 
-// point every dense particle straight at its current root
-__global__ void k_fof_compress(int* __restrict__ parent, int n) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < n && parent[s] >= 0) parent[s] = uf_root(parent, s);
-}
-
-// heads of the cells holding dense particles: position i of the dense list
-// starts a cell (the list is in cell order)
-__global__ void k_cell_heads(const int4* __restrict__ spos, CellGrid g, const int* __restrict__ didx,
-                             const uint32_t* __restrict__ nd_ptr, int n, uint32_t* __restrict__ head) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int nd = (int)*nd_ptr;
-  uint32_t h = 0;
-  if (i < nd) {
-    const int4 p = spos[didx[i]];
-    const size_t c = grid_cell(g, cell_coord(p.z, g.nc), cell_coord(p.y, g.nc), grid_col(g, p.x));
-    if (i == 0) {
-      h = 1;
-    } else {
-      const int4 q = spos[didx[i - 1]];
-      h = c != grid_cell(g, cell_coord(q.z, g.nc), cell_coord(q.y, g.nc), grid_col(g, q.x));
-    }
-  }
-  head[i] = h;
-}
-
-__global__ void k_cell_list(const uint32_t* __restrict__ head_scan, const int* __restrict__ didx,
-                            const uint32_t* __restrict__ nd_ptr, int* __restrict__ clist) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int)*nd_ptr) return;
-  if (head_scan[i + 1] != head_scan[i]) clist[head_scan[i]] = didx[i];
-}
-
-// Every cell that holds dense particles has a main tree: the tree of its
-// first dense particle after pass one, kept at slot start[c] of a
-// per-particle array (the first slot of every non-empty cell is its own) so
-// the summary costs n entries instead of one per cell of the sparse table;
-// CELL_EMPTY marks cells without dense particles.  A dense particle outside
-// its cell's main tree at that point is a straggler.
-constexpr int CELL_EMPTY = -2;
-
-__global__ void k_cell_root_init(int* __restrict__ cell_root, long long n) {
-  long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < n) cell_root[c] = CELL_EMPTY;
-}
-
+// the main tree of every cell that holds dense particles, after pass one
 __global__ void k_cell_main(const int4* __restrict__ spos, CellGrid g, const int* __restrict__ clist,
-                            const uint32_t* __restrict__ ncl_ptr, const int* __restrict__ parent,
-                            int* __restrict__ cell_root, uint2* __restrict__ srange) {
+                            const uint32_t* __restrict__ ncl_ptr, int* __restrict__ parent,
+                            int* __restrict__ cell_root) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int)*ncl_ptr) return;
   const int s0 = clist[i];
-  const int4 p = spos[s0];
-  const size_t c = grid_cell(g, cell_coord(p.z, g.nc), cell_coord(p.y, g.nc), grid_col(g, p.x));
-  cell_root[g.start[c]] = parent[s0];  // a root after compression
-  srange[g.start[c]] = make_uint2(0, 0);
+  cell_root[g.start[cell_id(g, spos[s0])]] = uf_root(parent, s0);
 }
 
-// srange[start[c]] = the run of cell c in the straggler list (in cell order)
-__global__ void k_straggler_ranges(const int4* __restrict__ spos, CellGrid g, const int* __restrict__ slist,
-                                   const uint32_t* __restrict__ ns_ptr, uint2* __restrict__ srange) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int ns = (int)*ns_ptr;
-  if (i >= ns) return;
-  auto cell_of = [&](int s) {
-    const int4 p = spos[s];
-    return grid_cell(g, cell_coord(p.z, g.nc), cell_coord(p.y, g.nc), grid_col(g, p.x));
-  };
-  const size_t c = cell_of(slist[i]);
-  const uint32_t slot = g.start[c];
-  if (i == 0 || cell_of(slist[i - 1]) != c) srange[slot].x = (uint32_t)i;
-  if (i == ns - 1 || cell_of(slist[i + 1]) != c) srange[slot].y = (uint32_t)i + 1;
-}
-
-__global__ void k_stragglers(const int4* __restrict__ spos, CellGrid g, const int* __restrict__ didx,
-                             const uint32_t* __restrict__ nd_ptr, int n, const int* __restrict__ parent,
-                             const int* __restrict__ cell_root, uint8_t* __restrict__ strag,
-                             uint32_t* __restrict__ sflag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t f = 0;
-  if (i < (int)*nd_ptr) {
-    const int s = didx[i];
-    const int4 p = spos[s];
-    const size_t c = grid_cell(g, cell_coord(p.z, g.nc), cell_coord(p.y, g.nc), grid_col(g, p.x));
-    f = parent[s] != cell_root[g.start[c]];
-    strag[s] = (uint8_t)f;
+// The stragglers, listed in cell order; srange[start[c]] = the run of cell c
+// (one with dense particles) in that list.  Also points every dense particle
+// straight at its root.  Tiles are of the dense list: those past its end have
+// nothing to publish.
+__global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restrict__ spos, CellGrid g,
+                                                           const int* __restrict__ didx, uint32_t* __restrict__ counts,
+                                                           int* __restrict__ parent, const int* __restrict__ cell_root,
+                                                           uint8_t* __restrict__ strag, int* __restrict__ slist,
+                                                           uint2* __restrict__ srange,
+                                                           unsigned long long* __restrict__ status, long long ntiles,
+                                                           int* __restrict__ err) {
+  __shared__ Rank2Shared S;
+  const long long nd = counts[0];
+  const long long tile = rank2_tile(S, status, ntiles);
+  if (tile * R2_TILE >= nd) return;  // counts[2] starts at zero
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
+  unsigned flag[R2_ITEMS];
+  uint32_t lo[R2_ITEMS];  // the cell's first slot; top bits: first and last dense particle of the cell
+  unsigned first = 0, last = 0;
+  uint32_t na = 0, nb = 0;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long i = base + q * 32 + lane;
+    bool f = false, a = false, z = false;
+    uint32_t c = 0;
+    const bool in = i < nd;
+    int s = 0;
+    if (in) {
+      s = didx[i];
+      c = cell_id(g, spos[s]);
+    }
+    uint32_t cp = __shfl_up_sync(0xffffffffu, c, 1), cn = __shfl_down_sync(0xffffffffu, c, 1);
+    lo[q] = 0;
+    if (in) {
+      if (lane == 0) cp = i > 0 ? cell_id(g, spos[didx[i - 1]]) : ~c;
+      if (lane == 31) cn = i + 1 < nd ? cell_id(g, spos[didx[i + 1]]) : ~c;
+      a = cp != c;
+      z = cn != c || i + 1 == nd;
+      lo[q] = g.start[c];
+      const int r = uf_root(parent, s);
+      parent[s] = r;
+      f = r != cell_root[lo[q]];
+      strag[s] = (uint8_t)f;
+    }
+    first |= (unsigned)a << q;
+    last |= (unsigned)z << q;
+    flag[q] = __ballot_sync(0xffffffffu, f);
+    na += __popc(flag[q]);
   }
-  sflag[i] = f;
-}
-
-// the stragglers in list order (flags scanned in place)
-__global__ void k_straggler_list(const uint32_t* __restrict__ sscan, const int* __restrict__ didx,
-                                 const uint32_t* __restrict__ nd_ptr, int* __restrict__ slist) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int)*nd_ptr) return;
-  if (sscan[i + 1] != sscan[i]) slist[sscan[i]] = didx[i];
+  uint32_t ta, tb;
+  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const uint32_t r = na + __popc(flag[q] & lt);
+    const uint32_t f = flag[q] >> lane & 1u;
+    if (f) slist[r] = didx[base + q * 32 + lane];
+    if (first >> q & 1u) srange[lo[q]].x = r;
+    if (last >> q & 1u) srange[lo[q]].y = r + f;
+    na += __popc(flag[q]);
+  }
+  if ((tile + 1) * R2_TILE >= nd && threadIdx.x == 0) counts[2] = ta;
 }
 
 // Pass two, main trees as units: for every cell with dense particles and
@@ -1191,44 +1228,41 @@ int cells_fof(const CellGrid& g, const int4* spos, int n, const long long* sigma
               Workspace& ws, cudaStream_t st) {
   if (n <= 0) return CSO_OK;
   const size_t mark = ws.off;
-  uint32_t* flag = ws.get<uint32_t>((size_t)n + 1);
+  const long long words = rank2_words(n);
   int* didx = ws.get<int>(n);
-  uint32_t* head = ws.get<uint32_t>((size_t)n + 1);
   int* clist = ws.get<int>(n);
   uint8_t* strag = ws.get<uint8_t>(n);
-  uint32_t* sflag = ws.get<uint32_t>((size_t)n + 1);
   int* slist = ws.get<int>(n);
   uint2* srange = ws.get<uint2>(n);
-  if (!flag || !didx || !head || !clist || !strag || !sflag || !slist || !srange) {
+  // status words of the two lists' ranks, then the list lengths: dense
+  // particles, cells that hold any, stragglers
+  unsigned long long* status = ws.get<unsigned long long>((size_t)(2 * words + 2));
+  if (!didx || !clist || !strag || !slist || !srange || !status) {
     cso_set_error("workspace exhausted in the FoF pass");
     return CSO_ERR_BUDGET;
   }
-  // the dense list and the cells that hold dense particles; launches over
-  // them are sized by n and blocks past the counts (read on the device)
-  // return at once
-  k_fof_init<<<CL(cdiv(n, 256)), 256, 0, st>>>(parent, flag, n, sigma, T_L0);
-  CSO_TRY(scan_u32(flag, n, flag + n, ws, st));
-  k_dense_list<<<CL(cdiv(n, 256)), 256, 0, st>>>(flag, parent, n, didx);
-  const uint32_t* nd = flag + n;
-  k_cell_heads<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, didx, nd, n, head);
-  CSO_TRY(scan_u32(head, n, head + n, ws, st));
-  k_cell_list<<<CL(cdiv(n, 256)), 256, 0, st>>>(head, didx, nd, clist);
-  const uint32_t* ncl = head + n;
+  if (!ws.err) {
+    cso_set_error("FoF lists without a device error word");
+    return CSO_ERR_STATE;
+  }
+  uint32_t* counts = reinterpret_cast<uint32_t*>(status + 2 * words);
+  const unsigned tiles = (unsigned)(words - 1);
+  CSO_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)(2 * words + 2), st));
+  // launches over the lists are sized by n and blocks past the counts (read
+  // on the device) return at once
+  k_fof_lists<<<CL(tiles), R2_THREADS, 0, st>>>(g, spos, n, sigma, T_L0, parent, cell_root, minid, didx, clist, counts,
+                                                status, words - 1, ws.err);
+  const uint32_t *nd = counts, *ncl = counts + 1, *ns = counts + 2;
   // pass one: bands inside cells; main trees and stragglers
   k_fof_sample<<<CL(cdiv(n, 256)), 256, 0, st>>>(g, spos, didx, nd, lfof2, parent);
-  k_fof_compress<<<CL(cdiv(n, 256)), 256, 0, st>>>(parent, n);
-  k_cell_root_init<<<CL(cdiv(n, 256)), 256, 0, st>>>(cell_root, n);
-  k_cell_main<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, clist, ncl, parent, cell_root, srange);
-  k_stragglers<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, didx, nd, n, parent, cell_root, strag, sflag);
-  CSO_TRY(scan_u32(sflag, n, sflag + n, ws, st));
-  k_straggler_list<<<CL(cdiv(n, 256)), 256, 0, st>>>(sflag, didx, nd, slist);
-  k_straggler_ranges<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, slist, sflag + n, srange);
+  k_cell_main<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, clist, ncl, parent, cell_root);
+  k_stragglers<<<CL(tiles), R2_THREADS, 0, st>>>(spos, g, didx, counts, parent, cell_root, strag, slist, srange,
+                                                 status + words, words - 1, ws.err);
   // pass two: main trees of adjacent cells; pass three: stragglers
   const int lreach = reach_below(lfof2);
   k_fof_cells<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, clist, ncl, lfof2, lreach, parent, cell_root, strag);
-  k_fof_stragglers<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, slist, sflag + n, lfof2, lreach, parent, cell_root,
+  k_fof_stragglers<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, slist, ns, lfof2, lreach, parent, cell_root,
                                                            strag, srange);
-  CSO_CUDA(cudaMemsetAsync(minid, 0xff, sizeof(unsigned long long) * n, st));
   k_fof_finish<<<CL(cdiv(n, 256)), 256, 0, st>>>(parent, n, sigma, T_L0, sid, root, minid);
   CSO_CUDA(cudaGetLastError());
   ws.off = mark;

@@ -19,20 +19,52 @@
 #include "cells.cuh"
 #include "compaso.cuh"
 #include "pipeline.cuh"
+#include "rank2.cuh"
 #include "radial.cuh"
 
 namespace {
 
 constexpr unsigned long long NONE = ~0ull;
 
-__global__ void k_flags(const int* __restrict__ root, int n, const uint8_t* __restrict__ select,
-                        uint32_t* __restrict__ dflag, uint32_t* __restrict__ rflag) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int r = root[s];
-  const bool in = r >= 0 && (!select || select[s]);
-  dflag[s] = in;
-  rflag[s] = in && r == s;
+// The dense particles taking part, listed in cell order, and the index of
+// every group at its root (groups in the order of their roots); the numbers of
+// both go to meta.
+__global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restrict__ root, int n,
+                                                            const uint8_t* __restrict__ select,
+                                                            uint32_t* __restrict__ dl, uint32_t* __restrict__ gidx,
+                                                            unsigned long long* __restrict__ status, long long ntiles,
+                                                            Meta* meta) {
+  __shared__ Rank2Shared S;
+  const long long tile = rank2_tile(S, status, ntiles);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
+  unsigned in[R2_ITEMS], head[R2_ITEMS];
+  uint32_t na = 0, nb = 0;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long i = base + q * 32 + lane;
+    const int r = i < n ? root[i] : -1;
+    const bool d = r >= 0 && (!select || select[i]);
+    in[q] = __ballot_sync(0xffffffffu, d);
+    head[q] = __ballot_sync(0xffffffffu, d && r == (int)i);
+    na += __popc(in[q]);
+    nb += __popc(head[q]);
+  }
+  uint32_t ta, tb;
+  rank2_prefix(S, status, tile, na, nb, ta, tb, &meta->timeout);
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const uint32_t i = (uint32_t)(base + q * 32 + lane);
+    if (in[q] >> lane & 1u) dl[na + __popc(in[q] & lt)] = i;
+    if (head[q] >> lane & 1u) gidx[i] = nb + __popc(head[q] & lt);
+    na += __popc(in[q]);
+    nb += __popc(head[q]);
+  }
+  if (tile == ntiles - 1 && threadIdx.x == 0) {
+    meta->n_dense = ta;
+    meta->n_groups = tb;
+  }
 }
 
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* sh) {
@@ -48,22 +80,21 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
   return v;
 }
 
-// compact the dense particles taking part, each with its group's index; block
-// maxima of Sigma and id, one atomic per block
-__global__ void __launch_bounds__(256) k_compact_dense(const int* __restrict__ root, const uint8_t* __restrict__ select,
-                                                       int n, const uint32_t* __restrict__ dscan,
-                                                       const uint32_t* __restrict__ rscan,
-                                                       const long long* __restrict__ sigma,
-                                                       const uint64_t* __restrict__ sid, uint32_t* __restrict__ dl,
-                                                       uint32_t* __restrict__ grp, Meta* meta) {
+// the group of every listed particle; block maxima of Sigma and id, one
+// atomic per block
+__global__ void __launch_bounds__(256) k_member_group(const uint32_t* __restrict__ dl, const int* __restrict__ root,
+                                                      const uint32_t* __restrict__ gidx,
+                                                      const long long* __restrict__ sigma,
+                                                      const uint64_t* __restrict__ sid, uint32_t* __restrict__ grp,
+                                                      Meta* meta) {
   __shared__ unsigned long long sh[8];
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned nd = meta->n_dense;
+  if (blockIdx.x * blockDim.x >= nd) return;
+  const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long ms = 0, mid = 0;
-  const int r = s < n ? root[s] : -1;
-  if (r >= 0 && (!select || select[s])) {
-    const uint32_t k = dscan[s];
-    dl[k] = (uint32_t)s;
-    grp[k] = rscan[r];
+  if (k < nd) {
+    const uint32_t s = dl[k];
+    grp[k] = gidx[root[s]];
     ms = (unsigned long long)sigma[s];
     mid = (unsigned long long)sid[s];
   }
@@ -89,28 +120,52 @@ __global__ void k_gather_pos(const uint32_t* __restrict__ gs, int nd, const int4
   if (k < nd) epos[k] = spos[gs[k]];
 }
 
-__global__ void k_flag_assigned(const int* __restrict__ eslot, int nd, uint32_t* __restrict__ f) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nd) f[k] = eslot[k] >= 0;
-}
-
-// the members of L1 haloes, each with its halo's index; their L1 labels, on
-// the device by cell-sorted index and (optional) in input order
-__global__ void k_compact_assigned(const int* __restrict__ eslot, const uint32_t* __restrict__ grp,
-                                   const uint32_t* __restrict__ hbase, int nd, const uint32_t* __restrict__ scan,
-                                   const uint32_t* __restrict__ gs, uint32_t* __restrict__ key,
-                                   uint32_t* __restrict__ val, int* __restrict__ lab1, const int4* __restrict__ spos,
-                                   const uint32_t* __restrict__ hnuc, const uint64_t* __restrict__ sid,
-                                   uint64_t* __restrict__ ol1) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nd) return;
-  const int q = eslot[k];
-  if (q < 0) return;
-  const uint32_t h = hbase[grp[k]] + (uint32_t)q, s = gs[k], d = scan[k];
-  key[d] = h;
-  val[d] = s;
-  lab1[s] = (int)h;
-  if (ol1) ol1[spos[s].w] = sid[hnuc[h]];
+// The members of L1 haloes, listed with their halo's index; their L1 labels,
+// on the device by cell-sorted index and (optional) in input order.  The
+// number of members goes to *total.
+__global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restrict__ eslot,
+                                                              const uint32_t* __restrict__ grp,
+                                                              const uint32_t* __restrict__ hbase,
+                                                              const uint32_t* __restrict__ seg_off,
+                                                              const uint32_t* __restrict__ nuc_member, int nd,
+                                                              const uint32_t* __restrict__ gs,
+                                                              const int4* __restrict__ epos,
+                                                              const uint64_t* __restrict__ sid,
+                                                              uint32_t* __restrict__ key, uint32_t* __restrict__ val,
+                                                              int* __restrict__ lab1, uint64_t* __restrict__ ol1,
+                                                              unsigned long long* __restrict__ status,
+                                                              long long ntiles, uint32_t* __restrict__ total,
+                                                              int* __restrict__ err) {
+  __shared__ Rank2Shared S;
+  const long long tile = rank2_tile(S, status, ntiles);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
+  unsigned in[R2_ITEMS];
+  int slot[R2_ITEMS];
+  uint32_t na = 0, nb = 0;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long k = base + q * 32 + lane;
+    slot[q] = k < nd ? eslot[k] : -1;
+    in[q] = __ballot_sync(0xffffffffu, slot[q] >= 0);
+    na += __popc(in[q]);
+  }
+  uint32_t ta, tb;
+  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long k = base + q * 32 + lane;
+    if (slot[q] >= 0) {
+      const uint32_t g = grp[k], h = hbase[g] + (uint32_t)slot[q], s = gs[k];
+      const uint32_t d = na + __popc(in[q] & ((1u << lane) - 1u));
+      key[d] = h;
+      val[d] = s;
+      lab1[s] = (int)h;
+      if (ol1) ol1[epos[k].w] = sid[nuc_member[seg_off[g] + slot[q]]];
+    }
+    na += __popc(in[q]);
+  }
+  if (tile == ntiles - 1 && threadIdx.x == 0) *total = ta;
 }
 
 __global__ void k_fill_u64(uint64_t* p, long long n, uint64_t v) {
@@ -284,13 +339,38 @@ __global__ void k_summary(const uint32_t* __restrict__ seg2, int H1, const uint3
   keep[h] = n >= np_min;
 }
 
-__global__ void k_catalogue_keys(const cso_halo* __restrict__ rows, const uint32_t* __restrict__ keep,
-                                 const uint32_t* __restrict__ kscan, int H, uint64_t* __restrict__ key,
-                                 uint32_t* __restrict__ val) {
-  int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= H || !keep[h]) return;
-  key[kscan[h]] = rows[h].nucleus_id;
-  val[kscan[h]] = (uint32_t)h;
+// the rows the catalogue keeps, listed by their index; their number goes to *total
+__global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* __restrict__ rows,
+                                                               const uint32_t* __restrict__ keep, int H,
+                                                               uint64_t* __restrict__ key, uint32_t* __restrict__ val,
+                                                               unsigned long long* __restrict__ status,
+                                                               long long ntiles, uint32_t* __restrict__ total,
+                                                               int* __restrict__ err) {
+  __shared__ Rank2Shared S;
+  const long long tile = rank2_tile(S, status, ntiles);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
+  unsigned in[R2_ITEMS];
+  uint32_t na = 0, nb = 0;
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long h = base + q * 32 + lane;
+    in[q] = __ballot_sync(0xffffffffu, h < H && keep[h]);
+    na += __popc(in[q]);
+  }
+  uint32_t ta, tb;
+  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+#pragma unroll
+  for (int q = 0; q < R2_ITEMS; ++q) {
+    const long long h = base + q * 32 + lane;
+    if (in[q] >> lane & 1u) {
+      const uint32_t d = na + __popc(in[q] & ((1u << lane) - 1u));
+      key[d] = rows[h].nucleus_id;
+      val[d] = (uint32_t)h;
+    }
+    na += __popc(in[q]);
+  }
+  if (tile == ntiles - 1 && threadIdx.x == 0) *total = ta;
 }
 
 // rows in nucleus-id order; optionally the input index of each row's nucleus
@@ -381,26 +461,22 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   }
   // ---- gather: dense particles by group ----
   S.mark("gather");
-  ALLOC(uint32_t, dscan, n + 1);
-  ALLOC(uint32_t, rscan, n + 1);
-  k_flags<<<G1(n)>>>(root, N, gi.select, dscan, rscan);
-  CSO_TRY(scan_u32(dscan, n, dscan + n, ws, st));
-  CSO_TRY(scan_u32(rscan, n, rscan + n, ws, st));
+  // status words of the three lists below
+  const long long words = rank2_words(n);
+  ALLOC(unsigned long long, rstat, 3 * words);
+  CSO_CUDA(cudaMemsetAsync(rstat, 0, sizeof(unsigned long long) * 3 * words, st));
   ALLOC(uint32_t, dl, n);
+  ALLOC(uint32_t, gidx, n);
   ALLOC(uint32_t, grp, n);
-  k_compact_dense<<<G1(n)>>>(root, gi.select, N, dscan, rscan, sigma, sid, dl, grp, meta);
+  k_member_list<<<CL((unsigned)(words - 1)), R2_THREADS, 0, st>>>(root, N, gi.select, dl, gidx, rstat, words - 1, meta);
+  k_member_group<<<G1(n)>>>(dl, root, gidx, sigma, sid, grp, meta);
   CSO_CUDA(cudaGetLastError());
-  // counters: n_dense, G, sigma_max, id_max, bad
-  {
-    CSO_CUDA(cudaMemcpyAsync(c->pinned, dscan + n, 4, cudaMemcpyDeviceToHost, st));
-    CSO_CUDA(cudaMemcpyAsync((char*)c->pinned + 4, rscan + n, 4, cudaMemcpyDeviceToHost, st));
-    CSO_CUDA(cudaMemcpyAsync(c->pinned + 1, meta, sizeof(Meta), cudaMemcpyDeviceToHost, st));
-    CSO_CUDA(cudaStreamSynchronize(st));
-  }
-  const int nd = (int)((uint32_t*)c->pinned)[0];
-  const int G = (int)((uint32_t*)c->pinned)[1];
+  // counters: dense particles, groups, sigma_max, id_max, bad
   Meta hm;
-  memcpy(&hm, c->pinned + 1, sizeof(Meta));
+  CSO_TRY(readback(c, meta, sizeof(Meta)));
+  memcpy(&hm, c->pinned, sizeof(Meta));
+  const int nd = (int)hm.n_dense;
+  const int G = (int)hm.n_groups;
   if (hm.bad) {
     cso_set_error("positions outside [0, 2^21)");
     return CSO_ERR_ARG;
@@ -482,32 +558,35 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
 
   // ---- prep2: L1 haloes, their members and labels ----
   S.mark("prep2");
-  ALLOC(uint32_t, hbase, G + 1);
+  // (hbase[G] the haloes, hbase[G + 1] their members)
+  ALLOC(uint32_t, hbase, G + 2);
   if (G > 0) CSO_CUDA(cudaMemcpyAsync(hbase, nnuc, sizeof(uint32_t) * G, cudaMemcpyDeviceToDevice, st));
   CSO_TRY(scan_u32(hbase, G, hbase + G, ws, st));
-  ALLOC(uint32_t, aflag, nd + 1);
-  if (nd > 0) k_flag_assigned<<<G1(nd)>>>(eslot, nd, aflag);  // slot >= 0 <=> assigned
-  CSO_TRY(scan_u32(aflag, nd, aflag + nd, ws, st));
-  CSO_CUDA(cudaMemcpyAsync(c->pinned, hbase + G, 4, cudaMemcpyDeviceToHost, st));
-  CSO_CUDA(cudaMemcpyAsync((char*)c->pinned + 4, aflag + nd, 4, cudaMemcpyDeviceToHost, st));
-  CSO_CUDA(cudaStreamSynchronize(st));
+  ALLOC(int, lab1, n);
+  CSO_CUDA(cudaMemsetAsync(lab1, 0xff, sizeof(int) * n, st));
+  ALLOC(uint32_t, akey, nd);
+  ALLOC(uint32_t, aval, nd);
+  uint32_t* egs2 = aval;   // cell-sorted index of each member
+  uint32_t* ehal2 = akey;  // its L1 halo, ascending
+  if (nd > 0) {
+    const long long w2 = rank2_words(nd);
+    k_assigned_list<<<CL((unsigned)(w2 - 1)), R2_THREADS, 0, st>>>(eslot, gseg, hbase, seg1, nucm, nd, gs, epos, sid,
+                                                                   akey, aval, lab1, ol1, rstat + words, w2 - 1,
+                                                                   hbase + G + 1, ws.err);
+  } else {
+    CSO_CUDA(cudaMemsetAsync(hbase + G + 1, 0, sizeof(uint32_t), st));
+  }
+  CSO_CUDA(cudaGetLastError());
+  CSO_TRY(readback(c, hbase + G, 2 * sizeof(uint32_t)));
   const int H1 = (int)((uint32_t*)c->pinned)[0];
   const int na = (int)((uint32_t*)c->pinned)[1];
   c->stats[3] = H1;
   ALLOC(uint32_t, hnuc, H1);
   ALLOC(long long, hR2, H1);
   CSO_TRY(level_halo(G, seg1, hbase, nucm, nucR2, hnuc, hR2, H1, st));
-  ALLOC(int, lab1, n);
-  CSO_CUDA(cudaMemsetAsync(lab1, 0xff, sizeof(int) * n, st));
-  ALLOC(uint32_t, akey, na);
-  ALLOC(uint32_t, aval, na);
   ALLOC(uint32_t, akey2, na);
   ALLOC(uint32_t, aval2, na);
   ALLOC(uint32_t, seg2, H1 + 1);
-  uint32_t* egs2 = aval;   // cell-sorted index of each member
-  uint32_t* ehal2 = akey;  // its L1 halo, ascending
-  if (nd > 0)
-    k_compact_assigned<<<G1(nd)>>>(eslot, gseg, hbase, nd, aflag, gs, akey, aval, lab1, spos, hnuc, sid, ol1);
   if (na > 0) {
     uint32_t *pk = akey, *pv = aval;
     CSO_TRY(radix_sort_32(&pk, &pv, akey2, aval2, na, bit_length_u64(H1 > 0 ? H1 - 1 : 0), ws, st));
@@ -602,17 +681,17 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
                          st, SideStreams{{c->side, c->side2, c->side3}, c->fork, {c->join, c->join2, c->join3}}));
       S.mark("catalogue");
     }
-    ALLOC(uint32_t, kscan, H1 + 1);
-    CSO_CUDA(cudaMemcpyAsync(kscan, keep, sizeof(uint32_t) * H1, cudaMemcpyDeviceToDevice, st));
-    CSO_TRY(scan_u32(kscan, H1, kscan + H1, ws, st));
-    CSO_TRY(readback(c, kscan + H1, 4));
+    ALLOC(uint64_t, ckey, H1);
+    ALLOC(uint32_t, cval, H1);
+    const long long w3 = rank2_words(H1);
+    k_catalogue_list<<<CL((unsigned)(w3 - 1)), R2_THREADS, 0, st>>>(rows, keep, H1, ckey, cval, rstat + 2 * words, w3 - 1,
+                                                                    keep + H1, ws.err);
+    CSO_CUDA(cudaGetLastError());
+    CSO_TRY(readback(c, keep + H1, 4));
     nrows = (int)((uint32_t*)c->pinned)[0];
-    ALLOC(uint64_t, ckey, nrows);
-    ALLOC(uint32_t, cval, nrows);
     ALLOC(uint64_t, ckey2, nrows);
     ALLOC(uint32_t, cval2, nrows);
     if (nrows > 0) {
-      k_catalogue_keys<<<G1(H1)>>>(rows, keep, kscan, H1, ckey, cval);
       uint64_t* ph = nullptr;
       uint64_t* pl = ckey;
       uint32_t* pv = cval;

@@ -1,0 +1,100 @@
+// Ranks of two sets of flagged elements in one pass over the array: the
+// single-pass scan of scan_sort.cu (decoupled look-back over tiles taken from
+// an atomic counter) for flags known inside the caller's kernel, so that a
+// list is written by the kernel that decides who is on it, with no flag
+// array, scan and second pass in between.
+#pragma once
+#include "cso_internal.cuh"
+
+constexpr int R2_THREADS = 256;
+constexpr int R2_WARPS = R2_THREADS / 32;
+constexpr int R2_ITEMS = 16;  // elements per lane: a warp holds 512 consecutive ones, 32 per item
+constexpr int R2_TILE = R2_THREADS * R2_ITEMS;
+
+// A status word: state << 62 | first count << 31 | second count (counts below
+// 2^31).  States: 0 not published, 1 the tile's own counts, 2 inclusive prefix.
+struct Rank2Shared {
+  uint32_t wa[R2_WARPS], wb[R2_WARPS];
+  uint32_t a0, b0;
+  long long tile;
+};
+
+// status words needed for n elements (tiles, then the tile counter), zeroed by the caller
+static inline long long rank2_words(long long n) { return cdiv(n, R2_TILE) + 1; }
+
+__device__ __forceinline__ long long rank2_tile(Rank2Shared& S, unsigned long long* status, long long ntiles) {
+  if (threadIdx.x == 0) S.tile = (long long)atomicAdd(&status[ntiles], 1ull);
+  __syncthreads();
+  return S.tile;
+}
+
+// wa, wb: the calling warp's counts (the same on every lane).  On return they
+// are the numbers of flagged elements before the warp's first one; ta, tb the
+// inclusive totals up to the end of this tile.
+__device__ __forceinline__ void rank2_prefix(Rank2Shared& S, unsigned long long* status, long long tile, uint32_t& wa,
+                                             uint32_t& wb, uint32_t& ta, uint32_t& tb, int* err) {
+  constexpr unsigned long long M31 = (1ull << 31) - 1;
+  constexpr long long SPIN_LIMIT = 1ll << 22;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) {
+    S.wa[w] = wa;
+    S.wb[w] = wb;
+  }
+  __syncthreads();
+  uint32_t suma = 0, sumb = 0, befa = 0, befb = 0;
+#pragma unroll
+  for (int k = 0; k < R2_WARPS; ++k) {
+    if (k == w) {
+      befa = suma;
+      befb = sumb;
+    }
+    suma += S.wa[k];
+    sumb += S.wb[k];
+  }
+  if (w == 0) {
+    uint32_t pa = 0, pb = 0;
+    if (tile > 0) {
+      auto put = [&](unsigned long long state, uint32_t a, uint32_t b) {
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(status + tile),
+                     "l"(state << 62 | (unsigned long long)a << 31 | b)
+                     : "memory");
+      };
+      if (lane == 0) put(1, suma, sumb);
+      long long top = tile - 1, spins = 0;
+      for (;;) {
+        const long long j = top - lane;
+        unsigned long long v = 2ull << 62;  // before tile 0: prefix 0
+        if (j >= 0) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(status + j) : "memory");
+        const unsigned pmask = __ballot_sync(0xffffffffu, v >> 62 == 2);
+        const unsigned xmask = __ballot_sync(0xffffffffu, v >> 62 == 0);
+        const int first = pmask ? __ffs(pmask) - 1 : 31;
+        const unsigned need = first == 31 ? 0xffffffffu : (2u << first) - 1u;
+        if (xmask & need) {  // a predecessor has not published yet
+          if (++spins > SPIN_LIMIT) {
+            if (lane == 0) atomicExch(err, 1);
+            break;
+          }
+          continue;
+        }
+        pa += __reduce_add_sync(0xffffffffu, lane <= first ? (uint32_t)(v >> 31 & M31) : 0u);
+        pb += __reduce_add_sync(0xffffffffu, lane <= first ? (uint32_t)(v & M31) : 0u);
+        if (pmask) break;
+        top -= 32;
+      }
+      if (lane == 0) put(2, pa + suma, pb + sumb);
+    } else if (lane == 0) {
+      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(status),
+                   "l"(2ull << 62 | (unsigned long long)suma << 31 | sumb)
+                   : "memory");
+    }
+    if (lane == 0) {
+      S.a0 = pa;
+      S.b0 = pb;
+    }
+  }
+  __syncthreads();
+  wa = S.a0 + befa;
+  wb = S.b0 + befb;
+  ta = S.a0 + suma;
+  tb = S.b0 + sumb;
+}
