@@ -428,6 +428,68 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_os_pass(const K* __restrict__
   }
 }
 
+// Small arrays by one block: the whole scan and the whole sort in one launch
+// each, where the general kernels need a clearing, a launch per digit and two
+// more (a launch costs 2-4 us beside others; the work itself less).
+constexpr int SMALL_SCAN = 8192;
+constexpr int SMALL_SORT = 2048;
+
+__global__ void __launch_bounds__(1024) k_scan_small(uint32_t* __restrict__ d, int n, uint32_t* __restrict__ total) {
+  __shared__ uint32_t sw[33];
+  uint32_t carry = 0;
+  for (int base = 0; base < n; base += 4096) {
+    const int i = base + threadIdx.x * 4;
+    uint32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = i + k < n ? d[i + k] : 0u;
+    uint32_t excl;
+    const uint32_t sum = block_excl_scan(v[0] + v[1] + v[2] + v[3], sw, excl);
+    uint32_t at = carry + excl;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (i + k < n) d[i + k] = at;
+      at += v[k];
+    }
+    carry += sum;
+  }
+  if (total && threadIdx.x == 0) *total = carry;
+}
+
+// Sorts (key, position) by the masked key in shared memory: bitonic over
+// twice as many elements as threads; the position makes it stable.
+template <class K>
+__global__ void __launch_bounds__(SMALL_SORT / 2) k_sort_small(const K* __restrict__ kin, const uint32_t* __restrict__ vin,
+                                                             K* __restrict__ kout, uint32_t* __restrict__ vout, int n,
+                                                             int m, K mask) {
+  __shared__ K sk[SMALL_SORT];
+  __shared__ uint16_t sp[SMALL_SORT];
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    sk[i] = i < n ? kin[i] & mask : K(~K(0));
+    sp[i] = (uint16_t)i;  // past the end: behind every element of the same key
+  }
+  __syncthreads();
+  for (int k = 2; k <= m; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < m / 2; t += blockDim.x) {
+        const int i = 2 * t - (t & (j - 1)), l = i + j;
+        const K a = sk[i], b = sk[l];
+        const uint16_t pa = sp[i], pb = sp[l];
+        const bool gt = a > b || (a == b && pa > pb);
+        if (gt == ((i & k) == 0)) {
+          sk[i] = b;
+          sk[l] = a;
+          sp[i] = pb;
+          sp[l] = pa;
+        }
+      }
+      __syncthreads();
+    }
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    kout[i] = kin[sp[i]];
+    vout[i] = vin[sp[i]];
+  }
+}
+
 }  // namespace
 
 int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaStream_t st) {
@@ -438,6 +500,11 @@ int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaSt
   if (!ws.err) {
     cso_set_error("scan without a device error word");
     return CSO_ERR_STATE;
+  }
+  if (n <= SMALL_SCAN) {
+    k_scan_small<<<CL(1), 1024, 0, st>>>(data, (int)n, total);
+    CSO_CUDA(cudaGetLastError());
+    return CSO_OK;
   }
   const bool big = n > SP_BIG;
   const long long ntiles = cdiv(n, (long long)SP_THREADS * (big ? 32 : 16));
@@ -463,6 +530,17 @@ static int onesweep(K** key, uint32_t** val, K* key_alt, uint32_t* val_alt, long
   if (!ws.err) {
     cso_set_error("sort without a device error word");
     return CSO_ERR_STATE;
+  }
+  if (n <= SMALL_SORT) {
+    int m = 2;
+    while (m < n) m <<= 1;
+    const int b8 = (bits + 7) / 8 * 8;  // whole digits, as the passes below
+    const K mask = b8 >= (int)(8 * sizeof(K)) ? K(~K(0)) : K((K(1) << b8) - 1);
+    k_sort_small<K><<<CL(1), m / 2 < 32 ? 32 : m / 2, 0, st>>>(*key, *val, key_alt, val_alt, (int)n, m, mask);
+    CSO_CUDA(cudaGetLastError());
+    std::swap(*key, key_alt);
+    std::swap(*val, val_alt);
+    return CSO_OK;
   }
   constexpr int TILE = OS_THREADS * OsItems<K>::v;
   const int passes = (bits + 7) / 8;

@@ -51,3 +51,19 @@ def test_fof_from_given_sums(ctx, n, dense):
 def test_whole_path(ctx, n):
     pos, ids = clumps(n, 100 + n)
     assert_matches_oracle(ctx.find_groups(pos, ids, cso.cso_params_default(U), halo_cap=max(16, n)), pos, ids, U)
+
+
+@pytest.mark.parametrize("n", [2, 1023, 1025, 2047, 2048, 2049])
+def test_levels_with_labels_about_the_one_block_sort(ctx, n):
+    pos, ids = clumps(n, 200 + n)
+    po = O.params(U)
+    sigma, _ = O.density(pos, po)
+    rng = np.random.default_rng(n)
+    l0 = np.full(n, np.iinfo(np.uint64).max, np.uint64)
+    which = rng.integers(0, 7, n)
+    for g in range(6):  # a seventh of the particles stays in no group
+        l0[which == g] = ids[which == g].min() if (which == g).any() else 0
+    l1, l2, halos = cso.cso_levels(ctx.h, pos, ids, sigma, l0, cso.cso_params_default(U))
+    w1, w2, wh, _ = O.compaso(pos, ids, sigma, l0, po)
+    assert np.array_equal(l1, w1) and np.array_equal(l2, w2)
+    assert np.array_equal(halos["nucleus_id"], wh["nucleus_id"]) and np.array_equal(halos["R2"], wh["R2"])
