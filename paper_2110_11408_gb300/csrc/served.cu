@@ -28,9 +28,12 @@ struct ServedState {
   std::vector<cso_ctx*> slots;
   std::unordered_map<uint64_t, StreamState*> streams;  // slab streams by request_id
   std::vector<std::thread> workers;
+  cudaMemPool_t pool = nullptr;  // device memory of the slab streams
   size_t in_use = 0;  // device bytes reserved by running requests
   bool stop = false;
 };
+
+constexpr uint64_t POOL_KEEP = 1ull << 30;
 
 static double now_s() {
   using namespace std::chrono;
@@ -125,7 +128,7 @@ static void run_slab(cso_ctx* slot, ServedState& S, ServedRequest* r) {
     }
     if (all && ss->x_received == CSO_BOX) {  // the stream is over
       S.streams.erase(ss->id);
-      stream_release(ss);
+      stream_release(ss, slot->stream);
       ss = nullptr;
     }
   }
@@ -152,7 +155,7 @@ static void worker_loop(cso_ctx* parent, int k) {
           st->second->busy = true;
         } else if (r->in.x_lo == 0) {  // the first slab opens the stream
           StreamState* ss = nullptr;
-          if (stream_begin(&ss, r->in.request_id, &r->p) == CSO_OK) {
+          if (stream_begin(&ss, r->in.request_id, &r->p, S.pool) == CSO_OK) {
             ss->busy = true;
             S.streams[r->in.request_id] = ss;
           }
@@ -180,6 +183,16 @@ static int served_start(cso_ctx* c) {
   if (c->served) return CSO_OK;
   ServedState* S = new ServedState();
   c->served = S;
+  // the slab streams' memory: a pool of this context's own, which keeps at
+  // most POOL_KEEP bytes that no stream uses and goes with the context
+  CSO_CUDA(cudaSetDevice(c->device));
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = c->device;
+  CSO_CUDA(cudaMemPoolCreate(&S->pool, &props));
+  uint64_t keep = POOL_KEEP;
+  CSO_CUDA(cudaMemPoolSetAttribute(S->pool, cudaMemPoolAttrReleaseThreshold, &keep));
   const int nslots = c->served_slots > 0 ? c->served_slots : 4;
   for (int k = 0; k < nslots; ++k) {
     cso_ctx* s = nullptr;
@@ -200,8 +213,11 @@ void served_stop(cso_ctx* c) {
   }
   S->cv_work.notify_all();
   for (auto& t : S->workers) t.join();
-  for (auto* s : S->slots) cso_free(s);
-  for (auto& kv : S->streams) stream_release(kv.second);
+  for (auto* s : S->slots) cso_free(s);  // (waits for the slots' streams)
+  cudaSetDevice(c->device);
+  for (auto& kv : S->streams) stream_release(kv.second, c->stream);
+  cudaStreamSynchronize(c->stream);
+  if (S->pool) cudaMemPoolDestroy(S->pool);
   for (auto& kv : S->tickets) delete kv.second;
   for (auto* r : S->queue) (void)r;  // owned through the ticket table
   delete S;

@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cells.cuh"
 #include "compaso.cuh"
@@ -180,52 +181,52 @@ __global__ void k_compact_resident(const uint32_t* __restrict__ keep, const uint
 
 // ---------------------------------------------------------------------------
 
-void stream_release(StreamState* S) {
+void stream_release(StreamState* S, cudaStream_t st) {
   if (!S) return;
   void* bufs[] = {S->rpos[0], S->rpos[1], S->rid[0], S->rid[1], S->rsig[0],  S->rsig[1],
                   S->rflag[0], S->rflag[1], S->rslab[0], S->rslab[1], S->ridx[0], S->ridx[1],
                   S->dslabs,  S->ddone,   S->dnrows, S->dhist,   S->dbad};
   for (void* b : bufs)
-    if (b) cudaFree(b);
+    if (b) cudaFreeAsync(b, st);
   delete S;
 }
 
-static int ensure_capacity(StreamState& S, long long need) {
+// Device memory of the stream, from the served path's pool in the order of
+// stream st.  (cudaMalloc and cudaFree for every growth of every stream wait
+// for the device: 14.1 against 12.7 ms for a 2M-particle box in eight slabs.)
+static int pool_get(StreamState& S, cudaStream_t st, void** p, size_t bytes) {
+  CSO_CUDA(cudaMallocFromPoolAsync(p, bytes, S.pool, st));
+  return CSO_OK;
+}
+
+static int ensure_capacity(StreamState& S, long long need, cudaStream_t st) {
   if (need <= S.cap) return CSO_OK;
   long long cap = std::max<long long>(need, S.cap * 3 / 2 + 1024);
   for (int k = 0; k < 2; ++k) {
-    void *a = nullptr, *b = nullptr, *c = nullptr, *d = nullptr, *e = nullptr, *f = nullptr;
-    CSO_CUDA(cudaMalloc(&a, sizeof(int32_t) * 3 * cap));
-    CSO_CUDA(cudaMalloc(&b, sizeof(uint64_t) * cap));
-    CSO_CUDA(cudaMalloc(&c, sizeof(long long) * cap));
-    CSO_CUDA(cudaMalloc(&d, sizeof(uint8_t) * cap));
-    CSO_CUDA(cudaMalloc(&e, sizeof(uint32_t) * cap));
-    CSO_CUDA(cudaMalloc(&f, sizeof(uint32_t) * cap));
-    if (k == S.cur && S.nr > 0) {  // keep the live copy
-      CSO_CUDA(cudaMemcpy(a, S.rpos[k], sizeof(int32_t) * 3 * S.nr, cudaMemcpyDeviceToDevice));
-      CSO_CUDA(cudaMemcpy(b, S.rid[k], sizeof(uint64_t) * S.nr, cudaMemcpyDeviceToDevice));
-      CSO_CUDA(cudaMemcpy(c, S.rsig[k], sizeof(long long) * S.nr, cudaMemcpyDeviceToDevice));
-      CSO_CUDA(cudaMemcpy(d, S.rflag[k], sizeof(uint8_t) * S.nr, cudaMemcpyDeviceToDevice));
-      CSO_CUDA(cudaMemcpy(e, S.rslab[k], sizeof(uint32_t) * S.nr, cudaMemcpyDeviceToDevice));
-      CSO_CUDA(cudaMemcpy(f, S.ridx[k], sizeof(uint32_t) * S.nr, cudaMemcpyDeviceToDevice));
-    }
-    void* old[] = {S.rpos[k], S.rid[k], S.rsig[k], S.rflag[k], S.rslab[k], S.ridx[k]};
-    for (void* o : old)
-      if (o) CSO_CUDA(cudaFree(o));
-    S.rpos[k] = (int32_t*)a;
-    S.rid[k] = (uint64_t*)b;
-    S.rsig[k] = (long long*)c;
-    S.rflag[k] = (uint8_t*)d;
-    S.rslab[k] = (uint32_t*)e;
-    S.ridx[k] = (uint32_t*)f;
+    const bool live = k == S.cur && S.nr > 0;  // the copy to keep
+    auto grow = [&](auto*& buf, size_t size) -> int {
+      void* p = nullptr;
+      CSO_TRY(pool_get(S, st, &p, size * (size_t)cap));
+      if (live) CSO_CUDA(cudaMemcpyAsync(p, buf, size * (size_t)S.nr, cudaMemcpyDeviceToDevice, st));
+      if (buf) CSO_CUDA(cudaFreeAsync(buf, st));
+      buf = static_cast<std::remove_reference_t<decltype(buf)>>(p);
+      return CSO_OK;
+    };
+    CSO_TRY(grow(S.rpos[k], sizeof(int32_t) * 3));
+    CSO_TRY(grow(S.rid[k], sizeof(uint64_t)));
+    CSO_TRY(grow(S.rsig[k], sizeof(long long)));
+    CSO_TRY(grow(S.rflag[k], sizeof(uint8_t)));
+    CSO_TRY(grow(S.rslab[k], sizeof(uint32_t)));
+    CSO_TRY(grow(S.ridx[k], sizeof(uint32_t)));
   }
   S.cap = cap;
   return CSO_OK;
 }
 
-int stream_begin(StreamState** out, uint64_t id, const cso_params* p) {
+int stream_begin(StreamState** out, uint64_t id, const cso_params* p, cudaMemPool_t pool) {
   StreamState* S = new StreamState();
   S->id = id;
+  S->pool = pool;
   S->p = *p;
   int rc = cso_params_derive(&S->p);
   if (rc == CSO_OK) rc = cells_choose(S->p.b2, &S->nc);
@@ -258,10 +259,10 @@ int stream_step(cso_ctx* c, StreamState& S, const cso_input* in, cso_output* out
 
   // ---- append the slab's particles to the resident store ----
   CSO_CUDA(cudaStreamSynchronize(st));
-  CSO_TRY(ensure_capacity(S, S.nr + n_new));
+  CSO_TRY(ensure_capacity(S, S.nr + n_new, st));
   if (!S.dhist) {
-    CSO_CUDA(cudaMalloc((void**)&S.dhist, sizeof(unsigned) * nc));
-    CSO_CUDA(cudaMalloc((void**)&S.dbad, sizeof(int)));
+    CSO_TRY(pool_get(S, st, (void**)&S.dhist, sizeof(unsigned) * nc));
+    CSO_TRY(pool_get(S, st, (void**)&S.dbad, sizeof(int)));
   }
   CSO_CUDA(cudaMemsetAsync(S.dbad, 0, sizeof(int), st));
   const int k = S.cur;
@@ -376,18 +377,17 @@ int stream_step(cso_ctx* c, StreamState& S, const cso_input* in, cso_output* out
     void* a = nullptr;
     void* b = nullptr;
     void* d = nullptr;
-    CSO_CUDA(cudaMalloc(&a, sizeof(SlabPtrs) * cap));
-    CSO_CUDA(cudaMalloc(&b, sizeof(unsigned long long) * cap));
-    CSO_CUDA(cudaMalloc(&d, sizeof(unsigned long long) * cap));
+    CSO_TRY(pool_get(S, st, &a, sizeof(SlabPtrs) * cap));
+    CSO_TRY(pool_get(S, st, &b, sizeof(unsigned long long) * cap));
+    CSO_TRY(pool_get(S, st, &d, sizeof(unsigned long long) * cap));
     CSO_CUDA(cudaMemsetAsync(b, 0, sizeof(unsigned long long) * cap, st));
     CSO_CUDA(cudaMemsetAsync(d, 0, sizeof(unsigned long long) * cap, st));
     if (S.slab_cap) {
       CSO_CUDA(cudaMemcpyAsync(b, S.ddone, sizeof(unsigned long long) * S.slab_cap, cudaMemcpyDeviceToDevice, st));
       CSO_CUDA(cudaMemcpyAsync(d, S.dnrows, sizeof(unsigned long long) * S.slab_cap, cudaMemcpyDeviceToDevice, st));
-      CSO_CUDA(cudaStreamSynchronize(st));
-      cudaFree(S.dslabs);
-      cudaFree(S.ddone);
-      cudaFree(S.dnrows);
+      CSO_CUDA(cudaFreeAsync(S.dslabs, st));
+      CSO_CUDA(cudaFreeAsync(S.ddone, st));
+      CSO_CUDA(cudaFreeAsync(S.dnrows, st));
     }
     S.dslabs = a;
     S.ddone = (unsigned long long*)b;

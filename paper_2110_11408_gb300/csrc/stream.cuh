@@ -16,6 +16,7 @@ struct StreamSlab {
 
 struct StreamState {
   uint64_t id = 0;
+  cudaMemPool_t pool = nullptr;  // of the served path
   cso_params p{};
   int nc = 0;
   long long x_received = 0;  // grid x up to which slabs have arrived
@@ -42,6 +43,7 @@ struct StreamState {
   std::vector<StreamSlab> slabs;
 };
 
-int stream_begin(StreamState** out, uint64_t id, const cso_params* p);
+int stream_begin(StreamState** out, uint64_t id, const cso_params* p, cudaMemPool_t pool);
 int stream_step(cso_ctx* c, StreamState& S, const cso_input* in, cso_output* out, ServedRequest* req);
-void stream_release(StreamState* S);
+// gives the stream's memory back to its pool, in the order of st
+void stream_release(StreamState* S, cudaStream_t st);
