@@ -10,10 +10,11 @@
 //
 // Almost every member has a denser neighbour close by, and cells are sorted
 // by x, so a lane first looks at the slots next to its own in the sorted
-// order; the few members left (about one per warp) are tested by the whole
-// warp over the 27-cell stencil, own row first, 128 neighbours a step; a
-// test still open after PEAK_STEPS steps (a true peak, mostly) goes to a
-// block of its own.
+// order; the few members left (about one per warp) get a warp each over the
+// 27-cell stencil, own row first, 128 neighbours a step; a test still open
+// after PEAK_STEPS steps (a true peak, mostly) goes to a block of its own.
+// Three kernels, so that the first, which sees every member, runs at full
+// occupancy.
 #include <limits.h>
 
 #include "peaks.cuh"
@@ -141,8 +142,10 @@ __device__ int warp_peak(const PeakArgs& a, uint32_t se, int glabel, int steps) 
 
 struct PeakOut {
   uint2* found;        // (segment, cell-sorted index) of every peak, unordered
-  uint2* open;         // tests handed to a block
-  unsigned* counts;    // [0] found, [1] open
+  uint2* left;         // members for a warp's test
+  uint2* open;         // tests for a block
+  unsigned m;          // members in all (room in each list)
+  unsigned* counts;    // [0] found, [1] left for a warp, [2] left for a block
   uint32_t* seg_count; // peaks per segment
 };
 
@@ -153,21 +156,23 @@ __device__ __forceinline__ void add_peak(const PeakOut& o, uint32_t seg, uint32_
 }
 
 __global__ void __launch_bounds__(256) k_peak_near(PeakArgs a, const uint32_t* __restrict__ gs,
-                                                   const uint32_t* __restrict__ seg, int m, long long T_min,
-                                                   long long T_test, int first, int* __restrict__ beater, PeakOut out) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const uint32_t s = k < m ? gs[k] : 0u;
-  const long long sp = k < m ? a.ssig[s] : LLONG_MIN;
-  bool todo = k < m && sp > T_test;
+                                                   const uint32_t* __restrict__ seg, long long T_min, long long T_test,
+                                                   int first, int* __restrict__ beater, PeakOut out) {
+  const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in = k < out.m;
+  const uint32_t s = in ? gs[k] : 0u;
+  const long long sp = in ? a.ssig[s] : LLONG_MIN;
+  const bool test = in && sp > T_test;
+  bool todo = test;
   int beat = BEAT_OPEN, lab = -1;
-  if (!first && todo) {
-    beat = beater[s];
-    lab = a.slab[s];
-    if (beat == BEAT_NONE || a.slab[beat] == lab) todo = false;  // known: a peak, or beaten inside its segment
-    else beat = BEAT_OPEN;
-  }
-  if (first) {
+  if (!first) {
+    if (todo) {
+      beat = beater[s];
+      lab = a.slab[s];
+      // known: a peak, or beaten inside its segment
+      if (beat != BEAT_NONE && a.slab[beat] != lab) beat = BEAT_OPEN;
+    }
+  } else {
     // the slots next to its own: any particle of the group there that is
     // within b and denser settles it
     int4 p = make_int4(0, 0, 0, 0);
@@ -177,14 +182,18 @@ __global__ void __launch_bounds__(256) k_peak_near(PeakArgs a, const uint32_t* _
       id = a.sid[s];
       lab = a.slab[s];
     }
-    for (int o = 1; o <= NEAR; ++o) {
+    for (int o0 = 1; o0 <= NEAR; o0 += 4) {
       if (!__any_sync(0xffffffffu, todo)) break;
+      long long st[8];  // eight loads in flight
 #pragma unroll
-      for (int side = -1; side <= 1; side += 2) {
-        const long long t = (long long)s + side * o;
-        if (!todo || t < 0 || t >= a.n) continue;
-        const long long st = a.ssig[t];
-        if (st < sp || a.slab[t] != lab) continue;
+      for (int u = 0; u < 8; ++u) {
+        const long long t = (long long)s + (u & 1 ? -(o0 + u / 2) : o0 + u / 2);
+        st[u] = todo && t >= 0 && t < a.n ? a.ssig[t] : LLONG_MIN;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = (int)s + (u & 1 ? -(o0 + u / 2) : o0 + u / 2);
+        if (!todo || st[u] < sp || a.slab[t] != lab) continue;
         const int4 q = a.spos[t];
         // nearest image by sign extension from 21 bits; a slot next to this
         // one may be anywhere, so each offset is bounded before it is squared
@@ -192,24 +201,36 @@ __global__ void __launch_bounds__(256) k_peak_near(PeakArgs a, const uint32_t* _
                   dz = (int)((unsigned)(p.z - q.z) << 11) >> 11;
         if (max(abs(dx), max(abs(dy), abs(dz))) > 16384) continue;  // b <= 16,384 grid units
         const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
-        if (d >= a.b2 || (st == sp && a.sid[t] > id)) continue;
-        beat = (int)t;
+        if (d >= a.b2 || (st[u] == sp && a.sid[t] > id)) continue;
+        beat = t;
         todo = false;
       }
     }
   }
-  // the whole warp tests the members left, one by one
-  for (unsigned left = __ballot_sync(0xffffffffu, todo); left; left &= left - 1) {
-    const int src = __ffs(left) - 1;
-    const int b = warp_peak(a, __shfl_sync(0xffffffffu, s, src), __shfl_sync(0xffffffffu, lab, src), PEAK_STEPS);
-    if (lane == src) beat = b;
-  }
-  if (k >= m || sp <= T_test) return;
+  if (!test) return;
   if (beat == BEAT_OPEN) {
-    out.open[atomicAdd(&out.counts[1], 1u)] = make_uint2(seg[k], s);
+    out.left[atomicAdd(&out.counts[1], 1u)] = make_uint2(seg[k], s);
   } else {
     if (first) beater[s] = beat;
-    if (beat == BEAT_NONE && sp > T_min) add_peak(out, seg[k], s);
+    else if (beat == BEAT_NONE && sp > T_min) add_peak(out, seg[k], s);
+  }
+}
+
+// the members left, a warp each for at most PEAK_STEPS steps
+__global__ void __launch_bounds__(256) k_peak_warp(PeakArgs a, long long T_min, int first, int* __restrict__ beater,
+                                                   PeakOut out) {
+  const int lane = threadIdx.x & 31;
+  const unsigned m = out.counts[1];
+  for (unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += gridDim.x * blockDim.x >> 5) {
+    const uint2 o = out.left[i];
+    const int b = warp_peak(a, o.y, a.slab[o.y], PEAK_STEPS);
+    if (lane != 0) continue;
+    if (b == BEAT_OPEN) {
+      out.open[atomicAdd(&out.counts[2], 1u)] = o;
+    } else {
+      if (first) beater[o.y] = b;
+      if (b == BEAT_NONE && a.ssig[o.y] > T_min) add_peak(out, o.x, o.y);
+    }
   }
 }
 
@@ -218,7 +239,7 @@ __global__ void __launch_bounds__(OPEN_NT) k_peak_open(PeakArgs a, long long T_m
                                                        int* __restrict__ beater, PeakOut out) {
   __shared__ int hit;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned m = out.counts[1];
+  const unsigned m = out.counts[2];
   for (unsigned i = blockIdx.x; i < m; i += gridDim.x) {
     const uint2 o = out.open[i];
     if (threadIdx.x == 0) hit = BEAT_NONE;
@@ -277,18 +298,21 @@ int peaks_find(const PeakArgs& a, const uint32_t* gs, const uint32_t* seg, int m
   const size_t mark = ws.off;
   PeakOut o;
   o.found = ws.get<uint2>(m);
+  o.left = ws.get<uint2>(m);
   o.open = ws.get<uint2>(m);
-  uint32_t* cursor = ws.get<uint32_t>((size_t)nseg + 2);
-  if (!P.off || !P.pos || !P.sig || !P.id || !P.out || !o.found || !o.open || !cursor) {
+  o.m = (unsigned)m;
+  uint32_t* cursor = ws.get<uint32_t>((size_t)nseg + 3);
+  if (!P.off || !P.pos || !P.sig || !P.id || !P.out || !o.found || !o.left || !o.open || !cursor) {
     cso_set_error("workspace exhausted in the peak search");
     return CSO_ERR_BUDGET;
   }
   o.counts = cursor + nseg;
   o.seg_count = P.off;
   CSO_CUDA(cudaMemsetAsync(P.off, 0, sizeof(uint32_t) * ((size_t)nseg + 1), st));
-  CSO_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * ((size_t)nseg + 2), st));
+  CSO_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * ((size_t)nseg + 3), st));
   if (m > 0) {
-    k_peak_near<<<CL(cdiv(m, 256)), 256, 0, st>>>(a, gs, seg, m, T_min, T_test, first, beater, o);
+    k_peak_near<<<CL(cdiv(m, 256)), 256, 0, st>>>(a, gs, seg, T_min, T_test, first, beater, o);
+    k_peak_warp<<<CL(cso_sm_count() * 8), 256, 0, st>>>(a, T_min, first, beater, o);
     k_peak_open<<<CL(cso_sm_count() * 8), OPEN_NT, 0, st>>>(a, T_min, first, beater, o);
     CSO_TRY(scan_u32(P.off, nseg, P.off + nseg, ws, st));
     k_peak_place<<<CL(cso_sm_count()), 256, 0, st>>>(a, o.found, o.counts, cursor, P);
