@@ -800,185 +800,6 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
   if ((tile + 1) * R2_TILE >= nd && threadIdx.x == 0) counts[2] = ta;
 }
 
-// Pass two, main trees as units: for every cell with dense particles and
-// each of its 13 forward neighbours (every adjacent pair of cells once), the
-// two main trees are joined if any pair of their members links.  A warp
-// holds the cell, 32 slots at a time, streams the neighbour through shared
-// memory and stops at the first link, so a pair of dense cells costs one
-// tile instead of a test per particle.
-__device__ __forceinline__ void fof_cell_pairs(const CellGrid& g, const int4* __restrict__ spos, int s0,
-                                               uint32_t lfof2, int lreach, int* __restrict__ parent,
-                                               const int* __restrict__ cell_root, const uint8_t* __restrict__ strag,
-                                               int4* tile, int* tmain, int4* tileA, int* hit, int lane) {
-  const int4 p0 = spos[s0];
-  const int nc = g.nc;
-  const int cy = cell_coord(p0.y, nc), cz = cell_coord(p0.z, nc), tc = grid_col(g, p0.x);
-  const size_t cA = grid_cell(g, cz, cy, tc);
-  const uint32_t a_lo = g.start[cA], a_hi = g.start[cA + 1];
-  const int crA = cell_root[a_lo];
-  const XCells X = x_cells(g, tc);
-  // lane r < 13: forward neighbour q = 14 + r, (dz, dy, dx) = (q / 9 - 1, q / 3 % 3 - 1, q % 3 - 1)
-  uint32_t b_lo = 0, b_hi = 0;
-  int crB = CELL_EMPTY, bsx = 0, bsy = 0, bsz = 0;
-  if (lane < 13) {
-    const int q = 14 + lane;
-    const int dz = q / 9 - 1, dy = q / 3 % 3 - 1, dx = q % 3 - 1;
-    int sz, sy;
-    const int zz = wrap_yz(cz + dz, nc, sz), yy = wrap_yz(cy + dy, nc, sy);
-    const int col = dx < 0 ? (X.a < tc ? X.a : X.wl) : (dx > 0 ? (X.b > tc ? X.b : X.wr) : tc);
-    const int sx = dx < 0 ? (X.a < tc ? 0 : CSO_BOX) : (dx > 0 ? (X.b > tc ? 0 : -CSO_BOX) : 0);
-    if (col >= 0) {
-      const size_t c = grid_cell(g, zz, yy, col);
-      b_lo = g.start[c];
-      b_hi = g.start[c + 1];
-      if (b_lo < b_hi) crB = cell_root[b_lo];
-      bsx = sx;
-      bsy = sy;
-      bsz = sz;
-    }
-  }
-  // every neighbour's tree against ours at once (a stale answer only costs a search)
-  const int rootA = uf_root(parent, crA);
-  const bool need = crB >= 0 && uf_root(parent, crB) != rootA;
-  const uint32_t mA = a_hi - a_lo, mB = b_hi - b_lo;
-  const bool small = mA <= 32 && mB <= 32;
-  if (mA <= 32 && __any_sync(0xffffffffu, need && small)) {
-    // Small pairs together: A's slots staged once, the warp's lanes take
-    // (neighbour, slot) pairs of all small neighbours in turn, and every lane
-    // tests its neighbour particle against all of A.
-    const uint32_t a = a_lo + lane;
-    const bool av = a < a_hi && parent[a] >= 0 && !strag[a];
-    tileA[lane] = av ? spos[a] : make_int4(0, 0, 0, 0);
-    if (lane < 13) hit[lane] = 0;
-    const unsigned amask = __ballot_sync(0xffffffffu, av);
-    const uint32_t cnt = (need && small) ? mB : 0;
-    uint32_t incl = cnt;
-    for (int o = 1; o < 16; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const uint32_t total = __shfl_sync(0xffffffffu, incl, 12);
-    const uint32_t excl = incl - cnt;
-    __syncwarp();
-    for (uint32_t base = 0; base < total; base += 32) {
-      const uint32_t gi = base + lane;
-      int r = 12;
-      for (int q = 11; q >= 0; --q) {
-        const uint32_t pr = __shfl_sync(0xffffffffu, incl, q);
-        if (gi < pr) r = q;
-      }
-      const uint32_t bl = __shfl_sync(0xffffffffu, b_lo, r), ex = __shfl_sync(0xffffffffu, excl, r);
-      const int sx = __shfl_sync(0xffffffffu, bsx, r), sy = __shfl_sync(0xffffffffu, bsy, r),
-                sz = __shfl_sync(0xffffffffu, bsz, r);
-      const uint32_t t = bl + (gi - ex);
-      if (gi < total && amask && parent[t] >= 0 && !strag[t]) {
-        const int4 q = spos[t];
-        const int qx = q.x - sx, qy = q.y - sy, qz = q.z - sz;
-        for (unsigned m = amask; m; m &= m - 1) {
-          const int4 pa = tileA[__ffs(m) - 1];
-          const int dx = pa.x - qx, dy = pa.y - qy, dz = pa.z - qz;
-          const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
-          if (d < lfof2) {
-            hit[r] = 1;
-            break;
-          }
-        }
-      }
-    }
-    __syncwarp();
-    if (lane < 13 && hit[lane]) uf_unite(parent, crA, crB);
-    __syncwarp();
-  }
-  // pairs with a big side: the neighbour streamed through shared memory
-  for (unsigned todo = __ballot_sync(0xffffffffu, need && !small); todo; todo &= todo - 1) {
-    const int r = __ffs(todo) - 1;
-    const uint32_t lo = __shfl_sync(0xffffffffu, b_lo, r), hi = __shfl_sync(0xffffffffu, b_hi, r);
-    const int cb = __shfl_sync(0xffffffffu, crB, r);
-    const int sx = __shfl_sync(0xffffffffu, bsx, r), sy = __shfl_sync(0xffffffffu, bsy, r),
-              sz = __shfl_sync(0xffffffffu, bsz, r);
-    int same = 0;
-    if (lane == 0) same = uf_root(parent, crA) == uf_root(parent, cb);
-    if (__shfl_sync(0xffffffffu, same, 0)) continue;
-    bool found = false;
-    // only our slots within l_FoF in x of the neighbour's x extent can link
-    uint32_t ta = a_lo, tb = a_hi;
-    if (lane == 0 && tb - ta > 32u) {
-      const int bx0 = spos[lo].x - sx, bx1 = spos[hi - 1].x - sx;
-      x_trim(spos, ta, tb, bx0 - lreach, bx1 + lreach);
-    }
-    ta = __shfl_sync(0xffffffffu, ta, 0);
-    tb = __shfl_sync(0xffffffffu, tb, 0);
-    for (uint32_t a0 = ta; a0 < tb && !found; a0 += 32) {
-      const uint32_t a = a0 + lane;
-      const bool av = a < tb && parent[a] >= 0 && !strag[a];
-      const int4 pa = av ? spos[a] : make_int4(0, 0, 0, 0);
-      const int xq = pa.x + sx, yq = pa.y + sy, zq = pa.z + sz;
-      if (!__any_sync(0xffffffffu, av)) continue;
-      // the neighbour's slots within l_FoF of this tile in x (cells are sorted by x)
-      const int xqmin = __reduce_min_sync(0xffffffffu, av ? xq : INT_MAX);
-      const int xqmax = __reduce_max_sync(0xffffffffu, av ? xq : INT_MIN);
-      uint32_t blo = lo, bhi = hi;
-      if (lane == 0 && bhi - blo > 32u) x_trim(spos, blo, bhi, xqmin - lreach, xqmax + lreach);
-      blo = __shfl_sync(0xffffffffu, blo, 0);
-      bhi = __shfl_sync(0xffffffffu, bhi, 0);
-      for (uint32_t b0 = blo; b0 < bhi; b0 += 32) {
-        const uint32_t t = b0 + lane;
-        const bool tv = t < bhi && parent[t] >= 0 && !strag[t];
-        tile[lane] = tv ? spos[t] : make_int4(0, 0, 0, 0);
-        tmain[lane] = tv;
-        __syncwarp();
-        const int m = bhi - b0 < 32 ? (int)(bhi - b0) : 32;
-        bool found_here = false;
-        if (av) {
-          for (int k = 0; k < m; ++k) {
-            if (!tmain[k]) continue;
-            const int4 qb = tile[k];
-            const int dx = xq - qb.x, dy = yq - qb.y, dz = zq - qb.z;
-            const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
-            if (d < lfof2) {
-              found_here = true;
-              break;
-            }
-          }
-        }
-        __syncwarp();
-        if (__any_sync(0xffffffffu, found_here)) {
-          found = true;
-          break;
-        }
-      }
-    }
-    if (found && lane == 0) uf_unite(parent, crA, cb);
-    __syncwarp();
-  }
-}
-
-__global__ void __launch_bounds__(256) k_fof_cells(CellGrid g, const int4* __restrict__ spos,
-                                                   const int* __restrict__ clist, const uint32_t* __restrict__ ncl_ptr,
-                                                   uint32_t lfof2, int lreach, int* __restrict__ parent,
-                                                   const int* __restrict__ cell_root,
-                                                   const uint8_t* __restrict__ strag) {
-  __shared__ int4 tile[8][32];
-  __shared__ int4 tileA[8][32];
-  __shared__ int tmain[8][32];
-  __shared__ int hit[8][16];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ncl = (int)*ncl_ptr;
-  for (int wi = blockIdx.x * 8 + w; wi < ncl; wi += gridDim.x * 8)
-    fof_cell_pairs(g, spos, clist[wi], lfof2, lreach, parent, cell_root, strag, tile[w], tmain[w], tileA[w], hit[w],
-                   lane);
-}
-
-// Pass three, the stragglers: against every neighbour cell in l_FoF reach (its
-// own included), the first link into the cell's main tree (skipped when that
-// tree is already the straggler's) and every link to a later straggler (each
-// straggler pair once).  A warp per straggler: lanes 0-26 look up one cell
-// each (skipping those out of reach by the particle's distance to the home
-// cell's faces, and trimming the rest to l_FoF in x), so the lookups' chain
-// of dependent loads is paid once and not once per cell, and the slots of all
-// cells are tested as one flat sequence, 32 at a time (a lane per straggler
-// walking its cells in turn: 202 us for the 3,000 stragglers of the side-64
-// box, where the longest walk set the time).
 __device__ __forceinline__ int fold21(int v) { return (int)((unsigned)v << 11) >> 11; }  // nearest image
 
 // lane whose run of the flat sequence holds f (incl: inclusive ends of the lanes' runs)
@@ -999,6 +820,203 @@ __device__ __forceinline__ uint32_t warp_incl_u32(uint32_t v, int lane) {
   return v;
 }
 
+// Pair of cells one of which holds more than 32 slots, by the whole warp:
+// whether any member of main tree A (slots a_lo .. a_hi) links with any of B
+// (slots lo .. hi, whose image our positions shifted by (sx, sy, sz) meet).
+// The warp holds 32 slots of A at a time, streams B through shared memory and
+// stops at the first link, so a pair of dense cells costs one tile instead of
+// a test per particle.
+__device__ __forceinline__ bool fof_big_pair(const int4* __restrict__ spos, uint32_t a_lo, uint32_t a_hi, uint32_t lo,
+                                             uint32_t hi, int sx, int sy, int sz, uint32_t lfof2, int lreach,
+                                             const int* __restrict__ parent, const uint8_t* __restrict__ strag,
+                                             int4* tile, int* tmain, int lane) {
+  bool found = false;
+  // only our slots within l_FoF in x of the neighbour's x extent can link
+  uint32_t ta = a_lo, tb = a_hi;
+  if (lane == 0 && tb - ta > 32u) {
+    const int bx0 = spos[lo].x - sx, bx1 = spos[hi - 1].x - sx;
+    x_trim(spos, ta, tb, bx0 - lreach, bx1 + lreach);
+  }
+  ta = __shfl_sync(0xffffffffu, ta, 0);
+  tb = __shfl_sync(0xffffffffu, tb, 0);
+  for (uint32_t a0 = ta; a0 < tb && !found; a0 += 32) {
+    const uint32_t a = a0 + lane;
+    const bool av = a < tb && parent[a] >= 0 && !strag[a];
+    const int4 pa = av ? spos[a] : make_int4(0, 0, 0, 0);
+    const int xq = pa.x + sx, yq = pa.y + sy, zq = pa.z + sz;
+    if (!__any_sync(0xffffffffu, av)) continue;
+    // the neighbour's slots within l_FoF of this tile in x (cells are sorted by x)
+    const int xqmin = __reduce_min_sync(0xffffffffu, av ? xq : INT_MAX);
+    const int xqmax = __reduce_max_sync(0xffffffffu, av ? xq : INT_MIN);
+    uint32_t blo = lo, bhi = hi;
+    if (lane == 0 && bhi - blo > 32u) x_trim(spos, blo, bhi, xqmin - lreach, xqmax + lreach);
+    blo = __shfl_sync(0xffffffffu, blo, 0);
+    bhi = __shfl_sync(0xffffffffu, bhi, 0);
+    for (uint32_t b0 = blo; b0 < bhi; b0 += 32) {
+      const uint32_t t = b0 + lane;
+      const bool tv = t < bhi && parent[t] >= 0 && !strag[t];
+      tile[lane] = tv ? spos[t] : make_int4(0, 0, 0, 0);
+      tmain[lane] = tv;
+      __syncwarp();
+      const int m = bhi - b0 < 32 ? (int)(bhi - b0) : 32;
+      bool found_here = false;
+      if (av) {
+        for (int k = 0; k < m; ++k) {
+          if (!tmain[k]) continue;
+          const int4 qb = tile[k];
+          const int dx = xq - qb.x, dy = yq - qb.y, dz = zq - qb.z;
+          const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
+          if (d < lfof2) {
+            found_here = true;
+            break;
+          }
+        }
+      }
+      __syncwarp();
+      if (__any_sync(0xffffffffu, found_here)) {
+        found = true;
+        break;
+      }
+    }
+  }
+  return found;
+}
+
+// Pass two, main trees as units: for every cell with dense particles and
+// each of its 13 forward neighbours (every adjacent pair of cells once), the
+// two main trees are joined if any pair of their members links.  Half a warp
+// per cell: lanes 0-12 of the half look up a neighbour each (its range, its
+// summary and both trees' roots: a chain of dependent loads that is all the
+// time there is to a small cell, so a warp runs two), pairs already in one
+// tree drop out, and the pairs of two cells of up to 32 slots are tested
+// together, the half's lanes spread over (neighbour, slot) pairs against the
+// cell staged once.  The whole warp then takes the other pairs of both cells
+// in turn.  (Those on a list of their own, a warp per cell or per pair, were
+// slower: joining one neighbour often joins the next, and sooner is better.)
+// Full occupancy (32 registers, a few spilled) is worth more here than none
+// spilled: FoF of the side-256 box 3.86 ms with a warp per cell, 3.75 with
+// half a warp, 3.46 at eight blocks per SM.
+__device__ __forceinline__ int forward_col(const XCells& X, int tc, int dx) {
+  return dx < 0 ? (X.a < tc ? X.a : X.wl) : (dx > 0 ? (X.b > tc ? X.b : X.wr) : tc);
+}
+
+__global__ void __launch_bounds__(256, 8) k_fof_cells(CellGrid g, const int4* __restrict__ spos,
+                                                   const int* __restrict__ clist, const uint32_t* __restrict__ ncl_ptr,
+                                                   uint32_t lfof2, int lreach, int* __restrict__ parent,
+                                                   const int* __restrict__ cell_root,
+                                                   const uint8_t* __restrict__ strag) {
+  __shared__ int4 tile[16][32];
+  __shared__ int tmains[8][32];
+  const int lane = threadIdx.x & 31, l16 = lane & 15, sub = lane >> 4;
+  int4* tileA = tile[threadIdx.x >> 4];
+  const int ncl = (int)*ncl_ptr;
+  const int nc = g.nc;
+  for (int i0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5 << 1; i0 < ncl; i0 += gridDim.x * blockDim.x >> 4) {
+    const bool valid = i0 + sub < ncl;
+    const int s0 = clist[valid ? i0 + sub : i0];
+    const int4 p0 = spos[s0];
+    const int cy = cell_coord(p0.y, nc), cz = cell_coord(p0.z, nc), tc = grid_col(g, p0.x);
+    const size_t cA = grid_cell(g, cz, cy, tc);
+    const uint32_t a_lo = g.start[cA], mA = g.start[cA + 1] - a_lo;
+    const int crA = cell_root[a_lo];
+    // lane r < 13: forward neighbour q = 14 + r, (dz, dy, dx) = (q / 9 - 1, q / 3 % 3 - 1, q % 3 - 1)
+    uint32_t b_hi = 0, mB = 0;
+    int crB = CELL_EMPTY, bsx = 0, bsy = 0, bsz = 0;
+    if (l16 < 13) {
+      const int q = 14 + l16, dx1 = q % 3 - 1;
+      const int zz = wrap_yz(cz + q / 9 - 1, nc, bsz), yy = wrap_yz(cy + q / 3 % 3 - 1, nc, bsy);
+      const XCells X = x_cells(g, tc);
+      const int col = forward_col(X, tc, dx1);
+      bsx = dx1 < 0 ? (X.a < tc ? 0 : CSO_BOX) : (dx1 > 0 ? (X.b > tc ? 0 : -CSO_BOX) : 0);
+      if (col >= 0) {
+        const size_t c = grid_cell(g, zz, yy, col);
+        const uint32_t lo = g.start[c];
+        b_hi = g.start[c + 1];
+        mB = b_hi - lo;
+        if (mB) crB = cell_root[lo];
+      }
+    }
+    // every neighbour's tree against ours at once (a stale answer only costs a search)
+    const bool need = valid && crB >= 0 && uf_root(parent, crB) != uf_root(parent, crA);
+    const bool small = mA <= 32 && mB <= 32;
+    unsigned big = __ballot_sync(0xffffffffu, need && !small);  // bit 16 sub + r
+    const uint32_t cnt = need && small ? mB : 0;
+    const unsigned any = __ballot_sync(0xffffffffu, cnt > 0);
+    if (any) {
+      const bool mine = any >> (16 * sub) & 0xffffu;
+      unsigned amask = 0;
+  #pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t o = l16 + 16 * k;
+        const bool av = mine && o < mA && parent[a_lo + o] >= 0 && !strag[a_lo + o];
+        if (av) tileA[o] = spos[a_lo + o];
+        amask |= (__ballot_sync(0xffffffffu, av) >> (16 * sub) & 0xffffu) << (16 * k);
+      }
+      uint32_t incl = cnt;
+  #pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o, 16);
+        if (l16 >= o) incl += t;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 15, 16);
+      const uint32_t longest = max(total, __shfl_xor_sync(0xffffffffu, total, 16));
+      __syncwarp();
+      unsigned hits = 0;  // bit 16 sub + r: pair r of the half links
+      for (uint32_t f0 = 0; f0 < longest; f0 += 16) {
+        const uint32_t f = f0 + l16;
+        int r = 0;
+  #pragma unroll
+        for (int o = 8; o; o >>= 1)
+          if (__shfl_sync(0xffffffffu, incl, r + o - 1, 16) <= f) r += o;
+        const uint32_t end = __shfl_sync(0xffffffffu, incl, r, 16), hi = __shfl_sync(0xffffffffu, b_hi, r, 16);
+        bool hit = false;
+        if (f < total && !(hits >> (16 * sub + r) & 1u)) {
+          const uint32_t t = hi - (end - f);
+          if (parent[t] >= 0 && !strag[t]) {
+            const int4 q = spos[t];
+            for (unsigned m = amask; m; m &= m - 1) {
+              const int4 pa = tileA[__ffs(m) - 1];
+              const int dx = fold21(pa.x - q.x), dy = fold21(pa.y - q.y), dz = fold21(pa.z - q.z);
+              if ((uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz) < lfof2) {
+                hit = true;
+                break;
+              }
+            }
+          }
+        }
+        hits |= __reduce_or_sync(0xffffffffu, hit ? 1u << (16 * sub + r) : 0u);
+      }
+      if (hits >> lane & 1u) uf_unite(parent, crA, crB);
+      __syncwarp();
+    }
+    for (; big; big &= big - 1) {
+      const int r = __ffs(big) - 1;
+      const uint32_t hi = __shfl_sync(0xffffffffu, b_hi, r), lo = hi - __shfl_sync(0xffffffffu, mB, r);
+      const uint32_t alo = __shfl_sync(0xffffffffu, a_lo, r), ahi = alo + __shfl_sync(0xffffffffu, mA, r);
+      const int ca = __shfl_sync(0xffffffffu, crA, r), cb = __shfl_sync(0xffffffffu, crB, r);
+      const int sx = __shfl_sync(0xffffffffu, bsx, r), sy = __shfl_sync(0xffffffffu, bsy, r),
+                sz = __shfl_sync(0xffffffffu, bsz, r);
+      int same = 0;
+      if (lane == 0) same = uf_root(parent, ca) == uf_root(parent, cb);
+      if (__shfl_sync(0xffffffffu, same, 0)) continue;
+      const bool found = fof_big_pair(spos, alo, ahi, lo, hi, sx, sy, sz, lfof2, lreach, parent, strag,
+                                      tile[threadIdx.x >> 5 << 1], tmains[threadIdx.x >> 5], lane);
+      if (found && lane == 0) uf_unite(parent, ca, cb);
+      __syncwarp();
+    }
+  }
+}
+
+// Pass three, the stragglers: against every neighbour cell in l_FoF reach (its
+// own included), the first link into the cell's main tree (skipped when that
+// tree is already the straggler's) and every link to a later straggler (each
+// straggler pair once).  A warp per straggler: lanes 0-26 look up one cell
+// each (skipping those out of reach by the particle's distance to the home
+// cell's faces, and trimming the rest to l_FoF in x), so the lookups' chain
+// of dependent loads is paid once and not once per cell, and the slots of all
+// cells are tested as one flat sequence, 32 at a time (a lane per straggler
+// walking its cells in turn: 202 us for the 3,000 stragglers of the side-64
+// box, where the longest walk set the time).
 __global__ void __launch_bounds__(256) k_fof_stragglers(CellGrid g, const int4* __restrict__ spos,
                                                         const int* __restrict__ slist,
                                                         const uint32_t* __restrict__ ns_ptr, uint32_t lfof2,
@@ -1234,7 +1252,7 @@ int cells_fof(const CellGrid& g, const int4* spos, int n, const long long* sigma
   uint8_t* strag = ws.get<uint8_t>(n);
   int* slist = ws.get<int>(n);
   uint2* srange = ws.get<uint2>(n);
-  // status words of the two lists' ranks, then the list lengths: dense
+  // status words of the two lists' ranks, then the lists' lengths: dense
   // particles, cells that hold any, stragglers
   unsigned long long* status = ws.get<unsigned long long>((size_t)(2 * words + 2));
   if (!didx || !clist || !strag || !slist || !srange || !status) {
