@@ -574,7 +574,8 @@ __device__ __forceinline__ uint32_t cell_id(const CellGrid& g, int4 p) {
 // holds any.  counts[0] and counts[1] receive their lengths.  (A pass each
 // for the flags, their scans and the lists: 0.39 ms on the side-256 box, this
 // one 0.16.)
-__global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4* __restrict__ spos, int n,
+template <int ITEMS>
+__global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const int4* __restrict__ spos, int n,
                                                           const long long* __restrict__ sigma, long long T_L0,
                                                           int* __restrict__ parent, int* __restrict__ cell_root,
                                                           unsigned long long* __restrict__ minid,
@@ -585,10 +586,10 @@ __global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
-  unsigned dense[R2_ITEMS], head[R2_ITEMS];
+  const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
+  unsigned dense[ITEMS], head[ITEMS];
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long i = base + q * 32 + lane;
     const bool in = i < n;
     const bool d = in && sigma[i] > T_L0;
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4
   }
   uint32_t na = 0, nb = 0;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     bool h = false;
     if (dense[q] >> lane & 1u) {
       // first of its cell: no dense slot before it there (the one next to it, mostly)
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4
   rank2_prefix(S, status, tile, na, nb, ta, tb, err);
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const int i = (int)(base + q * 32 + lane);
     if (dense[q] >> lane & 1u) didx[na + __popc(dense[q] & lt)] = i;
     if (head[q] >> lane & 1u) clist[nb + __popc(head[q] & lt)] = i;
@@ -636,9 +637,10 @@ __global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4
 }
 
 // Pass one (in the spirit of Afforest, Sutton et al. 2018): each dense
-// particle tests the W = 32 slots after it in its cell, cyclically, so every
-// pair of a cell of up to 33 particles is tested and a big cell is joined by
-// a band of links around it.  The band joins almost every dense particle of
+// particle tests the W = 16 slots after it in its cell, cyclically, so every
+// pair of a cell of up to 17 particles is tested and a big cell is joined by
+// a band of links around it (FoF of the side-256 box: 3.24 ms with W = 16, 3.31
+// with 32, 4.54 with 8, which leaves more stragglers).  The band joins almost every dense particle of
 // a big cell into one tree; the few it misses are handled one by one later.
 //
 // A warp whose particles share a cell streams the union of its lanes'
@@ -646,7 +648,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_fof_lists(CellGrid g, const int4
 // its current root (-1 if not dense), so a lane pays a forest update only for
 // a link into another tree.  A staged root that has since been hooked
 // elsewhere is still a member of its tree, so the test stays correct.
-constexpr uint32_t FOF_BAND = 32;
+constexpr uint32_t FOF_BAND = 16;
 
 __global__ void __launch_bounds__(256) k_fof_sample(CellGrid g, const int4* __restrict__ spos,
                                                     const int* __restrict__ didx, const uint32_t* __restrict__ nd_ptr,
@@ -739,6 +741,7 @@ __global__ void k_cell_main(const int4* __restrict__ spos, CellGrid g, const int
 // (one with dense particles) in that list.  Also points every dense particle
 // straight at its root.  Tiles are of the dense list: those past its end have
 // nothing to publish.
+template <int ITEMS>
 __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restrict__ spos, CellGrid g,
                                                            const int* __restrict__ didx, uint32_t* __restrict__ counts,
                                                            int* __restrict__ parent, const int* __restrict__ cell_root,
@@ -749,15 +752,15 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
   __shared__ Rank2Shared S;
   const long long nd = counts[0];
   const long long tile = rank2_tile(S, status, ntiles);
-  if (tile * R2_TILE >= nd) return;  // counts[2] starts at zero
+  if (tile * (R2_THREADS * ITEMS) >= nd) return;  // counts[2] starts at zero
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
-  unsigned flag[R2_ITEMS];
-  uint32_t lo[R2_ITEMS];  // the cell's first slot; top bits: first and last dense particle of the cell
+  const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
+  unsigned flag[ITEMS];
+  uint32_t lo[ITEMS];  // the cell's first slot; top bits: first and last dense particle of the cell
   unsigned first = 0, last = 0;
   uint32_t na = 0, nb = 0;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long i = base + q * 32 + lane;
     bool f = false, a = false, z = false;
     uint32_t c = 0;
@@ -789,7 +792,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
   rank2_prefix(S, status, tile, na, nb, ta, tb, err);
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const uint32_t r = na + __popc(flag[q] & lt);
     const uint32_t f = flag[q] >> lane & 1u;
     if (f) slist[r] = didx[base + q * 32 + lane];
@@ -797,7 +800,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
     if (last >> q & 1u) srange[lo[q]].y = r + f;
     na += __popc(flag[q]);
   }
-  if ((tile + 1) * R2_TILE >= nd && threadIdx.x == 0) counts[2] = ta;
+  if ((tile + 1) * (R2_THREADS * ITEMS) >= nd && threadIdx.x == 0) counts[2] = ta;
 }
 
 __device__ __forceinline__ int fold21(int v) { return (int)((unsigned)v << 11) >> 11; }  // nearest image
@@ -1017,7 +1020,7 @@ __global__ void __launch_bounds__(256, 8) k_fof_cells(CellGrid g, const int4* __
 // cells are tested as one flat sequence, 32 at a time (a lane per straggler
 // walking its cells in turn: 202 us for the 3,000 stragglers of the side-64
 // box, where the longest walk set the time).
-__global__ void __launch_bounds__(256) k_fof_stragglers(CellGrid g, const int4* __restrict__ spos,
+__global__ void __launch_bounds__(256, 8) k_fof_stragglers(CellGrid g, const int4* __restrict__ spos,
                                                         const int* __restrict__ slist,
                                                         const uint32_t* __restrict__ ns_ptr, uint32_t lfof2,
                                                         int lreach, int* __restrict__ parent,
@@ -1264,18 +1267,18 @@ int cells_fof(const CellGrid& g, const int4* spos, int n, const long long* sigma
     return CSO_ERR_STATE;
   }
   uint32_t* counts = reinterpret_cast<uint32_t*>(status + 2 * words);
-  const unsigned tiles = (unsigned)(words - 1);
+  const long long tiles = rank2_tiles(n);
   CSO_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)(2 * words + 2), st));
   // launches over the lists are sized by n and blocks past the counts (read
   // on the device) return at once
-  k_fof_lists<<<CL(tiles), R2_THREADS, 0, st>>>(g, spos, n, sigma, T_L0, parent, cell_root, minid, didx, clist, counts,
-                                                status, words - 1, ws.err);
+  RANK2_LAUNCH(k_fof_lists, n, st, g, spos, n, sigma, T_L0, parent, cell_root, minid, didx, clist, counts, status, tiles,
+               ws.err);
   const uint32_t *nd = counts, *ncl = counts + 1, *ns = counts + 2;
   // pass one: bands inside cells; main trees and stragglers
   k_fof_sample<<<CL(cdiv(n, 256)), 256, 0, st>>>(g, spos, didx, nd, lfof2, parent);
   k_cell_main<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, clist, ncl, parent, cell_root);
-  k_stragglers<<<CL(tiles), R2_THREADS, 0, st>>>(spos, g, didx, counts, parent, cell_root, strag, slist, srange,
-                                                 status + words, words - 1, ws.err);
+  RANK2_LAUNCH(k_stragglers, n, st, spos, g, didx, counts, parent, cell_root, strag, slist, srange, status + words, tiles,
+               ws.err);
   // pass two: main trees of adjacent cells; pass three: stragglers
   const int lreach = reach_below(lfof2);
   k_fof_cells<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, clist, ncl, lfof2, lreach, parent, cell_root, strag);

@@ -29,6 +29,7 @@ constexpr unsigned long long NONE = ~0ull;
 // The dense particles taking part, listed in cell order, and the index of
 // every group at its root (groups in the order of their roots); the numbers of
 // both go to meta.
+template <int ITEMS>
 __global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restrict__ root, int n,
                                                             const uint8_t* __restrict__ select,
                                                             uint32_t* __restrict__ dl, uint32_t* __restrict__ gidx,
@@ -37,11 +38,11 @@ __global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restric
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
-  unsigned in[R2_ITEMS], head[R2_ITEMS];
+  const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
+  unsigned in[ITEMS], head[ITEMS];
   uint32_t na = 0, nb = 0;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long i = base + q * 32 + lane;
     const int r = i < n ? root[i] : -1;
     const bool d = r >= 0 && (!select || select[i]);
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restric
   rank2_prefix(S, status, tile, na, nb, ta, tb, &meta->timeout);
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const uint32_t i = (uint32_t)(base + q * 32 + lane);
     if (in[q] >> lane & 1u) dl[na + __popc(in[q] & lt)] = i;
     if (head[q] >> lane & 1u) gidx[i] = nb + __popc(head[q] & lt);
@@ -123,6 +124,7 @@ __global__ void k_gather_pos(const uint32_t* __restrict__ gs, int nd, const int4
 // The members of L1 haloes, listed with their halo's index; their L1 labels,
 // on the device by cell-sorted index and (optional) in input order.  The
 // number of members goes to *total.
+template <int ITEMS>
 __global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restrict__ eslot,
                                                               const uint32_t* __restrict__ grp,
                                                               const uint32_t* __restrict__ hbase,
@@ -139,12 +141,12 @@ __global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restr
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
-  unsigned in[R2_ITEMS];
-  int slot[R2_ITEMS];
+  const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
+  unsigned in[ITEMS];
+  int slot[ITEMS];
   uint32_t na = 0, nb = 0;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long k = base + q * 32 + lane;
     slot[q] = k < nd ? eslot[k] : -1;
     in[q] = __ballot_sync(0xffffffffu, slot[q] >= 0);
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restr
   uint32_t ta, tb;
   rank2_prefix(S, status, tile, na, nb, ta, tb, err);
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long k = base + q * 32 + lane;
     if (slot[q] >= 0) {
       const uint32_t g = grp[k], h = hbase[g] + (uint32_t)slot[q], s = gs[k];
@@ -343,6 +345,7 @@ __global__ void k_summary(const uint32_t* __restrict__ seg2, int H1, const uint3
 }
 
 // the rows the catalogue keeps, listed by their index; their number goes to *total
+template <int ITEMS>
 __global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* __restrict__ rows,
                                                                const uint32_t* __restrict__ keep, int H,
                                                                uint64_t* __restrict__ key, uint32_t* __restrict__ val,
@@ -352,11 +355,11 @@ __global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* _
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long base = tile * R2_TILE + (long long)w * 32 * R2_ITEMS;
-  unsigned in[R2_ITEMS];
+  const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
+  unsigned in[ITEMS];
   uint32_t na = 0, nb = 0;
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long h = base + q * 32 + lane;
     in[q] = __ballot_sync(0xffffffffu, h < H && keep[h]);
     na += __popc(in[q]);
@@ -364,7 +367,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* _
   uint32_t ta, tb;
   rank2_prefix(S, status, tile, na, nb, ta, tb, err);
 #pragma unroll
-  for (int q = 0; q < R2_ITEMS; ++q) {
+  for (int q = 0; q < ITEMS; ++q) {
     const long long h = base + q * 32 + lane;
     if (in[q] >> lane & 1u) {
       const uint32_t d = na + __popc(in[q] & ((1u << lane) - 1u));
@@ -471,7 +474,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   ALLOC(uint32_t, dl, n);
   ALLOC(uint32_t, gidx, n);
   ALLOC(uint32_t, grp, n);
-  k_member_list<<<CL((unsigned)(words - 1)), R2_THREADS, 0, st>>>(root, N, gi.select, dl, gidx, rstat, words - 1, meta);
+  RANK2_LAUNCH(k_member_list, n, st, root, N, gi.select, dl, gidx, rstat, rank2_tiles(n), meta);
   k_member_group<<<G1(n)>>>(dl, root, gidx, sigma, sid, grp, meta);
   CSO_CUDA(cudaGetLastError());
   // counters: dense particles, groups, sigma_max, id_max, bad
@@ -572,10 +575,8 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   uint32_t* egs2 = aval;   // cell-sorted index of each member
   uint32_t* ehal2 = akey;  // its L1 halo, ascending
   if (nd > 0) {
-    const long long w2 = rank2_words(nd);
-    k_assigned_list<<<CL((unsigned)(w2 - 1)), R2_THREADS, 0, st>>>(eslot, gseg, hbase, seg1, nucm, nd, gs, epos, sid,
-                                                                   akey, aval, lab1, ol1, rstat + words, w2 - 1,
-                                                                   hbase + G + 1, ws.err);
+    RANK2_LAUNCH(k_assigned_list, (long long)nd, st, eslot, gseg, hbase, seg1, nucm, nd, gs, epos, sid, akey, aval, lab1, ol1,
+                 rstat + words, rank2_tiles(nd), hbase + G + 1, ws.err);
   } else {
     CSO_CUDA(cudaMemsetAsync(hbase + G + 1, 0, sizeof(uint32_t), st));
   }
@@ -689,9 +690,8 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
     }
     ALLOC(uint64_t, ckey, H1);
     ALLOC(uint32_t, cval, H1);
-    const long long w3 = rank2_words(H1);
-    k_catalogue_list<<<CL((unsigned)(w3 - 1)), R2_THREADS, 0, st>>>(rows, keep, H1, ckey, cval, rstat + 2 * words, w3 - 1,
-                                                                    keep + H1, ws.err);
+    RANK2_LAUNCH(k_catalogue_list, (long long)H1, st, rows, keep, H1, ckey, cval, rstat + 2 * words, rank2_tiles(H1),
+                 keep + H1, ws.err);
     CSO_CUDA(cudaGetLastError());
     CSO_TRY(readback(c, keep + H1, 4));
     nrows = (int)((uint32_t*)c->pinned)[0];

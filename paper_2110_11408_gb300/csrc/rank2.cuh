@@ -8,8 +8,11 @@
 
 constexpr int R2_THREADS = 256;
 constexpr int R2_WARPS = R2_THREADS / 32;
-constexpr int R2_ITEMS = 16;  // elements per lane: a warp holds 512 consecutive ones, 32 per item
-constexpr int R2_TILE = R2_THREADS * R2_ITEMS;
+// Elements per lane (a warp holds 32 ITEMS consecutive ones, 32 per item): 16,
+// or 4 for arrays of up to R2_SMALL elements, where tiles of 4,096 would leave
+// most SMs without one (131,000 dense particles: k_stragglers 52 -> 21 us).
+constexpr int R2_BIG = 16, R2_FEW = 4;
+constexpr long long R2_SMALL = 1ll << 21;
 
 // A status word: state << 62 | first count << 31 | second count (counts below
 // 2^31).  States: 0 not published, 1 the tile's own counts, 2 inclusive prefix.
@@ -19,8 +22,22 @@ struct Rank2Shared {
   long long tile;
 };
 
-// status words needed for n elements (tiles, then the tile counter), zeroed by the caller
-static inline long long rank2_words(long long n) { return cdiv(n, R2_TILE) + 1; }
+static inline long long rank2_tiles(long long n) {
+  return cdiv(n, R2_THREADS * (n > R2_SMALL ? R2_BIG : R2_FEW));
+}
+// status words needed for n elements or fewer (tiles, then the tile counter), zeroed by the caller
+static inline long long rank2_words(long long n) {
+  const long long few = n < R2_SMALL ? n : R2_SMALL, a = cdiv(few, R2_THREADS * R2_FEW), b = cdiv(n, R2_THREADS * R2_BIG);
+  return (a > b ? a : b) + 1;
+}
+
+// launches KERNEL<ITEMS> over n elements; the variadic arguments end in ..., status, tiles, ...
+#define RANK2_LAUNCH(KERNEL, n, st, ...)                                                             \
+  do {                                                                                               \
+    const unsigned tiles_ = (unsigned)rank2_tiles(n);                                                \
+    if ((n) > R2_SMALL) KERNEL<R2_BIG><<<CL(tiles_), R2_THREADS, 0, st>>>(__VA_ARGS__);              \
+    else KERNEL<R2_FEW><<<CL(tiles_), R2_THREADS, 0, st>>>(__VA_ARGS__);                             \
+  } while (0)
 
 __device__ __forceinline__ long long rank2_tile(Rank2Shared& S, unsigned long long* status, long long ntiles) {
   if (threadIdx.x == 0) S.tile = (long long)atomicAdd(&status[ntiles], 1ull);
