@@ -73,7 +73,11 @@ struct Workspace {
 // ---------------------------------------------------------------------------
 // exclusive scan of n uint32 values in place; *total (device, may be null)
 // receives the sum.  Scratch comes from ws.
-int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaStream_t st);
+// With `half` the values come from there (16 bits each, 8-byte aligned) unless
+// *over (device) is set, and data receives the result either way.  data is
+// 16-byte aligned.
+int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaStream_t st,
+             const uint16_t* half = nullptr, const int* over = nullptr);
 
 // Stable LSD radix sort of (key, val) pairs by the low `bits` bits of the
 // 128-bit key (hi:lo).  Sorted output ends in (*khi, *klo, *val) which point

@@ -1,5 +1,5 @@
 // Ranks of two sets of flagged elements in one pass over the array: the
-// single-pass scan of scan_sort.cu (decoupled look-back over tiles taken from
+// one-sweep sort of scan_sort.cu (decoupled look-back over tiles taken from
 // an atomic counter) for flags known inside the caller's kernel, so that a
 // list is written by the kernel that decides who is on it, with no flag
 // array, scan and second pass in between.

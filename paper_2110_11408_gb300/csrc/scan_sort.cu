@@ -1,5 +1,4 @@
-// Device-wide exclusive scan (single pass, decoupled look-back) and stable
-// LSD radix sorts (8-bit digits).
+// Device-wide exclusive scan and stable LSD radix sorts (8-bit digits).
 //
 // Both sorts rank elements inside a tile with warp-level matching
 // (__match_any_sync): warp w owns a contiguous run of the tile and keeps a
@@ -44,18 +43,9 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* smem_w
   return total;
 }
 
-// Single-pass exclusive scan with decoupled look-back (Merrill and Garland,
-// "Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016).  Tiles
-// take their index from an atomic counter in the order they start, so every
-// predecessor of a tile is already running; each tile publishes its aggregate
-// (flag A), then warp 0 walks back over 32 predecessors at a time, adding
-// aggregates until it meets an inclusive prefix (flag P), and publishes its
-// own inclusive prefix.  A status word is flag << 32 | value.
-// Tiles of 4,096 values (256 threads of 16), or of 32,768 (1,024 of 32) for
-// arrays of more than SP_BIG values, where fewer look-backs count for more
-// (binning of the side-256 box with its 262M-entry table 2.25 -> 2.18 ms
-// against tiles of 8,192).
-constexpr long long SP_BIG = 1ll << 22;
+// Look-back status words of the one-sweep sort (the decoupled look-back of
+// Merrill and Garland, "Single-pass Parallel Prefix Scan with Decoupled
+// Look-back", 2016): flag << 32 | value.
 constexpr unsigned long long SP_A = 1ull << 32, SP_P = 2ull << 32;
 constexpr long long SP_SPIN_LIMIT = 1ll << 22;
 
@@ -68,98 +58,108 @@ __device__ __forceinline__ void sp_store(unsigned long long* p, unsigned long lo
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// status[0 .. ntiles) and the tile counter status[ntiles] start at zero
-template <int SP_THREADS, int SP_ITEMS>
-__global__ void __launch_bounds__(SP_THREADS) k_scan_onepass(uint32_t* __restrict__ d, long long n,
-                                                             unsigned long long* __restrict__ status, long long ntiles,
-                                                             uint32_t* __restrict__ total, int* __restrict__ err) {
-  constexpr int SP_TILE = SP_THREADS * SP_ITEMS;
-  constexpr int R = SP_ITEMS / 4;  // rounds of four consecutive values per lane
-  __shared__ uint32_t sw[33];
-  __shared__ long long tile_sh;
-  __shared__ uint32_t prefix_sh;
-  if (threadIdx.x == 0) tile_sh = (long long)atomicAdd(&status[ntiles], 1ull);
-  __syncthreads();
-  const long long tile = tile_sh;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  // warp w holds a contiguous run of the tile; in round q its lanes hold 32
-  // consecutive groups of four values, so every load moves 512 contiguous bytes
-  const long long wb = tile * SP_TILE + (long long)w * 32 * SP_ITEMS;
-  const bool vec = wb + 32 * SP_ITEMS <= n && ((reinterpret_cast<uintptr_t>(d) & 15) == 0);
-  uint4 v[R];
-#pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const long long i = wb + ((long long)q * 32 + lane) * 4;
-    if (vec) {
-      v[q] = *reinterpret_cast<const uint4*>(d + i);
-    } else {
-      v[q].x = i < n ? d[i] : 0u;
-      v[q].y = i + 1 < n ? d[i + 1] : 0u;
-      v[q].z = i + 2 < n ? d[i + 2] : 0u;
-      v[q].w = i + 3 < n ? d[i + 3] : 0u;
+// Exclusive scan of a large array in two passes over it: sums of every warp's
+// run (k_scan_sums), the blocks' sums in one block (k_scan_small), then the runs
+// again with their bases (k_scan_apply).  Bound by its bytes: the second read
+// costs less than the waits of a single pass with look-back did, and no warp
+// waits for another.  Of 262M values 0.52 -> 0.47 ms against tiles of 32,768 by
+// look-back, of 2M to 4M 21-25 -> 15 us (with the clearing of its status words).
+// A run is `rounds` times 128 values (a multiple of 4 rounds, so that four loads
+// a lane are in flight); a block is 8 runs.
+constexpr int SC_WARPS = 8;
+
+struct ScanIn {
+  const uint32_t* w;     // the values,
+  const uint16_t* half;  // or (not null, and *over 0) the same in 16 bits
+  const int* over;
+  __device__ __forceinline__ bool narrow() const { return half && *over == 0; }
+};
+
+// values i .. i+3 (i a multiple of 4), zero past n
+template <bool HALF>
+__device__ __forceinline__ uint4 scan_load(const ScanIn& in, long long i, long long n) {
+  if (i + 4 <= n) {
+    if (HALF) {
+      const uint2 v = *reinterpret_cast<const uint2*>(in.half + i);
+      return make_uint4(v.x & 0xffffu, v.x >> 16, v.y & 0xffffu, v.y >> 16);
     }
+    return *reinterpret_cast<const uint4*>(in.w + i);
   }
-  // each round's exclusive prefix within the warp's run
-  uint32_t base[R];
-  uint32_t carry = 0;
+  uint32_t t[4];
 #pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const uint32_t sq = v[q].x + v[q].y + v[q].z + v[q].w;
-    const uint32_t inc = warp_incl_scan(sq);
-    base[q] = carry + inc - sq;
-    carry += __shfl_sync(0xffffffffu, inc, 31);
+  for (int k = 0; k < 4; ++k) t[k] = i + k < n ? (HALF ? (uint32_t)in.half[i + k] : in.w[i + k]) : 0u;
+  return make_uint4(t[0], t[1], t[2], t[3]);
+}
+
+template <bool HALF>
+__device__ __forceinline__ uint32_t scan_run_sum(const ScanIn& in, long long at, long long n, int rounds) {
+  uint32_t sum = 0;
+  for (int r = 0; r < rounds; r += 4) {
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = scan_load<HALF>(in, at + (long long)(r + k) * 128, n);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sum += v[k].x + v[k].y + v[k].z + v[k].w;
   }
-  // the warps' runs in order: lane 0 carries its warp's total into the block scan
-  uint32_t excl;
-  const uint32_t agg = block_excl_scan(lane == 0 ? carry : 0u, sw, excl);
-  const uint32_t woff = __shfl_sync(0xffffffffu, excl, 0);
-  if (threadIdx.x < 32) {
-    uint32_t prefix = 0;
-    if (tile > 0) {
-      if (lane == 0) sp_store(&status[tile], SP_A | agg);
-      long long top = tile - 1;
-      long long spins = 0;
-      for (;;) {
-        const long long j = top - lane;
-        const unsigned long long wv = j >= 0 ? sp_load(&status[j]) : SP_P;  // before tile 0: prefix 0
-        const unsigned long long flag = wv & ~0xffffffffull;
-        const unsigned pmask = __ballot_sync(0xffffffffu, flag == SP_P);
-        const unsigned xmask = __ballot_sync(0xffffffffu, flag == 0);
-        const int firstP = pmask ? __ffs(pmask) - 1 : 31;
-        const unsigned need = firstP == 31 ? 0xffffffffu : ((2u << firstP) - 1u);
-        if (xmask & need) {  // a predecessor has not published yet
-          if (++spins > SP_SPIN_LIMIT) {
-            if (lane == 0) atomicExch(err, 1);
-            break;
-          }
-          continue;
-        }
-        prefix += __reduce_add_sync(0xffffffffu, lane <= firstP ? (uint32_t)wv : 0u);
-        if (pmask) break;
-        top -= 32;
+  return __reduce_add_sync(0xffffffffu, sum);
+}
+
+// run_base[block * 8 + w]: the values of the block before warp w's run
+__global__ void __launch_bounds__(SC_WARPS * 32)
+    k_scan_sums(ScanIn in, long long n, int rounds, uint32_t* __restrict__ run_base, uint32_t* __restrict__ block_sum) {
+  __shared__ uint32_t sw[SC_WARPS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long run = (long long)blockIdx.x * SC_WARPS + w;
+  const long long at = run * rounds * 128 + lane * 4;
+  const uint32_t sum = in.narrow() ? scan_run_sum<true>(in, at, n, rounds) : scan_run_sum<false>(in, at, n, rounds);
+  if (lane == 0) sw[w] = sum;
+  __syncthreads();
+  uint32_t before = 0;
+  for (int k = 0; k < w; ++k) before += sw[k];
+  if (lane == 0) run_base[run] = before;
+  if (w == SC_WARPS - 1 && lane == 0) block_sum[blockIdx.x] = before + sum;
+}
+
+template <bool HALF>
+__device__ __forceinline__ void scan_run(const ScanIn& in, uint32_t* d, long long at, long long n, int rounds,
+                                         uint32_t carry) {
+  for (int r = 0; r < rounds; r += 4) {
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = scan_load<HALF>(in, at + (long long)(r + k) * 128, n);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long i = at + (long long)(r + k) * 128;
+      const uint32_t sum = v[k].x + v[k].y + v[k].z + v[k].w;
+      const uint32_t inc = warp_incl_scan(sum);
+      const uint32_t b0 = carry + inc - sum, b1 = b0 + v[k].x, b2 = b1 + v[k].y, b3 = b2 + v[k].z;
+      carry += __shfl_sync(0xffffffffu, inc, 31);
+      if (i + 4 <= n) {
+        *reinterpret_cast<uint4*>(d + i) = make_uint4(b0, b1, b2, b3);
+      } else {
+        if (i < n) d[i] = b0;
+        if (i + 1 < n) d[i + 1] = b1;
+        if (i + 2 < n) d[i + 2] = b2;
       }
     }
-    if (lane == 0) {
-      sp_store(&status[tile], SP_P | (uint32_t)(prefix + agg));
-      prefix_sh = prefix;
-      if (total && tile == ntiles - 1) *total = prefix + agg;
-    }
   }
-  __syncthreads();
-  const uint32_t off = prefix_sh + woff;
-#pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const long long i = wb + ((long long)q * 32 + lane) * 4;
-    const uint32_t b0 = off + base[q], b1 = b0 + v[q].x, b2 = b1 + v[q].y, b3 = b2 + v[q].z;
-    if (vec) {
-      *reinterpret_cast<uint4*>(d + i) = make_uint4(b0, b1, b2, b3);
-    } else {
-      if (i < n) d[i] = b0;
-      if (i + 1 < n) d[i + 1] = b1;
-      if (i + 2 < n) d[i + 2] = b2;
-      if (i + 3 < n) d[i + 3] = b3;
-    }
-  }
+}
+
+// The blocks go backwards: what the sums read last is still in L2.  A lane
+// reads its four values before it writes them and no other lane touches them,
+// so d may be in.w.
+__global__ void __launch_bounds__(SC_WARPS * 32)
+    k_scan_apply(ScanIn in, uint32_t* d, long long n, int rounds, const uint32_t* __restrict__ run_base,
+                 const uint32_t* __restrict__ block_base) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b = gridDim.x - 1 - blockIdx.x;
+  const long long run = (long long)b * SC_WARPS + w;
+  const long long at = run * rounds * 128 + lane * 4;
+  const uint32_t base = block_base[b] + run_base[run];
+  if (in.narrow())
+    scan_run<true>(in, d, at, n, rounds, base);
+  else
+    scan_run<false>(in, d, at, n, rounds, base);
 }
 
 // --------------------------------------------------------------------------
@@ -493,33 +493,31 @@ __global__ void __launch_bounds__(SMALL_SORT / 2) k_sort_small(const K* __restri
 
 }  // namespace
 
-int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaStream_t st) {
+int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaStream_t st, const uint16_t* half,
+             const int* over) {
   if (n <= 0) {
     if (total) CSO_CUDA(cudaMemsetAsync(total, 0, sizeof(uint32_t), st));
     return CSO_OK;
   }
-  if (!ws.err) {
-    cso_set_error("scan without a device error word");
-    return CSO_ERR_STATE;
-  }
-  if (n <= SMALL_SCAN) {
+  if (n <= SMALL_SCAN && !half) {
     k_scan_small<<<CL(1), 1024, 0, st>>>(data, (int)n, total);
     CSO_CUDA(cudaGetLastError());
     return CSO_OK;
   }
-  const bool big = n > SP_BIG;
-  const long long ntiles = cdiv(n, big ? 1024 * 32 : 256 * 16);
-  size_t mark = ws.off;
-  unsigned long long* status = ws.get<unsigned long long>(ntiles + 1);
-  if (!status) {
+  // at most SMALL_SCAN blocks, so that one block scans their sums
+  const int rounds = 4 * (int)cdiv(n, (long long)SMALL_SCAN * SC_WARPS * 128 * 4);
+  const int nb = (int)cdiv(n, (long long)SC_WARPS * 128 * rounds);
+  const size_t mark = ws.off;
+  uint32_t* run_base = ws.get<uint32_t>((size_t)nb * SC_WARPS);
+  uint32_t* block_sum = ws.get<uint32_t>(nb);
+  if (!run_base || !block_sum) {
     cso_set_error("workspace exhausted in scan");
     return CSO_ERR_BUDGET;
   }
-  CSO_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (ntiles + 1), st));
-  if (big)
-    k_scan_onepass<1024, 32><<<CL((unsigned)ntiles), 1024, 0, st>>>(data, n, status, ntiles, total, ws.err);
-  else
-    k_scan_onepass<256, 16><<<CL((unsigned)ntiles), 256, 0, st>>>(data, n, status, ntiles, total, ws.err);
+  const ScanIn in{data, half, over};
+  k_scan_sums<<<CL(nb), SC_WARPS * 32, 0, st>>>(in, n, rounds, run_base, block_sum);
+  k_scan_small<<<CL(1), 1024, 0, st>>>(block_sum, nb, total);
+  k_scan_apply<<<CL(nb), SC_WARPS * 32, 0, st>>>(in, data, n, rounds, run_base, block_sum);
   CSO_CUDA(cudaGetLastError());
   ws.off = mark;
   return CSO_OK;
