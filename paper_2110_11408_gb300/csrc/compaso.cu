@@ -301,6 +301,15 @@ __device__ __forceinline__ int level_of(unsigned long long d) {
   return 2 * m + (int)((d >> (m - 1)) & 1);
 }
 
+// Boxes of runs of `per` tiles (a multiple of 32), for a block that looks over
+// more tiles than two a thread.  Every tile's box of a group of 1.9M members is
+// 470 KB out of L2, 5.6 us a look; through its 456 runs the look takes 3.1.
+constexpr int SUPERS = 512;
+struct SuperBoxes {
+  int lo[3][SUPERS], hi[3][SUPERS];
+  int n, per;  // n = 0: none
+};
+
 // The tiles a CTA owns: rank, rank + cs, ... of the group's nt (cs = 1 for a block).
 struct Tiles {
   int nt, rank, cs;
@@ -359,15 +368,31 @@ __device__ __forceinline__ void for_members(const Tiles& T, int n, unsigned long
 
 // The CTA's tiles nearer than lim, listed (T.nlist = -1 if they are too many):
 // one look at every box, which the passes that follow then need not repeat.
-__device__ void list_tiles(Tiles& T, unsigned long long lim, uint32_t* list, int* count) {
+__device__ __forceinline__ void list_tiles(Tiles& T, unsigned long long lim, uint32_t* list, int* count,
+                                           const SuperBoxes* sup = nullptr) {
   if (threadIdx.x == 0) *count = 0;
   __syncthreads();
-  const int own = T.own();
-  for (int i = threadIdx.x; i < own; i += blockDim.x) {
-    const int t = T.rank + i * T.cs;
-    if (tile_gap2(T, t) >= lim) continue;
+  const auto take = [&](int t) {
+    if (tile_gap2(T, t) >= lim) return;
     const int k = atomicAdd(count, 1);
     if (k < TILE_LIST) list[k] = (uint32_t)t;
+  };
+  if (sup && sup->n > 0) {
+    // a warp opens every 32nd run, so that neighbours spread over the warps
+    const SuperBoxes& B = *sup;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int s0 = threadIdx.x >> 5; s0 < B.n; s0 += 32 * nw) {
+      const int s = s0 + lane * nw;
+      const bool in = s < B.n && axis_gap2(T.q.x, B.lo[0][s], B.hi[0][s]) + axis_gap2(T.q.y, B.lo[1][s], B.hi[1][s]) +
+                                            axis_gap2(T.q.z, B.lo[2][s], B.hi[2][s]) < lim;
+      for (unsigned m = __ballot_sync(0xffffffffu, in); m; m &= m - 1) {
+        const int first = (s0 + (__ffs(m) - 1) * nw) * B.per;
+        for (int t = first + lane; t < min(first + B.per, T.nt); t += 32) take(t);
+      }
+    }
+  } else {
+    const int own = T.own();
+    for (int i = threadIdx.x; i < own; i += blockDim.x) take(T.rank + i * T.cs);
   }
   __syncthreads();
   const int k = *count;
@@ -664,6 +689,119 @@ __device__ __forceinline__ unsigned long long try_bound(int k, const PredConst& 
 
 // ---------------------------------------------------------------------------
 // the choice of the next nucleus among a group's peaks
+// A try over so few tiles that every lane holds its members' distances: H tiles
+// a warp.  For the nuclei of the 16-CTA clusters, which are chosen one after the
+// other and mostly end in the first try, 25 tiles: 11.8 -> 7.5 us a try, and with
+// the runs above level 2 of the uneven groups (1.9M members in the largest, 193
+// nuclei) 4.96 -> 3.31 ms.  The smaller tiers gain nothing by it (8-CTA clusters
+// 0.334 -> 0.342 ms, blocks 0.197 -> 0.210: their tries are over fewer tiles or
+// the registers are missed) and stay on r_search.
+// r_search's select with one histogram over the window below lim, without its
+// second pass over memory and its sort: the members are put in bin order, and
+// each one of a bin that may hold the answer counts the nearer ones of its bin,
+// all bins at once.  R^2, -1 if nothing below lim qualifies, or -2 if the answer
+// may lie in or behind a bin of more than HELD_BIN members or past the list.
+constexpr int HELD = 2;
+constexpr unsigned HELD_BIN = 128;
+
+template <int NT>
+__device__ __forceinline__ bool held_fits(const Tiles& T) {
+  return T.nlist >= 0 && T.nlist <= HELD * (NT / 32);
+}
+
+template <int NT>
+__device__ long long held_search(const int4* __restrict__ epos, int n, int4 pc, const PredConst& c, SelShared& S, int nb,
+                                 const Tiles& T, unsigned long long lim) {
+  constexpr int per = NB / NT, H = HELD, TL = TILE / 32;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const float scale0 = bin_scale(n, lim, c, nb);
+  const Window W{0, lim - 1, 0, 0};
+  unsigned long long d[H][TL];  // ~0: none
+  unsigned at[H][TL];           // arrival in its bin << 10 | bin
+  static_assert(NB <= 1024 && H * NT * TL <= 1 << 21, "packed");
+#pragma unroll
+  for (int q = 0; q < per; ++q) S.cnt[tid * per + q] = 0;
+  if (tid == 0) {
+    S.best = NB;
+    S.lo = ~0ull;
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int i = w + h * (NT / 32);
+    const int t = i < T.nlist ? (int)T.list[i] : -1;
+#pragma unroll
+    for (int k = 0; k < TL; ++k) {
+      const int j = t * TILE + k * 32 + lane;
+      d[h][k] = t >= 0 && j < n ? (unsigned long long)dist2(pc, epos[j]) : ~0ull;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int k = 0; k < TL; ++k)
+      if (d[h][k] < lim) {
+        const int b = window_bin(W, d[h][k], c, scale0, nb);
+        at[h][k] = atomicAdd(&S.cnt[b], 1u) << 10 | (unsigned)b;
+      }
+  __syncthreads();
+  unsigned loc[per], sum = 0;
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    loc[q] = S.cnt[tid * per + q];
+    sum += loc[q];
+  }
+  unsigned first;
+  block_scan<NT>(sum, first, S.sw);
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int b = tid * per + q;
+    // could a member of the bin qualify?
+    bool ok = loc[q] && pred(first, bin_top(W, b, c, scale0, nb, W.whi), c);
+    if (ok && (loc[q] > HELD_BIN || first + loc[q] > CAP)) {
+      atomicMin(&S.best, b);
+      ok = false;
+    }
+    S.clo[b] = first | (ok ? 1u << 31 : 0u);
+    first += loc[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int k = 0; k < TL; ++k)
+      if (d[h][k] < lim) {
+        const unsigned f = S.clo[at[h][k] & 1023u];
+        if (f >> 31) S.list[(f & 0x7fffffffu) + (at[h][k] >> 10)] = (long long)d[h][k];
+      }
+  __syncthreads();
+  unsigned long long mine = ~0ull;
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int k = 0; k < TL; ++k)
+      if (d[h][k] < lim) {
+        const unsigned b = at[h][k] & 1023u, f = S.clo[b];
+        if (!(f >> 31) || d[h][k] >= mine) continue;
+        const unsigned lo = f & 0x7fffffffu, hi = lo + S.cnt[b];
+        unsigned nearer = lo;
+        for (unsigned j = lo; j < hi; ++j) nearer += S.list[j] < (long long)d[h][k];
+        if (pred(nearer, d[h][k], c)) mine = d[h][k];
+      }
+  if (__any_sync(0xffffffffu, mine != ~0ull)) {
+    mine = ~warp_max_u64(~mine);
+    if (lane == 0) atomicMin(&S.lo, mine);
+  }
+  __syncthreads();
+  const unsigned long long r = S.lo;
+  const int big = S.best;
+  if (big < NB && (r == ~0ull || window_bin(W, r, c, scale0, nb) > big)) {
+    __syncthreads();  // the search that follows clears the shared words
+    return -2;
+  }
+  return r == ~0ull ? -1 : (long long)r;
+}
+
 // ---------------------------------------------------------------------------
 struct Best {
   long long sig;
@@ -749,6 +887,33 @@ __device__ __forceinline__ Tiles group_tiles(const LevelArgs& a, int seg, unsign
   // at most n / TILE + 1 of them
   const size_t at = base / TILE + (size_t)seg;
   return Tiles{(n + TILE - 1) / TILE, rank, cs, a.tlo + at, a.thi + at, make_int4(0, 0, 0, 0), nullptr, -1};
+}
+
+// the runs' boxes from the tiles' (complete and visible to the block)
+__device__ void super_boxes(const Tiles& T, SuperBoxes& B) {
+  const int per = 32 * ((T.nt + 32 * SUPERS - 1) / (32 * SUPERS));
+  const int ns = T.nt <= 2 * (int)blockDim.x ? 0 : (T.nt + per - 1) / per;
+  if (threadIdx.x == 0) {
+    B.n = ns;
+    B.per = per;
+  }
+  const int lane = threadIdx.x & 31;
+  for (int s = threadIdx.x >> 5; s < ns; s += blockDim.x >> 5) {
+    int a[3] = {INT_MAX, INT_MAX, INT_MAX}, b[3] = {INT_MIN, INT_MIN, INT_MIN};
+    for (int t = s * per + lane; t < min((s + 1) * per, T.nt); t += 32) {
+      const int4 l = T.lo[t], h = T.hi[t];
+      a[0] = min(a[0], l.x), a[1] = min(a[1], l.y), a[2] = min(a[2], l.z);
+      b[0] = max(b[0], h.x), b[1] = max(b[1], h.y), b[2] = max(b[2], h.z);
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      a[x] = __reduce_min_sync(0xffffffffu, a[x]);
+      b[x] = __reduce_max_sync(0xffffffffu, b[x]);
+    }
+    if (lane == 0)
+      for (int x = 0; x < 3; ++x) B.lo[x][s] = a[x], B.hi[x][s] = b[x];
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ int4 tile_origin(const int4* epos, int4 pc) {
@@ -1171,10 +1336,12 @@ struct ClusterShared {
   PickShared K;
   uint32_t tiles[TILE_LIST];
   int ntiles;
+  SuperBoxes sup;
   unsigned h[LEVELS];
   int hbest;
 };
 
+template <int CS>
 __device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& B) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -1194,6 +1361,7 @@ __device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& 
   if (boxes) {
     tile_boxes(T, epos, n, a.tlo + (T.lo - a.tlo), a.thi + (T.hi - a.thi));
     cluster.sync();  // every CTA reads all boxes
+    if (CS == CL_HUGE_CS) super_boxes(T, B.sup);
   }
   unsigned long long gone = 0;
   int cur = next_nucleus(a, p0, m, -1, make_int4(0, 0, 0, 0), 0, gone, B.K);
@@ -1202,7 +1370,7 @@ __device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& 
     const int4 pc = a.peaks.pos[p0 + cur];
     long long R2 = -1;
     unsigned long long lim = 0;
-    bool tried = false;
+    bool tried = false, held = false;
     if (boxes && nn > 0) {
       T.q = tile_origin(epos, pc);
       if (private_flags(m)) {
@@ -1211,27 +1379,45 @@ __device__ void cluster_level(const LevelArgs& a, const int seg, ClusterShared& 
         // nuclei apart until the next search of the whole cluster, so a CTA
         // reads nothing here that another one writes on the way (distances,
         // flags and earlier radii are its own).
-        Tiles A = T;
-        A.rank = 0;
-        A.cs = 1;
+        T.rank = 0;
+        T.cs = 1;
         for (int k = 0; k < TRIES && R2 < 0; ++k) {
           const unsigned long long tl = try_bound(k, a.pc);
-          list_tiles(A, tl, B.tiles, &B.ntiles);
-          R2 = r_search<CL_NT>(epos, nullptr, n, pc, a.pc, B.S, 0, a.cap, a.nb, A, tl, false);
+          list_tiles(T, tl, B.tiles, &B.ntiles, CS == CL_HUGE_CS ? &B.sup : nullptr);
+          if (CS == CL_HUGE_CS && tl && held_fits<CL_NT>(T)) {
+            R2 = held_search<CL_NT>(epos, n, pc, a.pc, B.S, a.nb, T, tl);
+            held = R2 >= 0;
+            if (R2 != -2) continue;
+          }
+          R2 = r_search<CL_NT>(epos, nullptr, n, pc, a.pc, B.S, 0, a.cap, a.nb, T, tl, false);
         }
         tried = R2 >= 0;
+        T.rank = rank;
+        T.cs = cs;
       }
-      T.nlist = -1;
+      if (!held) T.nlist = -1;
       if (R2 < 0) lim = search_bound(T, n, a.pc, B.h, &B.hbest);
-      if (tried) list_tiles(T, (unsigned long long)R2, B.tiles, &B.ntiles);
+      if (tried && !held) list_tiles(T, (unsigned long long)R2, B.tiles, &B.ntiles);
       else if (lim) list_tiles(T, lim, B.tiles, &B.ntiles);
     }
     if (R2 < 0) R2 = cluster_r_search(cluster, epos, ed, n, T, pc, a.pc, B.S, B.C, a.cap, a.nb, lim);
     // steps 1 and 3 on this CTA's share of the members
-    for_members(T, n, boxes && nn > 0 ? (unsigned long long)R2 : 0, [&](int j) {
-      const long long d = tried ? dist2(pc, epos[j]) : ed[j];
-      if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
-    });
+    if (held) {
+      // this CTA's among the tiles that all of them listed
+      for (int i = tid >> 5; i < T.nlist; i += CL_NT / 32) {
+        const int t = (int)T.list[i];
+        if (t % cs == rank)
+          tile_members(t, n, [&](int j) {
+            const long long d = dist2(pc, epos[j]);
+            if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
+          });
+      }
+    } else {
+      for_members(T, n, boxes && nn > 0 ? (unsigned long long)R2 : 0, [&](int j) {
+        const long long d = tried ? dist2(pc, epos[j]) : ed[j];
+        if (d < R2) assign_member(a, base, eslot, edold, j, d, R2, nn);
+      });
+    }
     if (tid == 0) {  // every CTA: it reads the radii back in later assignments
       a.nuc_member[base + nn] = (uint32_t)pc.w;
       a.nuc_R2[base + nn] = R2;
@@ -1356,7 +1542,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(CL_NT)
     const unsigned it = *cluster.map_shared_rank(&item, 0);
     cluster.sync();  // every CTA has read the leader's item before it changes
     if (it >= cnt) return;
-    cluster_level(a, (int)order[first + it], B);
+    cluster_level<CS>(a, (int)order[first + it], B);
   }
 }
 
