@@ -670,18 +670,21 @@ __global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const i
 }
 
 // Pass one (in the spirit of Afforest, Sutton et al. 2018): each dense
-// particle tests the W = 16 slots after it in its cell, cyclically, so every
-// pair of a cell of up to 17 particles is tested and a big cell is joined by
-// a band of links around it (FoF of the side-256 box: 3.24 ms with W = 16, 3.31
-// with 32, 4.54 with 8, which leaves more stragglers).  The band joins almost every dense particle of
+// particle tests the W = 32 slots after it in its cell, cyclically, so every
+// pair of a cell of up to 33 particles is tested and a big cell is joined by
+// a band of links around it.  The band joins almost every dense particle of
 // a big cell into one tree; the few it misses are handled one by one later.
+// A narrower band gains 2% where it suffices (16: 3.24 against 3.31 ms on a
+// side-256 box) and costs 40% where it does not (16 on the benchmark's box of
+// that size: 4.64 against 3.30; 8 on the first: 4.54), by the cells whose trees
+// it leaves in pieces.
 //
 // A warp whose particles share a cell streams the union of its lanes'
 // windows through shared memory; the lane that stages a particle also stages
 // its current root (-1 if not dense), so a lane pays a forest update only for
 // a link into another tree.  A staged root that has since been hooked
 // elsewhere is still a member of its tree, so the test stays correct.
-constexpr uint32_t FOF_BAND = 16;
+constexpr uint32_t FOF_BAND = 32;
 
 __global__ void __launch_bounds__(256) k_fof_sample(CellGrid g, const int4* __restrict__ spos,
                                                     const int* __restrict__ didx, const uint32_t* __restrict__ nd_ptr,
@@ -1196,10 +1199,11 @@ int cells_check_dense(int nc) {
 
 // Tables from this size on count in 16 bits first: the clearing, the atomics and
 // the scan's two reads then move half the bytes.  Binning with a 262M-cell table
-// 2.13 -> 1.92 ms (2^24 particles), 0.87 -> 0.67 (2^20); with 34M cells 0.31 ->
+// 2.13 -> 1.92 ms (2^24 particles), 0.87 -> 0.67 (4M); with 34M cells 0.31 ->
 // 0.28.  At 2M to 4M cells the launches of the unused recount cost more than is
 // saved (0.039 -> 0.048 ms).
 static constexpr long long HALF_CELLS = 1ll << 24;
+static constexpr size_t HALF_ROOM = 1 << 20;  // left for the scan's sums: without it the count stays in 32 bits
 
 int cells_bin(const int32_t* pos, const uint64_t* ids, long long n, const CellGrid& g, uint32_t* start,
               int4* spos, uint64_t* sid, int* bad, Workspace& ws, cudaStream_t st, uint32_t* inv) {
@@ -1217,7 +1221,7 @@ int cells_bin(const int32_t* pos, const uint64_t* ids, long long n, const CellGr
     return CSO_ERR_BUDGET;
   }
   const size_t half_bytes = sizeof(uint16_t) * ((size_t)ncell + 8) / 16 * 16;
-  if (n > 0 && ncell + 1 >= HALF_CELLS && ws.off + half_bytes + 512 <= ws.cap) {
+  if (n > 0 && ncell + 1 >= HALF_CELLS && ws.off + half_bytes + HALF_ROOM <= ws.cap) {
     const size_t mark_half = ws.off;
     uint32_t* half = reinterpret_cast<uint32_t*>(ws.get<char>(half_bytes + sizeof(int)));
     int* over = reinterpret_cast<int*>(reinterpret_cast<char*>(half) + half_bytes);
