@@ -9,10 +9,12 @@
 //   select  R^2 = the smallest member distance d with n(<d)^2 u^6 < K d^3
 //           (exact), found without a full sort: a 1024-bin histogram over a
 //           window of d (first window binned by the threshold count
-//           sqrt(K) d^1.5 / u^3, later windows linearly), the first bin that
-//           could hold the answer (its interior count at its largest d) is
-//           sorted in shared memory and scanned, or narrowed further when it
-//           holds more than 2048 members; small groups are sorted whole;
+//           sqrt(K) d^1.5 / u^3, later windows linearly), the bins from the
+//           first that could hold the answer on (by its interior count at its
+//           largest d) are gathered into shared memory, up to 256 members, and
+//           each counts the nearer ones; a larger bin alone is sorted and
+//           scanned, or narrowed further when it holds more than 2048 members;
+//           small groups are counted or sorted whole;
 //   pass B  tentative membership / competitive reassignment (Eq. 3) and
 //           eligibility of the peaks left.
 //

@@ -43,8 +43,8 @@ struct LevelArgs {
 
 // size bins of the batched schedule: groups above `giant` members run on an
 // 8-CTA thread-block cluster, groups above large() on a 1024-thread block,
-// groups up to `small` members on one warp, the rest on a 256-thread block;
-// largest first within each bin
+// groups up to `small` members on one warp, up to 512 on a 128-thread block, the
+// rest on a 256-thread block; largest first within each bin
 struct LevelSchedule {
   int giant = 16384;
   int small = 64;
