@@ -56,7 +56,9 @@ extern "C" {
  * launch sizes are read back from the device between stages) */
 #define CSO_FLAG_GRAPH 4u
 #define CSO_FLAG_COUNT_PAIRS 8u /* count kernel pairs with d < b2 (cso_last_stats[6]); slows the density pass */
-#define CSO_FLAG_SELECT_STRESS 16u /* testing: tiny radius-search tiles so every select branch runs; same results */
+/* testing: tiny radius-search tiles so every select branch runs, and look-backs
+ * that do not wait for an earlier tile but count it themselves; same results */
+#define CSO_FLAG_SELECT_STRESS 16u
 /* threshold-radius search by the paper's radial bins (Sec. 2.3.4): members
  * are binned outward in steps of sqrt(3)/3 cell sides and a bin is skipped
  * while the members inside it, placed at its outer edge, still meet the

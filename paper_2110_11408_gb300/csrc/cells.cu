@@ -607,6 +607,17 @@ __device__ __forceinline__ uint32_t cell_id(const CellGrid& g, int4 p) {
 // holds any.  counts[0] and counts[1] receive their lengths.  (A pass each
 // for the flags, their scans and the lists: 0.39 ms on the side-256 box, this
 // one 0.16.)
+
+// dense slot i is the first one of its cell: no dense slot before it there (the
+// one next to it, mostly)
+__device__ __forceinline__ bool first_dense(const CellGrid& g, const int4* __restrict__ spos,
+                                            const long long* __restrict__ sigma, long long T_L0, long long i) {
+  const uint32_t c = cell_id(g, spos[i]);
+  for (long long t = i - 1; t >= 0 && cell_id(g, spos[t]) == c; --t)
+    if (sigma[t] > T_L0) return false;
+  return true;
+}
+
 template <int ITEMS>
 __global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const int4* __restrict__ spos, int n,
                                                           const long long* __restrict__ sigma, long long T_L0,
@@ -615,7 +626,7 @@ __global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const i
                                                           int* __restrict__ didx, int* __restrict__ clist,
                                                           uint32_t* __restrict__ counts,
                                                           unsigned long long* __restrict__ status, long long ntiles,
-                                                          int* __restrict__ err) {
+                                                          long long patience) {
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -636,24 +647,17 @@ __global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const i
   uint32_t na = 0, nb = 0;
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
-    bool h = false;
-    if (dense[q] >> lane & 1u) {
-      // first of its cell: no dense slot before it there (the one next to it, mostly)
-      const long long i = base + q * 32 + lane;
-      const uint32_t c = cell_id(g, spos[i]);
-      h = true;
-      for (long long t = i - 1; t >= 0 && cell_id(g, spos[t]) == c; --t)
-        if (sigma[t] > T_L0) {
-          h = false;
-          break;
-        }
-    }
+    const bool h = (dense[q] >> lane & 1u) && first_dense(g, spos, sigma, T_L0, base + q * 32 + lane);
     head[q] = __ballot_sync(0xffffffffu, h);
     na += __popc(dense[q]);
     nb += __popc(head[q]);
   }
   uint32_t ta, tb;
-  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  rank2_prefix(S, status, tile, na, nb, ta, tb, patience, [&](long long t) {
+    return rank2_count<ITEMS>(t, [&](long long i) {
+      return sigma[i] > T_L0 ? 1u | (first_dense(g, spos, sigma, T_L0, i) ? 2u : 0u) : 0u;
+    });
+  });
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
@@ -784,7 +788,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
                                                            uint8_t* __restrict__ strag, int* __restrict__ slist,
                                                            uint2* __restrict__ srange,
                                                            unsigned long long* __restrict__ status, long long ntiles,
-                                                           int* __restrict__ err) {
+                                                           long long patience) {
   __shared__ Rank2Shared S;
   const long long nd = counts[0];
   const long long tile = rank2_tile(S, status, ntiles);
@@ -792,7 +796,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long base = tile * (R2_THREADS * ITEMS) + (long long)w * 32 * ITEMS;
   unsigned flag[ITEMS];
-  uint32_t lo[ITEMS];  // the cell's first slot; top bits: first and last dense particle of the cell
+  uint32_t lo[ITEMS];  // the cell's first slot
   unsigned first = 0, last = 0;
   uint32_t na = 0, nb = 0;
 #pragma unroll
@@ -825,7 +829,13 @@ __global__ void __launch_bounds__(R2_THREADS) k_stragglers(const int4* __restric
     na += __popc(flag[q]);
   }
   uint32_t ta, tb;
-  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  // (roots do not change in this pass, so a tile counted here counts as it does itself)
+  rank2_prefix(S, status, tile, na, nb, ta, tb, patience, [&](long long t) {
+    return rank2_count<ITEMS>(t, [&](long long i) {
+      const int s = didx[i];
+      return uf_root(parent, s) != cell_root[g.start[cell_id(g, spos[s])]] ? 1u : 0u;
+    });
+  });
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
@@ -1321,23 +1331,19 @@ int cells_fof(const CellGrid& g, const int4* spos, int n, const long long* sigma
     cso_set_error("workspace exhausted in the FoF pass");
     return CSO_ERR_BUDGET;
   }
-  if (!ws.err) {
-    cso_set_error("FoF lists without a device error word");
-    return CSO_ERR_STATE;
-  }
   uint32_t* counts = reinterpret_cast<uint32_t*>(status + 2 * words);
   const long long tiles = rank2_tiles(n);
   CSO_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)(2 * words + 2), st));
   // launches over the lists are sized by n and blocks past the counts (read
   // on the device) return at once
   RANK2_LAUNCH(k_fof_lists, n, st, g, spos, n, sigma, T_L0, parent, cell_root, minid, didx, clist, counts, status, tiles,
-               ws.err);
+               ws.patience);
   const uint32_t *nd = counts, *ncl = counts + 1, *ns = counts + 2;
   // pass one: bands inside cells; main trees and stragglers
   k_fof_sample<<<CL(cdiv(n, 256)), 256, 0, st>>>(g, spos, didx, nd, lfof2, parent);
   k_cell_main<<<CL(cdiv(n, 256)), 256, 0, st>>>(spos, g, clist, ncl, parent, cell_root);
   RANK2_LAUNCH(k_stragglers, n, st, spos, g, didx, counts, parent, cell_root, strag, slist, srange, status + words, tiles,
-               ws.err);
+               ws.patience);
   // pass two: main trees of adjacent cells; pass three: stragglers
   const int lreach = reach_below(lfof2);
   k_fof_cells<<<CL(cso_sm_count() * 8), 256, 0, st>>>(g, spos, clist, ncl, lfof2, lreach, parent, cell_root, strag);

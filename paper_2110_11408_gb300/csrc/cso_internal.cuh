@@ -41,6 +41,13 @@ static inline T CL(T grid) {
   return grid;
 }
 
+// A tile of a look-back (scan_sort.cu, rank2.cuh) reads an earlier tile's status
+// word at most this often before it counts that tile's elements itself.  The
+// result does not depend on it: a wait ends with the right counts, whether the
+// earlier tile runs or not.  Far above the microseconds between two tiles, so that
+// nothing is counted twice in an ordinary run.
+constexpr long long LOOKBACK_PATIENCE = 1ll << 22;
+
 // ---------------------------------------------------------------------------
 // workspace: bump allocator over one device buffer owned by the context
 // ---------------------------------------------------------------------------
@@ -51,7 +58,7 @@ struct Workspace {
   size_t peak = 0;
   size_t need = 0;  // bytes requested during a sizing pass
   bool sizing = false;
-  int* err = nullptr;  // device word set by a kernel whose bounded wait gave up (CSO_ERR_TIMEOUT)
+  long long patience = LOOKBACK_PATIENCE;
   void* take(size_t bytes) {
     size_t o = (off + 255) & ~size_t(255);
     off = o + bytes;

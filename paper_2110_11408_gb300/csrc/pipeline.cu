@@ -30,11 +30,11 @@ constexpr unsigned long long NONE = ~0ull;
 // every group at its root (groups in the order of their roots); the numbers of
 // both go to meta.
 template <int ITEMS>
-__global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restrict__ root, int n,
+__global__ void __launch_bounds__(R2_THREADS, 5) k_member_list(const int* __restrict__ root, int n,
                                                             const uint8_t* __restrict__ select,
                                                             uint32_t* __restrict__ dl, uint32_t* __restrict__ gidx,
                                                             unsigned long long* __restrict__ status, long long ntiles,
-                                                            Meta* meta) {
+                                                            long long patience, Meta* meta) {
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -52,7 +52,12 @@ __global__ void __launch_bounds__(R2_THREADS) k_member_list(const int* __restric
     nb += __popc(head[q]);
   }
   uint32_t ta, tb;
-  rank2_prefix(S, status, tile, na, nb, ta, tb, &meta->timeout);
+  rank2_prefix(S, status, tile, na, nb, ta, tb, patience, [&](long long t) {
+    return rank2_count<ITEMS>(t, [&](long long i) {
+      const int r = root[i];
+      return r >= 0 && (!select || select[i]) ? 1u | (r == (int)i ? 2u : 0u) : 0u;
+    });
+  });
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
@@ -125,7 +130,7 @@ __global__ void k_gather_pos(const uint32_t* __restrict__ gs, int nd, const int4
 // on the device by cell-sorted index and (optional) in input order.  The
 // number of members goes to *total.
 template <int ITEMS>
-__global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restrict__ eslot,
+__global__ void __launch_bounds__(R2_THREADS, 6) k_assigned_list(const int* __restrict__ eslot,
                                                               const uint32_t* __restrict__ grp,
                                                               const uint32_t* __restrict__ hbase,
                                                               const uint32_t* __restrict__ seg_off,
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restr
                                                               int* __restrict__ lab1, uint64_t* __restrict__ ol1,
                                                               unsigned long long* __restrict__ status,
                                                               long long ntiles, uint32_t* __restrict__ total,
-                                                              int* __restrict__ err) {
+                                                              long long patience) {
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -153,7 +158,9 @@ __global__ void __launch_bounds__(R2_THREADS) k_assigned_list(const int* __restr
     na += __popc(in[q]);
   }
   uint32_t ta, tb;
-  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  rank2_prefix(S, status, tile, na, nb, ta, tb, patience, [&](long long t) {
+    return rank2_count<ITEMS>(t, [&](long long k) { return eslot[k] >= 0 ? 1u : 0u; });
+  });
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
     const long long k = base + q * 32 + lane;
@@ -351,7 +358,7 @@ __global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* _
                                                                uint64_t* __restrict__ key, uint32_t* __restrict__ val,
                                                                unsigned long long* __restrict__ status,
                                                                long long ntiles, uint32_t* __restrict__ total,
-                                                               int* __restrict__ err) {
+                                                               long long patience) {
   __shared__ Rank2Shared S;
   const long long tile = rank2_tile(S, status, ntiles);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -365,7 +372,9 @@ __global__ void __launch_bounds__(R2_THREADS) k_catalogue_list(const cso_halo* _
     na += __popc(in[q]);
   }
   uint32_t ta, tb;
-  rank2_prefix(S, status, tile, na, nb, ta, tb, err);
+  rank2_prefix(S, status, tile, na, nb, ta, tb, patience, [&](long long t) {
+    return rank2_count<ITEMS>(t, [&](long long h) { return keep[h] ? 1u : 0u; });
+  });
 #pragma unroll
   for (int q = 0; q < ITEMS; ++q) {
     const long long h = base + q * 32 + lane;
@@ -474,7 +483,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   ALLOC(uint32_t, dl, n);
   ALLOC(uint32_t, gidx, n);
   ALLOC(uint32_t, grp, n);
-  RANK2_LAUNCH(k_member_list, n, st, root, N, gi.select, dl, gidx, rstat, rank2_tiles(n), meta);
+  RANK2_LAUNCH(k_member_list, n, st, root, N, gi.select, dl, gidx, rstat, rank2_tiles(n), ws.patience, meta);
   k_member_group<<<G1(n)>>>(dl, root, gidx, sigma, sid, grp, meta);
   CSO_CUDA(cudaGetLastError());
   // counters: dense particles, groups, sigma_max, id_max, bad
@@ -486,10 +495,6 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   if (hm.bad) {
     cso_set_error("positions outside [0, 2^21)");
     return CSO_ERR_ARG;
-  }
-  if (hm.timeout) {
-    cso_set_error("a bounded device wait gave up");
-    return CSO_ERR_TIMEOUT;
   }
   c->stats[1] = nd;
   c->stats[2] = G;
@@ -576,7 +581,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   uint32_t* ehal2 = akey;  // its L1 halo, ascending
   if (nd > 0) {
     RANK2_LAUNCH(k_assigned_list, (long long)nd, st, eslot, gseg, hbase, seg1, nucm, nd, gs, epos, sid, akey, aval, lab1, ol1,
-                 rstat + words, rank2_tiles(nd), hbase + G + 1, ws.err);
+                 rstat + words, rank2_tiles(nd), hbase + G + 1, ws.patience);
   } else {
     CSO_CUDA(cudaMemsetAsync(hbase + G + 1, 0, sizeof(uint32_t), st));
   }
@@ -691,7 +696,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
     ALLOC(uint64_t, ckey, H1);
     ALLOC(uint32_t, cval, H1);
     RANK2_LAUNCH(k_catalogue_list, (long long)H1, st, rows, keep, H1, ckey, cval, rstat + 2 * words, rank2_tiles(H1),
-                 keep + H1, ws.err);
+                 keep + H1, ws.patience);
     CSO_CUDA(cudaGetLastError());
     CSO_TRY(readback(c, keep + H1, 4));
     nrows = (int)((uint32_t*)c->pinned)[0];
@@ -764,7 +769,6 @@ int pipeline_run(cso_ctx* c, const cso_input* in, const cso_params* p, cso_outpu
   }
   ALLOC(Meta, meta, 1);
   CSO_CUDA(cudaMemsetAsync(meta, 0, sizeof(Meta), st));
-  ws.err = &meta->timeout;
 
   // ---- bin ----
   S.mark("bin");
@@ -869,10 +873,6 @@ int pipeline_run(cso_ctx* c, const cso_input* in, const cso_params* p, cso_outpu
   c->stats[9] = (int64_t)ws.peak;
   c->stats[10] = g_cso_launches - launches0;
 #undef ALLOC
-  if (hm.timeout) {
-    cso_set_error("a bounded device wait gave up");
-    return CSO_ERR_TIMEOUT;
-  }
   if (nrows > out->halo_cap) {
     cso_set_error("catalogue has %d rows, halo_cap is %lld", nrows, (long long)out->halo_cap);
     return CSO_ERR_CAPACITY;

@@ -72,7 +72,6 @@ struct Meta {  // device counters read back by the host
   unsigned long long pairs, work1, work2;
   unsigned n_dense, n_groups;  // particles and groups taking part
   int bad;
-  int timeout;  // a bounded device wait gave up (Workspace::err points here)
 };
 
 // dense particles taking part (all, or those of selected groups) and group roots

@@ -45,13 +45,29 @@ __device__ __forceinline__ long long rank2_tile(Rank2Shared& S, unsigned long lo
   return S.tile;
 }
 
+// Both counts of a whole tile from its elements, by the calling warp: flags(i) has
+// bit 0 set if element i is in the first set, bit 1 if it is in the second.
+template <int ITEMS, class F>
+__device__ __forceinline__ uint2 rank2_count(long long tile, F flags) {
+  const long long base = tile * (R2_THREADS * ITEMS) + (threadIdx.x & 31);
+  uint2 c = make_uint2(0, 0);
+#pragma unroll 1
+  for (int q = 0; q < R2_THREADS * ITEMS; q += 32) {
+    const unsigned f = flags(base + q);
+    c.x += __popc(__ballot_sync(0xffffffffu, f & 1u));
+    c.y += __popc(__ballot_sync(0xffffffffu, f & 2u));
+  }
+  return c;
+}
+
 // wa, wb: the calling warp's counts (the same on every lane).  On return they
 // are the numbers of flagged elements before the warp's first one; ta, tb the
-// inclusive totals up to the end of this tile.
+// inclusive totals up to the end of this tile.  recount(t), called by one warp,
+// gives both counts of the whole tile t < tile (rank2_count).
+template <class R>
 __device__ __forceinline__ void rank2_prefix(Rank2Shared& S, unsigned long long* status, long long tile, uint32_t& wa,
-                                             uint32_t& wb, uint32_t& ta, uint32_t& tb, int* err) {
+                                             uint32_t& wb, uint32_t& ta, uint32_t& tb, long long patience, R recount) {
   constexpr unsigned long long M31 = (1ull << 31) - 1;
-  constexpr long long SPIN_LIMIT = 1ll << 22;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (lane == 0) {
     S.wa[w] = wa;
@@ -87,10 +103,13 @@ __device__ __forceinline__ void rank2_prefix(Rank2Shared& S, unsigned long long*
         const int first = pmask ? __ffs(pmask) - 1 : 31;
         const unsigned need = first == 31 ? 0xffffffffu : (2u << first) - 1u;
         if (xmask & need) {  // a predecessor has not published yet
-          if (++spins > SPIN_LIMIT) {
-            if (lane == 0) atomicExch(err, 1);
-            break;
-          }
+          if (spins++ < patience) continue;
+          // count the nearest such tile here and go on behind it
+          const int q = __ffs(xmask & need) - 1;
+          const uint2 c = recount(top - q);
+          pa += c.x + __reduce_add_sync(0xffffffffu, lane < q ? (uint32_t)(v >> 31 & M31) : 0u);
+          pb += c.y + __reduce_add_sync(0xffffffffu, lane < q ? (uint32_t)(v & M31) : 0u);
+          top -= q + 1;
           continue;
         }
         pa += __reduce_add_sync(0xffffffffu, lane <= first ? (uint32_t)(v >> 31 & M31) : 0u);

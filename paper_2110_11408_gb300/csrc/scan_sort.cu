@@ -45,10 +45,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* smem_w
 
 // Look-back status words of the one-sweep sort (the decoupled look-back of
 // Merrill and Garland, "Single-pass Parallel Prefix Scan with Decoupled
-// Look-back", 2016): flag << 32 | value.
-constexpr unsigned long long SP_A = 1ull << 32, SP_P = 2ull << 32;
-constexpr long long SP_SPIN_LIMIT = 1ll << 22;
-
+// Look-back", 2016).
 __device__ __forceinline__ unsigned long long sp_load(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -276,7 +273,6 @@ constexpr int OS_THREADS = 256;
 constexpr int OS_WARPS = OS_THREADS / 32;
 constexpr int OS_RADIX = 256;
 constexpr int OS_MAX_PASSES = 8;
-constexpr long long OS_SPIN_LIMIT = 1ll << 22;
 constexpr int OS_LB = 8;  // predecessors read per look-back round trip
 
 template <class K>
@@ -321,7 +317,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_os_pass(const K* __restrict__
                                                       K* __restrict__ kout, uint32_t* __restrict__ vout, long long n,
                                                       int pass, const uint32_t* __restrict__ gbase,
                                                       unsigned long long* __restrict__ status,
-                                                      unsigned* __restrict__ ctr, int* __restrict__ err) {
+                                                      unsigned* __restrict__ ctr, long long patience) {
   constexpr int ITEMS = OsItems<K>::v;
   constexpr int TILE = OS_THREADS * ITEMS;
   __shared__ K skey[TILE];
@@ -388,7 +384,8 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_os_pass(const K* __restrict__
   }
   // decoupled look-back over the earlier tiles' counts of digit d: OS_LB
   // predecessors per round trip, nearest first, adding counts up to the first
-  // inclusive prefix; a predecessor that has not published yet is read again
+  // inclusive prefix; a predecessor that has not published yet is read again,
+  // and counted here when the patience is used up
   uint32_t excl = 0;
   if (tile > 0) {
     long long j = tile - 1, spins = 0;
@@ -412,9 +409,13 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_os_pass(const K* __restrict__
       }
       if (done) break;
       j -= used;
-      if (wait && ++spins > OS_SPIN_LIMIT) {
-        atomicExch(err, 1);
-        break;  // excl stays below the true prefix: every write stays in range
+      if (wait && spins++ >= patience) {
+        const K* at = kin + j * TILE;
+        uint32_t c = 0;
+#pragma unroll 1
+        for (int e = 0; e < TILE; ++e) c += ((uint32_t)(at[e] >> shift) & 255u) == (uint32_t)d;
+        excl += c;
+        --j;
       }
     }
   }
@@ -528,10 +529,6 @@ int scan_u32(uint32_t* data, long long n, uint32_t* total, Workspace& ws, cudaSt
 template <class K>
 static int onesweep(K** key, uint32_t** val, K* key_alt, uint32_t* val_alt, long long n, int bits, Workspace& ws,
                     cudaStream_t st) {
-  if (!ws.err) {
-    cso_set_error("sort without a device error word");
-    return CSO_ERR_STATE;
-  }
   if (n <= SMALL_SORT) {
     int m = 2;
     while (m < n) m <<= 1;
@@ -561,7 +558,7 @@ static int onesweep(K** key, uint32_t** val, K* key_alt, uint32_t* val_alt, long
   for (int p = 0; p < passes; ++p) {
     k_os_pass<K><<<CL((unsigned)ntiles), OS_THREADS, 0, st>>>(*key, *val, key_alt, val_alt, n, p,
                                                                aux + (size_t)p * OS_RADIX, status,
-                                                               aux + (size_t)passes * OS_RADIX + p, ws.err);
+                                                               aux + (size_t)passes * OS_RADIX + p, ws.patience);
     K* t1 = *key;
     *key = key_alt;
     key_alt = t1;

@@ -411,7 +411,6 @@ int stream_step(cso_ctx* c, StreamState& S, const cso_input* in, cso_output* out
     ALLOC(Meta, meta, 1);
     // a window particle outside the window's columns sets meta->bad = 2
     CSO_CUDA(cudaMemsetAsync(meta, 0, sizeof(Meta), st));
-    ws.err = &meta->timeout;
     CSO_TRY(cells_bin(S.rpos[k], S.rid[k], NR, g, start, spos, sid, &meta->bad, ws, st));
 
     // ---- kernel sums of the columns that became final ----
@@ -468,15 +467,9 @@ int stream_step(cso_ctx* c, StreamState& S, const cso_input* in, cso_output* out
                                    S.ridx[k], S.rpos[o], S.rid[o], S.rsig[o], S.rflag[o], S.rslab[o], S.ridx[o]);
     CSO_CUDA(cudaGetLastError());
     CSO_CUDA(cudaMemcpyAsync(c->pinned, kscan + NR, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    CSO_CUDA(cudaMemcpyAsync((char*)c->pinned + 8, &meta->timeout, sizeof(int), cudaMemcpyDeviceToHost, st));
     CSO_CUDA(cudaStreamSynchronize(st));
     S.nr = *(uint32_t*)c->pinned;
     S.cur = o;
-    if (*(int*)((char*)c->pinned + 8)) {
-      cso_set_error("a bounded device wait gave up");
-      S.failed = true;
-      return CSO_ERR_TIMEOUT;
-    }
   }
   S.col_fin = fin;
 
