@@ -226,6 +226,7 @@ int ctx_reserve(cso_ctx* c, long long n, long long ncell, bool host_io) {
     cso_set_error("request needs %zu bytes of workspace, budget is %zu", need, c->budget);
     return CSO_ERR_BUDGET;
   }
+  served_fit(c, need);
   if (need > c->ws.cap) {
     if (c->ws.base) {
       CSO_CUDA(cudaStreamSynchronize(c->stream));

@@ -124,4 +124,7 @@ size_t workspace_bytes(long long n, long long ncell, bool host_io);
 int ctx_reserve(cso_ctx* c, long long n, long long ncell, bool host_io);
 int check_io(const cso_input* in, const cso_params* p, cso_output* out);
 void served_stop(cso_ctx* c);
+// room in the context's budget for `need` bytes of workspace beside what its
+// served path's pool keeps
+void served_fit(cso_ctx* c, size_t need);
 int pipeline_run(cso_ctx* c, const cso_input* in, const cso_params* p, cso_output* out);

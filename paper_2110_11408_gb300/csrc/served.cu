@@ -29,11 +29,29 @@ struct ServedState {
   std::unordered_map<uint64_t, StreamState*> streams;  // slab streams by request_id
   std::vector<std::thread> workers;
   cudaMemPool_t pool = nullptr;  // device memory of the slab streams
+  size_t budget = 0;  // of the context
   size_t in_use = 0;  // device bytes reserved by running requests
   bool stop = false;
 };
 
 constexpr uint64_t POOL_KEEP = 1ull << 30;
+
+// Freed memory that the pool keeps gives way to `need` bytes of running requests:
+// both fit the budget together, as they did when a stream's memory was freed with it.
+static void pool_fit(const ServedState& S, size_t need) {
+  if (S.budget == 0) return;
+  uint64_t held = 0, used = 0;
+  if (cudaMemPoolGetAttribute(S.pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+      cudaMemPoolGetAttribute(S.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+      need + (size_t)(held - used) > S.budget)
+    CSO_CUDA_VOID(cudaMemPoolTrimTo(S.pool, 0));
+}
+
+void served_fit(cso_ctx* c, size_t need) {
+  if (!c->served) return;
+  std::lock_guard<std::mutex> lock(c->served->mu);
+  pool_fit(*c->served, need);
+}
 
 static double now_s() {
   using namespace std::chrono;
@@ -130,6 +148,10 @@ static void run_slab(cso_ctx* slot, ServedState& S, ServedRequest* r) {
       S.streams.erase(ss->id);
       stream_release(ss, slot->stream);
       ss = nullptr;
+      if (S.budget) {  // (the stream's memory can only go once it is freed)
+        CSO_CUDA_VOID(cudaStreamSynchronize(slot->stream));
+        pool_fit(S, S.in_use);
+      }
     }
   }
   if (ss) ss->busy = false;
@@ -148,6 +170,7 @@ static void worker_loop(cso_ctx* parent, int k) {
       r = *it;
       S.queue.erase(it);
       S.in_use += r->need;
+      pool_fit(S, S.in_use);
       r->t_start = now_s();
       if (is_slab(r)) {
         auto st = S.streams.find(r->in.request_id);
@@ -183,15 +206,17 @@ static int served_start(cso_ctx* c) {
   if (c->served) return CSO_OK;
   ServedState* S = new ServedState();
   c->served = S;
+  S->budget = c->budget;
   // the slab streams' memory: a pool of this context's own, which keeps at
-  // most POOL_KEEP bytes that no stream uses and goes with the context
+  // most POOL_KEEP bytes that no stream uses (within a budget only what the
+  // running requests leave of it) and goes with the context
   CSO_CUDA(cudaSetDevice(c->device));
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = c->device;
   CSO_CUDA(cudaMemPoolCreate(&S->pool, &props));
-  uint64_t keep = POOL_KEEP;
+  uint64_t keep = c->budget && c->budget < POOL_KEEP ? c->budget : POOL_KEEP;
   CSO_CUDA(cudaMemPoolSetAttribute(S->pool, cudaMemPoolAttrReleaseThreshold, &keep));
   const int nslots = c->served_slots > 0 ? c->served_slots : 4;
   for (int k = 0; k < nslots; ++k) {
