@@ -12,6 +12,7 @@
 #include <condition_variable>
 #include <deque>
 #include <mutex>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 
@@ -202,10 +203,7 @@ static void worker_loop(cso_ctx* parent, int k) {
   }
 }
 
-static int served_start(cso_ctx* c) {
-  if (c->served) return CSO_OK;
-  ServedState* S = new ServedState();
-  c->served = S;
+static int served_open(cso_ctx* c, ServedState* S) {
   S->budget = c->budget;
   // the slab streams' memory: a pool of this context's own, which keeps at
   // most POOL_KEEP bytes that no stream uses (within a budget only what the
@@ -225,8 +223,23 @@ static int served_start(cso_ctx* c) {
     if (rc != CSO_OK) return rc;
     S->slots.push_back(s);
   }
-  for (int k = 0; k < nslots; ++k) S->workers.emplace_back(worker_loop, c, k);
+  try {
+    for (int k = 0; k < nslots; ++k) S->workers.emplace_back(worker_loop, c, k);
+  } catch (const std::system_error& e) {
+    cso_set_error("cannot start a worker thread: %s", e.what());
+    return CSO_ERR_STATE;
+  }
   return CSO_OK;
+}
+
+// The first submit's pool, slots and workers: all of them, or none (the next
+// submit then tries again).
+static int served_start(cso_ctx* c) {
+  if (c->served) return CSO_OK;
+  c->served = new ServedState();
+  const int rc = served_open(c, c->served);
+  if (rc != CSO_OK) served_stop(c);
+  return rc;
 }
 
 void served_stop(cso_ctx* c) {
