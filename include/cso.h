@@ -249,17 +249,19 @@ void cso_free(cso_ctx* ctx);
  * under each candidate pair of size bins -- groups above `giant` members on
  * 8-CTA thread-block clusters (4096, 8192, 16384, 65536, 262144), groups of at most
  * `small` members one per warp (32, 64); groups above max(giant / 16, 512)
- * run on 1024-thread blocks and the rest on 256-thread blocks -- times the
- * CompaSO levels, and keeps the fastest pair in the context for every later
- * call.  Outputs are written as by cso_find_groups (identical for every
+ * run on 1024-thread blocks, the rest on 128-thread (up to 512 members) and
+ * 256-thread blocks -- times the CompaSO levels, and keeps the fastest pair in
+ * the context for every later call; the default schedule (cso_set_schedule) is
+ * the candidate 16384, 64.  Outputs are written as by cso_find_groups (identical for every
  * pair).  giant/small (may be NULL) receive the choice. */
 int cso_autotune(cso_ctx* ctx, const cso_input* in, const cso_params* p, cso_output* out, int32_t* giant,
                  int32_t* small);
 
 /* Set the batched schedule's size bins directly (giant >= 64, 1 <= small
- * <= 64); the defaults are 16384 and 64, and until this or the autotuner is
- * called only as many of the groups above 16384 go to clusters as clusters
- * run at a time (and those of 131072 or more). */
+ * <= 64).  The defaults are 16384 and 64; with this pair only as many of the
+ * groups above 16384 go to clusters as clusters run at a time (and those of
+ * 131072 or more), the others to 1024-thread blocks.  Any other pair is taken
+ * as it is. */
 int cso_set_schedule(cso_ctx* ctx, int32_t giant, int32_t small);
 
 /* Groups above max(huge, giant) members run on 16-CTA thread-block clusters

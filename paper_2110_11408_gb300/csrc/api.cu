@@ -260,7 +260,6 @@ extern "C" int cso_set_schedule(cso_ctx* c, int32_t giant, int32_t small) {
   }
   c->sched.giant = giant;
   c->sched.small = small;
-  c->sched.set = true;
   return CSO_OK;
 }
 
@@ -287,7 +286,6 @@ extern "C" int cso_autotune(cso_ctx* c, const cso_input* in, const cso_params* p
     for (int si = 0; si < 2 && rc == CSO_OK; ++si) {
       c->sched.giant = giants[gi];
       c->sched.small = smalls[si];
-      c->sched.set = true;
       double t = 1e30;
       for (int rep = 0; rep < 2 && rc == CSO_OK; ++rep) {
         rc = cso_find_groups(c, in, p, out);

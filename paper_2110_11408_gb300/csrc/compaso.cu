@@ -1873,8 +1873,7 @@ int level_run_batched(const LevelArgs& a, const LevelSchedule& sc, Workspace& ws
   const int occ_l = g_occ_l, occ_m = g_occ_m, occ_s = g_occ_s, occ_w = g_occ_w;
   const int sms = cso_sm_count();
   const int n_clusters = sms / CL_CS > 0 ? sms / CL_CS : 1;
-  k_seg_order<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(bin, rank, a.nseg, sc.set ? UINT_MAX : (unsigned)n_clusters,
-                                                       order, q);
+  k_seg_order<<<CL(cdiv(a.nseg, 1024)), 1024, 0, st>>>(bin, rank, a.nseg, sc.max_giants(n_clusters), order, q);
   CSO_CUDA(cudaGetLastError());
   const int nseg = a.nseg;
   // no tier can hold more groups than there are: grids never exceed nseg

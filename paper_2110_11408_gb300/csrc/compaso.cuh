@@ -49,8 +49,13 @@ struct LevelSchedule {
   int giant = 16384;
   int small = 64;
   int huge = CSO_HUGE_GROUP;  // above max(huge, giant): 16-CTA clusters
-  bool set = false;  // bins chosen by the caller or the autotuner: taken as they are
   int large() const { return giant / 16 > 512 ? giant / 16 : 512; }
+  // giants that go to clusters, largest first, where `clusters` run at a time:
+  // the default bins send no more (k_seg_order), any others all of them
+  unsigned max_giants(int clusters) const {
+    const LevelSchedule d;
+    return giant == d.giant && small == d.small ? (unsigned)clusters : ~0u;
+  }
 };
 
 int level_run(const LevelArgs& a, cudaStream_t st);

@@ -417,7 +417,7 @@ int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched) {
     return level_run_batched(L, sched, c->ws, st, c->side, c->side2, c->side3, c->fork, c->join, c->join2, c->join3);
   for (int i = 0; i < CSO_LEVEL_GRAPHS; ++i) {
     LevelGraph& G = c->graphs[i];
-    if (G.exec && G.giant == sched.giant && G.small == sched.small && G.huge == sched.huge && G.set == sched.set &&
+    if (G.exec && G.giant == sched.giant && G.small == sched.small && G.huge == sched.huge &&
         !memcmp(&G.args, &L, sizeof(LevelArgs))) {
       ++c->graph_hits;
       CSO_CUDA(cudaGraphLaunch(G.exec, st));
@@ -450,7 +450,6 @@ int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched) {
   G.giant = sched.giant;
   G.small = sched.small;
   G.huge = sched.huge;
-  G.set = sched.set;
   ++c->graph_captures;
   CSO_CUDA(cudaGraphLaunch(G.exec, st));
   return CSO_OK;

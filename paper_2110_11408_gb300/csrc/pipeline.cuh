@@ -28,7 +28,6 @@ struct ServedState;
 struct LevelGraph {
   LevelArgs args;
   int giant = 0, small = 0, huge = 0;
-  bool set = false;
   cudaGraphExec_t exec = nullptr;
 };
 #define CSO_LEVEL_GRAPHS 4
