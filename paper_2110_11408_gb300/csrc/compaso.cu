@@ -862,18 +862,23 @@ struct Best {
   int i;  // -1: none
 };
 
-__device__ __forceinline__ void best_of(Best& a, const Best& b) {  // key order: Sigma desc, id asc
-  if (b.i >= 0 && (a.i < 0 || b.sig > a.sig || (b.sig == a.sig && b.id < a.id))) a = b;
+// Key order: Sigma desc, id asc, and cell order where a caller's ids repeat (the
+// list of peaks is in no order).  pos: the group's peaks.
+__device__ __forceinline__ void best_of(Best& a, const Best& b, const int4* pos) {
+  if (b.i < 0) return;
+  bool before = a.i < 0 || b.sig > a.sig || (b.sig == a.sig && b.id < a.id);
+  if (a.i >= 0 && b.sig == a.sig && b.id == a.id) before = pos[b.i].w < pos[a.i].w;
+  if (before) a = b;
 }
 
-__device__ __forceinline__ void warp_best(Best& a) {
+__device__ __forceinline__ void warp_best(Best& a, const int4* pos) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
     Best b;
     b.sig = __shfl_xor_sync(0xffffffffu, a.sig, o);
     b.id = __shfl_xor_sync(0xffffffffu, a.id, o);
     b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-    best_of(a, b);
+    best_of(a, b, pos);
   }
 }
 
@@ -894,25 +899,26 @@ __device__ int next_nucleus(const LevelArgs& a, unsigned p0, int m, int cur, int
                             unsigned long long& gone, PickShared& K) {
   const long long anum2 = (long long)a.alpha_num * a.alpha_num, aden2 = (long long)a.alpha_den * a.alpha_den;
   const bool priv = private_flags(m);
+  const int4* pos = a.peaks.pos + p0;
   Best mine{0, 0, -1};
   for (int i = threadIdx.x, k = 0; i < m; i += blockDim.x, ++k) {
     if (cur >= 0) {
       if (priv ? gone >> k & 1 : a.peaks.out[p0 + i] != 0) continue;
-      if (i == cur || (__int128)aden2 * dist2(pc, a.peaks.pos[p0 + i]) < (__int128)anum2 * R2) {
+      if (i == cur || (__int128)aden2 * dist2(pc, pos[i]) < (__int128)anum2 * R2) {
         if (priv) gone |= 1ull << k;
         else a.peaks.out[p0 + i] = 1;
         continue;
       }
     }
-    best_of(mine, Best{a.peaks.sig[p0 + i], a.peaks.id[p0 + i], i});
+    best_of(mine, Best{a.peaks.sig[p0 + i], a.peaks.id[p0 + i], i}, pos);
   }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  warp_best(mine);
+  warp_best(mine, pos);
   if (lane == 0) K.w[w] = mine;
   __syncthreads();
   if (w == 0) {
     Best b = lane < (int)(blockDim.x >> 5) ? K.w[lane] : Best{0, 0, -1};
-    warp_best(b);
+    warp_best(b, pos);
     if (lane == 0) K.all = b;
   }
   __syncthreads();
@@ -1694,8 +1700,8 @@ __device__ void level_warp(const LevelArgs& a, const int seg) {
   int nn = 0;
   while (true) {
     Best b = k0;
-    best_of(b, k1);
-    warp_best(b);
+    best_of(b, k1, a.peaks.pos + p0);
+    warp_best(b, a.peaks.pos + p0);
     if (b.i < 0) break;
     const int src = b.i & 31;
     const bool hi = b.i >= 32;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) k_peak_near(PeakArgs a, const uint32_t* _
                   dz = (int)((unsigned)(p.z - q.z) << 11) >> 11;
         if (max(abs(dx), max(abs(dy), abs(dz))) > 16384) continue;  // b <= 16,384 grid units
         const uint32_t d = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
-        if (d >= a.b2 || (st[u] == sp && a.sid[t] > id)) continue;
+        if (d >= a.b2 || (st[u] == sp && a.sid[t] >= id)) continue;
         beat = t;
         todo = false;
       }
