@@ -86,30 +86,24 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
   return v;
 }
 
-// the group of every listed particle; block maxima of Sigma and id, one
-// atomic per block
+// the group of every listed particle; block maxima of the ids (the catalogue's
+// sort key), one atomic per block
 __global__ void __launch_bounds__(256) k_member_group(const uint32_t* __restrict__ dl, const int* __restrict__ root,
                                                       const uint32_t* __restrict__ gidx,
-                                                      const long long* __restrict__ sigma,
                                                       const uint64_t* __restrict__ sid, uint32_t* __restrict__ grp,
                                                       Meta* meta) {
   __shared__ unsigned long long sh[8];
   const unsigned nd = meta->n_dense;
   if (blockIdx.x * blockDim.x >= nd) return;
   const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long ms = 0, mid = 0;
+  unsigned long long mid = 0;
   if (k < nd) {
     const uint32_t s = dl[k];
     grp[k] = gidx[root[s]];
-    ms = (unsigned long long)sigma[s];
     mid = (unsigned long long)sid[s];
   }
-  ms = block_max_u64(ms, sh);
   mid = block_max_u64(mid, sh);
-  if (threadIdx.x == 0) {
-    atomicMax(&meta->sigma_max, ms);
-    atomicMax(&meta->id_max, mid);
-  }
+  if (threadIdx.x == 0) atomicMax(&meta->id_max, mid);
 }
 
 __global__ void k_seg_bounds32(const uint32_t* __restrict__ key, int m, int nseg, uint32_t* __restrict__ seg_off) {
@@ -483,9 +477,9 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   ALLOC(uint32_t, gidx, n);
   ALLOC(uint32_t, grp, n);
   RANK2_LAUNCH(k_member_list, n, st, root, N, gi.select, dl, gidx, rstat, rank2_tiles(n), ws.patience, meta);
-  k_member_group<<<G1(n)>>>(dl, root, gidx, sigma, sid, grp, meta);
+  k_member_group<<<G1(n)>>>(dl, root, gidx, sid, grp, meta);
   CSO_CUDA(cudaGetLastError());
-  // counters: dense particles, groups, sigma_max, id_max, bad
+  // counters: dense particles, groups, id_max, bad
   Meta hm;
   CSO_TRY(readback(c, meta, sizeof(Meta)));
   memcpy(&hm, c->pinned, sizeof(Meta));
@@ -498,13 +492,7 @@ int run_groups(cso_ctx* c, const cso_params* p, const GroupsIn& gi, Stages& S, M
   c->stats[1] = nd;
   c->stats[2] = G;
 
-  const int bits_id = bit_length_u64(hm.id_max);
-  const int bits_sig = nd ? bit_length_u64(hm.sigma_max - (unsigned long long)(p->T_L0 + 1)) : 0;
   const int bits_g = bit_length_u64(G > 0 ? (unsigned long long)(G - 1) : 0);
-  if (bits_id + bits_sig + bits_g > 128) {
-    cso_set_error("sort key of %d bits exceeds 128", bits_id + bits_sig + bits_g);
-    return CSO_ERR_ARG;
-  }
   ALLOC(uint32_t, dl2, nd);
   ALLOC(uint32_t, grp2, nd);
   ALLOC(uint32_t, seg1, G + 1);

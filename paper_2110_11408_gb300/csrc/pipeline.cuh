@@ -67,7 +67,7 @@ struct cso_ctx {
 int level_stage(cso_ctx* c, const LevelArgs& L, const LevelSchedule& sched);
 
 struct Meta {  // device counters read back by the host
-  unsigned long long sigma_max, id_max;
+  unsigned long long id_max;
   unsigned long long pairs, work1, work2;
   unsigned n_dense, n_groups;  // particles and groups taking part
   int bad;
