@@ -49,7 +49,7 @@ extern "C" {
                               clusters, 16-CTA clusters for huge groups (cso_set_huge_group), largest first, on four
                               concurrent streams */
 #define CSO_FLAG_TIMING 2u  /* record per-stage CUDA events (cso_stage_times) */
-/* with CSO_FLAG_BATCHED: each CompaSO level stage (size sort, work queue and
+/* with CSO_FLAG_BATCHED: each CompaSO level stage (size bins, work queue and
  * the six persistent tier kernels) is captured once as a CUDA graph and
  * replayed by later calls with identical launch arguments (a box of the same
  * shape in the same context); the rest of the step is launched directly (its

@@ -249,10 +249,10 @@ __device__ __forceinline__ uint32_t kern(int4 q, int xq, int yq, int zq, uint32_
 //     exact because the true d of every staged pair is below 2^32 (max_span
 //     is chosen on the host so that ((max_span + 2)^2 + 8) cell^2 < 2^32).
 // The multiply-adds (half rate: 6 cycles of a sub-core per 32 pairs) are what
-// is left as the bound of the shared walk: of 4.64 ms on the side-256 box
-// (16.8M particles) its inner loop takes 2.7, the set-up of the rows 0.7 and
-// the lane-by-lane walks the rest.  One query per lane: 5.36 ms, and 1.03
-// ms against 0.70 on the side-128 box.
+// is left as the bound of the shared walk: of 4.69 ms on a side-256 box (16.8M
+// particles; another draw of the same recipe, the benchmark's, takes 4.9) its inner
+// loop takes 2.7, the set-up of the rows 0.7 and the lane-by-lane walks the rest.
+// One query per lane: 5.36 ms, and 1.03 ms against 0.70 on a side-128 box.
 //
 // Blocks run heaviest first: a cost pass files each block under
 // floor(log2) of its warps' summed cell counts and the density launch takes
@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(R2_THREADS, 8) k_fof_lists(CellGrid g, const i
 // pair of a cell of up to 33 particles is tested and a big cell is joined by
 // a band of links around it.  The band joins almost every dense particle of
 // a big cell into one tree; the few it misses are handled one by one later.
-// A narrower band gains 2% where it suffices (16: 3.24 against 3.31 ms on a
+// A narrower band gains 2% where it suffices (16: FoF 3.24 against 3.31 ms on a
 // side-256 box) and costs 40% where it does not (16 on the benchmark's box of
 // that size: 4.64 against 3.30; 8 on the first: 4.54), by the cells whose trees
 // it leaves in pieces.
@@ -1275,7 +1275,7 @@ static void density_span(int nc, int* max_span, bool* is_signed) {
       break;
     }
   // finer boxes share wider: up to nine cells while the signed form holds
-  // (side 256: 4.70 -> 4.64 ms with spans of up to 8 instead of 2)
+  // (side 256: 1.3% of the pass with spans of up to 8 instead of 2)
   while (sp >= 2 && sp < 8 && ((sp + 3.0) * (sp + 3.0) + 8.0) * side * side < 2147483648.0) ++sp;
   *max_span = sp;
   *is_signed = ((sp + 2.0) * (sp + 2.0) + 8.0) * side * side < 2147483648.0;

@@ -1,4 +1,4 @@
-// Cell-grid kernels (cells.cu): binning, density, FoF, peak test.
+// Cell-grid kernels (cells.cu): binning, density, FoF.
 #pragma once
 #include "cso_internal.cuh"
 

@@ -741,7 +741,6 @@ __device__ __forceinline__ unsigned long long try_bound(int k, const PredConst& 
 }
 
 // ---------------------------------------------------------------------------
-// the choice of the next nucleus among a group's peaks
 // A try over so few tiles that every lane holds its members' distances: H tiles
 // a warp.  For the nuclei of the 16-CTA clusters, which are chosen one after the
 // other and mostly end in the first try, 25 tiles: 11.8 -> 7.5 us a try, and with
@@ -855,6 +854,8 @@ __device__ long long held_search(const int4* __restrict__ epos, int n, int4 pc, 
   return r == ~0ull ? -1 : (long long)r;
 }
 
+// ---------------------------------------------------------------------------
+// the choice of the next nucleus among a group's peaks
 // ---------------------------------------------------------------------------
 struct Best {
   long long sig;
@@ -1049,7 +1050,11 @@ __device__ void level_block(const LevelArgs& a, const int seg, BlockShared& B) {
 }
 
 // The plain schedule: a block per group, of 1024 threads for groups above
-// PLAIN_BIG members and of 256 for the rest (each launch skips the other's).
+// PLAIN_BIG members and of 256 for the rest (each launch skips the other's): the
+// groups above small_n, whose members are walked in tiles.  The line is not sharp;
+// both levels together with 512 / 1,024 / 2,048 / 4,096 / 8,192, ms: 262,144
+// particles 0.51 / 0.54 / 0.57 / 0.58 / 0.58, 2.1M 1.90 / 1.94 / 2.03 / 2.04 / 2.06,
+// 16.8M 4.43 / 4.41 / 4.45 / 4.45 / 4.43.
 constexpr int PLAIN_BIG = 2048;
 
 template <int NT>
@@ -1565,6 +1570,11 @@ __global__ void __launch_bounds__(1024) k_seg_bins(const uint32_t* __restrict__ 
 // 152 of them finish seventy sooner than 19 clusters do (side-256 box, 74
 // groups above 16,384: level 1 2.05 -> 1.78 ms, level 2 1.05 -> 0.80; the
 // side-128 box has ten and keeps them all on clusters, 0.39 against 0.43 ms).
+// Levels 1 and 2 of the side-400 box (64M particles) with GIANT_ALWAYS of 15, 16,
+// 17, 18 and 30: 8.66, 8.03, 7.68, 7.68 and 7.68 ms, of the side-256 box 2.47, 2.32,
+// 2.32, 2.32, 2.32: a group has to be several times the bound before a cluster's
+// eight SMs are worth its wait, and these boxes have no more groups of 2^17 than
+// clusters run at once.
 constexpr int GIANT_ALWAYS = 17;
 __global__ void __launch_bounds__(1024) k_seg_order(const int* __restrict__ bin, const uint32_t* __restrict__ rank,
                                                     int nseg, unsigned max_giants, uint32_t* __restrict__ order,
