@@ -122,7 +122,9 @@ typedef struct cso_halo {
 
 /* Input particles.  pos is int32[n][3] (x, y, z), ids is uint64[n]; both host
  * or both device memory (on_device).  The caller owns them and keeps them
- * alive until the call (or, for cso_submit, the ticket) completes.
+ * alive until the call (or, for cso_submit, the ticket) completes.  ids name the
+ * particles in the labels and break ties of equal kernel sums; where they repeat,
+ * equal keys are taken in the order of the cell table (z, y, x cell, x, input).
  * x_lo/x_hi: reserved for slab requests; set both to 0 for a whole box. */
 typedef struct cso_input {
   const int32_t* pos;
